@@ -80,51 +80,90 @@ __device__ __forceinline__ double dist_rn(const double a[3], const double b[3]) 
   return sqrt(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
 }
 
-constexpr int kScanTile = 256;
+// Near pairs of every row: their counts, or (counts == nullptr) the columns themselves at
+// row_ptr[i] in increasing order.
+// Bound by FP32 issue (n^2 distance tests, ~8 instructions each). A warp owns four rows and
+// its lanes take 32 consecutive columns, so the grid has n / 32 blocks (a thread per row
+// left all but n / 256 SMs idle) and a staged column serves four tests. FP64 runs at 1/64 of
+// the FP32 rate here: a pair is decided in FP32 where the FP32 coordinates' rounding cannot
+// change the outcome and only the rest takes the exact FP64 test. Both passes at n = 20480:
+// 6.87 -> 0.5 ms; at n = 1452: 1.22 -> 0.045 ms.
+constexpr int kScanTile = 256;   // columns staged at a time (one per thread)
+constexpr int kScanRows = 4;     // rows per warp
+constexpr int kScanBlockRows = kScanRows * kScanTile / 32;
 
-// Near pairs of every row: counts (cols == nullptr) or the columns themselves at
-// row_ptr[i] in increasing order. One thread per row; the columns' centroids and
-// diameters are staged through shared memory, first tested in FP32 with a margin, then
-// exactly in FP64.
 __global__ void __launch_bounds__(kScanTile)
 near_scan_kernel(Geometry g, int32_t* __restrict__ counts, const int32_t* __restrict__ row_ptr,
                  int32_t* __restrict__ cols) {
   __shared__ float4 sc[kScanTile];
   const int64_t n = g.n;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double xi[3] = {0.0, 0.0, 0.0};
-  double hi = 0.0;
-  if (i < n) {
-    for (int c = 0; c < 3; ++c) xi[c] = g.cx[c * n + i];
-    hi = g.diam[i];
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int64_t i0 = (int64_t)blockIdx.x * kScanBlockRows + warp * kScanRows;
+  float fx[kScanRows], fy[kScanRows], fz[kScanRows], fh[kScanRows], fm[kScanRows];
+  int32_t cnt[kScanRows];
+#pragma unroll
+  for (int r = 0; r < kScanRows; ++r) {
+    const int64_t i = i0 + r;
+    const bool ok = i < n;
+    fx[r] = ok ? g.cx32[i] : -3e18f;   // rows past the end: nothing is near
+    fy[r] = ok ? g.cx32[n + i] : -3e18f;
+    fz[r] = ok ? g.cx32[2 * n + i] : -3e18f;
+    fh[r] = ok ? (float)g.diam[i] : 0.f;
+    fm[r] = fabsf(fx[r]) + fabsf(fy[r]) + fabsf(fz[r]);
+    cnt[r] = 0;
   }
-  const float fx = (float)xi[0], fy = (float)xi[1], fz = (float)xi[2], fh = (float)hi;
-  int32_t cnt = 0;
-  const int64_t base = (cols && i < n) ? row_ptr[i] : 0;
   for (int64_t l0 = 0; l0 < n; l0 += kScanTile) {
     __syncthreads();
     const int64_t lt = l0 + threadIdx.x;
-    sc[threadIdx.x] = lt < n ? make_float4((float)g.cx[lt], (float)g.cx[n + lt],
-                                           (float)g.cx[2 * n + lt], (float)g.diam[lt])
-                             : make_float4(3e30f, 3e30f, 3e30f, 0.f);
+    sc[threadIdx.x] = lt < n ? make_float4(g.cx32[lt], g.cx32[n + lt], g.cx32[2 * n + lt],
+                                           (float)g.diam[lt])
+                             : make_float4(3e18f, 3e18f, 3e18f, 0.f);
     __syncthreads();
-    if (i >= n) continue;
-    const int lim = (int)(n - l0 < kScanTile ? n - l0 : kScanTile);
-    for (int t = 0; t < lim; ++t) {
-      const float4 c = sc[t];
-      const float dx = fx - c.x, dy = fy - c.y, dz = fz - c.z;
-      const float hm = fmaxf(fh, c.w);
-      if (dx * dx + dy * dy + dz * dz > 4.02f * hm * hm + 1e-30f) continue;
-      const int64_t l = l0 + t;
-      if (l == i) continue;
-      const double xl[3] = {g.cx[l], g.cx[n + l], g.cx[2 * n + l]};
-      if (dist_rn(xi, xl) < 2.0 * fmax(hi, g.diam[l])) {
-        if (cols) cols[base + cnt] = (int32_t)l;
-        ++cnt;
+#pragma unroll 2
+    for (int t = 0; t < kScanTile; t += 32) {
+      const float4 c = sc[t + lane];
+      float d2[kScanRows];
+      bool hit[kScanRows];
+      bool any = false;
+#pragma unroll
+      for (int r = 0; r < kScanRows; ++r) {
+        const float dx = fx[r] - c.x, dy = fy[r] - c.y, dz = fz[r] - c.z;
+        const float hm = fmaxf(fh[r], c.w);
+        d2[r] = dx * dx + dy * dy + dz * dz;
+        hit[r] = !(d2[r] > 4.02f * hm * hm + 1e-30f);
+        any |= hit[r];
+      }
+      if (!__any_sync(0xffffffffu, any)) continue;
+      const int64_t l = l0 + t + lane;
+      const float cm = fabsf(c.x) + fabsf(c.y) + fabsf(c.z);
+#pragma unroll
+      for (int r = 0; r < kScanRows; ++r) {
+        const int64_t i = i0 + r;
+        bool in = hit[r] && l < n && i < n && l != i;
+        if (in) {
+          // the FP32 distance is off by at most 2^-23 sqrt(3) of the coordinates' size and a
+          // few ulps of itself; decided here unless the threshold lies within twice that
+          const float d = sqrtf(d2[r]), lim = 2.f * fmaxf(fh[r], c.w);
+          const float slack = 4.2e-7f * (fm[r] + cm) + 2e-6f * lim;
+          if (d > lim + slack) {
+            in = false;
+          } else if (!(d < lim - slack)) {
+            const double xi[3] = {g.cx[i], g.cx[n + i], g.cx[2 * n + i]};
+            const double xl[3] = {g.cx[l], g.cx[n + l], g.cx[2 * n + l]};
+            in = dist_rn(xi, xl) < 2.0 * fmax(g.diam[i], g.diam[l]);
+          }
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, in);
+        if (!counts && in)
+          cols[row_ptr[i] + cnt[r] + __popc(mask & ((1u << lane) - 1u))] = (int32_t)l;
+        cnt[r] += __popc(mask);
       }
     }
   }
-  if (i < n && !cols) counts[i] = cnt;
+  if (counts)
+#pragma unroll
+    for (int r = 0; r < kScanRows; ++r)
+      if (lane == 0 && i0 + r < n) counts[i0 + r] = cnt[r];
 }
 
 // The 8 x 8 rule's frame for panel l seen from x: collapsed vertex a (nearest x), the two
@@ -911,7 +950,7 @@ bem_status ensure_near(bem_ctx* ctx, cudaStream_t s) {
     }
     ctx->near_cap_n = n + 1;
   }
-  const unsigned blocks = (unsigned)((n + kScanTile - 1) / kScanTile);
+  const unsigned blocks = (unsigned)((n + kScanBlockRows - 1) / kScanBlockRows);
   near_scan_kernel<<<blocks, kScanTile, 0, s>>>(ctx->geo, ctx->d_near_ptr, nullptr, nullptr);
   ctx->launches++;
   std::vector<int32_t> h(n + 1);
@@ -942,9 +981,11 @@ bem_status ensure_near(bem_ctx* ctx, cudaStream_t s) {
                                        cudaMemcpyHostToDevice, s),
                   "near field copy");
   if (st != BEM_OK) return st;
-  near_scan_kernel<<<blocks, kScanTile, 0, s>>>(ctx->geo, nullptr, ctx->d_near_ptr,
-                                                ctx->d_near_cols);
-  ctx->launches++;
+  if (total > 0) {   // without pairs there is no column array, and nothing to write
+    near_scan_kernel<<<blocks, kScanTile, 0, s>>>(ctx->geo, nullptr, ctx->d_near_ptr,
+                                                  ctx->d_near_cols);
+    ctx->launches++;
+  }
   st = cuda_check(ctx, cudaGetLastError(), "near field kernels");
   if (st == BEM_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "near field build");
   if (st != BEM_OK) return st;

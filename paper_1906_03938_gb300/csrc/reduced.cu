@@ -20,7 +20,7 @@
 #include <vector>
 
 #include "internal.h"
-#include "small_eig.h"
+#include "small_eig_block.cuh"
 
 namespace bem {
 namespace {
@@ -281,12 +281,28 @@ __global__ void reduced_residual_kernel(const double2* __restrict__ Bhat, const 
   }
 }
 
+// Eigenvalues w and unit eigenvectors V of the p x p Rayleigh-Ritz matrix (one block).
 __global__ void small_eig_kernel(int m, double2* A, double2* w, double2* V, double2* Z,
                                  int* status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int rc = small::eig(m, reinterpret_cast<small::zc*>(A), reinterpret_cast<small::zc*>(w),
-                            reinterpret_cast<small::zc*>(V), reinterpret_cast<small::zc*>(Z));
-  if (rc != 0) atomicOr(status, kStatusNonFinite);
+  const int rc = small::eig_block(m, reinterpret_cast<small::zc*>(A),
+                                  reinterpret_cast<small::zc*>(w),
+                                  reinterpret_cast<small::zc*>(V),
+                                  reinterpret_cast<small::zc*>(Z));
+  if (rc != 0 && threadIdx.x == 0) atomicOr(status, kStatusNonFinite);
+}
+
+bem_status launch_small_eig(bem_ctx* ctx, int m, double2* A, double2* w, double2* V, double2* Z,
+                            cudaStream_t s) {
+  const size_t sm = small::eig_smem(m);
+  if (sm > 48 * 1024) {
+    const bem_status st = cuda_check(
+        ctx, cudaFuncSetAttribute(small_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sm), "small eigenproblem attribute");
+    if (st != BEM_OK) return st;
+  }
+  small_eig_kernel<<<1, small::eig_threads(m), sm, s>>>(m, A, w, V, Z, ctx->d_status);
+  ctx->launches++;
+  return cuda_check(ctx, cudaGetLastError(), "small eigenproblem");
 }
 
 // ---- Chebyshev variant (Eq. Chebyshev, Eq. sc1_chebyshev_red, Algorithm 2's setting) ----
@@ -610,8 +626,7 @@ extern "C" bem_status bem_solve_reduced(bem_ctx* ctx, const double* Bhat_dev, in
                                            nullptr, reinterpret_cast<double*>(G), s),
                       "reduced rayleigh-ritz");
       if (st != BEM_OK) return st;
-      small_eig_kernel<<<1, 32, 0, s>>>(p, G, mu, Vs, Zm, ctx->d_status);
-      ctx->launches++;
+      if ((st = launch_small_eig(ctx, p, G, mu, Vs, Zm, s)) != BEM_OK) return st;
       // Y = U Vs diag(1/mu): the y-parts of the Ritz vectors (U = S^{-1} C W)
       if (launch_zgemm(ctx, nu, p, p, reinterpret_cast<double*>(U), nu,
                        reinterpret_cast<double*>(Vs), p, Y_dev, nu, s) != cudaSuccess)
@@ -874,8 +889,7 @@ extern "C" bem_status bem_solve_chebyshev(bem_ctx* ctx, const double* B_dev, int
                                            nullptr, reinterpret_cast<double*>(op.Sm), s),
                       "chebyshev rayleigh-ritz");
       if (st != BEM_OK) return st;
-      small_eig_kernel<<<1, 32, 0, s>>>(p, op.Sm, op.mu, op.Vs, op.Zm, ctx->d_status);
-      ctx->launches++;
+      if ((st = launch_small_eig(ctx, p, op.Sm, op.mu, op.Vs, op.Zm, s)) != BEM_OK) return st;
       // y-parts of the Ritz vectors: the first block of W Vs (v_0 = T_0 y = y)
       if (launch_zgemm(ctx, nu, p, p, reinterpret_cast<double*>(W), rows,
                        reinterpret_cast<double*>(op.Vs), p, Y_dev, nu, s) != cudaSuccess)

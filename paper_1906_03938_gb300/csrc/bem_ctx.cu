@@ -3,9 +3,11 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
+#include "expand64.h"
 #include "internal.h"
 
 namespace bem {
@@ -31,6 +33,16 @@ bem_status ensure_scratch(bem_ctx* ctx, size_t bytes) {
   }
   ctx->scratch_bytes = bytes;
   return BEM_OK;
+}
+
+bool scratch_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s) {
+  if (bytes <= ctx->scratch_bytes) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  return ensure_scratch(ctx, bytes) == BEM_OK;
 }
 
 bem_status ensure_small(bem_ctx* ctx, size_t bytes) {
@@ -495,14 +507,24 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
     return project_hmatrix(ctx, V_dev, ldv, nu, Bhat_dev, AV_dev, s);
   st0 = ensure_self64(ctx, s);
   if (st0 != BEM_OK) return st0;
-  double* Y = AV_dev;
-  if (!Y) {
-    bem_status st = ensure_scratch(ctx, (size_t)N * n * nu * 2 * sizeof(double));
+  // one evaluation expanded over the nodes where that costs less than one per node, and its
+  // workspace can be had (a stream capture allocates nothing)
+  const size_t y_bytes = AV_dev ? 0 : (size_t)N * n * nu * 2 * sizeof(double);
+  ExpandPlan ex = expand_plan(ctx, N, ctx->con.c_re, ctx->con.c_im, std::max(ctx->con.a, ctx->con.b),
+                              nu, true, false);
+  if (ex.use) ex.use = scratch_ready(ctx, y_bytes + ex.bytes, s);
+  if (!ex.use) {
+    bem_status st = ensure_scratch(ctx, y_bytes);
     if (st != BEM_OK) return st;
-    Y = ctx->d_scratch;
   }
+  double* Y = AV_dev ? AV_dev : ctx->d_scratch;
   timing_begin(ctx, s);
-  bem_status st = cuda_check(ctx, launch_apply_fp64(ctx, V_dev, ldv, nu, Y, s), "apply kernel");
+  bem_status st = cuda_check(
+      ctx,
+      ex.use ? expand_apply_nodes(ctx, ex, V_dev, ldv, nu, Y,
+                                  reinterpret_cast<char*>(ctx->d_scratch) + y_bytes, s)
+             : launch_apply_fp64(ctx, V_dev, ldv, nu, Y, s),
+      "apply kernel");
   timing_end(ctx, s);
   if (st != BEM_OK) return st;
   if (near_active(ctx)) {

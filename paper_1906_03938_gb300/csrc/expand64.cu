@@ -1,0 +1,485 @@
+// FP64 products with A(k) at many wavenumbers from one evaluation of the operator.
+//
+// Every entry is A_il(k) = sum_q w_q e^{i k r_q} / r_q with r in [0, R]. About a centre c,
+// e^{i k r} = e^{i c r} e^{i (k - c) r}, and on [0, R] the second factor is a Chebyshev series
+// in x = 2 r / R - 1 whose terms fall like (|k - c| R / 4)^m / m!: M = 12 .. 20 terms give
+// FP64 rounding for a contour of radius ~1 about a body of diameter ~2, whatever the number
+// of wavenumbers. So
+//     A(k_j) = sum_m a_m(k_j) G_m,   G_m,il = sum_q w_q e^{i c r_q} / r_q T_m(x_q),
+// and A(k_j) X = sum_m a_m(k_j) (G_m X): one evaluation (a sine, cosine and root per point)
+// and M matrix products in the place of N of each. The general operator
+// c_G G + c_H (1/2 I + K) adds a second family of moments, H_m with the weight
+// w_q s_q / r_q, s = (y - x).n / r^2, and the coefficients of (i k r - 1) e^{i (k - c) r}; the
+// k-derivative only changes the coefficients.
+//
+// Bound by the FP64 pipe (1/64 of the FP32 rate on this part): per entry 7 (60 + 3 M) FP64
+// operations of evaluation and 3 M nu of products against N (7 x 77 + 4 nu) for the direct
+// form; the moments' round trip through memory (32 bytes a moment) is ~1 % of that. Measured:
+// the FP64 step of the 768-panel cube (N = 32, nu = 64) 32.2 -> 8.8 ms, residuals of 8 vectors
+// on 5120 panels 286 -> 80 ms (258 -> 52 in the operator), with the same or a smaller error
+// against 64-bit references.
+#include <math.h>
+
+#include <algorithm>
+
+#include "expand64.h"
+
+namespace bem {
+namespace {
+
+constexpr int kMaxTerms = 32;      // series length the evaluation kernel is built for
+constexpr int kCoefPoints = 64;    // Chebyshev points of the coefficients' quadrature
+constexpr int kRowsE = 128;        // rows per block of the evaluation (a thread each)
+constexpr int kColsE = 8;          // columns per block of the evaluation
+constexpr size_t kMomentBytes = (size_t)1 << 30;   // moments held at a time
+constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
+
+// a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
+// wavenumber k_j, times the operator's coefficient of the family.
+__global__ void expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R,
+                                   int M, int fams, int first_fam, bool deriv, OpCoef op,
+                                   double2* __restrict__ a) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= fams * nk * M) return;
+  const int m = t % M, j = (t / M) % nk, f = first_fam + t / (M * nk);
+  const double2 kj = k[j];
+  const double dr = kj.x - c.x, di = kj.y - c.y;
+  double2 s = make_double2(0.0, 0.0);
+  for (int q = 0; q < kCoefPoints; ++q) {
+    const double u = (q + 0.5) / kCoefPoints;
+    const double r = 0.5 * R * (cospi(u) + 1.0);
+    double sn, cs;
+    sincos(dr * r, &sn, &cs);
+    const double e = exp(-di * r);
+    // the family's factor at r: 1 or (i k r - 1), and their k-derivatives i r and -k r^2
+    double gr, gi;
+    if (f == 0) {
+      gr = deriv ? 0.0 : 1.0;
+      gi = deriv ? r : 0.0;
+    } else {
+      gr = deriv ? -kj.x * r * r : -kj.y * r - 1.0;
+      gi = deriv ? -kj.y * r * r : kj.x * r;
+    }
+    const double w = e * cospi(m * u);
+    s.x += w * (cs * gr - sn * gi);
+    s.y += w * (cs * gi + sn * gr);
+  }
+  const double sc = (m == 0 ? 1.0 : 2.0) / kCoefPoints;
+  const double or_ = f == 0 ? op.cgr : op.chr, oi = f == 0 ? op.cgi : op.chi;
+  a[t] = make_double2(sc * (s.x * or_ - s.y * oi), sc * (s.x * oi + s.y * or_));
+}
+
+// Moments of the columns [l0, l0 + kc): G[f M + m][l - l0][i] (i fastest). One thread per row;
+// the block's columns' geometry is staged in shared memory and read by broadcast. The
+// diagonal is zero (the self terms are added in closed form).
+template <int MT, bool kG, bool kH>
+__global__ void __launch_bounds__(kRowsE)
+expand_moments_kernel(Geometry g, double2 c, double two_over_R, int M, int64_t l0, int kc,
+                      double2* __restrict__ G) {
+  __shared__ double sq[kColsE][7][4];
+  __shared__ double sn3[kColsE][3];
+  const int64_t n = g.n;
+  const int64_t i = (int64_t)blockIdx.x * kRowsE + threadIdx.x;
+  const int c0 = blockIdx.y * kColsE;
+  const int nc = min(kColsE, kc - c0);
+  for (int t = threadIdx.x; t < nc * 7; t += kRowsE) {
+    const int cc = t / 7, q = t % 7;
+    const int64_t l = l0 + c0 + cc;
+    sq[cc][q][0] = g.qp[q * n + l];
+    sq[cc][q][1] = g.qp[(7 + q) * n + l];
+    sq[cc][q][2] = g.qp[(14 + q) * n + l];
+    sq[cc][q][3] = g.qw[q * n + l];
+  }
+  if (kH)
+    for (int t = threadIdx.x; t < nc * 3; t += kRowsE)
+      sn3[t / 3][t % 3] = g.nrm[(t % 3) * n + l0 + c0 + t / 3];
+  __syncthreads();
+  if (i >= n) return;
+  const double xi = g.cx[i], yi = g.cx[n + i], zi = g.cx[2 * n + i];
+  constexpr int F = (kG ? 1 : 0) + (kH ? 1 : 0);
+  for (int cc = 0; cc < nc; ++cc) {
+    const int64_t l = l0 + c0 + cc;
+    double ar[F][MT], ai[F][MT];
+#pragma unroll
+    for (int f = 0; f < F; ++f)
+#pragma unroll
+      for (int m = 0; m < MT; ++m) ar[f][m] = ai[f][m] = 0.0;
+    if (l != i) {
+#pragma unroll 1
+      for (int q = 0; q < 7; ++q) {
+        const double dx = sq[cc][q][0] - xi, dy = sq[cc][q][1] - yi, dz = sq[cc][q][2] - zi;
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        const double ri = rsqrt(r2);
+        double r = r2 * ri;
+        r = fma(0.5 * ri, fma(-r, r, r2), r);   // sqrt(r2) to its last bit or so
+        double s, co;
+        sincos(c.x * r, &s, &co);
+        double w = sq[cc][q][3] * ri;
+        if (c.y != 0.0) w *= exp(-c.y * r);
+        const double x = fma(r, two_over_R, -1.0), x2 = 2.0 * x;
+        double br[F], bi[F];
+        if (kG) {
+          br[0] = w * co;
+          bi[0] = w * s;
+        }
+        if (kH) {
+          const double h = w * ri * ri *
+                           (dx * sn3[cc][0] + dy * sn3[cc][1] + dz * sn3[cc][2]);
+          br[F - 1] = h * co;
+          bi[F - 1] = h * s;
+        }
+        double t0 = 1.0, t1 = x;
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+#pragma unroll
+          for (int f = 0; f < F; ++f) {
+            ar[f][m] = fma(br[f], t0, ar[f][m]);
+            ai[f][m] = fma(bi[f], t0, ai[f][m]);
+          }
+          const double t2 = fma(x2, t1, -t0);
+          t0 = t1;
+          t1 = t2;
+        }
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < F; ++f)
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+        if (m < M)
+          G[((int64_t)(f * M + m) * kc + c0 + cc) * n + i] = make_double2(ar[f][m], ai[f][m]);
+  }
+}
+
+constexpr int kTM = 32;    // rows of a product tile
+constexpr int kTK = 16;    // columns of the moments staged at a time
+constexpr int kThreadsM = 128;
+
+// Yp[split][s] (+)= G_s[:, ks] X[l0 + ks, :] for slot s = blockIdx.z % S and its share ks of
+// the kc columns. Three real products per complex term, as the Gram kernel's. FP64-bound: a
+// thread's 2 x (TN / 8) outputs take 6 .. 24 FP64 operations per k against 9 .. 18 8-byte
+// shared-memory reads at 1/16 of their cost.
+template <int TN>
+__global__ void __launch_bounds__(kThreadsM)
+expand_product_kernel(const double2* __restrict__ G, int64_t n, int kc, int S, int splits,
+                      const double2* __restrict__ X, int64_t ldx, int nu, int64_t l0, bool add,
+                      double2* __restrict__ Yp) {
+  __shared__ double ar[kTK][kTM], ai[kTK][kTM], as[kTK][kTM];
+  __shared__ double br[kTK][TN + 1], bi[kTK][TN + 1], bs[kTK][TN + 1];
+  constexpr int kCT = TN / 8;   // columns per thread (16 row pairs x 8 column groups)
+  const int s = blockIdx.z % S, split = blockIdx.z / S;
+  const int64_t i0 = (int64_t)blockIdx.x * kTM;
+  const int j0 = blockIdx.y * TN;
+  const int kb = (int)((int64_t)kc * split / splits), ke = (int)((int64_t)kc * (split + 1) / splits);
+  const int tid = threadIdx.x, tr = tid % 16, tc = tid / 16;
+  const double2* Gs = G + (int64_t)s * kc * n;
+  double s1[2][kCT], s2[2][kCT], s3[2][kCT];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < kCT; ++b) s1[a][b] = s2[a][b] = s3[a][b] = 0.0;
+  for (int k0 = kb; k0 < ke; k0 += kTK) {
+    __syncthreads();
+    for (int t = tid; t < kTK * kTM; t += kThreadsM) {
+      const int r = t % kTM, k = t / kTM;
+      const double2 v = (k0 + k < ke && i0 + r < n) ? Gs[(int64_t)(k0 + k) * n + i0 + r]
+                                                    : make_double2(0.0, 0.0);
+      ar[k][r] = v.x;
+      ai[k][r] = v.y;
+      as[k][r] = v.x + v.y;
+    }
+    for (int t = tid; t < kTK * TN; t += kThreadsM) {
+      const int k = t % kTK, cl = t / kTK;
+      const double2 v = (k0 + k < ke && j0 + cl < nu) ? X[(int64_t)(j0 + cl) * ldx + l0 + k0 + k]
+                                                      : make_double2(0.0, 0.0);
+      br[k][cl] = v.x;
+      bi[k][cl] = v.y;
+      bs[k][cl] = v.x + v.y;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kTK; ++k) {
+      double a1[2], a2[2], a3[2];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        a1[a] = ar[k][tr + 16 * a];
+        a2[a] = ai[k][tr + 16 * a];
+        a3[a] = as[k][tr + 16 * a];
+      }
+#pragma unroll
+      for (int b = 0; b < kCT; ++b) {
+        const int cl = tc + 8 * b;
+        const double b1 = br[k][cl], b2 = bi[k][cl], b3 = bs[k][cl];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          s1[a][b] = fma(a1[a], b1, s1[a][b]);
+          s2[a][b] = fma(a2[a], b2, s2[a][b]);
+          s3[a][b] = fma(a3[a], b3, s3[a][b]);
+        }
+      }
+    }
+  }
+  double2* Ys = Yp + ((int64_t)split * S + s) * n * nu;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int64_t i = i0 + tr + 16 * a;
+    if (i >= n) continue;
+#pragma unroll
+    for (int b = 0; b < kCT; ++b) {
+      const int cl = j0 + tc + 8 * b;
+      if (cl >= nu) continue;
+      double2 y = make_double2(s1[a][b] - s2[a][b], s3[a][b] - s1[a][b] - s2[a][b]);
+      if (add) {
+        const double2 o = Ys[(int64_t)cl * n + i];
+        y.x += o.x;
+        y.y += o.y;
+      }
+      Ys[(int64_t)cl * n + i] = y;
+    }
+  }
+}
+
+// Yp[0][s] = sum over the splits, in order.
+__global__ void expand_sum_kernel(int64_t count, int splits, double2* __restrict__ Yp) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= count) return;
+  double2 s = Yp[t];
+  for (int q = 1; q < splits; ++q) {
+    const double2 v = Yp[(int64_t)q * count + t];
+    s.x += v.x;
+    s.y += v.y;
+  }
+  Yp[t] = s;
+}
+
+constexpr int kNodesC = 8;   // wavenumbers per thread of the combination
+
+// Y_j = sum_s a_s(k_j) Y_s + self_j V (the self terms of the table, node-major), 8 nodes a thread.
+__global__ void __launch_bounds__(128)
+expand_nodes_kernel(const double2* __restrict__ Ys, int64_t n, int nu, int M, int fams, int N,
+                    const double2* __restrict__ a, const double2* __restrict__ self,
+                    const double2* __restrict__ V, int64_t ldv, double2* __restrict__ Y) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= n * nu) return;
+  const int64_t i = t % n;
+  const int cl = (int)(t / n);
+  const int j0 = blockIdx.y * kNodesC;
+  const double2 v = V[(int64_t)cl * ldv + i];
+  double2 acc[kNodesC];
+#pragma unroll
+  for (int u = 0; u < kNodesC; ++u) {
+    const int j = min(j0 + u, N - 1);
+    const double2 d = self[(int64_t)j * n + i];
+    acc[u] = make_double2(d.x * v.x - d.y * v.y, d.x * v.y + d.y * v.x);
+  }
+  for (int f = 0; f < fams; ++f)
+    for (int m = 0; m < M; ++m) {
+      const double2 y = Ys[(int64_t)(f * M + m) * n * nu + t];
+#pragma unroll
+      for (int u = 0; u < kNodesC; ++u) {
+        const double2 w = a[((int64_t)f * N + min(j0 + u, N - 1)) * M + m];
+        acc[u].x = fma(w.x, y.x, fma(-w.y, y.y, acc[u].x));
+        acc[u].y = fma(w.x, y.y, fma(w.y, y.x, acc[u].y));
+      }
+    }
+#pragma unroll
+  for (int u = 0; u < kNodesC; ++u)
+    if (j0 + u < N) Y[(int64_t)(j0 + u) * n * nu + t] = acc[u];
+}
+
+// R_c = sum_s a_s(k_c) Y_s,c + R_c x_c (R holds the self terms at k_c).
+__global__ void expand_columns_kernel(const double2* __restrict__ Ys, int64_t n, int m, int M,
+                                      int fams, const double2* __restrict__ a,
+                                      const double2* __restrict__ X, int64_t ldx,
+                                      double2* __restrict__ R) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= n * m) return;
+  const int64_t i = t % n;
+  const int c = (int)(t / n);
+  const double2 x = X[(int64_t)c * ldx + i], d = R[t];
+  double2 acc = make_double2(d.x * x.x - d.y * x.y, d.x * x.y + d.y * x.x);
+  for (int f = 0; f < fams; ++f)
+    for (int q = 0; q < M; ++q) {
+      const double2 y = Ys[(int64_t)(f * M + q) * n * m + t];
+      const double2 w = a[((int64_t)f * m + c) * M + q];
+      acc.x = fma(w.x, y.x, fma(-w.y, y.y, acc.x));
+      acc.y = fma(w.x, y.y, fma(w.y, y.x, acc.y));
+    }
+  R[t] = acc;
+}
+
+using MomentKernel = void (*)(Geometry, double2, double, int, int64_t, int, double2*);
+
+template <bool kG, bool kH>
+MomentKernel moment_kernel(int M) {
+  if (M <= 1) return expand_moments_kernel<1, kG, kH>;
+  if (M <= 8) return expand_moments_kernel<8, kG, kH>;
+  if (M <= 10) return expand_moments_kernel<10, kG, kH>;
+  if (M <= 12) return expand_moments_kernel<12, kG, kH>;
+  if (M <= 13) return expand_moments_kernel<13, kG, kH>;
+  if (M <= 14) return expand_moments_kernel<14, kG, kH>;
+  if (M <= 15) return expand_moments_kernel<15, kG, kH>;
+  if (M <= 16) return expand_moments_kernel<16, kG, kH>;
+  if (M <= 17) return expand_moments_kernel<17, kG, kH>;
+  if (M <= 18) return expand_moments_kernel<18, kG, kH>;
+  if (M <= 20) return expand_moments_kernel<20, kG, kH>;
+  if (M <= 24) return expand_moments_kernel<24, kG, kH>;
+  return expand_moments_kernel<kMaxTerms, kG, kH>;
+}
+
+// Largest distance between two points of the mesh, from above: the smaller of its box's
+// diagonal and twice the largest distance of a vertex from the box's centre.
+double mesh_reach(bem_ctx* ctx) {
+  if (ctx->reach_version == ctx->mesh_version) return ctx->reach;
+  double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  const std::vector<double>& p = ctx->h_xyz;
+  for (size_t t = 0; t < p.size(); ++t) {
+    lo[t % 3] = std::min(lo[t % 3], p[t]);
+    hi[t % 3] = std::max(hi[t % 3], p[t]);
+  }
+  double far2 = 0.0, diag2 = 0.0;
+  for (int c = 0; c < 3; ++c) diag2 += (hi[c] - lo[c]) * (hi[c] - lo[c]);
+  for (size_t t = 0; t + 2 < p.size(); t += 3) {
+    double d2 = 0.0;
+    for (int c = 0; c < 3; ++c) {
+      const double d = p[t + c] - 0.5 * (lo[c] + hi[c]);
+      d2 += d * d;
+    }
+    far2 = std::max(far2, d2);
+  }
+  ctx->reach = std::min(sqrt(diag2), 2.0 * sqrt(far2)) * (1.0 + 1e-12);
+  ctx->reach_version = ctx->mesh_version;
+  return ctx->reach;
+}
+
+// Terms after which the series of e^{i d r}, |d| <= dmax, on [0, R] is below 2^-56 of the
+// function's size (coefficients bounded by 2 (kappa / 2)^m / m!, kappa = dmax R / 2); the
+// factors r and r^2 of the other families cost two more.
+int series_terms(double dmax, double R) {
+  const double h = 0.25 * dmax * R;
+  if (!(h < 8.0)) return kMaxTerms + 1;
+  double t = 2.0;
+  int m = 0;
+  while (t > 0x1p-56 && m <= kMaxTerms) {
+    ++m;
+    t *= h / m;
+  }
+  return m;   // h = 0: the constant alone
+}
+
+}  // namespace
+
+ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dmax, int ncols,
+                       bool nodes, bool deriv) {
+  ExpandPlan p;
+  const OpCoef& op = ctx->op;
+  const bool hasG = op.cgr != 0.0 || op.cgi != 0.0, hasH = op.chr != 0.0 || op.chi != 0.0;
+  const int64_t n = ctx->geo.n;
+  p.R = mesh_reach(ctx);
+  if (!(p.R > 0.0) || !isfinite(p.R)) return p;
+  p.M = series_terms(dmax, p.R);
+  if (p.M > 1 && (hasH || deriv)) p.M += 2;
+  if (p.M == 1 && (hasH || deriv)) p.M = 3;   // factors 1, r, r^2
+  if (p.M < 1 || p.M > kMaxTerms) return p;
+  p.first = hasG ? 0 : 1;
+  p.fams = (hasG ? 1 : 0) + (hasH ? 1 : 0);
+  p.S = p.fams * p.M;
+  p.c = make_double2(c_re, c_im);
+  // FP64 operations per entry of the two forms; the smaller wins. Projection at n = 768,
+  // nu = 64: direct 5.56 ms at N = 5, expanded 5.41 ms at N = 6 and 5.48 ms at N = 16; at
+  // nu = 128: direct 10.2 ms at N = 6, expanded 8.4 ms at N = 7, 9.3 ms at N = 16. Residuals on
+  // 1280 panels: 5.9 ms for 2 to 8 columns (one product tile).
+  const int tn = ncols <= 8 ? 8 : 32;
+  const double padded = (double)((ncols + tn - 1) / tn * tn);
+  const double expand = 7.0 * (60.0 + (1.0 + 2.0 * p.fams) * p.M) + 3.0 * p.S * padded;
+  const double direct = nodes ? nk * (7.0 * 77.0 + 4.0 * ncols) : ncols * (7.0 * 77.0 + 4.0);
+  if (!(expand < direct)) return p;
+  // workspace: coefficients, moments of kc columns, slot products (per k split)
+  p.kc = (int)std::min<int64_t>(n, std::max<int64_t>(32, (int64_t)(kMomentBytes / ((size_t)p.S * n * 16))));
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  const int64_t tiles = (n + kTM - 1) / kTM * ((ncols + tn - 1) / tn) * p.S;
+  // enough blocks for eight small blocks on each SM, at least 64 columns each
+  p.splits = (int)std::max<int64_t>(1, std::min<int64_t>(8 * (int64_t)std::max(1, sms) / tiles, p.kc / 64));
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  p.coef_off = 0;
+  p.mom_off = up((size_t)p.S * nk * 16);
+  p.y_off = p.mom_off + up((size_t)p.S * p.kc * n * 16);
+  p.bytes = p.y_off + up((size_t)p.splits * p.S * n * ncols * 16);
+  p.use = p.bytes <= kMaxWork;
+  return p;
+}
+
+namespace {
+
+// The slot products Y_s = G_s X into the workspace.
+void expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const double* k_dev,
+                     const double* X, int64_t ldx, int ncols, bool deriv, char* work,
+                     cudaStream_t s) {
+  const int64_t n = ctx->geo.n;
+  double2* a = reinterpret_cast<double2*>(work + p.coef_off);
+  double2* G = reinterpret_cast<double2*>(work + p.mom_off);
+  double2* Yp = reinterpret_cast<double2*>(work + p.y_off);
+  const int total = p.S * nk;
+  expand_coef_kernel<<<(total + 63) / 64, 64, 0, s>>>(reinterpret_cast<const double2*>(k_dev), nk,
+                                                     p.c, p.R, p.M, p.fams, p.first, deriv,
+                                                     ctx->op, a);
+  MomentKernel mk = p.fams == 2 ? moment_kernel<true, true>(p.M)
+                                : (p.first == 0 ? moment_kernel<true, false>(p.M)
+                                                : moment_kernel<false, true>(p.M));
+  ctx->launches++;
+  for (int64_t l0 = 0; l0 < n; l0 += p.kc) {
+    const int kc = (int)std::min<int64_t>(p.kc, n - l0);
+    const dim3 ge((unsigned)((n + kRowsE - 1) / kRowsE), (unsigned)((kc + kColsE - 1) / kColsE));
+    mk<<<ge, kRowsE, 0, s>>>(ctx->geo, p.c, 2.0 / p.R, p.M, l0, kc, G);
+    const int tn = ncols <= 8 ? 8 : 32;
+    const dim3 gp((unsigned)((n + kTM - 1) / kTM), (unsigned)((ncols + tn - 1) / tn),
+                  (unsigned)(p.S * p.splits));
+    auto* pk = tn == 8 ? expand_product_kernel<8> : expand_product_kernel<32>;
+    pk<<<gp, kThreadsM, 0, s>>>(G, n, kc, p.S, p.splits, reinterpret_cast<const double2*>(X), ldx,
+                                ncols, l0, l0 > 0, Yp);
+    ctx->launches += 2;
+  }
+  if (p.splits > 1) {
+    const int64_t count = (int64_t)p.S * n * ncols;
+    expand_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, p.splits, Yp);
+    ctx->launches++;
+  }
+}
+
+}  // namespace
+
+cudaError_t expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
+                               int nu, double* Y, void* work, cudaStream_t s) {
+  char* w = static_cast<char*>(work);
+  const int N = ctx->con.N;
+  const int64_t n = ctx->geo.n;
+  expand_products(ctx, p, N, ctx->con.z, V, ldv, nu, false, w, s);
+  const dim3 g((unsigned)((n * nu + 127) / 128), (unsigned)((N + kNodesC - 1) / kNodesC));
+  expand_nodes_kernel<<<g, 128, 0, s>>>(reinterpret_cast<const double2*>(w + p.y_off), n, nu, p.M,
+                                        p.fams, N, reinterpret_cast<const double2*>(w + p.coef_off),
+                                        reinterpret_cast<const double2*>(ctx->con.self),
+                                        reinterpret_cast<const double2*>(V), ldv,
+                                        reinterpret_cast<double2*>(Y));
+  ctx->launches++;
+  return cudaGetLastError();
+}
+
+cudaError_t expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
+                                 const double* X, int64_t ldx, double* R, bool deriv, void* work,
+                                 cudaStream_t s) {
+  char* w = static_cast<char*>(work);
+  const int64_t n = ctx->geo.n;
+  const cudaError_t e = launch_self_at(ctx, m, lam_dev, R, deriv, s);
+  if (e != cudaSuccess) return e;
+  expand_products(ctx, p, m, lam_dev, X, ldx, m, deriv, w, s);
+  expand_columns_kernel<<<(unsigned)((n * m + 127) / 128), 128, 0, s>>>(
+      reinterpret_cast<const double2*>(w + p.y_off), n, m, p.M, p.fams,
+      reinterpret_cast<const double2*>(w + p.coef_off), reinterpret_cast<const double2*>(X), ldx,
+      reinterpret_cast<double2*>(R));
+  ctx->launches++;
+  if (near_active(ctx)) return launch_near_percol64(ctx, m, lam_dev, X, ldx, R, deriv, s);
+  return cudaGetLastError();
+}
+
+}  // namespace bem

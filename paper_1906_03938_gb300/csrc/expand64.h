@@ -1,0 +1,33 @@
+// FP64 products with the operator at many wavenumbers from one evaluation (expand64.cu).
+#pragma once
+
+#include "internal.h"
+
+namespace bem {
+
+struct ExpandPlan {
+  bool use = false;        // the expansion applies and costs less than the direct form
+  int M = 0;               // series terms
+  int fams = 0, first = 0; // moment families (0: single layer, 1: double layer), the first one
+  int S = 0;               // slots, fams M
+  int kc = 0;              // columns evaluated at a time
+  int splits = 1;          // shares of those columns in the products
+  double R = 0.0;          // largest distance
+  double2 c{};             // centre
+  size_t coef_off = 0, mom_off = 0, y_off = 0, bytes = 0;
+};
+
+// Plan for nk wavenumbers within dmax of the centre and ncols columns: every wavenumber times
+// every column (nodes), or wavenumber c times column c.
+ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dmax, int ncols,
+                       bool nodes, bool deriv);
+// Y_j = A(z_j) V for all nodes of the contour (its FP64 self-term table filled); Y as
+// launch_apply_fp64's.
+cudaError_t expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
+                               int nu, double* Y, void* work, cudaStream_t s);
+// As launch_apply_percol64, near field included.
+cudaError_t expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
+                                 const double* X, int64_t ldx, double* R, bool deriv, void* work,
+                                 cudaStream_t s);
+
+}  // namespace bem

@@ -161,6 +161,9 @@ struct bem_ctx {
   // host copy of the mesh (the cluster tree of the low-rank far field is built from it)
   std::vector<double> h_xyz;
   std::vector<int32_t> h_tri;
+  // upper bound of the distance between two points of the mesh, and its mesh (expand64.cu)
+  double reach = 0.0;
+  int64_t reach_version = -1;
   // low-rank far field (hmatrix.cu); null until bem_set_hmatrix
   bem::HMatrix* hm = nullptr;
 };
@@ -173,6 +176,9 @@ bem_status fail(bem_ctx* ctx, bem_status st, const std::string& msg);
 bem_status cuda_check(bem_ctx* ctx, cudaError_t e, const char* what);
 // Make sure the context's scratch holds at least `bytes`.
 bem_status ensure_scratch(bem_ctx* ctx, size_t bytes);
+// The same where a smaller workspace would do: false if it cannot be had (no memory, or the
+// stream is being captured and the buffer would have to grow).
+bool scratch_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s);
 bem_status ensure_small(bem_ctx* ctx, size_t bytes);
 void release_cublas(bem_ctx* ctx);
 // nodes z and weights w (2 N doubles each, interleaved) of a contour, on the host

@@ -6,9 +6,11 @@
 // reduction (deterministic).
 #include <math.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
+#include "expand64.h"
 #include "internal.h"
 #include "selfterm.cuh"
 
@@ -208,12 +210,28 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   const size_t small = (size_t)4 * m * sizeof(double);
   st = ensure_small(ctx, small);
   if (st != BEM_OK) return st;
-  double* R = R_dev;
-  if (!R) {
-    st = ensure_scratch(ctx, (size_t)2 * n * m * sizeof(double));
-    if (st != BEM_OK) return st;
-    R = ctx->d_scratch;
+  // FP64: one evaluation expanded about the middle of the given values for all columns, where
+  // that costs less than one per column and its workspace can be had
+  const size_t r_bytes = R_dev ? 0 : ((size_t)2 * n * m * sizeof(double) + 255) / 256 * 256;
+  ExpandPlan ex;
+  if (arith == 0) {
+    double lo[2] = {lam_host[0], lam_host[1]}, hi[2] = {lam_host[0], lam_host[1]};
+    for (int c = 0; c < 2 * m; ++c) {
+      lo[c % 2] = std::min(lo[c % 2], lam_host[c]);
+      hi[c % 2] = std::max(hi[c % 2], lam_host[c]);
+    }
+    const double cr = 0.5 * (lo[0] + hi[0]), ci = 0.5 * (lo[1] + hi[1]);
+    double dmax = 0.0;
+    for (int c = 0; c < m; ++c)
+      dmax = std::max(dmax, hypot(lam_host[2 * c] - cr, lam_host[2 * c + 1] - ci));
+    ex = expand_plan(ctx, m, cr, ci, dmax, m, false, Rd_dev != nullptr);
+    if (ex.use) ex.use = scratch_ready(ctx, r_bytes + ex.bytes, s);
   }
+  if (!ex.use) {
+    st = ensure_scratch(ctx, r_bytes);
+    if (st != BEM_OK) return st;
+  }
+  double* R = R_dev ? R_dev : ctx->d_scratch;
   double* dlam = ctx->d_small;
   double* dnorm = ctx->d_small + 2 * m;
   st = cuda_check(ctx, cudaMemcpyAsync(dlam, lam_host, 2 * m * sizeof(double),
@@ -222,6 +240,11 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   cudaError_t e;
   if (arith == 1) {
     e = launch_apply_ff(ctx, m, dlam, X_dev, ldx, R, Rd_dev, s);
+  } else if (ex.use) {
+    void* w = reinterpret_cast<char*>(ctx->d_scratch) + r_bytes;
+    e = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, false, w, s);
+    if (e == cudaSuccess && Rd_dev)
+      e = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, Rd_dev, true, w, s);
   } else {
     e = launch_apply_percol64(ctx, m, dlam, X_dev, ldx, R, false, s);
     if (e == cudaSuccess && Rd_dev) e = launch_apply_percol64(ctx, m, dlam, X_dev, ldx, Rd_dev, true, s);

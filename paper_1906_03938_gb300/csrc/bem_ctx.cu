@@ -512,22 +512,20 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
   const size_t y_bytes = AV_dev ? 0 : (size_t)N * n * nu * 2 * sizeof(double);
   ExpandPlan ex = expand_plan(ctx, N, ctx->con.c_re, ctx->con.c_im, std::max(ctx->con.a, ctx->con.b),
                               nu, true, false);
-  if (ex.use) ex.use = scratch_ready(ctx, y_bytes + ex.bytes, s);
+  ex.use = expand_ready(ctx, ex, y_bytes, nu, s);
   if (!ex.use) {
     bem_status st = ensure_scratch(ctx, y_bytes);
     if (st != BEM_OK) return st;
   }
   double* Y = AV_dev ? AV_dev : ctx->d_scratch;
   timing_begin(ctx, s);
-  bem_status st = cuda_check(
-      ctx,
+  bem_status st =
       ex.use ? expand_apply_nodes(ctx, ex, V_dev, ldv, nu, Y,
                                   reinterpret_cast<char*>(ctx->d_scratch) + y_bytes, s)
-             : launch_apply_fp64(ctx, V_dev, ldv, nu, Y, s),
-      "apply kernel");
+             : cuda_check(ctx, launch_apply_fp64(ctx, V_dev, ldv, nu, Y, s), "apply kernel");
   timing_end(ctx, s);
   if (st != BEM_OK) return st;
-  if (near_active(ctx)) {
+  if (near_active(ctx) && !ex.use) {
     st = near_apply64(ctx, V_dev, ldv, nu, Y, s);
     if (st != BEM_OK) return st;
   }

@@ -15,39 +15,38 @@
 // Bound by the FP64 pipe (1/64 of the FP32 rate on this part): per entry 7 (60 + 3 M) FP64
 // operations of evaluation and 3 M nu of products against N (7 x 77 + 4 nu) for the direct
 // form; the moments' round trip through memory (32 bytes a moment) is ~1 % of that. Measured:
-// the FP64 step of the 768-panel cube (N = 32, nu = 64) 32.2 -> 8.8 ms, residuals of 8 vectors
-// on 5120 panels 286 -> 80 ms (258 -> 52 in the operator), with the same or a smaller error
-// against 64-bit references.
+// the products of the 768-panel cube (N = 32, nu = 64) 28.1 -> 4.6 ms, of the residuals of 8
+// vectors on 5120 panels 258 -> 50 ms, with the same or a smaller error against 64-bit
+// references.
 #include <math.h>
 
 #include <algorithm>
 
+#include "expand64.cuh"
 #include "expand64.h"
 
 namespace bem {
 namespace {
 
-constexpr int kMaxTerms = 32;      // series length the evaluation kernel is built for
-constexpr int kCoefPoints = 64;    // Chebyshev points of the coefficients' quadrature
+constexpr int kCoefPoints = 64;    // Chebyshev points of the coefficients' quadrature (> kMaxTerms)
 constexpr int kRowsE = 128;        // rows per block of the evaluation (a thread each)
 constexpr int kColsE = 8;          // columns per block of the evaluation
 constexpr size_t kMomentBytes = (size_t)1 << 30;   // moments held at a time
 constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
 
 // a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
-// wavenumber k_j, times the operator's coefficient of the family.
-__global__ void expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R,
-                                   int M, int fams, int first_fam, bool deriv, OpCoef op,
-                                   double2* __restrict__ a) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= fams * nk * M) return;
-  const int m = t % M, j = (t / M) % nk, f = first_fam + t / (M * nk);
+// wavenumber k_j, times the operator's coefficient of the family. One block per (j, f): its
+// threads take one Chebyshev point each, then one coefficient each (a thread per coefficient
+// evaluated all points again: 196 us against 56 at 32 wavenumbers).
+__global__ void __launch_bounds__(kCoefPoints)
+expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, int M,
+                   int first_fam, bool deriv, OpCoef op, double2* __restrict__ a) {
+  __shared__ double2 fv[kCoefPoints];
+  const int j = blockIdx.x, f = first_fam + blockIdx.y, q = threadIdx.x;
   const double2 kj = k[j];
-  const double dr = kj.x - c.x, di = kj.y - c.y;
-  double2 s = make_double2(0.0, 0.0);
-  for (int q = 0; q < kCoefPoints; ++q) {
-    const double u = (q + 0.5) / kCoefPoints;
-    const double r = 0.5 * R * (cospi(u) + 1.0);
+  {
+    const double r = 0.5 * R * (cospi((q + 0.5) / kCoefPoints) + 1.0);
+    const double dr = kj.x - c.x, di = kj.y - c.y;
     double sn, cs;
     sincos(dr * r, &sn, &cs);
     const double e = exp(-di * r);
@@ -60,13 +59,21 @@ __global__ void expand_coef_kernel(const double2* __restrict__ k, int nk, double
       gr = deriv ? -kj.x * r * r : -kj.y * r - 1.0;
       gi = deriv ? -kj.y * r * r : kj.x * r;
     }
-    const double w = e * cospi(m * u);
-    s.x += w * (cs * gr - sn * gi);
-    s.y += w * (cs * gi + sn * gr);
+    fv[q] = make_double2(e * (cs * gr - sn * gi), e * (cs * gi + sn * gr));
+  }
+  __syncthreads();
+  if (q >= M) return;
+  const int m = q;
+  double2 s = make_double2(0.0, 0.0);
+  for (int p = 0; p < kCoefPoints; ++p) {
+    const double w = cospi(m * ((p + 0.5) / kCoefPoints));
+    s.x = fma(w, fv[p].x, s.x);
+    s.y = fma(w, fv[p].y, s.y);
   }
   const double sc = (m == 0 ? 1.0 : 2.0) / kCoefPoints;
   const double or_ = f == 0 ? op.cgr : op.chr, oi = f == 0 ? op.cgi : op.chi;
-  a[t] = make_double2(sc * (s.x * or_ - s.y * oi), sc * (s.x * oi + s.y * or_));
+  a[((int64_t)blockIdx.y * nk + j) * M + m] =
+      make_double2(sc * (s.x * or_ - s.y * oi), sc * (s.x * oi + s.y * or_));
 }
 
 // Moments of the columns [l0, l0 + kc): G[f M + m][l - l0][i] (i fastest). One thread per row;
@@ -106,41 +113,9 @@ expand_moments_kernel(Geometry g, double2 c, double two_over_R, int M, int64_t l
       for (int m = 0; m < MT; ++m) ar[f][m] = ai[f][m] = 0.0;
     if (l != i) {
 #pragma unroll 1
-      for (int q = 0; q < 7; ++q) {
-        const double dx = sq[cc][q][0] - xi, dy = sq[cc][q][1] - yi, dz = sq[cc][q][2] - zi;
-        const double r2 = dx * dx + dy * dy + dz * dz;
-        const double ri = rsqrt(r2);
-        double r = r2 * ri;
-        r = fma(0.5 * ri, fma(-r, r, r2), r);   // sqrt(r2) to its last bit or so
-        double s, co;
-        sincos(c.x * r, &s, &co);
-        double w = sq[cc][q][3] * ri;
-        if (c.y != 0.0) w *= exp(-c.y * r);
-        const double x = fma(r, two_over_R, -1.0), x2 = 2.0 * x;
-        double br[F], bi[F];
-        if (kG) {
-          br[0] = w * co;
-          bi[0] = w * s;
-        }
-        if (kH) {
-          const double h = w * ri * ri *
-                           (dx * sn3[cc][0] + dy * sn3[cc][1] + dz * sn3[cc][2]);
-          br[F - 1] = h * co;
-          bi[F - 1] = h * s;
-        }
-        double t0 = 1.0, t1 = x;
-#pragma unroll
-        for (int m = 0; m < MT; ++m) {
-#pragma unroll
-          for (int f = 0; f < F; ++f) {
-            ar[f][m] = fma(br[f], t0, ar[f][m]);
-            ai[f][m] = fma(bi[f], t0, ai[f][m]);
-          }
-          const double t2 = fma(x2, t1, -t0);
-          t0 = t1;
-          t1 = t2;
-        }
-      }
+      for (int q = 0; q < 7; ++q)
+        expand_point<MT, kG, kH>(ar, ai, sq[cc][q][3], sq[cc][q][0] - xi, sq[cc][q][1] - yi,
+                                 sq[cc][q][2] - zi, sn3[cc], c, two_over_R);
     }
 #pragma unroll
     for (int f = 0; f < F; ++f)
@@ -410,20 +385,23 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   return p;
 }
 
+bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, size_t before, int ncols, cudaStream_t s) {
+  return p.use && (!near_active(ctx) || near_expand_ready(ctx, p, ncols, s)) &&
+         scratch_ready(ctx, before + p.bytes, s);
+}
+
 namespace {
 
-// The slot products Y_s = G_s X into the workspace.
-void expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const double* k_dev,
+// The slot products Y_s = G_s X into the workspace, near-field corrections included.
+bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const double* k_dev,
                      const double* X, int64_t ldx, int ncols, bool deriv, char* work,
                      cudaStream_t s) {
   const int64_t n = ctx->geo.n;
   double2* a = reinterpret_cast<double2*>(work + p.coef_off);
   double2* G = reinterpret_cast<double2*>(work + p.mom_off);
   double2* Yp = reinterpret_cast<double2*>(work + p.y_off);
-  const int total = p.S * nk;
-  expand_coef_kernel<<<(total + 63) / 64, 64, 0, s>>>(reinterpret_cast<const double2*>(k_dev), nk,
-                                                     p.c, p.R, p.M, p.fams, p.first, deriv,
-                                                     ctx->op, a);
+  expand_coef_kernel<<<dim3((unsigned)nk, (unsigned)p.fams), kCoefPoints, 0, s>>>(
+      reinterpret_cast<const double2*>(k_dev), nk, p.c, p.R, p.M, p.first, deriv, ctx->op, a);
   MomentKernel mk = p.fams == 2 ? moment_kernel<true, true>(p.M)
                                 : (p.first == 0 ? moment_kernel<true, false>(p.M)
                                                 : moment_kernel<false, true>(p.M));
@@ -445,16 +423,18 @@ void expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const double* k_
     expand_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, p.splits, Yp);
     ctx->launches++;
   }
+  return near_active(ctx) ? near_expand64(ctx, p, X, ldx, ncols, Yp, s) : BEM_OK;
 }
 
 }  // namespace
 
-cudaError_t expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
+bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
                                int nu, double* Y, void* work, cudaStream_t s) {
   char* w = static_cast<char*>(work);
   const int N = ctx->con.N;
   const int64_t n = ctx->geo.n;
-  expand_products(ctx, p, N, ctx->con.z, V, ldv, nu, false, w, s);
+  const bem_status st = expand_products(ctx, p, N, ctx->con.z, V, ldv, nu, false, w, s);
+  if (st != BEM_OK) return st;
   const dim3 g((unsigned)((n * nu + 127) / 128), (unsigned)((N + kNodesC - 1) / kNodesC));
   expand_nodes_kernel<<<g, 128, 0, s>>>(reinterpret_cast<const double2*>(w + p.y_off), n, nu, p.M,
                                         p.fams, N, reinterpret_cast<const double2*>(w + p.coef_off),
@@ -462,24 +442,23 @@ cudaError_t expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* 
                                         reinterpret_cast<const double2*>(V), ldv,
                                         reinterpret_cast<double2*>(Y));
   ctx->launches++;
-  return cudaGetLastError();
+  return cuda_check(ctx, cudaGetLastError(), "expanded products");
 }
 
-cudaError_t expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
+bem_status expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
                                  const double* X, int64_t ldx, double* R, bool deriv, void* work,
                                  cudaStream_t s) {
   char* w = static_cast<char*>(work);
   const int64_t n = ctx->geo.n;
-  const cudaError_t e = launch_self_at(ctx, m, lam_dev, R, deriv, s);
-  if (e != cudaSuccess) return e;
-  expand_products(ctx, p, m, lam_dev, X, ldx, m, deriv, w, s);
+  bem_status st = cuda_check(ctx, launch_self_at(ctx, m, lam_dev, R, deriv, s), "self terms");
+  if (st == BEM_OK) st = expand_products(ctx, p, m, lam_dev, X, ldx, m, deriv, w, s);
+  if (st != BEM_OK) return st;
   expand_columns_kernel<<<(unsigned)((n * m + 127) / 128), 128, 0, s>>>(
       reinterpret_cast<const double2*>(w + p.y_off), n, m, p.M, p.fams,
       reinterpret_cast<const double2*>(w + p.coef_off), reinterpret_cast<const double2*>(X), ldx,
       reinterpret_cast<double2*>(R));
   ctx->launches++;
-  if (near_active(ctx)) return launch_near_percol64(ctx, m, lam_dev, X, ldx, R, deriv, s);
-  return cudaGetLastError();
+  return cuda_check(ctx, cudaGetLastError(), "expanded products");
 }
 
 }  // namespace bem

@@ -5,6 +5,8 @@
 
 namespace bem {
 
+constexpr int kMaxTerms = 32;   // longest series the kernels are built for
+
 struct ExpandPlan {
   bool use = false;        // the expansion applies and costs less than the direct form
   int M = 0;               // series terms
@@ -21,13 +23,21 @@ struct ExpandPlan {
 // every column (nodes), or wavenumber c times column c.
 ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dmax, int ncols,
                        bool nodes, bool deriv);
-// Y_j = A(z_j) V for all nodes of the contour (its FP64 self-term table filled); Y as
-// launch_apply_fp64's.
-cudaError_t expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
-                               int nu, double* Y, void* work, cudaStream_t s);
+// The workspace can be had: plan's bytes behind `before` bytes of the context's scratch, and the
+// near field's. False leaves the caller the direct form.
+bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, size_t before, int ncols, cudaStream_t s);
+// Y_j = A(z_j) V for all nodes of the contour (its FP64 self-term table filled), near field
+// included; Y as launch_apply_fp64's. work: plan's bytes.
+bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
+                              int nu, double* Y, void* work, cudaStream_t s);
 // As launch_apply_percol64, near field included.
-cudaError_t expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
-                                 const double* X, int64_t ldx, double* R, bool deriv, void* work,
-                                 cudaStream_t s);
+bem_status expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
+                                const double* X, int64_t ldx, double* R, bool deriv, void* work,
+                                cudaStream_t s);
+// Near pairs (near.cu): Y_s += C_s X for every slot, C_s the moments of the corrections
+// (A_near - A_7); its workspace.
+bool near_expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s);
+bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const double* X, int64_t ldx,
+                         int ncols, double2* Ys, cudaStream_t s);
 
 }  // namespace bem

@@ -171,23 +171,21 @@ __global__ void contour_kernel(int N, int kind, double c_re, double c_im, double
   w[2 * j + 1] = a * s / N;
 }
 
-// One thread per (panel l, node j).
+// Self entries of every panel at N wavenumbers, one warp per panel.
 // T's self entry: c_G times the single-layer self integral plus c_H / 2 (the jump of H).
-__global__ void self_term_kernel(Geometry g, int N, const double* z, GL16 gl, OpCoef op,
-                                 double* self) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= g.n * (int64_t)N) return;
-  const int64_t l = t % g.n;
-  const int j = (int)(t / g.n);
+__global__ void __launch_bounds__(128)
+self_term_kernel(Geometry g, int N, const double* z, GL16 gl, OpCoef op, bool deriv,
+                 double* self) {
+  const int64_t l = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
+  if (l >= g.n) return;
   double v[3][3], x[3];
   for (int e = 0; e < 3; ++e) {
     const int32_t vi = g.tri[3 * l + e];
     for (int c = 0; c < 3; ++c) v[e][c] = g.xyz[3 * (int64_t)vi + c];
   }
   for (int c = 0; c < 3; ++c) x[c] = g.cx[c * g.n + l];
-  const double2 a = self_term(v, x, make_double2(z[2 * j], z[2 * j + 1]), gl);
-  self[2 * (j * g.n + l)] = op.cgr * a.x - op.cgi * a.y + 0.5 * op.chr;
-  self[2 * (j * g.n + l) + 1] = op.cgr * a.y + op.cgi * a.x + 0.5 * op.chi;
+  self_entries_warp(v, x, l, g.n, N, reinterpret_cast<const double2*>(z), gl, deriv, op.cgr, op.cgi,
+                    op.chr, op.chi, threadIdx.x % 32, reinterpret_cast<double2*>(self));
 }
 
 // Moments of the FP32 self term. With f_g = half * w_g * d the angular weight of node g and
@@ -335,14 +333,17 @@ cudaError_t launch_self32(bem_ctx* ctx, int nk, const double* kz, float* out, cu
   return cudaGetLastError();
 }
 
-cudaError_t launch_self_terms(bem_ctx* ctx, cudaStream_t s) {
+cudaError_t launch_self_at(bem_ctx* ctx, int m, const double* lam_dev, double* R, bool deriv,
+                           cudaStream_t s) {
   static const GL16 gl = make_gl16();
-  const int64_t total = ctx->geo.n * (int64_t)ctx->con.N;
-  self_term_kernel<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(ctx->geo, ctx->con.N,
-                                                                   ctx->con.z, gl, ctx->op,
-                                                                   ctx->con.self);
+  self_term_kernel<<<(unsigned)((32 * ctx->geo.n + 127) / 128), 128, 0, s>>>(
+      ctx->geo, m, lam_dev, gl, ctx->op, deriv, R);
   ctx->launches++;
   return cudaGetLastError();
+}
+
+cudaError_t launch_self_terms(bem_ctx* ctx, cudaStream_t s) {
+  return launch_self_at(ctx, ctx->con.N, ctx->con.z, ctx->con.self, false, s);
 }
 
 }  // namespace bem

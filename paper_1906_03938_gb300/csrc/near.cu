@@ -23,8 +23,11 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
+#include "expand64.cuh"
+#include "expand64.h"
 #include "internal.h"
 #include "sm100.cuh"
 #include "surrogate.cuh"
@@ -396,6 +399,82 @@ near_apply64_kernel(Geometry g, const int32_t* __restrict__ ptr, const int32_t* 
       y.y += acc[cg].y;
       Yj[(int64_t)c * n + i] = y;
     }
+  }
+}
+
+// Moments of the corrections (A_near - A_7) in the expansion over wavenumbers (expand64.cu):
+// C[f M + m][e] for pair e, one thread per pair; its row by bisection of the row pointers. The
+// 71 points' roots and sines serve every wavenumber (near_apply64_kernel and
+// near_percol64_kernel evaluate them for each). FP64-bound: 71 (60 + 3 M) operations a pair.
+// Residuals of 8 vectors on 5120 panels: 23.0 -> 3.1 ms with near_slots64_kernel.
+template <int MT, bool kG, bool kH>
+__global__ void __launch_bounds__(128)
+near_moments64_kernel(Geometry g, const int32_t* __restrict__ ptr,
+                      const int32_t* __restrict__ cols, int64_t nnz, GL8 gl, double2 c,
+                      double two_over_R, int M, double2* __restrict__ C) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nnz) return;
+  const int64_t n = g.n;
+  int64_t lo = 0, hi = n - 1;   // the last row whose pairs start at or before e
+  while (lo < hi) {
+    const int64_t mid = (lo + hi + 1) / 2;
+    if (ptr[mid] <= e) lo = mid; else hi = mid - 1;
+  }
+  const int64_t i = lo, l = cols[e];
+  const double x[3] = {g.cx[i], g.cx[n + i], g.cx[2 * n + i]};
+  double nrm[3] = {0.0, 0.0, 0.0};
+  if (kH)
+    for (int d = 0; d < 3; ++d) nrm[d] = g.nrm[d * n + l];
+  NearFrame F;
+  near_frame(g, l, x, F);
+  constexpr int NF = (kG ? 1 : 0) + (kH ? 1 : 0);
+  double ar[NF][MT], ai[NF][MT];
+#pragma unroll
+  for (int f = 0; f < NF; ++f)
+#pragma unroll
+    for (int m = 0; m < MT; ++m) ar[f][m] = ai[f][m] = 0.0;
+#pragma unroll 1
+  for (int t = 0; t < 71; ++t) {
+    double w, y[3];
+    if (t < 64) {
+      const double sp = gl.x[t / 8], st = sp * gl.x[t % 8];
+      w = gl.w[t / 8] * gl.w[t % 8] * sp * F.scale;
+      for (int d = 0; d < 3; ++d) y[d] = F.a[d] + sp * F.ab[d] + st * F.bc[d];
+    } else {
+      const int q = t - 64;
+      w = -g.qw[q * n + l];
+      for (int d = 0; d < 3; ++d) y[d] = g.qp[(7 * d + q) * n + l];
+    }
+    expand_point<MT, kG, kH>(ar, ai, w, y[0] - x[0], y[1] - x[1], y[2] - x[2], nrm, c, two_over_R);
+  }
+#pragma unroll
+  for (int f = 0; f < NF; ++f)
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+      if (m < M) C[(int64_t)(f * M + m) * nnz + e] = make_double2(ar[f][m], ai[f][m]);
+}
+
+// Y_s += C_s X: one warp per (row i, slot s), lanes over the columns; Xt is X row-major.
+__global__ void __launch_bounds__(256)
+near_slots64_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ cols, int64_t n,
+                    int64_t nnz, int S, const double2* __restrict__ C,
+                    const double2* __restrict__ Xt, int nu, double2* __restrict__ Ys) {
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
+  const int lane = threadIdx.x % 32;
+  if (w >= n * S) return;
+  const int64_t i = w % n;
+  const int s = (int)(w / n);
+  const int32_t e0 = ptr[i], e1 = ptr[i + 1];
+  if (e0 == e1) return;
+  for (int c = lane; c < nu; c += 32) {
+    double2 acc = Ys[((int64_t)s * nu + c) * n + i];
+    for (int32_t e = e0; e < e1; ++e) {
+      const double2 m = C[(int64_t)s * nnz + e];
+      const double2 v = Xt[(int64_t)cols[e] * nu + c];
+      acc.x = fma(m.x, v.x, fma(-m.y, v.y, acc.x));
+      acc.y = fma(m.x, v.y, fma(m.y, v.x, acc.y));
+    }
+    Ys[((int64_t)s * nu + c) * n + i] = acc;
   }
 }
 
@@ -1007,6 +1086,47 @@ bem_status near_apply64(bem_ctx* ctx, const double* V, int64_t ldv, int nu, doub
       ctx->geo, ctx->d_near_ptr, ctx->d_near_cols, ctx->con.z, N, Vt, nu,
       reinterpret_cast<double2*>(Y), gl8(), ctx->op);
   ctx->launches += 2;
+  return cuda_check(ctx, cudaGetLastError(), "near field kernels");
+}
+
+bool near_expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s) {
+  const size_t need = ((size_t)ctx->geo.n * ncols + (size_t)p.S * ctx->near_nnz) * sizeof(double2);
+  if (need <= ctx->near_work_bytes) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  return ensure_near_work(ctx, need) == BEM_OK;
+}
+
+bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const double* X, int64_t ldx,
+                         int ncols, double2* Ys, cudaStream_t s) {
+  const int64_t n = ctx->geo.n, nnz = ctx->near_nnz;
+  if (nnz == 0) return BEM_OK;
+  double2* Xt = reinterpret_cast<double2*>(ctx->d_near_work);
+  double2* C = Xt + (size_t)n * ncols;
+  transpose64_kernel<<<(unsigned)((n * ncols + 255) / 256), 256, 0, s>>>(
+      reinterpret_cast<const double2*>(X), ldx, n, ncols, Xt);
+  const unsigned blocks = (unsigned)((nnz + 127) / 128);
+  auto go = [&](auto mt) {
+    constexpr int MT = decltype(mt)::value;
+    auto* k = p.fams == 2 ? near_moments64_kernel<MT, true, true>
+                          : (p.first == 0 ? near_moments64_kernel<MT, true, false>
+                                          : near_moments64_kernel<MT, false, true>);
+    k<<<blocks, 128, 0, s>>>(ctx->geo, ctx->d_near_ptr, ctx->d_near_cols, nnz, gl8(), p.c,
+                             2.0 / p.R, p.M, C);
+  };
+  if (p.M <= 1) go(std::integral_constant<int, 1>());
+  else if (p.M <= 12) go(std::integral_constant<int, 12>());
+  else if (p.M <= 14) go(std::integral_constant<int, 14>());
+  else if (p.M <= 16) go(std::integral_constant<int, 16>());
+  else if (p.M <= 18) go(std::integral_constant<int, 18>());
+  else if (p.M <= 24) go(std::integral_constant<int, 24>());
+  else go(std::integral_constant<int, kMaxTerms>());
+  near_slots64_kernel<<<(unsigned)((32 * n * (int64_t)p.S + 255) / 256), 256, 0, s>>>(
+      ctx->d_near_ptr, ctx->d_near_cols, n, nnz, p.S, C, Xt, ncols, Ys);
+  ctx->launches += 3;
   return cuda_check(ctx, cudaGetLastError(), "near field kernels");
 }
 

@@ -12,7 +12,6 @@
 
 #include "expand64.h"
 #include "internal.h"
-#include "selfterm.cuh"
 
 namespace bem {
 namespace {
@@ -93,33 +92,13 @@ residual_kernel(Geometry g, const double* __restrict__ lam, const double* __rest
     }
   }
   if (i < n) {
-    // R holds A_ii(lambda_c), written by self_at_kernel before this kernel runs
+    // R holds A_ii(lambda_c), written by launch_self_at before this kernel runs
     double2* Rc = reinterpret_cast<double2*>(R) + (int64_t)c * n;
     const double2 sd = Rc[i];
     acc.x += sd.x * self_x.x - sd.y * self_x.y;
     acc.y += sd.x * self_x.y + sd.y * self_x.x;
     Rc[i] = acc;
   }
-}
-
-// Self term A_ii(lambda_c) (or its k-derivative) of every row, written into R as the
-// multiplier of x_i.
-__global__ void self_at_kernel(Geometry g, const double* __restrict__ lam, GL16 gl,
-                               double* __restrict__ R, bool deriv, OpCoef op) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int c = blockIdx.y;
-  if (i >= g.n) return;
-  double v[3][3], x[3];
-  for (int e = 0; e < 3; ++e) {
-    const int32_t vi = g.tri[3 * i + e];
-    for (int d = 0; d < 3; ++d) v[e][d] = g.xyz[3 * (int64_t)vi + d];
-  }
-  for (int d = 0; d < 3; ++d) x[d] = g.cx[d * g.n + i];
-  // T's self entry: c_G A_ii (+ c_H / 2, whose k-derivative is 0)
-  const double2 a = self_term(v, x, make_double2(lam[2 * c], lam[2 * c + 1]), gl, deriv);
-  reinterpret_cast<double2*>(R)[(int64_t)c * g.n + i] =
-      make_double2(op.cgr * a.x - op.cgi * a.y + (deriv ? 0.0 : 0.5 * op.chr),
-                   op.cgr * a.y + op.cgi * a.x + (deriv ? 0.0 : 0.5 * op.chi));
 }
 
 __global__ void norms_kernel(const double* __restrict__ R, const double* __restrict__ X,
@@ -153,26 +132,16 @@ __global__ void norms_kernel(const double* __restrict__ R, const double* __restr
 
 cudaError_t launch_apply_percol64(bem_ctx* ctx, int m, const double* lam_dev, const double* X,
                                   int64_t ldx, double* R, bool deriv, cudaStream_t s) {
-  static const GL16 gl = make_gl16();
   const int64_t n = ctx->geo.n;
-  dim3 g1((unsigned)((n + 127) / 128), (unsigned)m);
-  self_at_kernel<<<g1, 128, 0, s>>>(ctx->geo, lam_dev, gl, R, deriv, ctx->op);
+  const cudaError_t e = launch_self_at(ctx, m, lam_dev, R, deriv, s);
+  if (e != cudaSuccess) return e;
   dim3 g2((unsigned)((n + kRowsPerBlock - 1) / kRowsPerBlock), (unsigned)m);
   if (deriv)
     residual_kernel<true><<<g2, kRowsPerBlock, 0, s>>>(ctx->geo, lam_dev, X, ldx, R, ctx->op);
   else
     residual_kernel<false><<<g2, kRowsPerBlock, 0, s>>>(ctx->geo, lam_dev, X, ldx, R, ctx->op);
-  ctx->launches += 2;
-  if (near_active(ctx)) return launch_near_percol64(ctx, m, lam_dev, X, ldx, R, deriv, s);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_self_at(bem_ctx* ctx, int m, const double* lam_dev, double* R, bool deriv,
-                           cudaStream_t s) {
-  static const GL16 gl = make_gl16();
-  dim3 g1((unsigned)((ctx->geo.n + 127) / 128), (unsigned)m);
-  self_at_kernel<<<g1, 128, 0, s>>>(ctx->geo, lam_dev, gl, R, deriv, ctx->op);
   ctx->launches++;
+  if (near_active(ctx)) return launch_near_percol64(ctx, m, lam_dev, X, ldx, R, deriv, s);
   return cudaGetLastError();
 }
 
@@ -225,7 +194,7 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
     for (int c = 0; c < m; ++c)
       dmax = std::max(dmax, hypot(lam_host[2 * c] - cr, lam_host[2 * c + 1] - ci));
     ex = expand_plan(ctx, m, cr, ci, dmax, m, false, Rd_dev != nullptr);
-    if (ex.use) ex.use = scratch_ready(ctx, r_bytes + ex.bytes, s);
+    ex.use = expand_ready(ctx, ex, r_bytes, m, s);
   }
   if (!ex.use) {
     st = ensure_scratch(ctx, r_bytes);
@@ -237,14 +206,15 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   st = cuda_check(ctx, cudaMemcpyAsync(dlam, lam_host, 2 * m * sizeof(double),
                                        cudaMemcpyHostToDevice, s), name);
   if (st != BEM_OK) return st;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   if (arith == 1) {
     e = launch_apply_ff(ctx, m, dlam, X_dev, ldx, R, Rd_dev, s);
   } else if (ex.use) {
     void* w = reinterpret_cast<char*>(ctx->d_scratch) + r_bytes;
-    e = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, false, w, s);
-    if (e == cudaSuccess && Rd_dev)
-      e = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, Rd_dev, true, w, s);
+    st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, false, w, s);
+    if (st == BEM_OK && Rd_dev)
+      st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, Rd_dev, true, w, s);
+    if (st != BEM_OK) return st;
   } else {
     e = launch_apply_percol64(ctx, m, dlam, X_dev, ldx, R, false, s);
     if (e == cudaSuccess && Rd_dev) e = launch_apply_percol64(ctx, m, dlam, X_dev, ldx, Rd_dev, true, s);

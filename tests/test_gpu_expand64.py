@@ -76,3 +76,15 @@ def test_residuals(op, m, k, spread, near):
         assert _err(Rd[:, c].cpu().numpy(), want_d) < 1e-11
         norm = np.linalg.norm(want) / np.linalg.norm(X[:, c])
         assert abs(rel[c] - norm) < 1e-11 * norm and abs(rel0[c] - norm) < 1e-11 * norm
+
+
+@pytest.mark.parametrize("k", [0.4, 7.0 + 0.5j, 24.0 - 1.0j, 60.0])
+def test_self_entries(k):
+    """One panel: the residual is the self entry (series below |k| rho = 2, angular sum above)."""
+    mesh = synth.cube_grid(4)
+    mesh = synth.Mesh("one", mesh.xyz, mesh.tri[:1])
+    _, ctx = _ctx(mesh, "single", 0)
+    _, R, Rd = ctx.residual_arith([k], _strided(np.ones((1, 1), dtype=complex), 1), arith=0, deriv=True)
+    ctx.close()
+    for got, d in ((R, 0), (Rd, 1)):
+        assert _err(got.cpu().numpy(), oasm.matrix(mesh, k, deriv=d, op=OPS["single"])) < 1e-11

@@ -137,14 +137,14 @@ bem_status bem_set_operator(bem_ctx* ctx, double cg_re, double cg_im, double ch_
  * The structure is built on the host at the first projection after a mesh change (from a
  * host copy of the mesh kept by bem_set_mesh) and reused; the compression runs at every
  * projection. The AV output holds the H-matrix products. Synchronises the stream (once per
- * node). bem_hmatrix_stats: far and dense block counts, the fraction of entries in far
+ * group of nodes compressed together). bem_hmatrix_stats: far and dense block counts, the fraction of entries in far
  * blocks, mean and largest rank of the last projection (host; BEM_ESTATE before
  * bem_set_hmatrix). bem_hmatrix_work: the algorithmic work of one node of the last
  * projection, averaged over its nodes: dense entries (each evaluated once and multiplied
  * into nu columns), sum over far blocks of rank x rows (the U_b T_b products) and of
  * rank x columns (the W_b^T V products); any pointer may be NULL (host; BEM_ESTATE before
- * bem_set_hmatrix). With bem_set_timing on, each node's leaf kernel (dense blocks and
- * U_b T_b) is timed by bem_kernel_times.
+ * bem_set_hmatrix). With bem_set_timing on, the nodes run one at a time and each node's leaf
+ * kernel (dense blocks and U_b T_b) is timed by bem_kernel_times.
  */
 bem_status bem_set_hmatrix(bem_ctx* ctx, int leaf, double eta, double eps, int rmax);
 bem_status bem_hmatrix_stats(const bem_ctx* ctx, int64_t* far_blocks, int64_t* dense_blocks,

@@ -8,13 +8,13 @@
 // when max(diam tau, diam sigma) <= eta dist(tau, sigma) and both hold more than two leaves
 // of panels, a pair of leaves that is not far is dense, any other pair splits into its
 // children's pairs.
-// Device, node by node:
-//   hm_aca_kernel        one CTA per far block: adaptive cross approximation with partial
+// Device, a group of nodes at a time (every launch covers the group's nodes):
+//   hm_aca_kernel        one CTA per far block and node: adaptive cross approximation with partial
 //                        pivoting on FP32 entries (block ~ U W^T, ranks up to rmax, stop at
 //                        ||u_k|| ||w_k|| <= eps ||S_k||_F with the exact norm update);
 //   hm_wtv_kernel        T_b = W_b^T V_sigma (rank x nu) per far block, as panel products in
 //                        shared memory;
-//   hm_leaf_kernel       one CTA per leaf row range: the leaf's dense column ranges evaluated
+//   hm_leaf_kernel       one CTA per leaf row range and node: the leaf's dense column ranges evaluated
 //                        32 panels at a time from geometry staged in shared memory and
 //                        multiplied with every basis column, then the rank-1 terms of every
 //                        far block above the leaf, 32 at a time, in a fixed order (no
@@ -76,7 +76,7 @@ struct HMatrix {
   size_t used_bytes = 0;
   int32_t* d_rank = nullptr;
   int64_t* d_toff = nullptr;
-  size_t rank_cap = 0;
+  size_t rank_cap = 0, toff_cap = 0;
   float2* d_t = nullptr;
   size_t t_bytes = 0;
   float2* d_vp = nullptr;      // V in cluster order, row-major (CW per panel, zero-padded), FP32
@@ -109,7 +109,7 @@ void free_work(HMatrix& h) {
   cudaFree(h.d_vp); cudaFree(h.d_y);
   h.d_uw = nullptr; h.d_used = nullptr; h.d_rank = nullptr; h.d_toff = nullptr; h.d_t = nullptr;
   h.d_vp = nullptr; h.d_y = nullptr;
-  h.uw_bytes = h.used_bytes = h.rank_cap = h.t_bytes = h.vp_bytes = h.y_bytes = 0;
+  h.uw_bytes = h.used_bytes = h.rank_cap = h.toff_cap = h.t_bytes = h.vp_bytes = h.y_bytes = 0;
 }
 
 double box_diam(const HMatrix::Cl& c) {
@@ -328,18 +328,29 @@ __device__ __forceinline__ void block_sum2(float& a, float& b, float* sa, float*
   __syncthreads();
 }
 
-// One CTA per far block: adaptive cross approximation with partial pivoting.
+// Buffers of a group of nodes (blockIdx.y = node of the group): strides between the nodes.
+struct HmGroup {
+  const double* z;        // the group's first node
+  int64_t uw, used, far;  // uw and used elements, far blocks per node
+};
+
+// One CTA per (far block, node of the group): adaptive cross approximation with partial
+// pivoting.
 template <bool general, int NT>
 __global__ void __launch_bounds__(NT)
-hm_aca_kernel(int base, HmGeom g, const int4* __restrict__ far,
+hm_aca_kernel(int base, HmGeom g, HmGroup grp, const int4* __restrict__ far,
               const int64_t* __restrict__ uw_off, const int64_t* __restrict__ used_off,
-              float kr, float ki, OpCoef op, float eps, int rmax, float2* __restrict__ uw,
+              OpCoef op, float eps, int rmax, float2* __restrict__ uw,
               uint8_t* __restrict__ used, int32_t* __restrict__ rank) {
   __shared__ float sv[NT / 32], sv2[NT / 32];
   __shared__ int si[NT / 32];
   __shared__ float2 ui[kMaxRank], wj[kMaxRank], au[kMaxRank], aw[kMaxRank];
   __shared__ float2 piv;
   const int b = base + (int)blockIdx.x, tid = threadIdx.x;
+  const float kr = (float)grp.z[2 * blockIdx.y], ki = (float)grp.z[2 * blockIdx.y + 1];
+  uw += blockIdx.y * grp.uw;
+  used += blockIdx.y * grp.used;
+  rank += blockIdx.y * grp.far;
   const int4 f = far[b];
   const int m = f.y - f.x, n = f.w - f.z;
   float2* U = uw + uw_off[b];
@@ -616,7 +627,7 @@ struct PanelRows : PanelTile<NCH> {
 template <int NCH>
 using PanelFor = typename std::conditional<NCH >= 4, PanelTile<NCH>, PanelRows<NCH>>::type;
 
-// Y_j for the rows of one leaf and every basis column (one CTA per leaf):
+// Y_j for the rows of one leaf and every basis column (one CTA per leaf and node of the group):
 //   dense part: the leaf's dense column ranges (contiguous in cluster order), 32 panels at a
 //   time: their quadrature points staged, the block T(z_j)[leaf, panels] evaluated into
 //   shared memory (self entries from the FP32 self terms), times the staged basis rows;
@@ -626,14 +637,20 @@ using PanelFor = typename std::conditional<NCH >= 4, PanelTile<NCH>, PanelRows<N
 // vp: V in cluster order, row-major with CW columns (zero beyond nu); T rows CW wide too.
 template <int NCH, bool general>
 __global__ void __launch_bounds__(kHmThreads, NCH >= 4 ? 2 : 4)
-hm_leaf_kernel(HmGeom g, const int4* __restrict__ leaves, const int2* __restrict__ near,
+hm_leaf_kernel(HmGeom g, HmGroup grp, const int4* __restrict__ leaves, const int2* __restrict__ near,
                const int32_t* __restrict__ leaf_far_ptr, const int32_t* __restrict__ leaf_far,
                const int4* __restrict__ far, const int64_t* __restrict__ uw_off,
                const int32_t* __restrict__ rank, const int64_t* __restrict__ toff,
                const float2* __restrict__ uw, const float2* __restrict__ T,
                const float2* __restrict__ vp, int nu, const float2* __restrict__ self32,
-               float kr, float ki, OpCoef op, float* __restrict__ Yp, int C, int64_t n_pad) {
+               OpCoef op, float* __restrict__ Yp, int64_t y_stride, int C, int64_t n_pad) {
   using P = PanelFor<NCH>;
+  const float kr = (float)grp.z[2 * blockIdx.y], ki = (float)grp.z[2 * blockIdx.y + 1];
+  uw += blockIdx.y * grp.uw;
+  rank += blockIdx.y * grp.far;
+  toff += blockIdx.y * grp.far;
+  self32 += blockIdx.y * g.n;
+  Yp += blockIdx.y * y_stride;
   extern __shared__ float4 hm_smem[];
   float2* sB = reinterpret_cast<float2*>(hm_smem);
   float2* sA = sB + kPanelK * P::CW;                          // A tile, slots P::aidx
@@ -733,11 +750,11 @@ hm_leaf_kernel(HmGeom g, const int4* __restrict__ leaves, const int2* __restrict
   }
 }
 
-// T_b = W_b^T V_sigma (rank x CW, row-major) per far block (one CTA each), 32 ranks and 32
-// panels of sigma per panel product.
+// T_b = W_b^T V_sigma (rank x CW, row-major) per far block and node of the group (one CTA
+// each), 32 ranks and 32 panels of sigma per panel product.
 template <int NCH>
 __global__ void __launch_bounds__(kHmThreads, NCH >= 4 ? 2 : 3)
-hm_wtv_kernel(const int4* __restrict__ far, const int64_t* __restrict__ uw_off,
+hm_wtv_kernel(HmGroup grp, const int4* __restrict__ far, const int64_t* __restrict__ uw_off,
               const int32_t* __restrict__ rank, const int64_t* __restrict__ toff, int rmax,
               const float2* __restrict__ uw, const float2* __restrict__ vp,
               float2* __restrict__ T) {
@@ -746,6 +763,9 @@ hm_wtv_kernel(const int4* __restrict__ far, const int64_t* __restrict__ uw_off,
   float2* sB = reinterpret_cast<float2*>(hm_smem);
   float2* sA = sB + kPanelK * P::CW;   // A tile, slots P::aidx
   const int b = blockIdx.x, tid = threadIdx.x;
+  uw += blockIdx.y * grp.uw;
+  rank += blockIdx.y * grp.far;
+  toff += blockIdx.y * grp.far;
   const int4 f = far[b];
   const int m = f.y - f.x, n = f.w - f.z;
   const int r = rank[b];
@@ -938,11 +958,11 @@ bem_status build_structure(bem_ctx* ctx, cudaStream_t s) {
 
 unsigned nblocks(int64_t count, int t = 256) { return (unsigned)((count + t - 1) / t); }
 
-// The W^T V and leaf kernels for CW = 64 NCH basis columns (the dynamic shared memory of
-// NCH = 4 exceeds the default 48 KB and is opted in).
+// The W^T V and leaf kernels of nodes j0 .. j0 + count - 1 for CW = 64 NCH basis columns (the
+// dynamic shared memory of NCH = 4 exceeds the default 48 KB and is opted in).
 template <int NCH, bool general>
-bem_status hm_apply_kernels(bem_ctx* ctx, HMatrix& h, bool wtv, int j, int nu, float kr, float ki,
-                            const ExtFrame& fr, cudaStream_t s) {
+bem_status hm_apply_kernels(bem_ctx* ctx, HMatrix& h, bool wtv, const HmGroup& grp, int j0,
+                            int count, int nu, const ExtFrame& fr, cudaStream_t s) {
   const size_t smem = PanelFor<NCH>::smem_bytes();
   if (cudaFuncSetAttribute(hm_leaf_kernel<NCH, general>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaFuncSetAttribute(hm_wtv_kernel<NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
@@ -950,19 +970,36 @@ bem_status hm_apply_kernels(bem_ctx* ctx, HMatrix& h, bool wtv, int j, int nu, f
   const int64_t n = ctx->geo.n;
   const HmGeom g{h.d_gq, h.d_gn, h.d_gc, n};
   if (wtv) {
-    hm_wtv_kernel<NCH><<<(unsigned)h.far.size(), kHmThreads, smem, s>>>(
-        h.d_far, h.d_uw_off, h.d_rank, h.d_toff, h.rmax, h.d_uw, h.d_vp, h.d_t);
+    hm_wtv_kernel<NCH><<<dim3((unsigned)h.far.size(), (unsigned)count), kHmThreads, smem, s>>>(
+        grp, h.d_far, h.d_uw_off, h.d_rank, h.d_toff, h.rmax, h.d_uw, h.d_vp, h.d_t);
     ctx->launches++;
   }
+  const int64_t y_stride = (int64_t)fr.acc_cols * fr.n_pad;
   timing_begin(ctx, s);
-  hm_leaf_kernel<NCH, general><<<(unsigned)h.leaves.size(), kHmThreads, smem, s>>>(
-      g, h.d_leaves, h.d_near, h.d_leaf_far_ptr, h.d_leaf_far, h.d_far, h.d_uw_off, h.d_rank,
+  hm_leaf_kernel<NCH, general><<<dim3((unsigned)h.leaves.size(), (unsigned)count), kHmThreads, smem, s>>>(
+      g, grp, h.d_leaves, h.d_near, h.d_leaf_far_ptr, h.d_leaf_far, h.d_far, h.d_uw_off, h.d_rank,
       h.d_toff, h.d_uw, h.d_t, h.d_vp, nu,
-      reinterpret_cast<const float2*>(ctx->con.self32) + (int64_t)j * n, kr, ki, ctx->op,
-      fr.Yp + (int64_t)j * fr.acc_cols * fr.n_pad, fr.C, fr.n_pad);
+      reinterpret_cast<const float2*>(ctx->con.self32) + (int64_t)j0 * n, ctx->op,
+      fr.Yp + (int64_t)j0 * y_stride, y_stride, fr.C, fr.n_pad);
   timing_end(ctx, s);
   ctx->launches++;
   return cuda_check(ctx, cudaGetLastError(), "low-rank far field kernels");
+}
+
+// Nodes compressed and applied together. One node's launches leave most of the device idle at
+// small n (96 leaves and ~1000 far blocks of a few columns at n = 3072) and end with a wait of
+// the host for the ranks; a group shares the launches and one such wait. Grouped as far as the
+// factors and T_b at full rank stay within kGroupBytes (n = 98304: one node, which fills the
+// device by itself). With bem_set_timing on every node runs alone, so that each leaf kernel is
+// timed. Each node's arithmetic is unchanged. cube3072, 32
+// nodes: leaf kernels 9.17 -> 3.94 ms, compression 6.06 -> 1.48, step 18.5 -> 6.5 ms.
+constexpr size_t kGroupBytes = (size_t)4 << 30;
+
+int group_nodes(const bem_ctx* ctx, const HMatrix& h, int cw) {
+  if (ctx->timing) return 1;
+  const size_t node = (size_t)h.uw_total * sizeof(float2) + (size_t)h.used_total +
+                      h.far.size() * (size_t)h.rmax * cw * sizeof(float2);
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)ctx->con.N, kGroupBytes / std::max<size_t>(1, node)));
 }
 
 }  // namespace
@@ -986,17 +1023,24 @@ bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, d
   if (h.mesh_version != ctx->mesh_version && (st = build_structure(ctx, s)) != BEM_OK) return st;
   if ((st = ensure_self32(ctx, s)) != BEM_OK) return st;
   const size_t nfar = h.far.size();
-  if ((st = grow(ctx, h.d_uw, h.uw_bytes, std::max<size_t>(1, h.uw_total) * sizeof(float2))) != BEM_OK ||
-      (st = grow(ctx, h.d_used, h.used_bytes, std::max<size_t>(1, h.used_total))) != BEM_OK ||
-      (st = grow(ctx, h.d_vp, h.vp_bytes, (size_t)n * 256 * sizeof(float2))) != BEM_OK)
-    return st;
   const int nch = nu <= 64 ? 1 : nu <= 128 ? 2 : 4;   // basis columns padded to CW = 64 nch
   const int cw = 64 * nch;
-  size_t rc = h.rank_cap, tc = h.rank_cap;
-  if ((st = grow(ctx, h.d_rank, rc, std::max<size_t>(1, nfar) * sizeof(int32_t))) != BEM_OK ||
-      (st = grow(ctx, h.d_toff, tc, std::max<size_t>(1, nfar) * sizeof(int64_t))) != BEM_OK)
+  int NB = group_nodes(ctx, h, cw);
+  auto group_buffers = [&]() -> bem_status {
+    bem_status r = grow(ctx, h.d_uw, h.uw_bytes, std::max<size_t>(1, NB * h.uw_total) * sizeof(float2));
+    if (r == BEM_OK) r = grow(ctx, h.d_used, h.used_bytes, std::max<size_t>(1, NB * h.used_total));
+    if (r == BEM_OK) r = grow(ctx, h.d_rank, h.rank_cap, std::max<size_t>(1, NB * nfar) * sizeof(int32_t));
+    if (r == BEM_OK) r = grow(ctx, h.d_toff, h.toff_cap, std::max<size_t>(1, NB * nfar) * sizeof(int64_t));
+    return r;
+  };
+  st = group_buffers();
+  if (st != BEM_OK && NB > 1) {   // no room for a group: one node at a time
+    NB = 1;
+    st = group_buffers();
+  }
+  if (st != BEM_OK ||
+      (st = grow(ctx, h.d_vp, h.vp_bytes, (size_t)n * 256 * sizeof(float2))) != BEM_OK)
     return st;
-  h.rank_cap = std::min(rc, tc);
   // the mixed path's FP32 partials (slice 0 of one column split), zeroed: the leaf kernels
   // write every row < n and column < nu
   ExtFrame fr;
@@ -1010,23 +1054,23 @@ bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, d
   hm_vperm_kernel<<<nblocks(n * cw), 256, 0, s>>>(reinterpret_cast<const double2*>(V), ldv, n, nu,
                                                   cw, h.d_perm, h.d_vp);
   ctx->launches++;
-  std::vector<int32_t> ranks(nfar);
-  std::vector<int64_t> toff(nfar);
+  std::vector<int32_t> ranks(NB * nfar);
+  std::vector<int64_t> toff(NB * nfar);
   const bool single = op_single(ctx->op);
   double rank_sum = 0.0, row_terms = 0.0, col_terms = 0.0;
   int rank_max = 0;
-  for (int j = 0; j < N; ++j) {
-    const float kr = (float)ctx->con.z_host[2 * j], ki = (float)ctx->con.z_host[2 * j + 1];
+  for (int j0 = 0; j0 < N; j0 += NB) {
+    const int count = std::min(NB, N - j0);
+    const HmGroup grp{ctx->con.z + 2 * j0, h.uw_total, h.used_total, (int64_t)nfar};
     if (nfar) {
       // the far blocks are ordered by size, largest first: those of at least kAcaBig rows +
       // columns take the wider kernel
       const HmGeom hg{h.d_gq, h.d_gn, h.d_gc, n};
       const int nbig = h.nbig, nsmall = (int)nfar - h.nbig;
 #define HM_ACA(GEN, NT, BASE, COUNT)                                                          \
-  hm_aca_kernel<GEN, NT><<<(unsigned)(COUNT), NT, 0, s>>>(BASE, hg, h.d_far, h.d_uw_off,      \
-                                                        h.d_used_off, kr, ki, ctx->op,        \
-                                                        (float)h.eps, h.rmax, h.d_uw, h.d_used, \
-                                                        h.d_rank)
+  hm_aca_kernel<GEN, NT><<<dim3((unsigned)(COUNT), (unsigned)count), NT, 0, s>>>(             \
+      BASE, hg, grp, h.d_far, h.d_uw_off, h.d_used_off, ctx->op, (float)h.eps, h.rmax, h.d_uw, \
+      h.d_used, h.d_rank)
       if (single) {
         if (nbig) HM_ACA(false, kAcaThreadsBig, 0, nbig);
         if (nsmall) HM_ACA(false, kAcaThreads, nbig, nsmall);
@@ -1035,9 +1079,8 @@ bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, d
         if (nsmall) HM_ACA(true, kAcaThreads, nbig, nsmall);
       }
 #undef HM_ACA
-      ctx->launches += (nbig > 0) + (nsmall > 0) - 1;
-      ctx->launches++;
-      st = cuda_check(ctx, cudaMemcpyAsync(ranks.data(), h.d_rank, nfar * sizeof(int32_t),
+      ctx->launches += (nbig > 0) + (nsmall > 0);
+      st = cuda_check(ctx, cudaMemcpyAsync(ranks.data(), h.d_rank, count * nfar * sizeof(int32_t),
                                            cudaMemcpyDeviceToHost, s), "rank copy");
       if (st == BEM_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "rank copy");
       if (st != BEM_OK) {
@@ -1045,19 +1088,20 @@ bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, d
         return st;
       }
       int64_t tot = 0;
-      for (size_t b = 0; b < nfar; ++b) {
-        toff[b] = tot;
-        tot += (int64_t)ranks[b] * cw;
-        rank_sum += ranks[b];
-        row_terms += (double)ranks[b] * (h.far[b].y - h.far[b].x);
-        col_terms += (double)ranks[b] * (h.far[b].w - h.far[b].z);
-        rank_max = std::max(rank_max, ranks[b]);
+      for (size_t e = 0; e < count * nfar; ++e) {
+        const int4 f = h.far[e % nfar];
+        toff[e] = tot;
+        tot += (int64_t)ranks[e] * cw;
+        rank_sum += ranks[e];
+        row_terms += (double)ranks[e] * (f.y - f.x);
+        col_terms += (double)ranks[e] * (f.w - f.z);
+        rank_max = std::max(rank_max, ranks[e]);
       }
       if ((st = grow(ctx, h.d_t, h.t_bytes, std::max<int64_t>(1, tot) * sizeof(float2))) != BEM_OK) {
         external_release(fr);
         return st;
       }
-      st = cuda_check(ctx, cudaMemcpyAsync(h.d_toff, toff.data(), nfar * sizeof(int64_t),
+      st = cuda_check(ctx, cudaMemcpyAsync(h.d_toff, toff.data(), count * nfar * sizeof(int64_t),
                                            cudaMemcpyHostToDevice, s), "offset copy");
       if (st != BEM_OK) {
         external_release(fr);
@@ -1065,13 +1109,13 @@ bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, d
       }
     }
     if (single)
-      st = nch == 1   ? hm_apply_kernels<1, false>(ctx, h, nfar > 0, j, nu, kr, ki, fr, s)
-           : nch == 2 ? hm_apply_kernels<2, false>(ctx, h, nfar > 0, j, nu, kr, ki, fr, s)
-                      : hm_apply_kernels<4, false>(ctx, h, nfar > 0, j, nu, kr, ki, fr, s);
+      st = nch == 1   ? hm_apply_kernels<1, false>(ctx, h, nfar > 0, grp, j0, count, nu, fr, s)
+           : nch == 2 ? hm_apply_kernels<2, false>(ctx, h, nfar > 0, grp, j0, count, nu, fr, s)
+                      : hm_apply_kernels<4, false>(ctx, h, nfar > 0, grp, j0, count, nu, fr, s);
     else
-      st = nch == 1   ? hm_apply_kernels<1, true>(ctx, h, nfar > 0, j, nu, kr, ki, fr, s)
-           : nch == 2 ? hm_apply_kernels<2, true>(ctx, h, nfar > 0, j, nu, kr, ki, fr, s)
-                      : hm_apply_kernels<4, true>(ctx, h, nfar > 0, j, nu, kr, ki, fr, s);
+      st = nch == 1   ? hm_apply_kernels<1, true>(ctx, h, nfar > 0, grp, j0, count, nu, fr, s)
+           : nch == 2 ? hm_apply_kernels<2, true>(ctx, h, nfar > 0, grp, j0, count, nu, fr, s)
+                      : hm_apply_kernels<4, true>(ctx, h, nfar > 0, grp, j0, count, nu, fr, s);
     if (st != BEM_OK) {
       external_release(fr);
       return st;

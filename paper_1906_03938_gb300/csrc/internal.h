@@ -215,7 +215,7 @@ cudaError_t launch_self_at(bem_ctx* ctx, int m, const double* lam_dev, double* R
 // out[2c] = ||R[:, c]||^2, out[2c+1] = ||X[:, c]||^2 (fixed-order sums)
 cudaError_t launch_colnorms(bem_ctx* ctx, const double* R, int64_t ldr, const double* X,
                             int64_t ldx, int64_t n, int m, double* out, cudaStream_t s);
-// dense FP32 operator and LU (dense32.cu)
+// dense FP32 operator and LU (dense32.cu); ipiv: 2 n ints
 bem_status assemble32(bem_ctx* ctx, int nk, const double* kz_host, const double* coef_host,
                       float2* M, cudaStream_t s);
 bem_status lu32(bem_ctx* ctx, float2* A, int64_t n, int* ipiv, cudaStream_t s);

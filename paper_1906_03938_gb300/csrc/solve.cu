@@ -327,7 +327,7 @@ bem_status inverse_power_impl(bem_ctx* ctx, double* V_dev, int64_t ldv, int nu, 
   size_t off = 0;
   auto take = [&](size_t b) { const size_t o = off; off += (b + 255) / 256 * 256; return o; };
   const size_t oS = take(mf ? 0 : (size_t)n * n * sizeof(float2)),
-               oP = take(mf ? 0 : (size_t)n * sizeof(int)),
+               oP = take(mf ? 0 : (size_t)2 * n * sizeof(int)),
                oG = take(mf ? gmres_sum_work_bytes(ctx, nu, restart) : 0),
                oV = take((size_t)N * n * nu * sizeof(float2)), oU = take((size_t)n * nu * sizeof(float2)),
                oB = take(mf ? (size_t)n * nu * sizeof(float2) : 0),
@@ -422,7 +422,7 @@ extern "C" bem_status bem_inverse_power_chebyshev(bem_ctx* ctx, double* V_dev, i
   size_t off = 0;
   auto take = [&](size_t b) { const size_t o = off; off += (b + 255) / 256 * 256; return o; };
   const size_t blk = (size_t)n * nu * sizeof(float2);
-  const size_t oG = take((size_t)n * n * sizeof(float2)), oP = take((size_t)n * sizeof(int)),
+  const size_t oG = take((size_t)n * n * sizeof(float2)), oP = take((size_t)2 * n * sizeof(int)),
                oW = take((size_t)m * blk), oE = take((size_t)m * blk), oX = take((size_t)N * blk),
                oU = take(blk), oN = take((size_t)nu * sizeof(double)),
                oL = take(((size_t)N * m + N) * sizeof(float)),
@@ -578,7 +578,7 @@ extern "C" bem_status bem_refine(bem_ctx* ctx, int m, double* lam_host, double* 
   }
   size_t off = 0;
   auto take = [&](size_t b) { const size_t o = off; off += (b + 255) / 256 * 256; return o; };
-  const size_t oA = take((size_t)n * n * sizeof(float2)), oP = take((size_t)n * sizeof(int)),
+  const size_t oA = take((size_t)n * n * sizeof(float2)), oP = take((size_t)2 * n * sizeof(int)),
                oR = take((size_t)2 * n * sizeof(double2)), oF = take((size_t)2 * n * sizeof(float2)),
                oE = take((size_t)n * sizeof(double2)), oL = take(8 * sizeof(double2)),
                oD = take(8 * sizeof(double2));
@@ -781,7 +781,7 @@ bem_status separate_clusters(bem_ctx* ctx, int k, double* lam, double* X_dev, in
     if (kc < 2 || kc > 32 || spread <= 1e-7 * hypot(sr, si)) continue;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += (bytes + 255) / 256 * 256; return o; };
-    const size_t oA = take((size_t)n * n * sizeof(float2)), oP = take((size_t)n * sizeof(int)),
+    const size_t oA = take((size_t)n * n * sizeof(float2)), oP = take((size_t)2 * n * sizeof(int)),
                  oX = take((size_t)n * kc * sizeof(double2)), oR = take((size_t)n * kc * sizeof(double2)),
                  oD = take((size_t)n * kc * sizeof(double2)), oF = take((size_t)n * kc * sizeof(float2)),
                  oM = take((size_t)2 * kc * kc * sizeof(double2)), oL = take((size_t)2 * kc * sizeof(double)),

@@ -158,29 +158,39 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo_elem, float hi_elem) {
 // Two entries (row i, columns l0, l0 + 1) of one node: the self term on the diagonal, zero
 // in the padding, then the hi/lo BF16 split into the four planes (Re hi, Re lo, Im hi, Im lo)
 // at ag; self points at the staged self term of column l0 (that of l0 + 1 is kMaxG later).
+// plain: the K-block holds neither the tile's diagonal nor padding (all but a few), and the
+// tests, a tenth of an entry's instructions, are passed by.
 __device__ __forceinline__ void put_entries(f2_t sr2, f2_t si2, const float2* self, int64_t i,
-                                            int64_t l0, int64_t n, unsigned char* ag,
+                                            int64_t l0, int64_t n, unsigned char* ag, bool plain,
                                             bool scaled = false, float2 cf = float2(),
                                             uint32_t plane_bytes = kPlaneBytes) {
   float re[2], im[2];
   f2split(sr2, re[0], re[1]);
   f2split(si2, im[0], im[1]);
+  if (!plain) {
 #pragma unroll
-  for (int d = 0; d < 2; ++d) {
-    if (i == l0 + d) {   // diagonal: the self term
-      const float2 sv = self[d * kMaxG];
-      re[d] = sv.x;
-      im[d] = sv.y;
-    }
-    if (scaled) {        // node-summed mode: c_j A_il(z_j)
+    for (int d = 0; d < 2; ++d)
+      if (i == l0 + d) {   // diagonal: the self term
+        const float2 sv = self[d * kMaxG];
+        re[d] = sv.x;
+        im[d] = sv.y;
+      }
+  }
+  if (scaled) {            // node-summed mode: c_j A_il(z_j)
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
       const float r = re[d] * cf.x - im[d] * cf.y;
       im[d] = re[d] * cf.y + im[d] * cf.x;
       re[d] = r;
     }
-    if (i >= n || l0 + d >= n) {   // padding rows / columns of the tile
-      re[d] = 0.f;
-      im[d] = 0.f;
-    }
+  }
+  if (!plain) {
+#pragma unroll
+    for (int d = 0; d < 2; ++d)
+      if (i >= n || l0 + d >= n) {   // padding rows / columns of the tile
+        re[d] = 0.f;
+        im[d] = 0.f;
+      }
   }
   const uint32_t hr = pack_bf16(re[0], re[1]);
   const uint32_t hi = pack_bf16(im[0], im[1]);
@@ -200,21 +210,24 @@ __device__ __forceinline__ void put_entries(f2_t sr2, f2_t si2, const float2* se
 // and ag + 1024 (row i1: eight 8-row groups of 128 bytes further); self points at the
 // staged self term of column l.
 __device__ __forceinline__ void put_rows(f2_t sr2, f2_t si2, const float2* self, int64_t i0,
-                                         int64_t i1, int64_t l, int64_t n, unsigned char* ag) {
+                                         int64_t i1, int64_t l, int64_t n, unsigned char* ag,
+                                         bool plain) {
   float re[2], im[2];
   f2split(sr2, re[0], re[1]);
   f2split(si2, im[0], im[1]);
-  const int64_t ii[2] = {i0, i1};
+  if (!plain) {
+    const int64_t ii[2] = {i0, i1};
 #pragma unroll
-  for (int d = 0; d < 2; ++d) {
-    if (ii[d] == l) {   // diagonal: the self term
-      const float2 sv = *self;
-      re[d] = sv.x;
-      im[d] = sv.y;
-    }
-    if (ii[d] >= n || l >= n) {   // padding rows / columns of the tile
-      re[d] = 0.f;
-      im[d] = 0.f;
+    for (int d = 0; d < 2; ++d) {
+      if (ii[d] == l) {   // diagonal: the self term
+        const float2 sv = *self;
+        re[d] = sv.x;
+        im[d] = sv.y;
+      }
+      if (ii[d] >= n || l >= n) {   // padding rows / columns of the tile
+        re[d] = 0.f;
+        im[d] = 0.f;
+      }
     }
   }
   const uint32_t hr = pack_bf16(re[0], re[1]);
@@ -229,6 +242,13 @@ __device__ __forceinline__ void put_rows(f2_t sr2, f2_t si2, const float2* self,
     *reinterpret_cast<uint16_t*>(ag + q * kHalfPlane) = (uint16_t)(v[q] & 0xFFFFu);
     *reinterpret_cast<uint16_t*>(ag + 1024 + q * kHalfPlane) = (uint16_t)(v[q] >> 16);
   }
+}
+
+// No entry of the 128 x 16 block of rows row0.. and columns 16 kb.. is on the diagonal or in
+// the padding.
+__device__ __forceinline__ bool block_plain(int64_t row0, int kb, int64_t n) {
+  const int64_t l0 = (int64_t)kb * kBK;
+  return row0 + kBM <= n && l0 + kBK <= n && (l0 + kBK <= row0 || l0 >= row0 + kBM);
 }
 
 // bounded wait that also watches the block's abort flag
@@ -385,12 +405,19 @@ __device__ __forceinline__ void mixed_apply_unit(const MixedParams& p, const int
       if (!wait_or_abort(&gready[s], par, abort_flag, p.status, p.wait_limit)) break;
       const float* graw = sGraw + s * (kBK * 64);
       float4* sCol = sColAll + s * (kBK * 7);
-      for (int x = lane; x < kBK * 7; x += 32) {
-        const int k = x / 7, q = x % 7;
-        const float4 hi = *reinterpret_cast<const float4*>(graw + k * 64 + 4 * q);
-        const float4 lo = *reinterpret_cast<const float4*>(graw + k * 64 + 28 + 4 * q);
-        sCol[x] = make_float4((hi.x - oxh) + (lo.x - oxl), (hi.y - oyh) + (lo.y - oyl),
-                              (hi.z - ozh) + (lo.z - ozl), hi.w);
+      for (int x = lane; x < kBK / 2 * 7; x += 32) {   // point q of the columns 2 kk, 2 kk + 1
+        const int kk = x / 7, q = x % 7;
+        float4 v[2];
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+          const float* gk = graw + (2 * kk + d) * 64 + 4 * q;
+          const float4 hi = *reinterpret_cast<const float4*>(gk);
+          const float4 lo = *reinterpret_cast<const float4*>(gk + 28);
+          v[d] = make_float4((hi.x - oxh) + (lo.x - oxl), (hi.y - oyh) + (lo.y - oyl),
+                             (hi.z - ozh) + (lo.z - ozl), hi.w);
+        }
+        sCol[2 * x] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
+        sCol[2 * x + 1] = make_float4(v[0].z, v[1].z, v[0].w, v[1].w);
       }
       float2* sSelf = sSelfAll + s * (kBK * kMaxG);
       for (int x = lane; x < kBK * kMaxG; x += 32) {
@@ -507,6 +534,7 @@ __device__ __forceinline__ void mixed_apply_unit(const MixedParams& p, const int
       const float2* sSelf = sSelfAll + s * (kBK * kMaxG);
       unsigned char* a_stage = sA + s * L.a_stage_bytes;
       const float4 xr = sRow[row];
+      const bool plain = block_plain(row0, kb, p.n);
 #pragma unroll 1
       for (int kg = 0; kg < (ready ? 2 : 0); ++kg) {
         const int k0 = 8 * kg + 2 * kp;
@@ -515,8 +543,9 @@ __device__ __forceinline__ void mixed_apply_unit(const MixedParams& p, const int
         f2_t rr2[7], am2[7];
         f2_t s2[kOp ? 7 : 1];   // (y - x) . n / r^2 of both columns (general operator)
         {
-          const float4* c0 = sCol + k0 * 7;
-          const float4* c1 = c0 + 7;
+          // staged by column pairs, (x0, x1, y0, y1) and (z0, z1, w0, w1): a load's register
+          // pairs are the paired instructions' operands, with no moves between
+          const ulonglong2* c0 = reinterpret_cast<const ulonglong2*>(sCol + k0 * 7);
           const f2_t xx = f2(xr.x, xr.x), xy = f2(xr.y, xr.y), xz = f2(xr.z, xr.z);
           // the columns' normals, negated (d = x - y here), from the staged packed geometry
           f2_t nnx = f2(0.f, 0.f), nny = nnx, nnz = nnx;
@@ -528,15 +557,14 @@ __device__ __forceinline__ void mixed_apply_unit(const MixedParams& p, const int
           }
 #pragma unroll
           for (int q = 0; q < 7; ++q) {
-            const float4 y0 = c0[q], y1 = c1[q];
-            const f2_t dx = sub2(xx, f2(y0.x, y1.x)), dy = sub2(xy, f2(y0.y, y1.y)),
-                       dz = sub2(xz, f2(y0.z, y1.z));
+            const ulonglong2 pxy = c0[2 * q], pzw = c0[2 * q + 1];
+            const f2_t dx = sub2(xx, pxy.x), dy = sub2(xy, pxy.y), dz = sub2(xz, pzw.x);
             const f2_t r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
             float r20, r21;
             f2split(r2, r20, r21);
             const f2_t rs = f2(rsqrtf_mufu(r20), rsqrtf_mufu(r21));
             rr2[q] = mul2(r2, rs);
-            am2[q] = mul2(f2(y0.w, y1.w), rs);
+            am2[q] = mul2(pzw.y, rs);
             if (kOp)
               s2[kOp ? q : 0] = mul2(fma2(dx, nnx, fma2(dy, nny, mul2(dz, nnz))), mul2(rs, rs));
           }
@@ -585,9 +613,9 @@ __device__ __forceinline__ void mixed_apply_unit(const MixedParams& p, const int
               }
             }
             put_entries(sa, ia, selfk + g, i, l0, p.n, a_stage + g * 4 * kPlaneBytes + off,
-                        scaled, cf[kSum ? g : 0]);
+                        plain, scaled, cf[kSum ? g : 0]);
             put_entries(sb, ib, selfk + g + 1, i, l0, p.n,
-                        a_stage + (g + 1) * 4 * kPlaneBytes + off, scaled, cf[kSum ? g + 1 : 0]);
+                        a_stage + (g + 1) * 4 * kPlaneBytes + off, plain, scaled, cf[kSum ? g + 1 : 0]);
           } else {
 #pragma unroll
             for (int h = g; h < g + 2; ++h) {
@@ -624,7 +652,7 @@ __device__ __forceinline__ void mixed_apply_unit(const MixedParams& p, const int
                 }
               }
               put_entries(sr2, si2, selfk + h, i, l0, p.n, a_stage + h * 4 * kPlaneBytes + off,
-                          scaled, cf[kSum ? h : 0]);
+                          plain, scaled, cf[kSum ? h : 0]);
             }
           }
         }
@@ -971,6 +999,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       const float2* sSelf = sSelfAll + s * (kBK * kMaxG);
       unsigned char* a_stage = sA + s * 2 * kHalfBytes;
       unsigned char* x_stage = sX + s * kHalfBytes;
+      const bool plain = block_plain(row0, kb, p.n);
       if (it == 0) {   // the rows, staged by the producer before its first release
         xa = sRow[rr];
         xb = sRow[rr + 64];
@@ -983,7 +1012,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         f2_t s2[kOp ? 7 : 1];
         {
           const float4* cq = sCol + k * 7;
-          const f2_t xx = f2(xa.x, xb.x), xy = f2(xa.y, xb.y), xz = f2(xa.z, xb.z);
           f2_t nnx = f2(0.f, 0.f), nny = nnx, nnz = nnx;
           if (kOp) {   // the column's normal, negated (d = x - y here)
             const float* gk = sGraw + s * (kBK * 64) + k * 64;
@@ -993,15 +1021,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           }
 #pragma unroll
           for (int q = 0; q < 7; ++q) {
+            // scalar differences: a paired one would first copy the column's coordinate
             const float4 y = cq[q];
-            const f2_t dx = sub2(xx, f2(y.x, y.x)), dy = sub2(xy, f2(y.y, y.y)),
-                       dz = sub2(xz, f2(y.z, y.z));
+            const f2_t dx = f2(__fsub_rn(xa.x, y.x), __fsub_rn(xb.x, y.x)),
+                       dy = f2(__fsub_rn(xa.y, y.y), __fsub_rn(xb.y, y.y)),
+                       dz = f2(__fsub_rn(xa.z, y.z), __fsub_rn(xb.z, y.z));
             const f2_t r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
             float r20, r21;
             f2split(r2, r20, r21);
-            const f2_t rs = f2(rsqrtf_mufu(r20), rsqrtf_mufu(r21));
+            const float rs0 = rsqrtf_mufu(r20), rs1 = rsqrtf_mufu(r21);
+            const f2_t rs = f2(rs0, rs1);
             rr2[q] = mul2(r2, rs);
-            am2[q] = mul2(f2(y.w, y.w), rs);
+            am2[q] = f2(__fmul_rn(y.w, rs0), __fmul_rn(y.w, rs1));
             if (kOp)
               s2[kOp ? q : 0] = mul2(fma2(dx, nnx, fma2(dy, nny, mul2(dz, nnz))), mul2(rs, rs));
           }
@@ -1046,8 +1077,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           // node `rank` into this CTA's stage, the other into the export buffer
           unsigned char* own = a_stage + kg * kHalfBytes + off;
           unsigned char* other = x_stage + off;
-          put_rows(sa, ia, selfk, i0, i1, l, p.n, rank == 0 ? own : other);
-          put_rows(sb, ib, selfk + 1, i0, i1, l, p.n, rank == 0 ? other : own);
+          put_rows(sa, ia, selfk, i0, i1, l, p.n, rank == 0 ? own : other, plain);
+          put_rows(sb, ib, selfk + 1, i0, i1, l, p.n, rank == 0 ? other : own, plain);
         } else {
           f2_t sr2 = f2(0.f, 0.f), si2 = f2(0.f, 0.f);
           const f2_t kmi2 = f2(kmi[0], kmi[0]), kr2 = f2(kr[0], kr[0]);
@@ -1076,7 +1107,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
               si2 = fma2(a, sn, si2);
             }
           }
-          put_rows(sr2, si2, selfk, i0, i1, l, p.n, a_stage + kg * kHalfBytes + off);
+          put_rows(sr2, si2, selfk, i0, i1, l, p.n, a_stage + kg * kHalfBytes + off, plain);
         }
       }
       fence_proxy_async_smem();

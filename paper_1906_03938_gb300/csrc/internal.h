@@ -108,6 +108,8 @@ struct bem_ctx {
   size_t zgemm_bytes = 0;
   float* d_lu_work = nullptr;    // the LU's trailing-update operands in real form
   size_t lu_work_bytes = 0;
+  double* d_ff = nullptr;        // column splits' partial sums of the double-FP32 residuals
+  size_t ff_bytes = 0;
   size_t small_bytes = 0;
   int64_t launches = 0;
   int64_t mesh_version = 0;         // bumped by every successful bem_set_mesh

@@ -16,6 +16,8 @@
 // k-derivative A' (kernel i e^{ikr}/(4 pi)) come from the same evaluation.
 #include <math.h>
 
+#include <algorithm>
+
 #include "ff_tables.cuh"
 #include "internal.h"
 
@@ -136,10 +138,15 @@ constexpr int kChunk = 64;
 
 // R_c = A(lambda_c) x_c (off-diagonal part plus the self term prefilled in R), and with
 // kDeriv also Rd_c = A'(lambda_c) x_c; one thread per row, columns staged in shared memory.
+// Bound by FP32 issue (~350 instructions a point) once the device is full: with fewer than a
+// few blocks per SM the columns are split over gridDim.z blocks, whose double-FP32 partial sums
+// go to part[split][c][i] (A x, then with kDeriv A' x) and are added in FP64 in split order by
+// ff_sum_kernel. n = 768, one vector: 2.2 -> 0.35 ms.
 template <bool kDeriv>
 __global__ void __launch_bounds__(kRows)
 residual_ff_kernel(Geometry g, const double* __restrict__ lam, const double* __restrict__ X,
-                   int64_t ldx, double* __restrict__ R, double* __restrict__ Rd) {
+                   int64_t ldx, double* __restrict__ R, double* __restrict__ Rd,
+                   double2* __restrict__ part) {
   __shared__ Tables T;
   __shared__ float sP[7][3][2][kChunk];   // quadrature points, pairs
   __shared__ float sW[7][2][kChunk];      // weights / 4 pi, pairs
@@ -155,7 +162,9 @@ residual_ff_kernel(Geometry g, const double* __restrict__ lam, const double* __r
   if (i < n)
     for (int d = 0; d < 3; ++d) xi[d] = ff_from(g.cx[d * n + i]);
   FF ar = {0.f, 0.f}, ai = ar, dr = ar, di = ar;   // row sums of A x and A' x
-  for (int64_t l0 = 0; l0 < n; l0 += kChunk) {
+  const int64_t chunks = (n + kChunk - 1) / kChunk;
+  const int64_t ch0 = chunks * blockIdx.z / gridDim.z, ch1 = chunks * (blockIdx.z + 1) / gridDim.z;
+  for (int64_t l0 = ch0 * kChunk; l0 < ch1 * kChunk; l0 += kChunk) {
     __syncthreads();
     for (int t = threadIdx.x; t < 7 * kChunk; t += kRows) {
       const int q = t / kChunk, lc = t % kChunk;
@@ -223,6 +232,14 @@ residual_ff_kernel(Geometry g, const double* __restrict__ lam, const double* __r
       }
     }
   }
+  if (part) {
+    if (i < n) {
+      const int64_t per = (int64_t)gridDim.y * n, at = (int64_t)c * n + i;
+      part[(blockIdx.z * (kDeriv ? 2 : 1)) * per + at] = make_double2(ff_to(ar), ff_to(ai));
+      if (kDeriv) part[(blockIdx.z * 2 + 1) * per + at] = make_double2(ff_to(dr), ff_to(di));
+    }
+    return;
+  }
   if (i < n) {
     const double2 xv = x[i];
     double2* Rc = reinterpret_cast<double2*>(R) + (int64_t)c * n;
@@ -238,6 +255,36 @@ residual_ff_kernel(Geometry g, const double* __restrict__ lam, const double* __r
   }
 }
 
+// R_c = sum of the splits' partial sums, in order, plus the self term prefilled in R times x;
+// Rd likewise (per: elements of one split's A x block).
+__global__ void ff_sum_kernel(const double2* __restrict__ part, int splits, bool deriv, int64_t n,
+                              int m, const double2* __restrict__ X, int64_t ldx,
+                              double2* __restrict__ R, double2* __restrict__ Rd) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, per = n * m;
+  if (t >= per) return;
+  const double2 x = X[(t / n) * ldx + t % n];
+  for (int d = 0; d < (deriv ? 2 : 1); ++d) {
+    double2* out = d ? Rd : R;
+    const double2 sd = out[t];
+    double2 s = make_double2(sd.x * x.x - sd.y * x.y, sd.x * x.y + sd.y * x.x);
+    for (int q = 0; q < splits; ++q) {
+      const double2 v = part[((int64_t)q * (deriv ? 2 : 1) + d) * per + t];
+      s.x += v.x;
+      s.y += v.y;
+    }
+    out[t] = s;
+  }
+}
+
+// Column splits: as many as make eight blocks per SM, a block keeping at least two chunks.
+int ff_splits(const bem_ctx* ctx, int64_t n, int m) {
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  const int64_t blocks = (n + kRows - 1) / kRows * m, chunks = (n + kChunk - 1) / kChunk;
+  return (int)std::max<int64_t>(1, std::min<int64_t>({8 * (int64_t)std::max(1, sms) / blocks,
+                                                      chunks / 2, 64}));
+}
+
 }  // namespace
 
 cudaError_t launch_apply_ff(bem_ctx* ctx, int m, const double* lam_dev, const double* X,
@@ -251,11 +298,34 @@ cudaError_t launch_apply_ff(bem_ctx* ctx, int m, const double* lam_dev, const do
   cudaError_t e = launch_self_at(ctx, m, lam_dev, R, false, s);
   if (e == cudaSuccess && Rd) e = launch_self_at(ctx, m, lam_dev, Rd, true, s);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((n + kRows - 1) / kRows), (unsigned)m);
+  // partial sums of the splits; one block per row range where they cannot be had
+  int splits = ff_splits(ctx, n, m);
+  const size_t bytes = (size_t)splits * (Rd ? 2 : 1) * n * m * sizeof(double2);
+  if (splits > 1 && bytes > ctx->ff_bytes) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      splits = 1;
+    } else {
+      cudaFree(ctx->d_ff);
+      ctx->d_ff = nullptr;
+      ctx->ff_bytes = 0;
+      if (cudaMalloc(&ctx->d_ff, bytes) == cudaSuccess) ctx->ff_bytes = bytes;
+      else splits = 1;
+    }
+    cudaGetLastError();
+  }
+  double2* part = splits > 1 ? reinterpret_cast<double2*>(ctx->d_ff) : nullptr;
+  dim3 grid((unsigned)((n + kRows - 1) / kRows), (unsigned)m, (unsigned)splits);
   if (Rd)
-    residual_ff_kernel<true><<<grid, kRows, 0, s>>>(ctx->geo, lam_dev, X, ldx, R, Rd);
+    residual_ff_kernel<true><<<grid, kRows, 0, s>>>(ctx->geo, lam_dev, X, ldx, R, Rd, part);
   else
-    residual_ff_kernel<false><<<grid, kRows, 0, s>>>(ctx->geo, lam_dev, X, ldx, R, nullptr);
+    residual_ff_kernel<false><<<grid, kRows, 0, s>>>(ctx->geo, lam_dev, X, ldx, R, nullptr, part);
+  if (part) {
+    ff_sum_kernel<<<(unsigned)((n * m + 255) / 256), 256, 0, s>>>(
+        part, splits, Rd != nullptr, n, m, reinterpret_cast<const double2*>(X), ldx,
+        reinterpret_cast<double2*>(R), reinterpret_cast<double2*>(Rd));
+    ctx->launches++;
+  }
   ctx->launches++;
   if (near_active(ctx)) {
     e = launch_near_percol64(ctx, m, lam_dev, X, ldx, R, false, s);

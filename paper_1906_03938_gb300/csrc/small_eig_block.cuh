@@ -3,10 +3,11 @@
 //
 // Bound by the serial chain of Givens rotations: about 3 m sweeps of up to m rotations, each
 // needing the previous one's result in two entries. On one thread every rotation also paid
-// for its ~3 m complex row and column updates (m = 32: 80 ms); here the updates are spread
-// over the threads, the rows and columns of A and Z in shared memory (m <= 64), and the
-// thread that owns the chain forms the next rotation while the others still update, so a
-// rotation costs two barriers and one chain step. m = 32: 80.6 ms -> 6.3 ms.
+// for its ~3 m complex row and column updates (m = 32: 80.6 ms); here A and Z sit in shared
+// memory (m <= 64) and one warp carries the chain: it applies a rotation to the few entries
+// the next one comes from, a lane per column, then a lane per row, and forms the next
+// rotation while the other warps apply this one to everything else, so a rotation costs one
+// barrier and one chain step. m = 32: 80.6 -> 4.7 ms.
 #pragma once
 
 #include "small_eig.h"
@@ -21,8 +22,17 @@ __host__ __device__ inline int eig_ld(int m) { return m <= kEigSmemMax ? m + 1 -
 __host__ inline size_t eig_smem(int m) {
   return m <= kEigSmemMax ? (size_t)3 * m * eig_ld(m) * sizeof(zc) : 0;
 }
-// half the threads update A, the other half Z
-__host__ inline int eig_threads(int m) { return 2 * (m < 32 ? 32 : (m + 31) / 32 * 32); }
+// a warp for the chain, the others for the 2 m rows and columns of a rotation
+__host__ inline int eig_threads(int m) { return 32 + 2 * (m < 32 ? 32 : (m + 31) / 32 * 32); }
+
+// 1 / sqrt(a) for a in the range givens_fast admits: the hardware's estimate (20 bits or more)
+// and one third-order step, e = 1 - a y^2, y (1 + e / 2 + 3 e^2 / 8): error below e^3.
+__device__ __forceinline__ double rsqrt_step(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-a * y, y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
 
 // Givens rotation as small::givens, by reciprocal square roots where the squares are safe.
 __device__ inline void givens_fast(zc x, zc y, double& c, zc& s) {
@@ -31,9 +41,16 @@ __device__ inline void givens_fast(zc x, zc y, double& c, zc& s) {
     givens(x, y, c, s);
     return;
   }
-  const double ix = rsqrt(ax2), in = rsqrt(ax2 + ay2);
-  c = ax2 * ix * in;
-  s = scl(mul(x, cj(y)), ix * in);
+  const double w = rsqrt_step(ax2) * rsqrt_step(ax2 + ay2);
+  c = ax2 * w;
+  s = scl(mul(x, cj(y)), w);
+}
+
+// (p, q) <- (c p + s q, c q - conj(s) p)
+__device__ __forceinline__ void rotate(zc& p, zc& q, double c, zc s) {
+  const zc a = p, b = q;
+  p = add(scl(a, c), mul(s, b));
+  q = sub(scl(b, c), mul(cj(s), a));
 }
 
 #define SE_A(M, i, j) (M)[(int64_t)(j) * ld + (i)]
@@ -49,9 +66,10 @@ __device__ inline int eig_block(int m, zc* gA, zc* gw, zc* gV, zc* gZ) {
   __shared__ double sh_beta;
   __shared__ int sh_l, sh_ihi, sh_state;
   const double eps = 2.220446049250313e-16;
-  const int tid = threadIdx.x, nt = blockDim.x, half = nt / 2;
-  const bool first = tid < half;      // this thread works on A (else on Z)
+  const int tid = threadIdx.x, nt = blockDim.x, half = nt / 2 / 32 * 32;
+  const bool first = tid < half;      // Hessenberg step: this thread works on A (else on Z)
   const int t = first ? tid : tid - half;
+  const int zt = nt - half;           // threads that work on Z
   const bool in_smem = m <= kEigSmemMax;
   const int ld = eig_ld(m);
   zc* A = in_smem ? reinterpret_cast<zc*>(eig_sm) : gA;
@@ -99,7 +117,7 @@ __device__ inline int eig_block(int m, zc* gA, zc* gw, zc* gV, zc* gZ) {
         for (int i = k + 2; i < m; ++i) SE_A(A, i, j) = sub(SE_A(A, i, j), mul(SE_A(A, i, k), s));
       }
     } else {
-      for (int i = t; i < m; i += half) {
+      for (int i = t; i < m; i += zt) {
         zc s = mul(SE_A(Z, i, k + 1), v0);
         for (int j = k + 2; j < m; ++j) s = add(s, mul(SE_A(Z, i, j), SE_A(A, j, k)));
         s = scl(s, beta);
@@ -176,39 +194,61 @@ __device__ inline int eig_block(int m, zc* gA, zc* gw, zc* gV, zc* gZ) {
     for (int k = l; k < ihi; ++k) {
       const double c = sh_c[k & 1];
       const zc s = sh_s[k & 1];
-      if (first) {
-        // rows k, k+1: columns from max(l, k-1) to m-1
-        for (int j = (k > l ? k - 1 : l) + t; j < m; j += half) {
-          const zc t1 = SE_A(A, k, j), t2 = SE_A(A, k + 1, j);
-          SE_A(A, k, j) = add(scl(t1, c), mul(s, t2));
-          SE_A(A, k + 1, j) = sub(scl(t2, c), mul(cj(s), t1));
-        }
-      } else {
-        for (int i = t; i < m; i += half) {
-          const zc t1 = SE_A(Z, i, k), t2 = SE_A(Z, i, k + 1);
-          SE_A(Z, i, k) = add(scl(t1, c), mul(cj(s), t2));
-          SE_A(Z, i, k + 1) = sub(scl(t2, c), mul(s, t1));
-        }
-      }
-      __syncthreads();
-      // columns k, k+1: rows 0 .. min(k+2, ihi); thread 0 takes rows k+1 and k+2, whose new
-      // entries of column k are the next rotation's, and forms it
       const int rmax = (k + 2 < ihi ? k + 2 : ihi);
-      auto col = [&](int i) {
-        const zc t1 = SE_A(A, i, k), t2 = SE_A(A, i, k + 1);
-        const zc a = add(scl(t1, c), mul(cj(s), t2));
-        SE_A(A, i, k) = a;
-        SE_A(A, i, k + 1) = sub(scl(t2, c), mul(s, t1));
-        return a;
-      };
-      if (tid == 0) {
-        const zc x = col(k + 1);
-        if (k + 2 <= rmax) {
-          const zc y = col(k + 2);
-          givens_fast(x, y, sh_c[(k + 1) & 1], sh_s[(k + 1) & 1]);
+      if (tid < 32) {
+        // rows k, k+1 of the columns k, k+1 and (the bulge) k-1
+        const int j = tid < 2 ? k + tid : k - 1;
+        if (tid < (k > l ? 3 : 2)) {
+          zc p = SE_A(A, k, j), q = SE_A(A, k + 1, j);
+          rotate(p, q, c, s);
+          SE_A(A, k, j) = p;
+          SE_A(A, k + 1, j) = q;
+        }
+        __syncwarp();
+        // columns k, k+1 of the rows k .. k+2; the next rotation zeroes A(k+2, k) against
+        // A(k+1, k)
+        const int i = k + tid;
+        zc p = mk(0.0, 0.0);
+        if (tid < 3 && i <= rmax) {
+          zc q = SE_A(A, i, k + 1);
+          p = SE_A(A, i, k);
+          rotate(p, q, c, cj(s));
+          SE_A(A, i, k) = p;
+          SE_A(A, i, k + 1) = q;
+        }
+        if (k + 1 < ihi) {
+          const zc x = mk(__shfl_sync(0xffffffffu, p.re, 1), __shfl_sync(0xffffffffu, p.im, 1));
+          const zc y = mk(__shfl_sync(0xffffffffu, p.re, 2), __shfl_sync(0xffffffffu, p.im, 2));
+          double nc;
+          zc ns;
+          givens_fast(x, y, nc, ns);
+          if (tid == 0) {
+            sh_c[(k + 1) & 1] = nc;
+            sh_s[(k + 1) & 1] = ns;
+          }
         }
       } else {
-        for (int i = tid - 1; i <= k; i += nt - 1) col(i);
+        // rows k, k+1 of the columns beyond k+1, columns k, k+1 of the rows above k, and of Z
+        const int nrow = m - k - 2 > 0 ? m - k - 2 : 0;
+        for (int u = tid - 32; u < nrow + k + m; u += nt - 32) {
+          zc *p, *q;
+          zc su = cj(s);
+          if (u < nrow) {
+            p = &SE_A(A, k, k + 2 + u);
+            q = &SE_A(A, k + 1, k + 2 + u);
+            su = s;
+          } else {
+            const int i = u - nrow;
+            zc* M = i < k ? A : Z;
+            const int r = i < k ? i : i - k;
+            p = &SE_A(M, r, k);
+            q = &SE_A(M, r, k + 1);
+          }
+          zc pv = *p, qv = *q;
+          rotate(pv, qv, c, su);
+          *p = pv;
+          *q = qv;
+        }
       }
       __syncthreads();
     }

@@ -189,9 +189,11 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
  * once; on return V (n x nu, column-major, leading dimension ldv) has orthonormal
  * columns and, if R_dev is not NULL, R_dev (nu x nu, column-major) holds R = R2 R1 with
  * V_in = V_out R. The second pass is FP64 throughout and sets the final orthogonality;
- * when R_dev is NULL and nu <= 128 the first pass (whose only job is to make V well
- * conditioned) runs its Gram matrix, Cholesky factor and triangular inverse in FP32 and
- * applies the inverse to V in FP64. Fails with BEM_EKERNEL if a Gram matrix is not
+ * when R_dev is NULL the first pass (whose only job is to make V well conditioned) runs its
+ * Cholesky factor and triangular inverse (and the smaller Gram matrices) in FP32 and applies
+ * the inverse to V in FP64. From n nu^2 = 2^25 the FP64 products are exact sums of BF16 digit
+ * products; their workspace (10 bytes per byte of V at nu = 32, 5 at 256; at most 8 GiB,
+ * else the FP64 pipe) stays with the context. Fails with BEM_EKERNEL if a Gram matrix is not
  * numerically positive definite (rank-deficient V). Synchronises the stream.
  */
 bem_status bem_cholqr2(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int nu,

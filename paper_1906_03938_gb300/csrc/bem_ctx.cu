@@ -228,6 +228,7 @@ void bem_destroy(bem_ctx* ctx) {
   cudaFree(ctx->d_piv_idx);
   cudaFree(ctx->d_lu_work);
   cudaFree(ctx->d_ff);
+  cudaFree(ctx->d_split);
   cudaFree(ctx->d_zgemm);
   release_cublas(ctx);
   cudaFree(ctx->d_solve);

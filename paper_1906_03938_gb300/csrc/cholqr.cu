@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "split64.h"
 
 namespace bem {
 namespace {
@@ -263,16 +264,18 @@ sum_parts_kernel(const double2* __restrict__ part, int parts, int nu, double2* _
   if (live && q == 0) G[t] = sum;
 }
 
-// FP32 first-pass factor: Z = R^{-1} for G = R^H R (nu <= 128), one block, by Gaussian
+// FP32 first-pass factor: Z = R^{-1} for G = R^H R (nu <= 128; wider ones in two diagonal
+// blocks, chol_block32_kernel), one block, by Gaussian
 // elimination of [G | I] without pivoting: the left part becomes D L^H and the right part
 // L^{-1} (G = L D L^H, L unit lower), so Z = L^{-H} D^{-1/2}. Shared memory holds G's
 // trailing lower triangle (G[r][c], r >= c) and W = L^{-1} transposed in the strict upper
 // triangle (W[c][r] at row r, column c); step k changes only columns c > k and reads
 // column k, so one barrier per step suffices. A pivot below 1e-6 of the largest diagonal
-// entry sets *fallback (V too ill-conditioned for an FP32 pass) and Z is not written.
+// entry (of Gd, nd columns) sets *fallback (V too ill-conditioned for an FP32 pass) and Z is not written.
 template <int kSlots>   // ceil(nu^2 / 1024)
 __global__ void __launch_bounds__(1024)
-chol_inv32_kernel(const double2* __restrict__ Gg, int nu, double2* __restrict__ Z, int* fallback) {
+chol_inv32_kernel(const double2* __restrict__ Gg, int ldg, int nu, const double2* __restrict__ Gd,
+                  int nd, double2* __restrict__ Z, int ldz, int* fallback) {
   extern __shared__ float2 S[];
   __shared__ float dmax_s;
   const int tid = threadIdx.x;
@@ -281,14 +284,14 @@ chol_inv32_kernel(const double2* __restrict__ Gg, int nu, double2* __restrict__ 
     const int r = e % nu, c = e / nu;
     float2 v = make_float2(0.f, 0.f);
     if (r >= c) {
-      const double2 g = Gg[(int64_t)r * nu + c];   // G[r][c] = conj(G[c][r]), upper stored
+      const double2 g = Gg[(int64_t)r * ldg + c];   // G[r][c] = conj(G[c][r]), upper stored
       v = make_float2((float)g.x, -(float)g.y);
     }
     S[e] = v;
   }
   if (tid < 32) {
     float m = 0.f;
-    for (int k = tid; k < nu; k += 32) m = fmaxf(m, (float)Gg[(int64_t)k * nu + k].x);
+    for (int k = tid; k < nd; k += 32) m = fmaxf(m, (float)Gd[(int64_t)k * nd + k].x);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     if (tid == 0) dmax_s = m;
@@ -345,7 +348,50 @@ chol_inv32_kernel(const double2* __restrict__ Gg, int nu, double2* __restrict__ 
         out = make_double2(w.x * inv, -w.y * inv);
       }
     }
-    Z[e] = out;
+    Z[(int64_t)k * ldz + c] = out;
+  }
+}
+
+// Inverse factor of a wider Gram matrix from two diagonal blocks, G = [G11 G12; . G22] at
+// kChol32 columns: Z11 = chol_inv32(G11), W = Z11^H G12 (= R12), S = G22 - W^H W,
+// Z22 = chol_inv32(S), T = W Z22, Z12 = -Z11 T. FP32 products (the first pass only has to make V
+// well conditioned); one thread per entry, 16 x 16 a block.
+//  kMode 0: W (h x r), 1: S (upper, r x r), 2: T (h x r), 3: Z12, with h = kChol32, r = nu - h.
+constexpr int kChol32 = 128;
+
+template <int kMode>
+__global__ void __launch_bounds__(256)
+chol_block32_kernel(const double2* __restrict__ G, double2* __restrict__ Z, int nu,
+                    double2* __restrict__ W, double2* __restrict__ S, double2* __restrict__ T) {
+  constexpr int h = kChol32;
+  const int r = nu - h;
+  const int i = blockIdx.x * 16 + threadIdx.x % 16, j = blockIdx.y * 16 + threadIdx.x / 16;
+  if (j >= r || i >= (kMode == 1 ? r : h)) return;
+  float2 acc = make_float2(0.f, 0.f);
+  auto f2of = [](double2 v) { return make_float2((float)v.x, (float)v.y); };
+  auto mac = [&](float2 a, float2 b) {   // a b
+    acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
+    acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
+  };
+  auto cj = [](float2 a) { return make_float2(a.x, -a.y); };
+  if (kMode == 0) {
+    for (int k = 0; k <= i; ++k)
+      mac(cj(f2of(Z[(int64_t)i * nu + k])), f2of(G[(int64_t)(h + j) * nu + k]));
+    W[(int64_t)j * h + i] = make_double2(acc.x, acc.y);
+  } else if (kMode == 1) {
+    if (i > j) return;
+    for (int k = 0; k < h; ++k)
+      mac(cj(f2of(W[(int64_t)i * h + k])), f2of(W[(int64_t)j * h + k]));
+    const double2 g = G[(int64_t)(h + j) * nu + h + i];
+    S[(int64_t)j * r + i] = make_double2(g.x - acc.x, i == j ? 0.0 : g.y - acc.y);
+  } else if (kMode == 2) {
+    for (int k = 0; k <= j; ++k)
+      mac(f2of(W[(int64_t)k * h + i]), f2of(Z[(int64_t)(h + j) * nu + h + k]));
+    T[(int64_t)j * h + i] = make_double2(acc.x, acc.y);
+  } else {
+    for (int k = i; k < h; ++k)
+      mac(f2of(Z[(int64_t)k * nu + i]), f2of(T[(int64_t)j * h + k]));
+    Z[(int64_t)(h + j) * nu + i] = make_double2(-acc.x, -acc.y);
   }
 }
 
@@ -767,6 +813,7 @@ namespace {
 struct CqLayout {
   int tiles_u = 0;           // upper Gram tiles
   int64_t parts = 0, rows_per_part = 0;
+  int64_t parts_max = 0;     // with those of the split products
   int near_blocks = 0;       // blocks of the near-identity element kernels (64 threads)
   int near_tiles = 0;        // 8 x 8 tiles of the near-identity products
   unsigned sum_blocks = 0;   // blocks of sum_parts_kernel (eight threads per element)
@@ -782,6 +829,7 @@ CqLayout cq_layout(bem_ctx* ctx, int64_t n, int nu) {
                                                    (2 * (int64_t)sms + L.tiles_u - 1) / L.tiles_u));
   L.rows_per_part = (n + L.parts - 1) / L.parts;
   L.parts = (n + L.rows_per_part - 1) / L.rows_per_part;
+  L.parts_max = std::max<int64_t>(L.parts, split64_parts(ctx, n, nu));
   L.near_blocks = (int)(((int64_t)nu * nu + 63) / 64);
   L.near_tiles = ((nu + 7) / 8) * ((nu + 7) / 8);
   L.sum_blocks = (unsigned)((8 * (int64_t)nu * nu + 255) / 256);
@@ -803,7 +851,7 @@ CqWork cq_work(void* work, int nu, const CqLayout& L) {
   const size_t m = (size_t)nu * nu;
   w.G = p; w.Z = p + m; w.R1 = p + 2 * m; w.R2 = p + 3 * m; w.P = p + 4 * m; w.Q = p + 5 * m;
   w.Y = p + 6 * m; w.P1 = p + 7 * m; w.Q1 = p + 8 * m; w.part = p + 9 * m;
-  w.deficient = reinterpret_cast<int*>(w.part + (size_t)L.parts * m);
+  w.deficient = reinterpret_cast<int*>(w.part + (size_t)L.parts_max * m);
   w.flags = w.deficient + 256;
   w.epsp = reinterpret_cast<float*>(w.flags + 8);
   return w;
@@ -822,21 +870,38 @@ bem_status set_smem(bem_ctx* ctx, const void* fn, size_t bytes) {
                     "cholqr attribute");
 }
 
+// Partial sums of the FP64 Gram matrix into w.part, added into G: on the tensor core where the
+// plan says so (split64.cu), else on the FP64 pipe.
+bem_status gram64(bem_ctx* ctx, const Split64& sp, double2* V, int64_t ldv, int64_t n, int nu,
+                  const CqLayout& L, const CqWork& w, double2* G, const int* gate, cudaStream_t s) {
+  int parts = (int)L.parts;
+  if (sp.use) {
+    const bem_status st = split64_gram(ctx, sp, V, w.part, gate, s);
+    if (st != BEM_OK) return st;
+    parts = sp.parts;
+  } else {
+    gram_partial_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
+        V, ldv, n, nu, L.rows_per_part, w.part, gate);
+    ctx->launches++;
+  }
+  sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, parts, nu, G, gate);
+  ctx->launches++;
+  return BEM_OK;
+}
+
 // One FP64 pass V <- V R^{-1} whose Gram matrix is expected near the identity: the
 // near-identity factor, or the classic Cholesky factorisation and triangular inverse when
 // ||G - I||_F > kNearEps (flag *classic, set on the device). Everything is skipped unless
 // *gate != 0 (gate null: always runs).
 bem_status near_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu,
-                     const CqLayout& L, const CqWork& w, const int* gate, int* classic,
-                     cudaStream_t s) {
+                     const CqLayout& L, const CqWork& w, const Split64& sp, const int* gate,
+                     int* classic, cudaStream_t s) {
   int* done = classic + 2;   // classic flag and its "second step not needed" companion
   bem_status st = cuda_check(ctx, cudaMemsetAsync(classic, 0, 3 * sizeof(int), s), "cholqr flag");
   if (st != BEM_OK) return st;
   double2* V = reinterpret_cast<double2*>(V_dev);
   const unsigned nb = (unsigned)L.near_blocks;
-  gram_partial_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
-      V, ldv, n, nu, L.rows_per_part, w.part, gate);
-  sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, (int)L.parts, nu, w.G, gate);
+  if ((st = gram64(ctx, sp, V, ldv, n, nu, L, w, w.G, gate, s)) != BEM_OK) return st;
   const unsigned nt = (unsigned)((nu + kNT - 1) / kNT);
   const dim3 tgrid(nt, nt);
   near_tile_kernel<0><<<tgrid, 64, 0, s>>>(w.G, nullptr, nullptr, nullptr, nu, w.P, w.Q, nullptr,
@@ -850,7 +915,10 @@ bem_status near_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu
                                            nullptr, gate, done);
   near_tile_kernel<2><<<tgrid, 64, 0, s>>>(w.G, w.Y, w.P1, w.Q1, nu, nullptr, nullptr, w.Z,
                                            nullptr, gate, done);
-  // V <- V Z: the classic inverse in FP64, the near-identity factor as V + V (Z - I)
+  ctx->launches += 6;
+  // V <- V Z: on the tensor core; else the classic inverse in FP64, the near-identity factor as
+  // V + V (Z - I)
+  if (sp.use) return split64_multiply(ctx, sp, V, w.Z, gate, nullptr, s);
   const unsigned rb = (unsigned)((n + kRMRows - 1) / kRMRows);
   right_multiply_kernel<<<rb, 256, right_multiply_smem(nu), s>>>(V, ldv, n, nu, w.Z, gate,
                                                                  nullptr, classic);
@@ -859,26 +927,34 @@ bem_status near_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu
                                                                             classic);
   right_multiply_near_df_kernel<<<rb, 256, right_multiply_df_smem(nu), s>>>(V, ldv, n, nu, Zs,
                                                                             gate, classic);
-  ctx->launches += 11;
+  ctx->launches += 3;
   return cuda_check(ctx, cudaGetLastError(), "cholqr kernels");
+}
+
+// V <- V Z in FP64 (skipped when skip and *skip != 0).
+bem_status multiply64(bem_ctx* ctx, const Split64& sp, double2* V, int64_t ldv, int64_t n, int nu,
+                      const double2* Z, const int* skip, cudaStream_t s) {
+  if (sp.use) return split64_multiply(ctx, sp, V, Z, nullptr, skip, s);
+  right_multiply_kernel<<<(unsigned)((n + kRMRows - 1) / kRMRows), 256, right_multiply_smem(nu),
+                          s>>>(V, ldv, n, nu, Z, nullptr, skip, nullptr);
+  ctx->launches++;
+  return BEM_OK;
 }
 
 // Classic FP64 pass: Gram, Cholesky (optionally refreshing collapsed columns), inverse,
 // V <- V R^{-1}; R kept in R_out.
 bem_status classic_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu,
-                        const CqLayout& L, const CqWork& w, double2* R_out, uint64_t refresh_seed,
-                        cudaStream_t s) {
+                        const CqLayout& L, const CqWork& w, const Split64& sp, double2* R_out,
+                        uint64_t refresh_seed, cudaStream_t s) {
   double2* V = reinterpret_cast<double2*>(V_dev);
-  gram_partial_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
-      V, ldv, n, nu, L.rows_per_part, w.part, nullptr);
-  sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, (int)L.parts, nu, R_out, nullptr);
+  bem_status st = gram64(ctx, sp, V, ldv, n, nu, L, w, R_out, nullptr, s);
+  if (st != BEM_OK) return st;
   const size_t chol_smem = nu <= 64 ? (size_t)nu * nu * sizeof(double2) : 0;
   cholesky_kernel<<<1, 1024, chol_smem, s>>>(R_out, nu, ctx->d_status,
                                              refresh_seed ? w.deficient : nullptr, nullptr);
   triangular_inverse_kernel<<<nu, 128, 0, s>>>(R_out, nu, w.Z, nullptr);
-  right_multiply_kernel<<<(unsigned)((n + kRMRows - 1) / kRMRows), 256, right_multiply_smem(nu),
-                          s>>>(V, ldv, n, nu, w.Z, nullptr, nullptr, nullptr);
-  ctx->launches += 5;
+  ctx->launches += 2;
+  if ((st = multiply64(ctx, sp, V, ldv, n, nu, w.Z, nullptr, s)) != BEM_OK) return st;
   if (refresh_seed) {
     refresh_columns_kernel<<<(unsigned)((n * nu + 255) / 256), 256, 0, s>>>(V, ldv, n, nu,
                                                                            w.deficient,
@@ -892,7 +968,7 @@ bem_status classic_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int
 
 size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu) {
   const CqLayout L = cq_layout(ctx, n, nu);
-  return (9 + (size_t)L.parts) * (size_t)nu * nu * sizeof(double2) +
+  return (9 + (size_t)L.parts_max) * (size_t)nu * nu * sizeof(double2) +
          (256 + 8) * sizeof(int) + (size_t)L.near_tiles * sizeof(float);
 }
 
@@ -900,8 +976,8 @@ size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu) {
 // asynchronous; a Gram matrix that is not positive definite is flagged in the context's
 // status word.
 //
-// Without R: the first pass runs in FP32 (nu <= 128, no refresh): it only has to make V
-// well conditioned. The FP64 second pass then sees G = I + E with small E and uses the
+// Without R (and no refresh): the first pass runs in FP32: it only has to make V well
+// conditioned. The FP64 second pass then sees G = I + E with small E and uses the
 // near-identity factor. If V is too ill-conditioned for FP32 the first pass leaves V alone
 // (device flag) and a third pass runs (its kernels return at once otherwise); the second
 // pass then falls back to the classic factorisation by itself. With R: two classic passes
@@ -918,39 +994,57 @@ bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int
   if ((st = set_smem(ctx, (const void*)right_multiply_near_df_kernel,
                      right_multiply_df_smem(nu))) != BEM_OK)
     return st;
+  Split64 sp;
+  split64_plan(ctx, V_dev, ldv, n, nu, sp, s);
   if (R_dev) {
-    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, w.R1, refresh_seed, s)) != BEM_OK) return st;
-    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, w.R2, 0, s)) != BEM_OK) return st;
+    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R1, refresh_seed, s)) != BEM_OK) return st;
+    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R2, 0, s)) != BEM_OK) return st;
     upper_product_kernel<<<1, 256, 0, s>>>(w.R2, w.R1, nu, reinterpret_cast<double2*>(R_dev));
     ctx->launches++;
     return cuda_check(ctx, cudaGetLastError(), "cholqr kernels");
   }
-  const bool fp32_first = refresh_seed == 0 && nu <= 128;
-  if (!fp32_first) {
-    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, w.R1, refresh_seed, s)) != BEM_OK) return st;
-    return near_pass(ctx, V_dev, ldv, n, nu, L, w, nullptr, w.flags + 1, s);
+  if (refresh_seed != 0) {
+    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R1, refresh_seed, s)) != BEM_OK) return st;
+    return near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, s);
   }
   int* fallback = w.flags;
-  const size_t ci_smem = (size_t)nu * nu * sizeof(float2);
-  if ((st = set_smem(ctx, (const void*)chol_inv32_kernel<4>, ci_smem)) != BEM_OK ||
+  const int h = std::min(nu, kChol32), r = nu - h;   // diagonal blocks of the FP32 factor
+  const size_t ci_smem = (size_t)h * h * sizeof(float2);
+  if ((st = set_smem(ctx, (const void*)chol_inv32_kernel<4>, std::min(ci_smem, (size_t)64 * 64 * sizeof(float2)))) != BEM_OK ||
       (st = set_smem(ctx, (const void*)chol_inv32_kernel<16>, ci_smem)) != BEM_OK)
     return st;
   st = cuda_check(ctx, cudaMemsetAsync(fallback, 0, sizeof(int), s), "cholqr flag");
   if (st != BEM_OK) return st;
   double2* V = reinterpret_cast<double2*>(V_dev);
-  gram_partial32_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
-      V, ldv, n, nu, L.rows_per_part, w.part);
-  sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, (int)L.parts, nu, w.G, nullptr);
-  if (nu <= 64)
-    chol_inv32_kernel<4><<<1, 1024, ci_smem, s>>>(w.G, nu, w.Z, fallback);
-  else
-    chol_inv32_kernel<16><<<1, 1024, ci_smem, s>>>(w.G, nu, w.Z, fallback);
-  right_multiply_kernel<<<(unsigned)((n + kRMRows - 1) / kRMRows), 256, right_multiply_smem(nu),
-                          s>>>(V, ldv, n, nu, w.Z, nullptr, fallback, nullptr);
-  ctx->launches += 4;
+  if (sp.use && nu > kChol32) {
+    if ((st = gram64(ctx, sp, V, ldv, n, nu, L, w, w.G, nullptr, s)) != BEM_OK) return st;
+  } else {
+    gram_partial32_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
+        V, ldv, n, nu, L.rows_per_part, w.part);
+    sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, (int)L.parts, nu, w.G, nullptr);
+    ctx->launches += 2;
+  }
+  auto inverse32 = [&](const double2* G, int ldg, int m, double2* Z) {
+    if (m <= 64)
+      chol_inv32_kernel<4><<<1, 1024, (size_t)m * m * sizeof(float2), s>>>(G, ldg, m, w.G, nu, Z, nu, fallback);
+    else
+      chol_inv32_kernel<16><<<1, 1024, (size_t)m * m * sizeof(float2), s>>>(G, ldg, m, w.G, nu, Z, nu, fallback);
+    ctx->launches++;
+  };
+  inverse32(w.G, nu, h, w.Z);
+  if (r > 0) {
+    const dim3 gh((unsigned)((h + 15) / 16), (unsigned)((r + 15) / 16)), gr(gh.y, gh.y);
+    chol_block32_kernel<0><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+    chol_block32_kernel<1><<<gr, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+    inverse32(w.Q, r, r, w.Z + (size_t)h * nu + h);
+    chol_block32_kernel<2><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+    chol_block32_kernel<3><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+    ctx->launches += 4;
+  }
+  if ((st = multiply64(ctx, sp, V, ldv, n, nu, w.Z, fallback, s)) != BEM_OK) return st;
   if ((st = cuda_check(ctx, cudaGetLastError(), "cholqr kernels")) != BEM_OK) return st;
-  if ((st = near_pass(ctx, V_dev, ldv, n, nu, L, w, nullptr, w.flags + 1, s)) != BEM_OK) return st;
-  return near_pass(ctx, V_dev, ldv, n, nu, L, w, fallback, w.flags + 4, s);
+  if ((st = near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, s)) != BEM_OK) return st;
+  return near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, fallback, w.flags + 4, s);
 }
 
 }  // namespace bem

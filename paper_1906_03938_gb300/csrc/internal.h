@@ -108,6 +108,8 @@ struct bem_ctx {
   size_t zgemm_bytes = 0;
   float* d_lu_work = nullptr;    // the LU's trailing-update operands in real form
   size_t lu_work_bytes = 0;
+  void* d_split = nullptr;       // digit planes of the split FP64 products (split64.cu)
+  size_t split_bytes = 0;
   double* d_ff = nullptr;        // column splits' partial sums of the double-FP32 residuals
   size_t ff_bytes = 0;
   size_t small_bytes = 0;

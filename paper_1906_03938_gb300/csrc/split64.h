@@ -1,0 +1,36 @@
+// FP64-accurate products of tall matrices on the tensor core (split64.cu).
+#pragma once
+
+#include "internal.h"
+
+namespace bem {
+
+// Workspace of the split products of an n x nu basis (Gram matrix and multiplication).
+struct Split64 {
+  bool use = false;
+  int64_t n = 0, ldv = 0;
+  int nu = 0;
+  int kbn = 0, kbu = 0;      // 16-deep K-blocks along the rows, along the columns
+  int mtu = 0, ntu = 0;      // 128-wide and 32-wide tiles of the columns
+  int64_t mtn = 0;           // 128-row tiles
+  int parts = 0;             // row ranges of the Gram matrix (its partial sums)
+  unsigned char *a = nullptr, *b = nullptr;   // digit planes of the two operands
+  int *emax = nullptr, *erow = nullptr, *ez = nullptr;   // exponents: columns, rows, factor
+};
+
+// Fills sp for V; use is false where the FP64 kernels are the better choice (small products) or
+// the workspace cannot be had.
+void split64_plan(bem_ctx* ctx, const double* V, int64_t ldv, int64_t n, int nu, Split64& sp,
+                  cudaStream_t s);
+// Row ranges of the Gram matrix of an n x nu basis (partial sums to provide for).
+int split64_parts(const bem_ctx* ctx, int64_t n, int nu);
+// part[r][b nu + a] = sum over row range r of conj(V[i][a]) V[i][b] for the upper 32 x 32 tiles
+// (sp.parts ranges). Skipped on the device when gate is given and *gate == 0.
+bem_status split64_gram(bem_ctx* ctx, const Split64& sp, const double2* V, double2* part,
+                        const int* gate, cudaStream_t s);
+// V <- V Z, Z nu x nu upper triangular. Skipped when (gate and *gate == 0) or
+// (skip and *skip != 0).
+bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, double2* V, const double2* Z,
+                            const int* gate, const int* skip, cudaStream_t s);
+
+}  // namespace bem

@@ -46,7 +46,7 @@ def test_large_sizes_match_the_matrix_free_solve(m):
     mesh = synth.cube_sphere(m, (1.0, 0.8, 0.55))
     bem, ctx, z, w = _ctx(mesh.xyz, mesh.tri)
     V0 = torch.from_numpy(synth.complex_gaussian(mesh.n, 3, 4)).to("cuda:0")
-    V, W = bem.fortran(V0), bem.fortran(V0)
+    V, W = bem.fortran(V0), bem.fortran(V0.clone())
     ctx.inverse_power(V, 1, 4.5 + 0.3j)
     ctx.inverse_power_mf(W, 1, 4.5 + 0.3j, tol=2e-5, max_iter=2000)
     ctx.close()

@@ -191,7 +191,7 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
  * V_in = V_out R. The second pass is FP64 throughout and sets the final orthogonality;
  * when R_dev is NULL the first pass (whose only job is to make V well conditioned) runs its
  * Cholesky factor and triangular inverse (and the smaller Gram matrices) in FP32 and applies
- * the inverse to V in FP64. From n nu^2 = 2^25 the FP64 products are exact sums of BF16 digit
+ * the inverse to V in FP64. From n nu^2 = 2^23 the FP64 products are exact sums of BF16 digit
  * products; their workspace (10 bytes per byte of V at nu = 32, 5 at 256; at most 8 GiB,
  * else the FP64 pipe) stays with the context. Fails with BEM_EKERNEL if a Gram matrix is not
  * numerically positive definite (rank-deficient V). Synchronises the stream.

@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "sm100.cuh"
 #include "split64.h"
 
 namespace bem {
@@ -235,11 +236,12 @@ gram_partial32_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int
 
 // G = sum of the partials (deterministic): eight threads per element, thread q adding the
 // parts q, q + 8, ... in order, then a fixed shuffle tree. Elements of lower tiles are not
-// formed.
+// formed. epsp, if given: the block's sum of |G - I|^2 (off-diagonal entries twice).
 __global__ void __launch_bounds__(256)
 sum_parts_kernel(const double2* __restrict__ part, int parts, int nu, double2* __restrict__ G,
-                 const int* gate) {
+                 float* __restrict__ epsp, const int* gate) {
   if (gate && *gate == 0) return;
+  __shared__ float red[32];
   const int64_t count = (int64_t)nu * nu;
   const int64_t gt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t t = gt / 8;
@@ -262,94 +264,124 @@ sum_parts_kernel(const double2* __restrict__ part, int parts, int nu, double2* _
     sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
   }
   if (live && q == 0) G[t] = sum;
+  if (!epsp) return;
+  if (q == 0) {
+    const int a = (int)(t % nu), b = (int)(t / nu);
+    const float er = (float)(sum.x - (a == b ? 1.0 : 0.0)), ei = a == b ? 0.f : (float)sum.y;
+    red[threadIdx.x / 8] = live && a <= b ? (er * er + ei * ei) * (a == b ? 1.f : 2.f) : 0.f;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    float e2 = red[threadIdx.x];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+    if (threadIdx.x == 0) epsp[blockIdx.x] = e2;
+  }
 }
 
 // FP32 first-pass factor: Z = R^{-1} for G = R^H R (nu <= 128; wider ones in two diagonal
-// blocks, chol_block32_kernel), one block, by Gaussian
-// elimination of [G | I] without pivoting: the left part becomes D L^H and the right part
-// L^{-1} (G = L D L^H, L unit lower), so Z = L^{-H} D^{-1/2}. Shared memory holds G's
-// trailing lower triangle (G[r][c], r >= c) and W = L^{-1} transposed in the strict upper
-// triangle (W[c][r] at row r, column c); step k changes only columns c > k and reads
-// column k, so one barrier per step suffices. A pivot below 1e-6 of the largest diagonal
-// entry (of Gd, nd columns) sets *fallback (V too ill-conditioned for an FP32 pass) and Z is not written.
-template <int kSlots>   // ceil(nu^2 / 1024)
-__global__ void __launch_bounds__(1024)
-chol_inv32_kernel(const double2* __restrict__ Gg, int ldg, int nu, const double2* __restrict__ Gd,
-                  int nd, double2* __restrict__ Z, int ldz, int* fallback) {
-  extern __shared__ float2 S[];
+// blocks, chol_block32_kernel), one block, by Gaussian elimination of [G | I] without pivoting:
+// the left part becomes D L^H and the right part L^{-1} (G = L D L^H, L unit lower), so
+// Z = L^{-H} D^{-1/2}. Element (r, c) of the working matrix is the trailing G[r][c] for r >= c
+// and W[c][r], W = L^{-1}, for r < c; step k changes only columns c > k and reads column k. A
+// pivot below 1e-6 of the largest diagonal entry (of Gd, nd columns) sets *fallback (V too
+// ill-conditioned for an FP32 pass) and Z is not written.
+//
+// nu dependent steps of little work each: kGrid x kGrid threads keep kT x kT elements each in
+// registers (rows and columns kGrid apart, so that the shrinking part stays spread over all
+// warps), and only the next column goes through shared memory, in two buffers with one barrier a
+// step. With the whole matrix in shared memory its bandwidth set the time: 41 us at nu = 64,
+// 237 us at 128; now 29 us and 107 us. Run by the first kGrid^2 threads of a block.
+template <int kGrid, int kT>   // nu <= kGrid kT
+__device__ void chol_inv32_block(const double2* Gg, int ldg, int nu, const double2* Gd, int nd,
+                                 double2* __restrict__ Z, int ldz, int* fallback) {
+  __shared__ float2 col[2][kGrid * kT];
+  __shared__ float diag[kGrid * kT];
   __shared__ float dmax_s;
-  const int tid = threadIdx.x;
-  const int total = nu * nu;
-  for (int e = tid; e < total; e += blockDim.x) {
-    const int r = e % nu, c = e / nu;
-    float2 v = make_float2(0.f, 0.f);
-    if (r >= c) {
-      const double2 g = Gg[(int64_t)r * ldg + c];   // G[r][c] = conj(G[c][r]), upper stored
-      v = make_float2((float)g.x, -(float)g.y);
+  const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
+  const int tr = lane % 8 + 8 * (w % (kGrid / 8)), tc = lane / 8 + 4 * (w / (kGrid / 8));
+  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kGrid * kGrid) : "memory"); };
+  float2 g[kT][kT];   // [row slot][column slot]
+#pragma unroll
+  for (int i = 0; i < kT; ++i)
+#pragma unroll
+    for (int j = 0; j < kT; ++j) {
+      const int r = tr + kGrid * i, c = tc + kGrid * j;
+      g[i][j] = make_float2(0.f, 0.f);
+      if (r >= c && r < nu) {
+        const double2 v = __ldcg(Gg + (int64_t)r * ldg + c);   // G[r][c] = conj(G[c][r])
+        g[i][j] = make_float2((float)v.x, -(float)v.y);
+      }
     }
-    S[e] = v;
-  }
   if (tid < 32) {
     float m = 0.f;
-    for (int k = tid; k < nd; k += 32) m = fmaxf(m, (float)Gd[(int64_t)k * nd + k].x);
+    for (int k = tid; k < nd; k += 32) m = fmaxf(m, (float)__ldcg(Gd + (int64_t)k * nd + k).x);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     if (tid == 0) dmax_s = m;
   }
-  __syncthreads();
-  const float dmax = dmax_s;
-  int sr[kSlots], sc[kSlots];
+  if (tc == 0)
 #pragma unroll
-  for (int m = 0; m < kSlots; ++m) {
-    const int e = tid + m * 1024;
-    sr[m] = e < total ? e % nu : 0;
-    sc[m] = e < total ? e / nu : -1;
-  }
+    for (int i = 0; i < kT; ++i) col[0][tr + kGrid * i] = g[i][0];
+  sync();
+  const float dmax = dmax_s;
   for (int k = 0; k < nu; ++k) {
-    const float d = S[k * nu + k].x;
+    const float2* s = col[k & 1];
+    const float d = s[k].x;
     if (!(d > 1e-6f * dmax) || !isfinite(d)) {
       if (tid == 0) *fallback = 1;
       return;   // d is the same for every thread: the whole block leaves
     }
+    if (tid == 0) diag[k] = d;
     const float rd = 1.f / d;
+    float2 a[kT];   // column k at this thread's rows: G[r][k], 1 at r = k, W[k][r] above
 #pragma unroll
-    for (int m = 0; m < kSlots; ++m) {
-      const int r = sr[m], c = sc[m];
-      if (c <= k) continue;
-      if (r >= c) {
-        // G[r][c] -= G[r][k] conj(G[c][k]) / d
-        const float2 a = S[k * nu + r], b = S[k * nu + c];
-        float2 g = S[c * nu + r];
-        g.x -= (a.x * b.x + a.y * b.y) * rd;
-        g.y -= (a.y * b.x - a.x * b.y) * rd;
-        S[c * nu + r] = g;
-      } else if (r <= k) {
-        // W[c][r] -= (G[c][k] / d) W[k][r], W[k][k] = 1
-        const float2 l = S[k * nu + c];
-        const float2 w = (r == k) ? make_float2(1.f, 0.f) : S[k * nu + r];
-        float2 g = S[c * nu + r];
-        g.x -= (l.x * w.x - l.y * w.y) * rd;
-        g.y -= (l.x * w.y + l.y * w.x) * rd;
-        S[c * nu + r] = g;
+    for (int i = 0; i < kT; ++i) a[i] = tr + kGrid * i == k ? make_float2(1.f, 0.f) : s[tr + kGrid * i];
+#pragma unroll
+    for (int j = 0; j < kT; ++j) {
+      if (kGrid * j + kGrid - 1 <= k) continue;
+      const int c = tc + kGrid * j;
+      float2 l = s[c];
+      l = c > k ? make_float2(l.x * rd, l.y * rd) : make_float2(0.f, 0.f);   // L[c][k]
+#pragma unroll
+      for (int i = 0; i < kT; ++i) {
+        if (i < j && kGrid * i > k) continue;
+        const int r = tr + kGrid * i;
+        // r >= c: G[r][c] -= G[r][k] conj(L[c][k]); r <= k: W[c][r] -= L[c][k] W[k][r]
+        const float ly = r >= c ? -l.y : l.y;
+        if (r >= c || r <= k) {
+          g[i][j].x -= a[i].x * l.x - a[i].y * ly;
+          g[i][j].y -= a[i].x * ly + a[i].y * l.x;
+        }
       }
+      if (c == k + 1)
+#pragma unroll
+        for (int i = 0; i < kT; ++i) col[(k + 1) & 1][tr + kGrid * i] = g[i][j];
     }
-    __syncthreads();
+    sync();
   }
   // Z[c][k] = conj(W[k][c]) / sqrt(d_k) for c <= k, zero below the diagonal
-  for (int e = tid; e < total; e += blockDim.x) {
-    const int c = e % nu, k = e / nu;
-    double2 out = make_double2(0.0, 0.0);
-    if (c <= k) {
-      const float inv = 1.f / sqrtf(S[k * nu + k].x);
-      if (c == k) {
-        out = make_double2(inv, 0.0);
-      } else {
-        const float2 w = S[k * nu + c];
-        out = make_double2(w.x * inv, -w.y * inv);
-      }
+#pragma unroll
+  for (int j = 0; j < kT; ++j) {
+    const int c = tc + kGrid * j;
+    if (c >= nu) continue;
+    const float inv = 1.f / sqrtf(diag[c]);
+#pragma unroll
+    for (int i = 0; i < kT; ++i) {
+      const int r = tr + kGrid * i;
+      if (r >= nu) continue;
+      Z[(int64_t)c * ldz + r] = r > c ? make_double2(0.0, 0.0)
+                                : r == c ? make_double2(inv, 0.0)
+                                         : make_double2(g[i][j].x * inv, -g[i][j].y * inv);
     }
-    Z[(int64_t)k * ldz + c] = out;
   }
+}
+
+template <int kT>
+__global__ void __launch_bounds__(1024)
+chol_inv32_kernel(const double2* __restrict__ Gg, int ldg, int nu, const double2* __restrict__ Gd,
+                  int nd, double2* __restrict__ Z, int ldz, int* fallback) {
+  chol_inv32_block<32, kT>(Gg, ldg, nu, Gd, nd, Z, ldz, fallback);
 }
 
 // Inverse factor of a wider Gram matrix from two diagonal blocks, G = [G11 G12; . G22] at
@@ -395,6 +427,12 @@ chol_block32_kernel(const double2* __restrict__ G, double2* __restrict__ Z, int 
   }
 }
 
+// ||G - I||_F up to which the near-identity factor is used; its error is O(||G - I||^4)
+// (at 8e-4 it still matches the Cholesky factor to rounding)
+constexpr float kNearEps = 5e-4f;
+// ||G - I||_F up to which the first step alone is exact to rounding
+constexpr float kNearEpsSmall = 1e-5f;
+
 // ---- second pass near the identity ----
 //
 // After a first pass G = V^H V = I + E with ||E|| small. The inverse factor Z = R^{-1} is
@@ -415,9 +453,8 @@ __device__ __forceinline__ double2 e_entry(const double2* G, int nu, int m, int 
   return make_double2(g.x, -g.y);
 }
 
-// Y entry (m, i), m <= i: explicit (Yx non-null) or Y0 = -U(E) from G.
-__device__ __forceinline__ double2 y_entry(const double2* G, const double2* Yx, int nu, int m, int i) {
-  if (Yx) return Yx[(int64_t)i * nu + m];
+// Y0 = -U(E) entry (m, i), m <= i.
+__device__ __forceinline__ double2 y_entry(const double2* G, int nu, int m, int i) {
   const double2 g = G[(int64_t)i * nu + m];
   return m < i ? make_double2(-g.x, -g.y) : make_double2(-0.5 * (g.x - 1.0), 0.0);
 }
@@ -425,10 +462,8 @@ __device__ __forceinline__ double2 y_entry(const double2* G, const double2* Yx, 
 constexpr int kNT = 8;     // output tile of the near-identity products (kNT x kNT per block)
 constexpr int kNM = 16;    // inner-dimension chunk staged in shared memory
 
-// Tiled small products of the near-identity factor; one 8 x 8 output tile per block of 64
-// threads, the inner dimension staged 16 at a time in shared memory.
-//  kMode 0: P = Y0^H E (all entries), Q = Y0^H Y0 (upper), Y0 = -U(E) formed from G, and
-//           the block sums of |E_ij|^2 (upper triangle, off-diagonal entries twice);
+// Tiled small products of the near-identity factor's second step; one 8 x 8 output tile per
+// block of 64 threads, the inner dimension staged 16 at a time in shared memory.
 //  kMode 1: P = Y^H E, Q = Y^H Y for the explicit Y;
 //  kMode 2: Z = I + Y2, Y2 = -U(E + P + P^H + Q + P Y) (P, Q, Y of mode 1).
 template <int kMode>
@@ -436,10 +471,9 @@ __global__ void __launch_bounds__(64)
 near_tile_kernel(const double2* __restrict__ G, const double2* __restrict__ Y,
                  const double2* __restrict__ Pin, const double2* __restrict__ Qin, int nu,
                  double2* __restrict__ P, double2* __restrict__ Q, double2* __restrict__ Z,
-                 float* epsp, const int* gate, const int* skip_if) {
+                 const int* gate, const int* skip_if) {
   if ((gate && *gate == 0) || (skip_if && *skip_if != 0)) return;
   __shared__ double2 sA[kNM][kNT], sB[kNM][kNT], sC[kNM][kNT];
-  __shared__ float red[64];
   const int tid = threadIdx.x;
   const int ti = tid % kNT, tj = tid / kNT;
   const int i0 = blockIdx.x * kNT, j0 = blockIdx.y * kNT;
@@ -458,10 +492,10 @@ near_tile_kernel(const double2* __restrict__ G, const double2* __restrict__ Y,
         sA[mm][cc] = (mv && ic < nu) ? Pin[(int64_t)m * nu + ic] : make_double2(0.0, 0.0);   // P(i, m)
         sB[mm][cc] = (mv && jc < nu && m <= jc) ? Y[(int64_t)jc * nu + m] : make_double2(0.0, 0.0);
       } else {
-        sA[mm][cc] = (mv && ic < nu && m <= ic) ? y_entry(G, kMode == 0 ? nullptr : Y, nu, m, ic)
+        sA[mm][cc] = (mv && ic < nu && m <= ic) ? Y[(int64_t)ic * nu + m]
                                                 : make_double2(0.0, 0.0);
         sB[mm][cc] = (mv && jc < nu) ? e_entry(G, nu, m, jc) : make_double2(0.0, 0.0);
-        sC[mm][cc] = (mv && jc < nu && m <= jc) ? y_entry(G, kMode == 0 ? nullptr : Y, nu, m, jc)
+        sC[mm][cc] = (mv && jc < nu && m <= jc) ? Y[(int64_t)jc * nu + m]
                                                 : make_double2(0.0, 0.0);
       }
     }
@@ -501,60 +535,98 @@ near_tile_kernel(const double2* __restrict__ G, const double2* __restrict__ Y,
     P[t] = p;
     if (i <= j) Q[t] = q;
   }
-  if (kMode == 0) {
-    float e2 = 0.f;
-    if (in && i <= j) {
-      const double2 e = e_entry(G, nu, i, j);
-      e2 = (float)((e.x * e.x + e.y * e.y) * (i == j ? 1.0 : 2.0));
-    }
-    red[tid] = e2;
-    __syncthreads();
-    for (int s = 32; s > 0; s >>= 1) {
-      if (tid < s) red[tid] += red[tid + s];
-      __syncthreads();
-    }
-    if (tid == 0) epsp[blockIdx.y * gridDim.x + blockIdx.x] = red[0];
-  }
 }
 
-// Y1 = -U(E + P + P^H + Q). Every block first sums the block sums of |E|^2 in order; if
-// ||E||_F exceeds eps_max the near-identity route is abandoned (*classic = 1) and the
-// classic Cholesky factorisation runs instead. *done = 1 tells the second step to skip.
-__global__ void __launch_bounds__(64)
-near_y1_kernel(const double2* __restrict__ G, const double2* __restrict__ P,
-               const double2* __restrict__ Q, const float* __restrict__ epsp, int nparts,
-               int nu, float eps_max, float eps_small, double2* __restrict__ Y,
-               double2* __restrict__ Z, int* classic, int* done, const int* gate) {
-  if (gate && *gate == 0) return;
-  __shared__ float e2s;
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int b = 0; b < nparts; ++b) s += epsp[b];
-    e2s = s;
+// The first step, Y1 = -U(E + Y0^H E + E Y0 + Y0^H Y0), Y0 = -U(E). E = -(Y0 + Y0^H), so the
+// second-order terms are -(Y0^H Y0 + Y0^2 + (Y0^2)^H), triangular products with a third of the
+// terms. Every block first sums the block sums of |E|^2 in order:
+//  ||E||_F > eps_max: the near-identity route is abandoned (*classic = 1) and the classic
+//    Cholesky factorisation runs instead;
+//  ||E||_F <= eps_small: Y1 is exact to rounding (its error is O(||E||^3)), Z = I + Y1 is
+//    written here and the second step is skipped (*done = 1). The second-order terms are then
+//    below 1e-10 and their rounding in FP32 (6e-18) far below Z's own in FP64, so they are
+//    formed on the FP32 pipe (at nu = 256 42 us; all terms in FP64 took 298 + 20 us).
+// One 8 x 8 output tile per block of 64 threads, upper tiles only.
+template <typename T, typename T2>
+__device__ __forceinline__ T2 near_second_order(const double2* __restrict__ G, int nu, int i0, int j0) {
+  __shared__ T2 sA[kNM][kNT], sB[kNM][kNT], sC[kNM][kNT];   // Y0(m, i), Y0(m, j), Y0(i, m)
+  const int tid = threadIdx.x, ti = tid % kNT, tj = tid / kNT;
+  T2 h;
+  h.x = h.y = 0;
+  T tdiag = 0;   // Re of Y0^2 on the diagonal once more: its conjugate
+  const int mend = min(nu, j0 + kNT);
+  for (int m0 = 0; m0 < mend; m0 += kNM) {
+    __syncthreads();
+    for (int x = tid; x < kNM * kNT; x += 64) {
+      const int mm = x / kNT, cc = x % kNT, m = m0 + mm;
+      auto y0 = [&](int r, int c) {
+        const double2 v = r <= c && c < nu ? y_entry(G, nu, r, c) : make_double2(0.0, 0.0);
+        T2 o;
+        o.x = (T)v.x;
+        o.y = (T)v.y;
+        return o;
+      };
+      sA[mm][cc] = y0(m, i0 + cc);
+      sB[mm][cc] = y0(m, j0 + cc);
+      sC[mm][cc] = y0(i0 + cc, m);
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int mm = 0; mm < kNM; ++mm) {
+      const T2 a = sA[mm][ti], b = sB[mm][tj], c = sC[mm][ti];
+      h.x += a.x * b.x + a.y * b.y + (c.x * b.x - c.y * b.y);
+      h.y += a.x * b.y - a.y * b.x + (c.x * b.y + c.y * b.x);
+      tdiag += c.x * b.x - c.y * b.y;
+    }
   }
+  if (i0 + ti == j0 + tj) h.x += tdiag;
+  return h;
+}
+
+__global__ void __launch_bounds__(64)
+near_y1_kernel(const double2* __restrict__ G, const float* __restrict__ epsp, int nparts, int nu,
+               float eps_max, float eps_small, double2* __restrict__ Y, double2* __restrict__ Z,
+               int* classic, int* done, const int* gate) {
+  if (gate && *gate == 0) return;
+  __shared__ float red[64];
+  const int tid = threadIdx.x;
+  float s = 0.f;
+  for (int b = tid; b < nparts; b += 64) s += epsp[b];
+  red[tid] = s;
   __syncthreads();
+  for (int k = 32; k > 0; k >>= 1) {
+    if (tid < k) red[tid] += red[tid + k];
+    __syncthreads();
+  }
+  const float e2s = red[0];
+  const bool first = blockIdx.x == 0 && blockIdx.y == 0 && tid == 0;
   if (!(e2s <= eps_max * eps_max)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (first) {
       *classic = 1;
       *done = 1;
     }
     return;
   }
-  // ||E|| <= eps_small: Y1 is already exact to rounding (its error is O(||E||^3)), so
-  // Z = I + Y1 is written here and the second step is skipped
   const bool small = e2s <= eps_small * eps_small;
-  if (small && blockIdx.x == 0 && threadIdx.x == 0) *done = 1;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nu * nu) return;
-  const int i = (int)(t % nu), j = (int)(t / nu);
+  if (small && first) *done = 1;
+  const int i0 = blockIdx.x * kNT, j0 = blockIdx.y * kNT;
+  const int i = i0 + tid % kNT, j = j0 + tid / kNT;
   double2 y = make_double2(0.0, 0.0);
-  if (i < j) {
-    const double2 e = e_entry(G, nu, i, j), p = P[t], pt = P[(int64_t)i * nu + j], q = Q[t];
-    y = make_double2(-(e.x + p.x + pt.x + q.x), -(e.y + p.y - pt.y + q.y));
-  } else if (i == j) {
-    const double2 e = e_entry(G, nu, i, i), p = P[t], q = Q[t];
-    y = make_double2(-0.5 * (e.x + 2.0 * p.x + q.x), 0.0);
+  if (i0 <= j0) {
+    double2 h;
+    if (small) {
+      const float2 f = near_second_order<float, float2>(G, nu, i0, j0);
+      h = make_double2(f.x, f.y);
+    } else {
+      h = near_second_order<double, double2>(G, nu, i0, j0);
+    }
+    if (i <= j && j < nu) {
+      const double2 e = e_entry(G, nu, i, j);
+      y = i < j ? make_double2(h.x - e.x, h.y - e.y) : make_double2(-0.5 * (e.x - h.x), 0.0);
+    }
   }
+  if (i >= nu || j >= nu) return;
+  const int64_t t = (int64_t)j * nu + i;
   if (small)
     Z[t] = i == j ? make_double2(1.0 + y.x, 0.0) : y;
   else
@@ -614,13 +686,10 @@ size_t right_multiply_smem(int nu) {
 // V <- V M in place, M nu x nu upper triangular (column-major, zero below the diagonal);
 // each block owns kRMRows complete rows of V, staged in shared memory before any is
 // overwritten. Three real products per complex term: a b = (S1 - S2) + i (S3 - S1 - S2),
-// S1 = a.re b.re, S2 = a.im b.im, S3 = (a.re + a.im)(b.re + b.im).
-// gate, need: skip unless *gate != 0 and *need != 0; skip_if: skip when *skip_if != 0.
-__global__ void __launch_bounds__(256)
-right_multiply_kernel(double2* V, int64_t ldv, int64_t n, int nu, const double2* __restrict__ M,
-                      const int* gate, const int* skip_if, const int* need) {
-  if ((gate && *gate == 0) || (need && *need == 0) || (skip_if && *skip_if != 0)) return;
-  extern __shared__ double rm_smem[];
+// S1 = a.re b.re, S2 = a.im b.im, S3 = (a.re + a.im)(b.re + b.im). kOut: outputs a thread.
+template <int kOut>
+__device__ __forceinline__ void multiply64_rows(double* rm_smem, double2* V, int64_t ldv, int64_t n,
+                                                int nu, const double2* __restrict__ M) {
   double* vr = rm_smem;                  // [nu][kRMRows]
   double* vi = vr + nu * kRMRows;
   double* vs = vi + nu * kRMRows;
@@ -637,7 +706,6 @@ right_multiply_kernel(double2* V, int64_t ldv, int64_t n, int nu, const double2*
     vi[c * kRMRows + rr] = v.y;
     vs[c * kRMRows + rr] = v.x + v.y;
   }
-  constexpr int kOut = kMaxNu * kRMRows / 256;   // outputs per thread at nu = kMaxNu
   const int outs = kRMRows * nu;
   double s1[kOut], s2[kOut], s3[kOut];
 #pragma unroll
@@ -675,6 +743,15 @@ right_multiply_kernel(double2* V, int64_t ldv, int64_t n, int nu, const double2*
     const int64_t r = r0 + rr;
     if (r < n) V[(int64_t)c * ldv + r] = make_double2(s1[m] - s2[m], s3[m] - s1[m] - s2[m]);
   }
+}
+
+// gate, need: skip unless *gate != 0 and *need != 0; skip_if: skip when *skip_if != 0.
+__global__ void __launch_bounds__(256)
+right_multiply_kernel(double2* V, int64_t ldv, int64_t n, int nu, const double2* __restrict__ M,
+                      const int* gate, const int* skip_if, const int* need) {
+  if ((gate && *gate == 0) || (need && *need == 0) || (skip_if && *skip_if != 0)) return;
+  extern __shared__ double rm_smem[];
+  multiply64_rows<kMaxNu * kRMRows / 256>(rm_smem, V, ldv, n, nu, M);
 }
 
 // V <- V + V (M - I) for the near-identity factor M = I + Y (upper triangular), with the
@@ -722,11 +799,9 @@ __global__ void split_near_factor_kernel(const double2* __restrict__ M, int nu,
   Ms[t] = make_float4(br, bi, (float)(b.x - br), (float)(b.y - bi));
 }
 
-__global__ void __launch_bounds__(256)
-right_multiply_near_df_kernel(double2* V, int64_t ldv, int64_t n, int nu,
-                              const float4* __restrict__ Ms, const int* gate, const int* skip_if) {
-  if ((gate && *gate == 0) || (skip_if && *skip_if != 0)) return;
-  extern __shared__ float4 df_smem[];
+template <int kOut>
+__device__ __forceinline__ void multiply_df_rows(float4* df_smem, double2* V, int64_t ldv, int64_t n,
+                                                 int nu, const float4* __restrict__ Ms) {
   float4* sV = df_smem;                 // [nu][kRMRows]: (re hi, im hi, re lo, im lo)
   float4* sM = sV + nu * kRMRows;       // [kDFK][nu]
   const int tid = threadIdx.x;
@@ -738,7 +813,6 @@ right_multiply_near_df_kernel(double2* V, int64_t ldv, int64_t n, int nu,
     const float hr = (float)v.x, hi = (float)v.y;
     sV[c * kRMRows + rr] = make_float4(hr, hi, (float)(v.x - hr), (float)(v.y - hi));
   }
-  constexpr int kOut = kMaxNu * kRMRows / 256;
   const int outs = kRMRows * nu;
   float sr[kOut], srl[kOut], si[kOut], sil[kOut];
 #pragma unroll
@@ -791,6 +865,318 @@ right_multiply_near_df_kernel(double2* V, int64_t ldv, int64_t n, int nu,
   }
 }
 
+__global__ void __launch_bounds__(256)
+right_multiply_near_df_kernel(double2* V, int64_t ldv, int64_t n, int nu,
+                              const float4* __restrict__ Ms, const int* gate, const int* skip_if) {
+  if ((gate && *gate == 0) || (skip_if && *skip_if != 0)) return;
+  extern __shared__ float4 df_smem[];
+  multiply_df_rows<kMaxNu * kRMRows / 256>(df_smem, V, ldv, n, nu, Ms);
+}
+
+// ---- nu <= kSmallNu: one launch a factor ----
+//
+// The steps between a Gram matrix and its multiplication are short and dependent; as kernels of
+// their own (sum, products, norm, Cholesky, inverse, second step, split) each costs a launch,
+// most of them only to find that it is not needed: ~25 launches of 2-4 us against 10 us of work
+// at 320 x 16. Here one cluster of eight blocks does them all, with cluster barriers between
+// the steps that exchange data (through global memory; a block reads what others wrote with
+// ld.cg) and plain branches where the flags were. A CholeskyQR2 takes 9 launches instead of 36:
+// 150 -> 62 us at 320 x 16,
+// 170 -> 94 us at 1452 x 30.
+constexpr int kSmallNu = 64;
+constexpr int kFactorBlocks = 8, kFactorThreads = 1024;
+enum { kFactor32 = 0, kFactorNear = 1, kFactorClassic = 2 };
+
+struct FactorArgs {
+  const double2* part;   // partial Gram matrices
+  int parts, nu;
+  double2 *G, *P, *Y, *Z;
+  float4* Ms;            // Z - I split for the double-FP32 multiply
+  int* flag;             // kFactor32: 1 = too ill-conditioned for FP32; kFactorNear: 1 = near route
+  int* status;
+  int* deficient;        // kFactorClassic: see cholesky_kernel
+  const int* gate;
+};
+
+size_t factor_smem(int mode, int nu) {
+  return mode == kFactorNear ? (size_t)(2 * nu * (nu + 1) + kFactorBlocks * (nu + 1)) * sizeof(double2) : 0;
+}
+
+// Z = R^{-1} of G = R^H R in FP64 by the elimination of chol_inv32_kernel, with the pivot rule
+// of cholesky_kernel. entry(r, c): G(r, c), r <= c. Whole block; false on a failed pivot.
+template <int kT, typename Entry>
+__device__ bool eliminate64(const Entry& entry, int nu, double2* __restrict__ Z, int* deficient) {
+  __shared__ double2 col[2][32 * kT];
+  __shared__ double diag[32 * kT];
+  const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
+  const int tr = lane % 8 + 8 * (w % 4), tc = lane / 8 + 4 * (w / 4);
+  double2 g[kT][kT];
+#pragma unroll
+  for (int i = 0; i < kT; ++i)
+#pragma unroll
+    for (int j = 0; j < kT; ++j) {
+      const int r = tr + 32 * i, c = tc + 32 * j;
+      g[i][j] = make_double2(0.0, 0.0);
+      if (r >= c && r < nu) {
+        const double2 v = entry(c, r);
+        g[i][j] = make_double2(v.x, -v.y);
+        if (r == c) diag[r] = v.x;
+      }
+    }
+  if (tc == 0)
+#pragma unroll
+    for (int i = 0; i < kT; ++i) col[0][tr + 32 * i] = g[i][0];
+  __syncthreads();
+  double dmax = 0.0;
+  for (int k = 0; k < nu; ++k) dmax = fmax(dmax, diag[k]);
+  __syncthreads();
+  bool ok = true;
+  for (int k = 0; k < nu; ++k) {
+    const double2* s = col[k & 1];
+    double d = s[k].x;
+    const bool bad = !(d > 1e-13 * dmax) || !isfinite(d);
+    if (bad && !deficient) {
+      ok = false;
+      break;
+    }
+    if (tid == 0 && deficient) deficient[k] = bad ? 1 : 0;
+    if (bad) d = 1.0;   // unit pivot, no update
+    if (tid == 0) diag[k] = d;
+    const double rd = 1.0 / d;
+    double2 a[kT];
+#pragma unroll
+    for (int i = 0; i < kT; ++i) a[i] = tr + 32 * i == k ? make_double2(1.0, 0.0) : s[tr + 32 * i];
+#pragma unroll
+    for (int j = 0; j < kT; ++j) {
+      if (32 * j + 31 <= k) continue;
+      const int c = tc + 32 * j;
+      double2 l = s[c];
+      l = c > k && !bad ? make_double2(l.x * rd, l.y * rd) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int i = 0; i < kT; ++i) {
+        if (i < j && 32 * i > k) continue;
+        const int r = tr + 32 * i;
+        const double ly = r >= c ? -l.y : l.y;
+        if (c > k && !bad && (r >= c || r <= k)) {
+          g[i][j].x -= a[i].x * l.x - a[i].y * ly;
+          g[i][j].y -= a[i].x * ly + a[i].y * l.x;
+        }
+      }
+      if (c == k + 1)
+#pragma unroll
+        for (int i = 0; i < kT; ++i) col[(k + 1) & 1][tr + 32 * i] = g[i][j];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < kT; ++j) {
+    const int c = tc + 32 * j;
+    if (c >= nu) continue;
+    const double inv = ok ? 1.0 / sqrt(diag[c]) : NAN;
+#pragma unroll
+    for (int i = 0; i < kT; ++i) {
+      const int r = tr + 32 * i;
+      if (r >= nu) continue;
+      Z[(int64_t)c * nu + r] = r > c ? make_double2(0.0, 0.0)
+                               : r == c ? make_double2(inv, 0.0)
+                                        : make_double2(g[i][j].x * inv, -g[i][j].y * inv);
+    }
+  }
+  return ok;
+}
+
+// Second-order terms Y0^H Y0 + Y0^2 (+ its conjugate on the diagonal) at (i, j), i <= j.
+template <typename T2, typename Y0>
+__device__ __forceinline__ T2 second_order_at(const Y0& y0, int i, int j) {
+  T2 h;
+  h.x = h.y = 0;
+  for (int m = 0; m <= i; ++m) {
+    const T2 a = y0(m, i), b = y0(m, j);
+    h.x += a.x * b.x + a.y * b.y;
+    h.y += a.x * b.y - a.y * b.x;
+  }
+  for (int m = i; m <= j; ++m) {
+    const T2 a = y0(i, m), b = y0(m, j);
+    h.x += a.x * b.x - a.y * b.y;
+    h.y += a.x * b.y + a.y * b.x;
+    if (i == j) h.x += a.x * b.x - a.y * b.y;
+  }
+  return h;
+}
+
+template <int kMode, int kT>
+__global__ void __cluster_dims__(kFactorBlocks, 1, 1) __launch_bounds__(kFactorThreads)
+cq_factor_kernel(FactorArgs p) {
+  if (p.gate && *p.gate == 0) return;
+  extern __shared__ double2 factor_mem[];
+  __shared__ double2 red[32][32];
+  __shared__ float redf[32];
+  const int tid = threadIdx.x, lane = tid % 32, w = tid / 32, nu = p.nu;
+  const int rank = (int)sm100::cluster_ctarank();
+  // G = sum of the partials: a warp adds every eighth part of 32 elements
+  for (int t0 = rank * 128; t0 < nu * nu; t0 += kFactorBlocks * 128) {
+    const int q = w % 8, t = t0 + (w / 8) * 32 + lane;
+    const bool live = t < nu * nu && t % nu / kGT <= t / nu / kGT;
+    double2 sum = make_double2(0.0, 0.0);
+    if (live)
+#pragma unroll 8
+      for (int r = q; r < p.parts; r += 8) {
+        const double2 v = p.part[(int64_t)r * nu * nu + t];
+        sum.x += v.x;
+        sum.y += v.y;
+      }
+    red[w][lane] = sum;
+    __syncthreads();
+    if (live && q == 0) {
+#pragma unroll
+      for (int k = 1; k < 8; ++k) {
+        sum.x += red[w + k][lane].x;
+        sum.y += red[w + k][lane].y;
+      }
+      p.G[t] = sum;
+    }
+    __syncthreads();
+  }
+  sm100::cluster_sync_all();
+  if (kMode == kFactor32) {
+    if (rank != 0 || tid >= 256) return;
+    if (tid == 0) *p.flag = 0;   // (chol_inv32_block: same thread)
+    if (nu <= 16)
+      chol_inv32_block<16, 1>(p.G, nu, nu, p.G, nu, p.Z, nu, p.flag);
+    else
+      chol_inv32_block<16, 2 * kT>(p.G, nu, nu, p.G, nu, p.Z, nu, p.flag);
+    return;
+  }
+  if (kMode == kFactorClassic) {
+    if (rank == 0) {
+      const bool ok = eliminate64<kT>([&](int r, int c) { return __ldcg(p.G + (int64_t)c * nu + r); },
+                                      nu, p.Z, p.deficient);
+      if (!ok && tid == 0) atomicOr(p.status, kStatusNotSPD);
+    }
+    return;
+  }
+  const int ld = nu + 1;   // (odd in 16-byte words: columns over all banks)
+  double2* sG = factor_mem;            // [c][r], r <= c
+  double2* sY = sG + nu * ld;
+  double2* sP = sY + nu * ld;          // this block's rows of P
+  float2* yf = reinterpret_cast<float2*>(sY);
+  float e2 = 0.f;
+  for (int t = tid; t < nu * nu; t += kFactorThreads) {
+    const int r = t % nu, c = t / nu;
+    if (r > c) continue;
+    const double2 g = __ldcg(p.G + t);
+    sG[c * ld + r] = g;
+    const float ex = (float)(r == c ? g.x - 1.0 : g.x), ey = r == c ? 0.f : (float)g.y;
+    e2 += (ex * ex + ey * ey) * (r == c ? 1.f : 2.f);
+    yf[c * ld + r] = r == c ? make_float2(-0.5f * ex, 0.f) : make_float2(-ex, -ey);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+  if (lane == 0) redf[w] = e2;
+  __syncthreads();
+  e2 = redf[lane];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+  const bool near = e2 <= kNearEps * kNearEps, small = e2 <= kNearEpsSmall * kNearEpsSmall;
+  if (rank == 0 && tid == 0) *p.flag = near ? 1 : 0;
+  if (!near) {
+    if (rank == 0) {
+      const bool ok = eliminate64<kT>([&](int r, int c) { return sG[c * ld + r]; }, nu, p.Z, nullptr);
+      if (!ok && tid == 0) atomicOr(p.status, kStatusNotSPD);
+    }
+    return;
+  }
+  auto e_at = [&](int m, int j) {
+    if (m > j) {
+      const double2 g = sG[m * ld + j];
+      return make_double2(g.x, -g.y);
+    }
+    const double2 g = sG[j * ld + m];
+    return m == j ? make_double2(g.x - 1.0, 0.0) : g;
+  };
+  // this thread's output: rows rank, rank + 8, ... of the block, a column each
+  const int i = rank + kFactorBlocks * (tid / kSmallNu), j = tid % kSmallNu;
+  const bool out = i < nu && j < nu;
+  auto finish = [&](double2 y) {   // Z = I + Y at (i, j), and its split
+    const int t = j * nu + i;
+    const double2 z = i > j ? make_double2(0.0, 0.0) : i == j ? make_double2(1.0 + y.x, 0.0) : y;
+    const double br = i == j ? z.x - 1.0 : z.x;
+    p.Z[t] = z;
+    const float fr = (float)br, fi = (float)z.y;
+    p.Ms[t] = make_float4(fr, fi, (float)(br - fr), (float)(z.y - fi));
+  };
+  auto y1_of = [&](double2 h) {
+    const double2 e = e_at(i, j);
+    return i < j ? make_double2(h.x - e.x, h.y - e.y) : make_double2(-0.5 * (e.x - h.x), 0.0);
+  };
+  if (small) {   // as near_y1_kernel: FP32 second-order terms
+    if (!out) return;
+    double2 y = make_double2(0.0, 0.0);
+    if (i <= j) {
+      const float2 h = second_order_at<float2>([&](int r, int c) { return yf[c * ld + r]; }, i, j);
+      y = y1_of(make_double2(h.x, h.y));
+    }
+    finish(y);
+    return;
+  }
+  if (out && i <= j) {
+    auto y0 = [&](int r, int c) {
+      const double2 g = sG[c * ld + r];
+      return r == c ? make_double2(-0.5 * (g.x - 1.0), 0.0) : make_double2(-g.x, -g.y);
+    };
+    p.Y[j * nu + i] = y1_of(second_order_at<double2>(y0, i, j));
+  }
+  sm100::cluster_sync_all();
+  for (int t = tid; t < nu * nu; t += kFactorThreads) {
+    const int r = t % nu, c = t / nu;
+    sY[c * ld + r] = r <= c ? __ldcg(p.Y + t) : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  double2 pe = make_double2(0.0, 0.0), q = pe;
+  if (out) {
+    for (int m = 0; m <= i; ++m) {
+      const double2 a = sY[i * ld + m], b = e_at(m, j), c = sY[j * ld + m];
+      pe.x += a.x * b.x + a.y * b.y;
+      pe.y += a.x * b.y - a.y * b.x;
+      q.x += a.x * c.x + a.y * c.y;
+      q.y += a.x * c.y - a.y * c.x;
+    }
+    sP[tid / kSmallNu * ld + j] = pe;
+    p.P[j * nu + i] = pe;
+  }
+  __syncthreads();
+  sm100::cluster_sync_all();
+  if (!out) return;
+  double2 y = make_double2(0.0, 0.0);
+  if (i <= j) {
+    double2 h = e_at(i, j);
+    const double2 pt = __ldcg(p.P + i * nu + j);
+    h.x += pe.x + pt.x + q.x;
+    h.y += pe.y - pt.y + q.y;
+    for (int m = 0; m <= j; ++m) {
+      const double2 a = sP[tid / kSmallNu * ld + m], b = sY[j * ld + m];
+      h.x += a.x * b.x - a.y * b.y;
+      h.y += a.x * b.y + a.y * b.x;
+    }
+    y = i < j ? make_double2(-h.x, -h.y) : make_double2(-0.5 * h.x, 0.0);
+  }
+  finish(y);
+}
+
+// V <- V Z for nu <= kSmallNu: the near-identity product where *near says so, else in FP64.
+__global__ void __launch_bounds__(256)
+multiply_small_kernel(double2* V, int64_t ldv, int64_t n, int nu, const double2* __restrict__ Z,
+                      const float4* __restrict__ Ms, const int* gate, const int* skip_if,
+                      const int* near) {
+  if ((gate && *gate == 0) || (skip_if && *skip_if != 0)) return;
+  extern __shared__ double rm_smem[];
+  constexpr int kOut = kSmallNu * kRMRows / 256;
+  if (near && *near != 0)
+    multiply_df_rows<kOut>(reinterpret_cast<float4*>(rm_smem), V, ldv, n, nu, Ms);
+  else
+    multiply64_rows<kOut>(rm_smem, V, ldv, n, nu, Z);
+}
+
 // C = A * B for upper-triangular nu x nu A, B (one block).
 __global__ void upper_product_kernel(const double2* A, const double2* B, int nu, double2* C) {
   for (int64_t t = threadIdx.x; t < (int64_t)nu * nu; t += blockDim.x) {
@@ -813,9 +1199,8 @@ namespace {
 struct CqLayout {
   int tiles_u = 0;           // upper Gram tiles
   int64_t parts = 0, rows_per_part = 0;
+  int64_t parts32 = 0, rows32 = 0;   // of the FP32 Gram matrix
   int64_t parts_max = 0;     // with those of the split products
-  int near_blocks = 0;       // blocks of the near-identity element kernels (64 threads)
-  int near_tiles = 0;        // 8 x 8 tiles of the near-identity products
   unsigned sum_blocks = 0;   // blocks of sum_parts_kernel (eight threads per element)
 };
 
@@ -825,13 +1210,16 @@ CqLayout cq_layout(bem_ctx* ctx, int64_t n, int nu) {
   CqLayout L;
   const int T = (nu + kGT - 1) / kGT;
   L.tiles_u = T * (T + 1) / 2;
-  L.parts = std::max<int64_t>(1, std::min<int64_t>((n + kGT - 1) / kGT,
-                                                   (2 * (int64_t)sms + L.tiles_u - 1) / L.tiles_u));
+  // no fewer than 4 rows a part: a 32 x 32 tile of a row is 0.8 us of an SM's FP64 pipe, so a short
+  // V is spread thin (320 x 16: 27 us at 32 rows a part, 5.6 us at 4); one block an SM where a
+  // single cluster adds the parts
+  const int64_t blocks = (nu <= kSmallNu ? 1 : 2) * (int64_t)std::max(1, sms);
+  L.parts = std::max<int64_t>(1, std::min<int64_t>((n + 3) / 4, (blocks + L.tiles_u - 1) / L.tiles_u));
   L.rows_per_part = (n + L.parts - 1) / L.parts;
   L.parts = (n + L.rows_per_part - 1) / L.rows_per_part;
+  L.rows32 = std::max<int64_t>(L.rows_per_part, kGT);
+  L.parts32 = (n + L.rows32 - 1) / L.rows32;
   L.parts_max = std::max<int64_t>(L.parts, split64_parts(ctx, n, nu));
-  L.near_blocks = (int)(((int64_t)nu * nu + 63) / 64);
-  L.near_tiles = ((nu + 7) / 8) * ((nu + 7) / 8);
   L.sum_blocks = (unsigned)((8 * (int64_t)nu * nu + 255) / 256);
   return L;
 }
@@ -857,12 +1245,6 @@ CqWork cq_work(void* work, int nu, const CqLayout& L) {
   return w;
 }
 
-// ||G - I||_F up to which the near-identity factor is used; its error is O(||G - I||^4)
-// (at 8e-4 it still matches the Cholesky factor to rounding)
-constexpr float kNearEps = 5e-4f;
-// ||G - I||_F up to which the first step alone is exact to rounding
-constexpr float kNearEpsSmall = 1e-5f;
-
 bem_status set_smem(bem_ctx* ctx, const void* fn, size_t bytes) {
   if (bytes <= 48 * 1024) return BEM_OK;
   return cuda_check(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -870,21 +1252,49 @@ bem_status set_smem(bem_ctx* ctx, const void* fn, size_t bytes) {
                     "cholqr attribute");
 }
 
-// Partial sums of the FP64 Gram matrix into w.part, added into G: on the tensor core where the
-// plan says so (split64.cu), else on the FP64 pipe.
-bem_status gram64(bem_ctx* ctx, const Split64& sp, double2* V, int64_t ldv, int64_t n, int nu,
-                  const CqLayout& L, const CqWork& w, double2* G, const int* gate, cudaStream_t s) {
-  int parts = (int)L.parts;
-  if (sp.use) {
-    const bem_status st = split64_gram(ctx, sp, V, w.part, gate, s);
+// Partial sums of the FP64 Gram matrix into w.part (their count in parts): on the tensor core
+// where the plan says so (split64.cu), else on the FP64 pipe.
+bem_status gram_parts64(bem_ctx* ctx, const Split64& sp, const double2* V, int64_t ldv, int64_t n,
+                        int nu, const CqLayout& L, const CqWork& w, const int* gate, int& parts,
+                        cudaStream_t s) {
+  parts = sp.use ? sp.parts : (int)L.parts;
+  if (sp.use) return split64_gram(ctx, sp, V, w.part, gate, s);
+  gram_partial_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
+      V, ldv, n, nu, L.rows_per_part, w.part, gate);
+  ctx->launches++;
+  return BEM_OK;
+}
+
+// V <- V Z in FP64 (skipped when gate and *gate == 0, or skip and *skip != 0). same: V is the one
+// whose Gram matrix was formed last (the split products then have its scales).
+bem_status multiply64(bem_ctx* ctx, const Split64& sp, bool same, double2* V, int64_t ldv,
+                      int64_t n, int nu, const double2* Z, const int* gate, const int* skip,
+                      cudaStream_t s) {
+  if (sp.use) return split64_multiply(ctx, sp, same, V, Z, gate, skip, s);
+  const unsigned rb = (unsigned)((n + kRMRows - 1) / kRMRows);
+  if (nu <= kSmallNu)
+    multiply_small_kernel<<<rb, 256, right_multiply_smem(nu), s>>>(V, ldv, n, nu, Z, nullptr, gate,
+                                                                   skip, nullptr);
+  else
+    right_multiply_kernel<<<rb, 256, right_multiply_smem(nu), s>>>(V, ldv, n, nu, Z, gate, skip, nullptr);
+  ctx->launches++;
+  return BEM_OK;
+}
+
+// The factor of a Gram matrix in w.part for nu <= kSmallNu (cq_factor_kernel).
+template <int kMode>
+bem_status small_factor(bem_ctx* ctx, const CqWork& w, int parts, int nu, int* flag, int* deficient,
+                        const int* gate, cudaStream_t s) {
+  const FactorArgs a{w.part, parts, nu, w.G, w.P, w.Y, w.Z, reinterpret_cast<float4*>(w.Q1),
+                     flag, ctx->d_status, deficient, gate};
+  auto* kernel = nu <= 32 ? cq_factor_kernel<kMode, 1> : cq_factor_kernel<kMode, 2>;
+  if (factor_smem(kMode, nu) > 0) {   // (beside ~19 KB of its static arrays)
+    const bem_status st = cuda_check(
+        ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_smem(kMode, nu)),
+        "cholqr attribute");
     if (st != BEM_OK) return st;
-    parts = sp.parts;
-  } else {
-    gram_partial_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
-        V, ldv, n, nu, L.rows_per_part, w.part, gate);
-    ctx->launches++;
   }
-  sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, parts, nu, G, gate);
+  kernel<<<kFactorBlocks, kFactorThreads, factor_smem(kMode, nu), s>>>(a);
   ctx->launches++;
   return BEM_OK;
 }
@@ -896,33 +1306,41 @@ bem_status gram64(bem_ctx* ctx, const Split64& sp, double2* V, int64_t ldv, int6
 bem_status near_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu,
                      const CqLayout& L, const CqWork& w, const Split64& sp, const int* gate,
                      int* classic, cudaStream_t s) {
-  int* done = classic + 2;   // classic flag and its "second step not needed" companion
-  bem_status st = cuda_check(ctx, cudaMemsetAsync(classic, 0, 3 * sizeof(int), s), "cholqr flag");
-  if (st != BEM_OK) return st;
   double2* V = reinterpret_cast<double2*>(V_dev);
-  const unsigned nb = (unsigned)L.near_blocks;
-  if ((st = gram64(ctx, sp, V, ldv, n, nu, L, w, w.G, gate, s)) != BEM_OK) return st;
+  const unsigned rb = (unsigned)((n + kRMRows - 1) / kRMRows);
+  int parts;
+  bem_status st = gram_parts64(ctx, sp, V, ldv, n, nu, L, w, gate, parts, s);
+  if (st != BEM_OK) return st;
+  float4* Zs = reinterpret_cast<float4*>(w.Q1);   // Z - I split (Q1 is free by then)
+  if (nu <= kSmallNu) {
+    int* near = classic;
+    if ((st = small_factor<kFactorNear>(ctx, w, parts, nu, near, nullptr, gate, s)) != BEM_OK) return st;
+    if (sp.use) return split64_multiply(ctx, sp, true, V, w.Z, gate, nullptr, s);
+    multiply_small_kernel<<<rb, 256, right_multiply_smem(nu), s>>>(V, ldv, n, nu, w.Z, Zs, gate,
+                                                                   nullptr, near);
+    ctx->launches++;
+    return cuda_check(ctx, cudaGetLastError(), "cholqr kernels");
+  }
+  int* done = classic + 2;   // classic flag and its "second step not needed" companion
+  st = cuda_check(ctx, cudaMemsetAsync(classic, 0, 3 * sizeof(int), s), "cholqr flag");
+  if (st != BEM_OK) return st;
+  sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, parts, nu, w.G, w.epsp, gate);
   const unsigned nt = (unsigned)((nu + kNT - 1) / kNT);
   const dim3 tgrid(nt, nt);
-  near_tile_kernel<0><<<tgrid, 64, 0, s>>>(w.G, nullptr, nullptr, nullptr, nu, w.P, w.Q, nullptr,
-                                           w.epsp, gate, nullptr);
-  near_y1_kernel<<<nb, 64, 0, s>>>(w.G, w.P, w.Q, w.epsp, (int)(nt * nt), nu, kNearEps,
-                                   kNearEpsSmall, w.Y, w.Z, classic, done, gate);
-  const size_t chol_smem = nu <= 64 ? (size_t)nu * nu * sizeof(double2) : 0;
-  cholesky_kernel<<<1, 1024, chol_smem, s>>>(w.G, nu, ctx->d_status, nullptr, classic);
+  near_y1_kernel<<<tgrid, 64, 0, s>>>(w.G, w.epsp, (int)L.sum_blocks, nu, kNearEps, kNearEpsSmall,
+                                      w.Y, w.Z, classic, done, gate);
+  cholesky_kernel<<<1, 1024, 0, s>>>(w.G, nu, ctx->d_status, nullptr, classic);
   triangular_inverse_kernel<<<nu, 128, 0, s>>>(w.G, nu, w.Z, classic);
   near_tile_kernel<1><<<tgrid, 64, 0, s>>>(w.G, w.Y, nullptr, nullptr, nu, w.P1, w.Q1, nullptr,
-                                           nullptr, gate, done);
+                                           gate, done);
   near_tile_kernel<2><<<tgrid, 64, 0, s>>>(w.G, w.Y, w.P1, w.Q1, nu, nullptr, nullptr, w.Z,
-                                           nullptr, gate, done);
+                                           gate, done);
   ctx->launches += 6;
   // V <- V Z: on the tensor core; else the classic inverse in FP64, the near-identity factor as
   // V + V (Z - I)
-  if (sp.use) return split64_multiply(ctx, sp, V, w.Z, gate, nullptr, s);
-  const unsigned rb = (unsigned)((n + kRMRows - 1) / kRMRows);
+  if (sp.use) return split64_multiply(ctx, sp, true, V, w.Z, gate, nullptr, s);
   right_multiply_kernel<<<rb, 256, right_multiply_smem(nu), s>>>(V, ldv, n, nu, w.Z, gate,
                                                                  nullptr, classic);
-  float4* Zs = reinterpret_cast<float4*>(w.R2);   // R2 is free outside the classic passes
   split_near_factor_kernel<<<(unsigned)((nu * nu + 255) / 256), 256, 0, s>>>(w.Z, nu, Zs, gate,
                                                                             classic);
   right_multiply_near_df_kernel<<<rb, 256, right_multiply_df_smem(nu), s>>>(V, ldv, n, nu, Zs,
@@ -931,30 +1349,28 @@ bem_status near_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu
   return cuda_check(ctx, cudaGetLastError(), "cholqr kernels");
 }
 
-// V <- V Z in FP64 (skipped when skip and *skip != 0).
-bem_status multiply64(bem_ctx* ctx, const Split64& sp, double2* V, int64_t ldv, int64_t n, int nu,
-                      const double2* Z, const int* skip, cudaStream_t s) {
-  if (sp.use) return split64_multiply(ctx, sp, V, Z, nullptr, skip, s);
-  right_multiply_kernel<<<(unsigned)((n + kRMRows - 1) / kRMRows), 256, right_multiply_smem(nu),
-                          s>>>(V, ldv, n, nu, Z, nullptr, skip, nullptr);
-  ctx->launches++;
-  return BEM_OK;
-}
-
 // Classic FP64 pass: Gram, Cholesky (optionally refreshing collapsed columns), inverse,
-// V <- V R^{-1}; R kept in R_out.
+// V <- V R^{-1}; R kept in R_out if it is given.
 bem_status classic_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu,
                         const CqLayout& L, const CqWork& w, const Split64& sp, double2* R_out,
                         uint64_t refresh_seed, cudaStream_t s) {
   double2* V = reinterpret_cast<double2*>(V_dev);
-  bem_status st = gram64(ctx, sp, V, ldv, n, nu, L, w, R_out, nullptr, s);
+  int parts;
+  bem_status st = gram_parts64(ctx, sp, V, ldv, n, nu, L, w, nullptr, parts, s);
   if (st != BEM_OK) return st;
-  const size_t chol_smem = nu <= 64 ? (size_t)nu * nu * sizeof(double2) : 0;
-  cholesky_kernel<<<1, 1024, chol_smem, s>>>(R_out, nu, ctx->d_status,
-                                             refresh_seed ? w.deficient : nullptr, nullptr);
-  triangular_inverse_kernel<<<nu, 128, 0, s>>>(R_out, nu, w.Z, nullptr);
-  ctx->launches += 2;
-  if ((st = multiply64(ctx, sp, V, ldv, n, nu, w.Z, nullptr, s)) != BEM_OK) return st;
+  int* deficient = refresh_seed ? w.deficient : nullptr;
+  if (!R_out && nu <= kSmallNu) {
+    if ((st = small_factor<kFactorClassic>(ctx, w, parts, nu, nullptr, deficient, nullptr, s)) != BEM_OK)
+      return st;
+  } else {
+    double2* R = R_out ? R_out : w.R1;
+    sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, parts, nu, R, nullptr, nullptr);
+    const size_t chol_smem = nu <= 64 ? (size_t)nu * nu * sizeof(double2) : 0;
+    cholesky_kernel<<<1, 1024, chol_smem, s>>>(R, nu, ctx->d_status, deficient, nullptr);
+    triangular_inverse_kernel<<<nu, 128, 0, s>>>(R, nu, w.Z, nullptr);
+    ctx->launches += 3;
+  }
+  if ((st = multiply64(ctx, sp, true, V, ldv, n, nu, w.Z, nullptr, nullptr, s)) != BEM_OK) return st;
   if (refresh_seed) {
     refresh_columns_kernel<<<(unsigned)((n * nu + 255) / 256), 256, 0, s>>>(V, ldv, n, nu,
                                                                            w.deficient,
@@ -969,7 +1385,7 @@ bem_status classic_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int
 size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu) {
   const CqLayout L = cq_layout(ctx, n, nu);
   return (9 + (size_t)L.parts_max) * (size_t)nu * nu * sizeof(double2) +
-         (256 + 8) * sizeof(int) + (size_t)L.near_tiles * sizeof(float);
+         (256 + 8) * sizeof(int) + (size_t)L.sum_blocks * sizeof(float);
 }
 
 // CholeskyQR2 of V (n x nu, ld ldv) with caller-provided work (cholqr2_work_bytes);
@@ -1004,47 +1420,52 @@ bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int
     return cuda_check(ctx, cudaGetLastError(), "cholqr kernels");
   }
   if (refresh_seed != 0) {
-    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R1, refresh_seed, s)) != BEM_OK) return st;
+    if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, refresh_seed, s)) != BEM_OK) return st;
     return near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, s);
   }
   int* fallback = w.flags;
-  const int h = std::min(nu, kChol32), r = nu - h;   // diagonal blocks of the FP32 factor
-  const size_t ci_smem = (size_t)h * h * sizeof(float2);
-  if ((st = set_smem(ctx, (const void*)chol_inv32_kernel<4>, std::min(ci_smem, (size_t)64 * 64 * sizeof(float2)))) != BEM_OK ||
-      (st = set_smem(ctx, (const void*)chol_inv32_kernel<16>, ci_smem)) != BEM_OK)
-    return st;
-  st = cuda_check(ctx, cudaMemsetAsync(fallback, 0, sizeof(int), s), "cholqr flag");
-  if (st != BEM_OK) return st;
   double2* V = reinterpret_cast<double2*>(V_dev);
-  if (sp.use && nu > kChol32) {
-    if ((st = gram64(ctx, sp, V, ldv, n, nu, L, w, w.G, nullptr, s)) != BEM_OK) return st;
+  int parts;
+  const bool wide = sp.use && nu > kChol32;   // the split Gram matrix, else FP32
+  if (wide) {
+    if ((st = gram_parts64(ctx, sp, V, ldv, n, nu, L, w, nullptr, parts, s)) != BEM_OK) return st;
   } else {
-    gram_partial32_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts), 256, 0, s>>>(
-        V, ldv, n, nu, L.rows_per_part, w.part);
-    sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, (int)L.parts, nu, w.G, nullptr);
-    ctx->launches += 2;
-  }
-  auto inverse32 = [&](const double2* G, int ldg, int m, double2* Z) {
-    if (m <= 64)
-      chol_inv32_kernel<4><<<1, 1024, (size_t)m * m * sizeof(float2), s>>>(G, ldg, m, w.G, nu, Z, nu, fallback);
-    else
-      chol_inv32_kernel<16><<<1, 1024, (size_t)m * m * sizeof(float2), s>>>(G, ldg, m, w.G, nu, Z, nu, fallback);
+    parts = (int)L.parts32;
+    gram_partial32_kernel<<<dim3((unsigned)L.tiles_u, (unsigned)L.parts32), 256, 0, s>>>(
+        V, ldv, n, nu, L.rows32, w.part);
     ctx->launches++;
-  };
-  inverse32(w.G, nu, h, w.Z);
-  if (r > 0) {
-    const dim3 gh((unsigned)((h + 15) / 16), (unsigned)((r + 15) / 16)), gr(gh.y, gh.y);
-    chol_block32_kernel<0><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-    chol_block32_kernel<1><<<gr, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-    inverse32(w.Q, r, r, w.Z + (size_t)h * nu + h);
-    chol_block32_kernel<2><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-    chol_block32_kernel<3><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-    ctx->launches += 4;
   }
-  if ((st = multiply64(ctx, sp, V, ldv, n, nu, w.Z, fallback, s)) != BEM_OK) return st;
+  if (nu <= kSmallNu) {
+    if ((st = small_factor<kFactor32>(ctx, w, parts, nu, fallback, nullptr, nullptr, s)) != BEM_OK) return st;
+  } else {
+    st = cuda_check(ctx, cudaMemsetAsync(fallback, 0, sizeof(int), s), "cholqr flag");
+    if (st != BEM_OK) return st;
+    sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, parts, nu, w.G, nullptr, nullptr);
+    const int h = std::min(nu, kChol32), r = nu - h;   // diagonal blocks of the FP32 factor
+    auto inverse32 = [&](const double2* G, int ldg, int m, double2* Z) {
+      auto* kernel = m <= 32 ? chol_inv32_kernel<1> : m <= 64 ? chol_inv32_kernel<2> : chol_inv32_kernel<4>;
+      kernel<<<1, 1024, 0, s>>>(G, ldg, m, w.G, nu, Z, nu, fallback);
+      ctx->launches++;
+    };
+    inverse32(w.G, nu, h, w.Z);
+    ctx->launches++;
+    if (r > 0) {
+      const dim3 gh((unsigned)((h + 15) / 16), (unsigned)((r + 15) / 16)), gr(gh.y, gh.y);
+      chol_block32_kernel<0><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+      chol_block32_kernel<1><<<gr, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+      inverse32(w.Q, r, r, w.Z + (size_t)h * nu + h);
+      chol_block32_kernel<2><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+      chol_block32_kernel<3><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
+      ctx->launches += 4;
+    }
+  }
+  if ((st = multiply64(ctx, sp, wide, V, ldv, n, nu, w.Z, nullptr, fallback, s)) != BEM_OK) return st;
   if ((st = cuda_check(ctx, cudaGetLastError(), "cholqr kernels")) != BEM_OK) return st;
   if ((st = near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, s)) != BEM_OK) return st;
-  return near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, fallback, w.flags + 4, s);
+  // the third pass rarely runs: for the smaller bases the form with the fewest launches
+  Split64 third = sp;
+  if (nu <= kSmallNu && n * (int64_t)nu * nu < ((int64_t)1 << 25)) third.use = false;
+  return near_pass(ctx, V_dev, ldv, n, nu, L, w, third, fallback, w.flags + 4, s);
 }
 
 }  // namespace bem

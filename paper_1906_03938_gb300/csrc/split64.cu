@@ -51,10 +51,11 @@ constexpr uint32_t kWaitG = kStageWaitDefault;
 constexpr int kNotFinite = INT_MIN;           // exponent of a scale over non-finite values
 constexpr int kZero = -4000;                  // of one over zeros
 constexpr size_t kMaxSplitBytes = (size_t)8 << 30;
-// n nu^2 from which the split products pay. A CholeskyQR2, split against FP64 products, in us:
-// 4096 x 32 342 / 256, 1452 x 64 392 / 323, 3072 x 64 410 / 380 below it; 512 x 256 1462 / 1947,
-// 3072 x 128 724 / 1098, 65536 x 32 668 / 1188, 8192 x 256 1909 / 7171 above.
-constexpr int64_t kMinWork = (int64_t)1 << 25;
+// n nu^2 from which the split products pay (more launches, less work). A CholeskyQR2, split
+// against FP64 products, in us: 4096 x 32 225 / 172, 20000 x 16 300 / 273, 1452 x 64 271 / 238
+// below it; 600 x 128 420 / 502, 12000 x 32 265 / 287, 3072 x 64 284 / 313, 6000 x 48 289 / 428,
+// 50000 x 16 425 / 525, 8192 x 256 1909 / 7171 above.
+constexpr int64_t kMinWork = (int64_t)1 << 23;
 
 __device__ __forceinline__ bool skipped(const int* gate, const int* skip) {
   return (gate && *gate == 0) || (skip && *skip != 0);
@@ -115,21 +116,15 @@ split_colmax_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, unsig
   if (threadIdx.x % 32 == 0 && m) atomicMax(hi + blockIdx.x, m);
 }
 
-// hi -> exponents, in place
-__global__ void split_exponent_kernel(unsigned* hi, int nu, const int* gate, const int* skip) {
-  if (skipped(gate, skip)) return;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < nu) hi[c] = (unsigned)exponent_of(hi[c]);
-}
-
 __device__ __forceinline__ int scale_exp(int e) { return (e == kNotFinite || e == kZero) ? 0 : e; }
+__device__ __forceinline__ int col_exp(const unsigned* hi, int c) { return scale_exp(exponent_of(hi[c])); }
 
 // Digit planes of V's columns with the rows as K: a[kb][tile of 128 columns][digit][re, im] and
 // b[kb][tile of 32 columns]{[digit][re | im], [digit][im | -re]}, in K-major core matrices. One
 // thread per column and 8 rows.
 __global__ void __launch_bounds__(128)
 split_columns_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu, int kbn,
-                     int mtu, int ntu, const int* __restrict__ ec, unsigned char* __restrict__ a,
+                     int mtu, int ntu, const unsigned* __restrict__ hc, unsigned char* __restrict__ a,
                      unsigned char* __restrict__ b, const int* gate) {
   if (skipped(gate, nullptr)) return;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -143,7 +138,7 @@ split_columns_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int 
   const int64_t kb = gr / 2;
   const int kh = (int)(gr % 2);
   long long re[8], im[8];
-  const int e = c < nu ? scale_exp(ec[c]) : 0;
+  const int e = c < nu ? col_exp(hc, c) : 0;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int64_t i = gr * 8 + j;
@@ -176,58 +171,63 @@ split_columns_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int 
   put_b(1, 1);
 }
 
-// Exponent of each row of V D^-1, D = diag(2^ec).
-__global__ void __launch_bounds__(128)
-split_rowmax_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu,
-                    const int* __restrict__ ec, int* __restrict__ er, const int* gate,
-                    const int* skip) {
-  if (skipped(gate, skip)) return;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int e = kZero;
-  bool bad = false;
-  for (int c = 0; c < nu; ++c) {
-    const double2 v = V[(int64_t)c * ldv + i];
-    const int x = exponent_of(max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu,
-                                  (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
-    if (x == kNotFinite || ec[c] == kNotFinite) bad = true;
-    else if (x != kZero) e = max(e, x - scale_exp(ec[c]));
-  }
-  er[i] = bad ? kNotFinite : e;
-}
-
-// Digit planes of the rows of V D^-1 with the columns as K: a[kb][tile of 128 rows][digit]
-// [re, im]. One thread per row and 8 columns.
-__global__ void __launch_bounds__(128)
+// Exponents of the rows of V D^-1, D the columns' scales, and their digit planes with the
+// columns as K: a[kb][tile of 128 rows][digit][re, im]. 32 rows a block, eight threads a row; the
+// second pass over the block's rows comes from the caches.
+__global__ void __launch_bounds__(256)
 split_rows_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu, int kbu,
-                  int64_t mtn, const int* __restrict__ ec, const int* __restrict__ er,
+                  int64_t mtn, const unsigned* __restrict__ hc, int* __restrict__ er,
                   unsigned char* __restrict__ a, const int* gate, const int* skip) {
   if (skipped(gate, skip)) return;
-  const int64_t i = blockIdx.x * (int64_t)kTileM + threadIdx.x;
-  const int gr = blockIdx.y, kb = gr / 2, kh = gr % 2;
-  const int e = i < n ? scale_exp(er[i]) : 0;
-  long long re[8], im[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int c = gr * 8 + j;
-    double2 v = make_double2(0.0, 0.0);
-    int ej = 0;
-    if (i < n && c < nu) {
-      v = V[(int64_t)c * ldv + i];
-      ej = e + scale_exp(ec[c]);
-    }
-    re[j] = fixed55(v.x, ej);
-    im[j] = fixed55(v.y, ej);
+  __shared__ int ec[kMaxNu], se[8][32], sbad;
+  const int lane = threadIdx.x % 32, q = threadIdx.x / 32;
+  const int64_t i = blockIdx.x * (int64_t)32 + lane;
+  if (threadIdx.x == 0) sbad = 0;
+  __syncthreads();
+  for (int c = threadIdx.x; c < nu; c += 256) {
+    const int e = exponent_of(hc[c]);
+    if (e == kNotFinite) sbad = 1;
+    ec[c] = scale_exp(e);
   }
-  const int m = threadIdx.x;
-  unsigned char* ap = a + ((size_t)kb * mtn + blockIdx.x) * kABytes + (m / 8) * 256 + kh * 128 + (m % 8) * 16;
-  uint4 d[kDigits];
-  digits8(re, d, false);
+  __syncthreads();
+  int e = kZero;
+  if (i < n)
+#pragma unroll 4
+    for (int c = q; c < nu; c += 8) {
+      const double2 v = V[(int64_t)c * ldv + i];
+      const int x = exponent_of(max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu,
+                                    (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
+      // (a value that is not finite makes its column's scale so: sbad)
+      if (x != kNotFinite && x != kZero) e = max(e, x - ec[c]);
+    }
+  se[q][lane] = e;
+  __syncthreads();
 #pragma unroll
-  for (int s = 0; s < kDigits; ++s) *reinterpret_cast<uint4*>(ap + (2 * s) * 4096) = d[s];
-  digits8(im, d, false);
+  for (int k = 0; k < 8; ++k) e = max(e, se[k][lane]);
+  if (q == 0 && i < n) er[i] = sbad ? kNotFinite : e;
+  e = scale_exp(e);
+  const int m = (int)(i % kTileM);
+  for (int gr = q; gr < 2 * kbu; gr += 8) {
+    const int kb = gr / 2, kh = gr % 2;
+    long long re[8], im[8];
 #pragma unroll
-  for (int s = 0; s < kDigits; ++s) *reinterpret_cast<uint4*>(ap + (2 * s + 1) * 4096) = d[s];
+    for (int j = 0; j < 8; ++j) {
+      const int c = gr * 8 + j;
+      const bool in = i < n && c < nu;
+      const double2 v = in ? V[(int64_t)c * ldv + i] : make_double2(0.0, 0.0);
+      const int ej = in ? e + ec[c] : 0;
+      re[j] = fixed55(v.x, ej);
+      im[j] = fixed55(v.y, ej);
+    }
+    unsigned char* ap = a + ((size_t)kb * mtn + i / kTileM) * kABytes + (m / 8) * 256 + kh * 128 + (m % 8) * 16;
+    uint4 d[kDigits];
+    digits8(re, d, false);
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s) *reinterpret_cast<uint4*>(ap + (2 * s) * 4096) = d[s];
+    digits8(im, d, false);
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s) *reinterpret_cast<uint4*>(ap + (2 * s + 1) * 4096) = d[s];
+  }
 }
 
 // Digit planes of the columns of D Z (Z upper triangular) with the rows as K:
@@ -235,7 +235,7 @@ split_rows_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu,
 // exponent.
 __global__ void __launch_bounds__(64)
 split_factor_kernel(const double2* __restrict__ Z, int nu, int kbu, int ntu,
-                    const int* __restrict__ ec, int* __restrict__ ez, unsigned char* __restrict__ b,
+                    const unsigned* __restrict__ hc, int* __restrict__ ez, unsigned char* __restrict__ b,
                     const int* gate, const int* skip) {
   if (skipped(gate, skip)) return;
   __shared__ int se[2], sbad;
@@ -249,7 +249,7 @@ split_factor_kernel(const double2* __restrict__ Z, int nu, int kbu, int ntu,
       const int x = exponent_of(max((unsigned)__double2hiint(z.x) & 0x7FFFFFFFu,
                                     (unsigned)__double2hiint(z.y) & 0x7FFFFFFFu));
       if (x == kNotFinite) sbad = 1;
-      else if (x != kZero) e = max(e, x + scale_exp(ec[k]));
+      else if (x != kZero) e = max(e, x + col_exp(hc, k));
     }
   for (int off = 16; off > 0; off >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
   if (tid % 32 == 0) se[tid / 32] = e;
@@ -268,7 +268,7 @@ split_factor_kernel(const double2* __restrict__ Z, int nu, int kbu, int ntu,
       int ej = 0;
       if (c < nu && k <= c && !sbad) {
         z = Z[(int64_t)c * nu + k];
-        ej = e - scale_exp(ec[k]);
+        ej = e - col_exp(hc, k);
       }
       re[j] = fixed55(z.x, ej);
       im[j] = fixed55(z.y, ej);
@@ -296,7 +296,7 @@ struct GemmArgs {
   int nu;
   int64_t n, ldv;
   int kb_total, parts; // Gram: K-blocks and row ranges
-  const int *ea, *eb;  // exponents of the output's rows and columns
+  const int *ea, *eb;  // exponents of the output's rows and columns (Gram: largest high words)
   double2* out;        // Gram partial sums, or V
   int* status;
   const int *gate, *skip;
@@ -511,12 +511,13 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
       // value = (hi 2^32 + lo) 2^(ea + eb - 70)
       const int64_t row = t.ta * kTileM + quarter * 32 + lane;
       const int64_t rows = kGram ? p.nu : p.n;
-      const int er = row < rows ? p.ea[row] : 0;
+      auto exp_at = [](const int* e, int64_t k) { return kGram ? exponent_of((unsigned)e[k]) : e[k]; };
+      const int er = row < rows ? exp_at(p.ea, row) : 0;
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
         const int col = t.tb * kTileN + k;
         if (row >= rows || col >= p.nu) continue;
-        const int ec = p.eb[col];
+        const int ec = exp_at(p.eb, col);
         const int e = scale_exp(er) + scale_exp(ec) - 70;
         double v = fma((double)hi[k], 4294967296.0, (double)lo[k]);
         v = e > -1022 && e < 1023 ? v * __longlong_as_double((long long)(e + 1023) << 52) : ldexp(v, e);
@@ -596,24 +597,21 @@ void split64_plan(bem_ctx* ctx, const double* V, int64_t ldv, int64_t n, int nu,
   unsigned char* base = static_cast<unsigned char*>(ctx->d_split);
   sp.a = base;
   sp.b = base + a_bytes;
-  sp.emax = reinterpret_cast<int*>(base + a_bytes + b_bytes);
-  sp.ez = sp.emax + nu;
+  sp.hcol = reinterpret_cast<unsigned*>(base + a_bytes + b_bytes);
+  sp.ez = reinterpret_cast<int*>(sp.hcol + nu);
   sp.erow = sp.ez + nu;
   sp.use = set_gemm_smem(ctx) == BEM_OK;
 }
 
 namespace {
 
-bem_status column_exponents(bem_ctx* ctx, const Split64& sp, const double2* V, const int* gate,
-                            const int* skip, cudaStream_t s) {
-  const bem_status st = cuda_check(ctx, cudaMemsetAsync(sp.emax, 0, sp.nu * sizeof(int), s), "split exponents");
+bem_status column_maxima(bem_ctx* ctx, const Split64& sp, const double2* V, const int* gate,
+                         const int* skip, cudaStream_t s) {
+  const bem_status st = cuda_check(ctx, cudaMemsetAsync(sp.hcol, 0, sp.nu * sizeof(int), s), "split scales");
   if (st != BEM_OK) return st;
   const unsigned ys = (unsigned)std::max<int64_t>(1, std::min<int64_t>((sp.n + 2047) / 2048, 64));
-  split_colmax_kernel<<<dim3((unsigned)sp.nu, ys), 256, 0, s>>>(V, sp.ldv, sp.n,
-                                                               reinterpret_cast<unsigned*>(sp.emax), gate, skip);
-  split_exponent_kernel<<<(unsigned)((sp.nu + 127) / 128), 128, 0, s>>>(
-      reinterpret_cast<unsigned*>(sp.emax), sp.nu, gate, skip);
-  ctx->launches += 2;
+  split_colmax_kernel<<<dim3((unsigned)sp.nu, ys), 256, 0, s>>>(V, sp.ldv, sp.n, sp.hcol, gate, skip);
+  ctx->launches++;
   return BEM_OK;
 }
 
@@ -621,29 +619,29 @@ bem_status column_exponents(bem_ctx* ctx, const Split64& sp, const double2* V, c
 
 bem_status split64_gram(bem_ctx* ctx, const Split64& sp, const double2* V, double2* part,
                         const int* gate, cudaStream_t s) {
-  bem_status st = column_exponents(ctx, sp, V, gate, nullptr, s);
+  bem_status st = column_maxima(ctx, sp, V, gate, nullptr, s);
   if (st != BEM_OK) return st;
   const int64_t threads = 2 * (int64_t)sp.kbn * sp.mtu * kTileM;
   split_columns_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(
-      V, sp.ldv, sp.n, sp.nu, sp.kbn, sp.mtu, sp.ntu, sp.emax, sp.a, sp.b, gate);
+      V, sp.ldv, sp.n, sp.nu, sp.kbn, sp.mtu, sp.ntu, sp.hcol, sp.a, sp.b, gate);
   int tiles = 0;
   for (int a = 0; a < sp.mtu; ++a) tiles += sp.ntu - a * (kTileM / kTileN);
-  GemmArgs g{sp.a, sp.b, sp.mtu, sp.ntu, sp.nu, sp.n, sp.ldv, sp.kbn, sp.parts, sp.emax, sp.emax,
-             part, ctx->d_status, gate, nullptr};
+  GemmArgs g{sp.a, sp.b, sp.mtu, sp.ntu, sp.nu, sp.n, sp.ldv, sp.kbn, sp.parts,
+             reinterpret_cast<const int*>(sp.hcol), reinterpret_cast<const int*>(sp.hcol), part, ctx->d_status, gate, nullptr};
   split_gemm_kernel<true><<<dim3((unsigned)tiles, (unsigned)sp.parts), kThreadsG, GemmSmem::total, s>>>(g);
   ctx->launches += 2;
   return cuda_check(ctx, cudaGetLastError(), "split Gram matrix");
 }
 
-bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, double2* V, const double2* Z,
-                            const int* gate, const int* skip, cudaStream_t s) {
-  bem_status st = column_exponents(ctx, sp, V, gate, skip, s);
-  if (st != BEM_OK) return st;
-  split_rowmax_kernel<<<(unsigned)((sp.n + 127) / 128), 128, 0, s>>>(V, sp.ldv, sp.n, sp.nu, sp.emax,
-                                                                   sp.erow, gate, skip);
-  split_rows_kernel<<<dim3((unsigned)sp.mtn, 2u * sp.kbu), kTileM, 0, s>>>(
-      V, sp.ldv, sp.n, sp.nu, sp.kbu, sp.mtn, sp.emax, sp.erow, sp.a, gate, skip);
-  split_factor_kernel<<<(unsigned)(sp.ntu * kTileN), 64, 0, s>>>(Z, sp.nu, sp.kbu, sp.ntu, sp.emax,
+bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, bool same, double2* V,
+                            const double2* Z, const int* gate, const int* skip, cudaStream_t s) {
+  if (!same) {
+    const bem_status st = column_maxima(ctx, sp, V, gate, skip, s);
+    if (st != BEM_OK) return st;
+  }
+  split_rows_kernel<<<(unsigned)(sp.mtn * (kTileM / 32)), 256, 0, s>>>(
+      V, sp.ldv, sp.n, sp.nu, sp.kbu, sp.mtn, sp.hcol, sp.erow, sp.a, gate, skip);
+  split_factor_kernel<<<(unsigned)(sp.ntu * kTileN), 64, 0, s>>>(Z, sp.nu, sp.kbu, sp.ntu, sp.hcol,
                                                                 sp.ez, sp.b, gate, skip);
   GemmArgs g{sp.a, sp.b, sp.mtn, sp.ntu, sp.nu, sp.n, sp.ldv, sp.kbu, 1, sp.erow, sp.ez, V,
              ctx->d_status, gate, skip};
@@ -651,7 +649,7 @@ bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, double2* V, const d
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const unsigned grid = (unsigned)std::min<int64_t>(std::max(1, sms), sp.mtn * sp.ntu);
   split_gemm_kernel<false><<<grid, kThreadsG, GemmSmem::total, s>>>(g);
-  ctx->launches += 4;
+  ctx->launches += 3;
   return cuda_check(ctx, cudaGetLastError(), "split product");
 }
 

@@ -15,7 +15,8 @@ struct Split64 {
   int64_t mtn = 0;           // 128-row tiles
   int parts = 0;             // row ranges of the Gram matrix (its partial sums)
   unsigned char *a = nullptr, *b = nullptr;   // digit planes of the two operands
-  int *emax = nullptr, *erow = nullptr, *ez = nullptr;   // exponents: columns, rows, factor
+  unsigned* hcol = nullptr;                   // largest high words of the columns
+  int *erow = nullptr, *ez = nullptr;         // exponents of the rows and of the factor
 };
 
 // Fills sp for V; use is false where the FP64 kernels are the better choice (small products) or
@@ -28,9 +29,9 @@ int split64_parts(const bem_ctx* ctx, int64_t n, int nu);
 // (sp.parts ranges). Skipped on the device when gate is given and *gate == 0.
 bem_status split64_gram(bem_ctx* ctx, const Split64& sp, const double2* V, double2* part,
                         const int* gate, cudaStream_t s);
-// V <- V Z, Z nu x nu upper triangular. Skipped when (gate and *gate == 0) or
-// (skip and *skip != 0).
-bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, double2* V, const double2* Z,
-                            const int* gate, const int* skip, cudaStream_t s);
+// V <- V Z, Z nu x nu upper triangular. same: V is unchanged since split64_gram (its scales are
+// there). Skipped when (gate and *gate == 0) or (skip and *skip != 0).
+bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, bool same, double2* V,
+                            const double2* Z, const int* gate, const int* skip, cudaStream_t s);
 
 }  // namespace bem

@@ -1,5 +1,5 @@
 """CholeskyQR2 on its two sets of kernels: the split products on the tensor core
-(csrc/split64.cu, from n nu^2 = 2^25) and the FP64 pipe below, with the FP32 first factor in one
+(csrc/split64.cu, from n nu^2 = 2^23) and the FP64 pipe below, with the FP32 first factor in one
 or two diagonal blocks (nu > 128). Sizes around the 16-, 32- and 128-wide tiles and the 64- and
 128-row flushes; columns of one sign (the digits' sums at their largest), columns scaled by
 1e30 .. 1e35 (a spread of 1e7 or squares beyond FP32's range squared are refused), strided

@@ -17,7 +17,8 @@
 // form; the moments' round trip through memory (32 bytes a moment) is ~1 % of that. Measured:
 // the products of the 768-panel cube (N = 32, nu = 64) 28.1 -> 4.6 ms, of the residuals of 8
 // vectors on 5120 panels 258 -> 50 ms, with the same or a smaller error against 64-bit
-// references.
+// references. The larger products run on the tensor core (split64.cu): 4.6 -> 0.41 ms and
+// 15.8 -> 9 ms.
 #include <math.h>
 
 #include <algorithm>
@@ -32,6 +33,11 @@ constexpr int kCoefPoints = 64;    // Chebyshev points of the coefficients' quad
 constexpr int kRowsE = 128;        // rows per block of the evaluation (a thread each)
 constexpr int kColsE = 8;          // columns per block of the evaluation
 constexpr size_t kMomentBytes = (size_t)1 << 30;   // moments held at a time
+// n^2 S (padded columns - 4) from which the split products pay (split64.cu; conversions of 24 ps a
+// moment and three more launches against 5.6 ps a moment and column). Split against FP64, in us:
+// 300 panels, 8 residuals 505 / 457, 588 panels, 2 residuals 978 / 955 below it; projections of
+// 300 panels, 10 columns 751 / 958, 588 x 60 1687 / 3695, 1728 panels, 2 residuals 5247 / 5518 above.
+constexpr int64_t kSplitWork = (int64_t)1 << 25;
 constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
 
 // a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
@@ -374,13 +380,19 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const int64_t tiles = (n + kTM - 1) / kTM * ((ncols + tn - 1) / tn) * p.S;
+  p.split = n * n * p.S * (int64_t)(padded - 4.0) >= kSplitWork;
+  if (p.split) {
+    p.kc = (int)std::min<int64_t>(n, std::max<int64_t>(64, (int64_t)(kMomentBytes / ((size_t)p.S * n * 16)) / 16 * 16));
+    p.batch = split64_batch_plan(n, p.kc, p.S, ncols);
+  }
   // enough blocks for eight small blocks on each SM, at least 64 columns each
-  p.splits = (int)std::max<int64_t>(1, std::min<int64_t>(8 * (int64_t)std::max(1, sms) / tiles, p.kc / 64));
+  p.splits = p.split ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(8 * (int64_t)std::max(1, sms) / tiles, p.kc / 64));
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   p.coef_off = 0;
   p.mom_off = up((size_t)p.S * nk * 16);
   p.y_off = p.mom_off + up((size_t)p.S * p.kc * n * 16);
-  p.bytes = p.y_off + up((size_t)p.splits * p.S * n * ncols * 16);
+  p.batch_off = p.y_off + up((size_t)p.splits * p.S * n * ncols * 16);
+  p.bytes = p.batch_off + p.batch.bytes;
   p.use = p.bytes <= kMaxWork;
   return p;
 }
@@ -406,17 +418,29 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
                                 : (p.first == 0 ? moment_kernel<true, false>(p.M)
                                                 : moment_kernel<false, true>(p.M));
   ctx->launches++;
+  const double2* Xd = reinterpret_cast<const double2*>(X);
+  if (p.split) {
+    const bem_status st = split64_batch_scales(ctx, p.batch, work + p.batch_off, Xd, ldx, s);
+    if (st != BEM_OK) return st;
+  }
   for (int64_t l0 = 0; l0 < n; l0 += p.kc) {
     const int kc = (int)std::min<int64_t>(p.kc, n - l0);
     const dim3 ge((unsigned)((n + kRowsE - 1) / kRowsE), (unsigned)((kc + kColsE - 1) / kColsE));
     mk<<<ge, kRowsE, 0, s>>>(ctx->geo, p.c, 2.0 / p.R, p.M, l0, kc, G);
+    ctx->launches++;
+    if (p.split) {
+      const bem_status st = split64_batch(ctx, p.batch, work + p.batch_off, G, (int64_t)kc * n, kc,
+                                          Xd + l0, ldx, l0 > 0, Yp, s);
+      if (st != BEM_OK) return st;
+      continue;
+    }
     const int tn = ncols <= 8 ? 8 : 32;
     const dim3 gp((unsigned)((n + kTM - 1) / kTM), (unsigned)((ncols + tn - 1) / tn),
                   (unsigned)(p.S * p.splits));
     auto* pk = tn == 8 ? expand_product_kernel<8> : expand_product_kernel<32>;
-    pk<<<gp, kThreadsM, 0, s>>>(G, n, kc, p.S, p.splits, reinterpret_cast<const double2*>(X), ldx,
+    pk<<<gp, kThreadsM, 0, s>>>(G, n, kc, p.S, p.splits, Xd, ldx,
                                 ncols, l0, l0 > 0, Yp);
-    ctx->launches += 2;
+    ctx->launches++;
   }
   if (p.splits > 1) {
     const int64_t count = (int64_t)p.S * n * ncols;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "internal.h"
+#include "split64.h"
 
 namespace bem {
 
@@ -16,7 +17,9 @@ struct ExpandPlan {
   int splits = 1;          // shares of those columns in the products
   double R = 0.0;          // largest distance
   double2 c{};             // centre
-  size_t coef_off = 0, mom_off = 0, y_off = 0, bytes = 0;
+  bool split = false;      // products on the tensor core (split64.cu)
+  SplitBatch batch;
+  size_t coef_off = 0, mom_off = 0, y_off = 0, batch_off = 0, bytes = 0;
 };
 
 // Plan for nk wavenumbers within dmax of the centre and ncols columns: every wavenumber times

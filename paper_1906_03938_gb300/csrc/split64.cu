@@ -171,24 +171,29 @@ split_columns_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int 
   put_b(1, 1);
 }
 
-// Exponents of the rows of V D^-1, D the columns' scales, and their digit planes with the
-// columns as K: a[kb][tile of 128 rows][digit][re, im]. 32 rows a block, eight threads a row; the
-// second pass over the block's rows comes from the caches.
+// Exponents of the rows of V D^-1, D the columns' scales (hc null: 1), and their digit planes with
+// the columns as K: a[kb][matrix][tile of 128 rows][digit][re, im], blockIdx.y of gridDim.y
+// matrices vstep apart. 32 rows a block, eight threads a row; the second pass over the block's
+// rows comes from the caches.
 __global__ void __launch_bounds__(256)
-split_rows_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu, int kbu,
-                  int64_t mtn, const unsigned* __restrict__ hc, int* __restrict__ er,
+split_rows_kernel(const double2* __restrict__ V, int64_t ldv, int64_t vstep, int64_t n, int nu,
+                  int kbu, int64_t mtn, const unsigned* __restrict__ hc, int* __restrict__ er,
                   unsigned char* __restrict__ a, const int* gate, const int* skip) {
   if (skipped(gate, skip)) return;
   __shared__ int ec[kMaxNu], se[8][32], sbad;
+  V += blockIdx.y * vstep;
+  er += blockIdx.y * n;
+  a += blockIdx.y * (size_t)mtn * kABytes;
   const int lane = threadIdx.x % 32, q = threadIdx.x / 32;
   const int64_t i = blockIdx.x * (int64_t)32 + lane;
   if (threadIdx.x == 0) sbad = 0;
   __syncthreads();
-  for (int c = threadIdx.x; c < nu; c += 256) {
-    const int e = exponent_of(hc[c]);
-    if (e == kNotFinite) sbad = 1;
-    ec[c] = scale_exp(e);
-  }
+  if (hc)
+    for (int c = threadIdx.x; c < nu; c += 256) {
+      const int e = exponent_of(hc[c]);
+      if (e == kNotFinite) sbad = 1;
+      ec[c] = scale_exp(e);
+    }
   __syncthreads();
   int e = kZero;
   if (i < n)
@@ -197,14 +202,15 @@ split_rows_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu,
       const double2 v = V[(int64_t)c * ldv + i];
       const int x = exponent_of(max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu,
                                     (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
-      // (a value that is not finite makes its column's scale so: sbad)
-      if (x != kNotFinite && x != kZero) e = max(e, x - ec[c]);
+      if (x == kNotFinite) e = INT_MAX;
+      else if (x != kZero) e = max(e, x - (hc ? ec[c] : 0));
     }
   se[q][lane] = e;
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < 8; ++k) e = max(e, se[k][lane]);
-  if (q == 0 && i < n) er[i] = sbad ? kNotFinite : e;
+  if (sbad || e == INT_MAX) e = kNotFinite;
+  if (q == 0 && i < n) er[i] = e;
   e = scale_exp(e);
   const int m = (int)(i % kTileM);
   for (int gr = q; gr < 2 * kbu; gr += 8) {
@@ -215,11 +221,11 @@ split_rows_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu,
       const int c = gr * 8 + j;
       const bool in = i < n && c < nu;
       const double2 v = in ? V[(int64_t)c * ldv + i] : make_double2(0.0, 0.0);
-      const int ej = in ? e + ec[c] : 0;
+      const int ej = in ? e + (hc ? ec[c] : 0) : 0;
       re[j] = fixed55(v.x, ej);
       im[j] = fixed55(v.y, ej);
     }
-    unsigned char* ap = a + ((size_t)kb * mtn + i / kTileM) * kABytes + (m / 8) * 256 + kh * 128 + (m % 8) * 16;
+    unsigned char* ap = a + ((size_t)kb * gridDim.y * mtn + i / kTileM) * kABytes + (m / 8) * 256 + kh * 128 + (m % 8) * 16;
     uint4 d[kDigits];
     digits8(re, d, false);
 #pragma unroll
@@ -290,14 +296,52 @@ split_factor_kernel(const double2* __restrict__ Z, int nu, int kbu, int ntu,
   }
 }
 
+// Digit planes of the columns of X with the rows [0, n) as K, for a plain product:
+// b[kb][tile of 32 columns]{[digit][re | im], [digit][-im | re]}. A thread per column and 8 rows.
+__global__ void __launch_bounds__(128)
+split_rhs_kernel(const double2* __restrict__ X, int64_t ldx, int n, int nu, int kbn, int ntu,
+                 const unsigned* __restrict__ hc, unsigned char* __restrict__ b) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t gr = t % (2 * kbn);
+  const int c = (int)(t / (2 * kbn));
+  if (c >= ntu * kTileN) return;
+  long long re[8], im[8];
+  const int e = c < nu ? col_exp(hc, c) : 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int64_t i = gr * 8 + j;
+    const double2 v = (c < nu && i < n) ? X[(int64_t)c * ldx + i] : make_double2(0.0, 0.0);
+    re[j] = fixed55(v.x, e);
+    im[j] = fixed55(v.y, e);
+  }
+  const int r = c % kTileN;
+  unsigned char* bp = b + ((size_t)(gr / 2) * ntu + c / kTileN) * kBBytes + (r / 8) * 256 + (gr % 2) * 128 + (r % 8) * 16;
+  uint4 d[kDigits];
+  auto put_b = [&](int w, int h) {
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s)
+      *reinterpret_cast<uint4*>(bp + w * kBHalf + s * 2048 + h * 1024) = d[s];
+  };
+  digits8(re, d, false);
+  put_b(0, 0);
+  put_b(1, 1);
+  digits8(im, d, false);
+  put_b(0, 1);
+  digits8(im, d, true);
+  put_b(1, 0);
+}
+
 struct GemmArgs {
   const unsigned char *a, *b;
   int64_t ta, tb;      // tiles per K-block of a and b
+  int64_t mtn;         // batch: row tiles of one matrix (ta / mtn matrices)
+  bool add;            // batch: add to out
   int nu;
   int64_t n, ldv;
   int kb_total, parts; // Gram: K-blocks and row ranges
-  const int *ea, *eb;  // exponents of the output's rows and columns (Gram: largest high words)
-  double2* out;        // Gram partial sums, or V
+  const int *ea, *eb;  // exponents of the output's rows and columns (Gram, and the columns of a
+                       // batch: largest high words)
+  double2* out;        // Gram partial sums, V, or the products of a batch
   int* status;
   const int *gate, *skip;
 };
@@ -326,13 +370,15 @@ struct Tile {
 };
 
 // Tile i of this block (false: no more).
+enum { kGramSum = 0, kTriangle = 1, kBatch = 2 };
+
 // Gram: one tile per block, the upper ones only, counted along b within a; blockIdx.y the row
-// range. Product: whole rows of tiles per block (the row tile's planes stay in L2), widest
+// range. Products: whole rows of tiles per block (the row tile's planes stay in L2), widest
 // first; the rows left over after the last full round are dealt tile by tile.
-template <bool kGram>
+template <int kMode>
 __device__ __forceinline__ bool tile_of(const GemmArgs& p, int i, Tile& t) {
   const int nt = (int)p.tb;
-  if (kGram) {
+  if (kMode == kGramSum) {
     if (i > 0) return false;
     int rest = blockIdx.x, at = 0;
     while (rest >= nt - at * (kTileM / kTileN)) {
@@ -356,14 +402,15 @@ __device__ __forceinline__ bool tile_of(const GemmArgs& p, int i, Tile& t) {
     t.tb = nt - 1 - (int)(w / left);
   }
   t.kb0 = 0;
-  t.kb1 = min(p.kb_total, (t.tb + 1) * (kTileN / 16));
+  t.kb1 = kMode == kTriangle ? min(p.kb_total, (t.tb + 1) * (kTileN / 16)) : p.kb_total;
   return true;
 }
 
-// kGram: out[part][b nu + a] = sum of the rows of part blockIdx.y, with [re | im] and
-// [im | -re] for conj(V)^T V. else: V[i][c] = sum_k V[i][k] Z[k][c], with [re | im] and
-// [-im | re]; the K-blocks of the upper triangle only.
-template <bool kGram>
+// kGramSum: out[part][b nu + a] = sum of the rows of part blockIdx.y, with [re | im] and
+// [im | -re] for conj(V)^T V. kTriangle: V[i][c] = sum_k V[i][k] Z[k][c], with [re | im] and
+// [-im | re]; the K-blocks of the upper triangle only. kBatch: out_s (+)= A_s X likewise, all
+// K-blocks, the row tiles of the matrices one after the other.
+template <int kMode>
 __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
   if (skipped(p.gate, p.skip)) return;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -404,7 +451,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
     if (lane == 0) {
       int issued = 0;   // K-blocks over all tiles
       bool ok = true;
-      for (int i = 0; ok && tile_of<kGram>(p, i, t); ++i)
+      for (int i = 0; ok && tile_of<kMode>(p, i, t); ++i)
         for (int kb = t.kb0; kb < t.kb1; ++kb, ++issued) {
           const int s = issued % kStagesG;
           ok = wait_flag(&empty[s], ((issued / kStagesG) & 1) ^ 1, abort_flag, p.status);
@@ -424,7 +471,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
       int it = 0;               // K-blocks over all tiles
       int done[2] = {0, 0};     // chunks of the two groups handed over
       bool ok = true;
-      for (int i = 0; ok && tile_of<kGram>(p, i, t); ++i)
+      for (int i = 0; ok && tile_of<kMode>(p, i, t); ++i)
         for (int kb = t.kb0; ok && kb < t.kb1; ++kb, ++it) {
           const int s = it % kStagesG, at = kb - t.kb0;
           const bool end = kb + 1 == t.kb1;
@@ -476,7 +523,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
     const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + side * 32;
     int done[2] = {0, 0};
     bool ok = true;
-    for (int i = 0; ok && tile_of<kGram>(p, i, t); ++i) {
+    for (int i = 0; ok && tile_of<kMode>(p, i, t); ++i) {
       const int nkb = t.kb1 - t.kb0;
       long long hi[32], lo[32];   // sums of d < 4 and d >= 4
 #pragma unroll
@@ -509,23 +556,24 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
       }
       if (!ok) break;
       // value = (hi 2^32 + lo) 2^(ea + eb - 70)
-      const int64_t row = t.ta * kTileM + quarter * 32 + lane;
-      const int64_t rows = kGram ? p.nu : p.n;
-      auto exp_at = [](const int* e, int64_t k) { return kGram ? exponent_of((unsigned)e[k]) : e[k]; };
-      const int er = row < rows ? exp_at(p.ea, row) : 0;
+      const int64_t slot = kMode == kBatch ? t.ta / p.mtn : 0;
+      const int64_t row = (t.ta - slot * p.mtn) * kTileM + quarter * 32 + lane;
+      const int64_t rows = kMode == kGramSum ? p.nu : p.n;
+      int er = row < rows ? p.ea[slot * p.n + row] : 0;
+      if (kMode == kGramSum) er = exponent_of((unsigned)er);
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
         const int col = t.tb * kTileN + k;
         if (row >= rows || col >= p.nu) continue;
-        const int ec = exp_at(p.eb, col);
+        const int ec = kMode == kTriangle ? p.eb[col] : exponent_of((unsigned)p.eb[col]);
         const int e = scale_exp(er) + scale_exp(ec) - 70;
         double v = fma((double)hi[k], 4294967296.0, (double)lo[k]);
         v = e > -1022 && e < 1023 ? v * __longlong_as_double((long long)(e + 1023) << 52) : ldexp(v, e);
         if (er == kNotFinite || ec == kNotFinite) v = NAN;
         double* o = reinterpret_cast<double*>(
-            kGram ? p.out + (int64_t)blockIdx.y * p.nu * p.nu + (int64_t)col * p.nu + row
-                  : p.out + (int64_t)col * p.ldv + row);
-        o[side] = v;
+            kMode == kGramSum ? p.out + (int64_t)blockIdx.y * p.nu * p.nu + (int64_t)col * p.nu + row
+                              : p.out + (slot * p.nu + col) * p.ldv + row);
+        o[side] = kMode == kBatch && p.add ? o[side] + v : v;
       }
     }
   }
@@ -540,7 +588,8 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
 }
 
 bem_status set_gemm_smem(bem_ctx* ctx) {
-  for (const void* f : {(const void*)split_gemm_kernel<true>, (const void*)split_gemm_kernel<false>}) {
+  for (const void* f : {(const void*)split_gemm_kernel<kGramSum>, (const void*)split_gemm_kernel<kTriangle>,
+                        (const void*)split_gemm_kernel<kBatch>}) {
     const bem_status st = cuda_check(
         ctx, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmSmem::total),
         "split product attribute");
@@ -605,12 +654,12 @@ void split64_plan(bem_ctx* ctx, const double* V, int64_t ldv, int64_t n, int nu,
 
 namespace {
 
-bem_status column_maxima(bem_ctx* ctx, const Split64& sp, const double2* V, const int* gate,
-                         const int* skip, cudaStream_t s) {
-  const bem_status st = cuda_check(ctx, cudaMemsetAsync(sp.hcol, 0, sp.nu * sizeof(int), s), "split scales");
+bem_status column_maxima(bem_ctx* ctx, unsigned* hcol, const double2* V, int64_t ldv, int64_t n,
+                         int nu, const int* gate, const int* skip, cudaStream_t s) {
+  const bem_status st = cuda_check(ctx, cudaMemsetAsync(hcol, 0, nu * sizeof(int), s), "split scales");
   if (st != BEM_OK) return st;
-  const unsigned ys = (unsigned)std::max<int64_t>(1, std::min<int64_t>((sp.n + 2047) / 2048, 64));
-  split_colmax_kernel<<<dim3((unsigned)sp.nu, ys), 256, 0, s>>>(V, sp.ldv, sp.n, sp.hcol, gate, skip);
+  const unsigned ys = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, 64));
+  split_colmax_kernel<<<dim3((unsigned)nu, ys), 256, 0, s>>>(V, ldv, n, hcol, gate, skip);
   ctx->launches++;
   return BEM_OK;
 }
@@ -619,16 +668,16 @@ bem_status column_maxima(bem_ctx* ctx, const Split64& sp, const double2* V, cons
 
 bem_status split64_gram(bem_ctx* ctx, const Split64& sp, const double2* V, double2* part,
                         const int* gate, cudaStream_t s) {
-  bem_status st = column_maxima(ctx, sp, V, gate, nullptr, s);
+  bem_status st = column_maxima(ctx, sp.hcol, V, sp.ldv, sp.n, sp.nu, gate, nullptr, s);
   if (st != BEM_OK) return st;
   const int64_t threads = 2 * (int64_t)sp.kbn * sp.mtu * kTileM;
   split_columns_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(
       V, sp.ldv, sp.n, sp.nu, sp.kbn, sp.mtu, sp.ntu, sp.hcol, sp.a, sp.b, gate);
   int tiles = 0;
   for (int a = 0; a < sp.mtu; ++a) tiles += sp.ntu - a * (kTileM / kTileN);
-  GemmArgs g{sp.a, sp.b, sp.mtu, sp.ntu, sp.nu, sp.n, sp.ldv, sp.kbn, sp.parts,
+  GemmArgs g{sp.a, sp.b, sp.mtu, sp.ntu, 0, false, sp.nu, sp.n, sp.ldv, sp.kbn, sp.parts,
              reinterpret_cast<const int*>(sp.hcol), reinterpret_cast<const int*>(sp.hcol), part, ctx->d_status, gate, nullptr};
-  split_gemm_kernel<true><<<dim3((unsigned)tiles, (unsigned)sp.parts), kThreadsG, GemmSmem::total, s>>>(g);
+  split_gemm_kernel<kGramSum><<<dim3((unsigned)tiles, (unsigned)sp.parts), kThreadsG, GemmSmem::total, s>>>(g);
   ctx->launches += 2;
   return cuda_check(ctx, cudaGetLastError(), "split Gram matrix");
 }
@@ -636,21 +685,66 @@ bem_status split64_gram(bem_ctx* ctx, const Split64& sp, const double2* V, doubl
 bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, bool same, double2* V,
                             const double2* Z, const int* gate, const int* skip, cudaStream_t s) {
   if (!same) {
-    const bem_status st = column_maxima(ctx, sp, V, gate, skip, s);
+    const bem_status st = column_maxima(ctx, sp.hcol, V, sp.ldv, sp.n, sp.nu, gate, skip, s);
     if (st != BEM_OK) return st;
   }
   split_rows_kernel<<<(unsigned)(sp.mtn * (kTileM / 32)), 256, 0, s>>>(
-      V, sp.ldv, sp.n, sp.nu, sp.kbu, sp.mtn, sp.hcol, sp.erow, sp.a, gate, skip);
+      V, sp.ldv, 0, sp.n, sp.nu, sp.kbu, sp.mtn, sp.hcol, sp.erow, sp.a, gate, skip);
   split_factor_kernel<<<(unsigned)(sp.ntu * kTileN), 64, 0, s>>>(Z, sp.nu, sp.kbu, sp.ntu, sp.hcol,
                                                                 sp.ez, sp.b, gate, skip);
-  GemmArgs g{sp.a, sp.b, sp.mtn, sp.ntu, sp.nu, sp.n, sp.ldv, sp.kbu, 1, sp.erow, sp.ez, V,
+  GemmArgs g{sp.a, sp.b, sp.mtn, sp.ntu, sp.mtn, false, sp.nu, sp.n, sp.ldv, sp.kbu, 1, sp.erow, sp.ez, V,
              ctx->d_status, gate, skip};
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const unsigned grid = (unsigned)std::min<int64_t>(std::max(1, sms), sp.mtn * sp.ntu);
-  split_gemm_kernel<false><<<grid, kThreadsG, GemmSmem::total, s>>>(g);
+  split_gemm_kernel<kTriangle><<<grid, kThreadsG, GemmSmem::total, s>>>(g);
   ctx->launches += 3;
   return cuda_check(ctx, cudaGetLastError(), "split product");
+}
+
+SplitBatch split64_batch_plan(int64_t n, int kc, int S, int ncols) {
+  SplitBatch b;
+  b.n = n;
+  b.S = S;
+  b.nu = ncols;
+  b.kc = kc;
+  b.mtn = (n + kTileM - 1) / kTileM;
+  b.ntu = (ncols + kTileN - 1) / kTileN;
+  const size_t kb = (size_t)(kc + 15) / 16;
+  auto up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
+  b.b_off = up(kb * S * (size_t)b.mtn * kABytes);
+  b.e_off = b.b_off + up(kb * b.ntu * kBBytes);
+  b.bytes = b.e_off + up(((size_t)ncols + (size_t)S * n) * sizeof(int));
+  return b;
+}
+
+bem_status split64_batch_scales(bem_ctx* ctx, const SplitBatch& b, char* work, const double2* X,
+                                int64_t ldx, cudaStream_t s) {
+  const bem_status st = set_gemm_smem(ctx);
+  if (st != BEM_OK) return st;
+  return column_maxima(ctx, reinterpret_cast<unsigned*>(work + b.e_off), X, ldx, b.n, b.nu, nullptr, nullptr, s);
+}
+
+bem_status split64_batch(bem_ctx* ctx, const SplitBatch& b, char* work, const double2* A,
+                         int64_t astep, int kc, const double2* X, int64_t ldx, bool add,
+                         double2* out, cudaStream_t s) {
+  unsigned char* ap = reinterpret_cast<unsigned char*>(work);
+  unsigned char* bp = ap + b.b_off;
+  unsigned* hcol = reinterpret_cast<unsigned*>(work + b.e_off);
+  int* er = reinterpret_cast<int*>(hcol + b.nu);
+  const int kb = (kc + 15) / 16;
+  split_rows_kernel<<<dim3((unsigned)(b.mtn * (kTileM / 32)), (unsigned)b.S), 256, 0, s>>>(
+      A, b.n, astep, b.n, kc, kb, b.mtn, nullptr, er, ap, nullptr, nullptr);
+  const int64_t threads = 2 * (int64_t)kb * b.ntu * kTileN;
+  split_rhs_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(X, ldx, kc, b.nu, kb, b.ntu, hcol, bp);
+  GemmArgs g{ap, bp, b.S * b.mtn, b.ntu, b.mtn, add, b.nu, b.n, b.n, kb, 1, er,
+             reinterpret_cast<const int*>(hcol), out, ctx->d_status, nullptr, nullptr};
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  const unsigned grid = (unsigned)std::min<int64_t>(std::max(1, sms), g.ta * g.tb);
+  split_gemm_kernel<kBatch><<<grid, kThreadsG, GemmSmem::total, s>>>(g);
+  ctx->launches += 3;
+  return cuda_check(ctx, cudaGetLastError(), "split products");
 }
 
 }  // namespace bem

@@ -34,4 +34,21 @@ bem_status split64_gram(bem_ctx* ctx, const Split64& sp, const double2* V, doubl
 bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, bool same, double2* V,
                             const double2* Z, const int* gate, const int* skip, cudaStream_t s);
 
+// Products A_s X, s < S, of n x kc matrices A_s (column-major, ld n) with the rows of X, in
+// `bytes` of workspace; X is taken kc rows at a time.
+struct SplitBatch {
+  int64_t n = 0, mtn = 0;   // rows and their 128-row tiles
+  int S = 0, nu = 0, ntu = 0, kc = 0;
+  size_t b_off = 0, e_off = 0, bytes = 0;
+};
+SplitBatch split64_batch_plan(int64_t n, int kc, int S, int ncols);
+// The scales of X's columns (all n rows), once before the products.
+bem_status split64_batch_scales(bem_ctx* ctx, const SplitBatch& b, char* work, const double2* X,
+                                int64_t ldx, cudaStream_t s);
+// out_s (n x nu, ld n, one after the other) (+)= A_s X for kc <= b.kc columns of the A_s (astep
+// elements apart) and rows of X.
+bem_status split64_batch(bem_ctx* ctx, const SplitBatch& b, char* work, const double2* A,
+                         int64_t astep, int kc, const double2* X, int64_t ldx, bool add,
+                         double2* out, cudaStream_t s);
+
 }  // namespace bem

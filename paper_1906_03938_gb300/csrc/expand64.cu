@@ -12,13 +12,13 @@
 // w_q s_q / r_q, s = (y - x).n / r^2, and the coefficients of (i k r - 1) e^{i (k - c) r}; the
 // k-derivative only changes the coefficients.
 //
-// Bound by the FP64 pipe (1/64 of the FP32 rate on this part): per entry 7 (60 + 3 M) FP64
-// operations of evaluation and 3 M nu of products against N (7 x 77 + 4 nu) for the direct
-// form; the moments' round trip through memory (32 bytes a moment) is ~1 % of that. Measured:
-// the products of the 768-panel cube (N = 32, nu = 64) 28.1 -> 4.6 ms, of the residuals of 8
-// vectors on 5120 panels 258 -> 50 ms, with the same or a smaller error against 64-bit
-// references. The larger products run on the tensor core (split64.cu): 4.6 -> 0.41 ms and
-// 15.8 -> 9 ms.
+// Bound by arithmetic: 7 points of 15 FP64 operations and ~(110 + 26 M) integer ones per entry
+// (below), and M nu products, in FP64 (1/64 of the FP32 rate on this part) or, the larger ones,
+// on the tensor core (split64.cu), against N (7 x 77 + 4 nu) FP64 operations of the direct form;
+// the moments' round trip through memory (32 bytes a moment, three times that with the digits) is
+// ~20 %. Measured: the products of the 768-panel cube (N = 32, nu = 64) 28.1 -> 0.95 ms, of the
+// residuals of 8 vectors on 5120 panels 258 -> 19 ms, with the same or a smaller error against
+// 64-bit references.
 #include <math.h>
 
 #include <algorithm>
@@ -82,20 +82,114 @@ expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, i
       make_double2(sc * (s.x * or_ - s.y * oi), sc * (s.x * oi + s.y * or_));
 }
 
+// ---- the moments ----
+//
+// In FP64 a point took ~98 operations on a pipe of 2 a clock and SM: distance, root, sine and
+// cosine, and 3 a term for the Chebyshev polynomials and the sums; 34 ms for 5120 panels and 14
+// terms. Only the distance and its root need a floating exponent. With r <= R and |T_m| <= 1
+// the rest is fixed-point arithmetic of 62 fractional bits, on the integer pipe: a product is
+// three 32 x 32 -> 64 multiply-adds, rounded to 2^-60 of its operands' bounds, finer than FP64's
+// 2^-53. So a point takes 15 FP64 operations and ~(110 + 26 M) integer instructions beside them.
+//   rho = r / R -> x = 2 rho - 1; the phase c r in turns, K rho mod 1, exact to 2^-60 max(1, K);
+//   its sine and cosine from a table of 1024 angles and a Taylor series of the rest (|t| <=
+//   pi / 1024: t - t^3 / 6 + t^5 / 120 and 1 - t^2 / 2 + t^4 / 24, the next terms below 2^-59);
+//   the seven weights w / r scaled together so that their sum fills 62 bits.
+// Measured: 5120 panels, 14 terms 34.3 -> 11.0 ms; 768 panels, 17 terms 730 -> 319 us; the residuals
+// and products keep their error against 64-bit references (7.6e-16, 9.5e-16).
+constexpr int kAngles = 1024;
+constexpr long long kOne = 1ll << 62;
+
+struct FixedPhase {
+  double inv_R;   // rho = r inv_R
+  long long K;    // turns per unit of rho, times 2^(62 - kb)
+  int kb;
+};
+
+struct Split {   // x = h 2^32 + l, both signed
+  int h, l;
+};
+__device__ __forceinline__ Split split(long long x) {
+  return Split{(int)((x + 0x80000000ll) >> 32), (int)x};
+}
+// a b 2^-64 to about a unit, plus add; |a|, |b| <= 2^62
+__device__ __forceinline__ long long mulh(Split a, Split b, long long add = 0) {
+  const long long m = (long long)a.h * b.l + ((long long)a.l * b.h + 0x80000000ll);
+  return (long long)a.h * b.h + add + (m >> 32);
+}
+// round(v 2^(62 - e)), 0 <= v < 2^e (or = 2^e)
+__device__ __forceinline__ long long fixed62(double v, int e) {
+  const unsigned long long bits = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+  const int be = (int)(bits >> 52);
+  const long long m = (long long)((bits & 0xFFFFFFFFFFFFFull) | (be ? 0x10000000000000ull : 0ull));
+  const int sh = max(be, 1) - 1013 - e;
+  if (sh >= 0) return m << min(sh, 10);
+  return sh > -63 ? (m + (1ll << (-sh - 1))) >> -sh : 0;
+}
+// a 2^(e - 60), rounded to FP64
+__device__ __forceinline__ double from_fixed60(long long a, int e) {
+  if (a == 0) return 0.0;
+  const unsigned long long u = (unsigned long long)llabs(a);
+  const int lz = __clzll((long long)u);
+  const int be = 1023 + 3 - lz + e;
+  if (be < 1 || be > 2045) return ldexp((double)a, e - 60);
+  // 53 bits at the top, rounded half up; a carry runs into the exponent
+  const unsigned long long m = ((u << lz) >> 10) + 1;
+  return __longlong_as_double((long long)((((unsigned long long)(be - 1) << 52) + (m >> 1)) |
+                                          ((unsigned long long)a & 0x8000000000000000ull)));
+}
+
+// cos and sin of 2 pi q / kAngles as 62-bit fractions, split: (cos h, cos l, sin h, sin l).
+__global__ void expand_angles_kernel(int4* __restrict__ table) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= kAngles) return;
+  double sn, cs;
+  sincospi(2.0 * q / kAngles, &sn, &cs);
+  const Split c = split(llrint(ldexp(cs, 62))), s = split(llrint(ldexp(sn, 62)));
+  table[q] = make_int4(c.h, c.l, s.h, s.l);
+}
+
+// cos and sin (62 fractional bits) of the angle phi 2^-64 turns.
+__device__ __forceinline__ void fixed_sincos(unsigned long long phi, const int4* table, long long& co,
+                                             long long& si) {
+  const unsigned q = (unsigned)((phi + (1ull << 53)) >> 54);   // (mod kAngles below)
+  const long long d = (long long)(phi - ((unsigned long long)q << 54));   // |d| <= 2^53
+  constexpr long long kTwoPi = 0x3243F6A8885A308Dll;    // 2 pi 2^59
+  constexpr long long kTwoThirds = 0x2AAAAAAAAAAAAAABll;   // 2 / 3 2^62
+  const long long th = mulh(split(d << 9), split(kTwoPi)) << 2;   // t 2^70
+  const Split t = split(th);
+  const long long u = mulh(t, t);                        // t^2 2^76
+  const int u47 = (int)(u >> 29);                        // t^2 2^47
+  const int f62 = (int)(((long long)u47 * u47) >> 32);   // t^4 2^62
+  // t^2 / 6 - t^4 / 120 in 2^-81
+  const long long v = (mulh(split(u), split(kTwoThirds)) - (((long long)f62 * 572662306) >> 22)) << 5;
+  const Split sn = split(th - (mulh(t, split(v)) >> 17));                       // sin t 2^70
+  const Split cm = split((u << 1) - (((long long)f62 * 357913941) >> 17));      // (1 - cos t) 2^78
+  const int4 e = table[q % kAngles];
+  const Split C{e.x, e.y}, S{e.z, e.w};
+  co = (((long long)e.x << 32) + e.y) - (((mulh(C, cm) >> 8) + mulh(S, sn)) >> 6);
+  si = (((long long)e.z << 32) + e.w) - (((mulh(S, cm) >> 8) - mulh(C, sn)) >> 6);
+}
+
 // Moments of the columns [l0, l0 + kc): G[f M + m][l - l0][i] (i fastest). One thread per row;
 // the block's columns' geometry is staged in shared memory and read by broadcast. The
 // diagonal is zero (the self terms are added in closed form).
 template <int MT, bool kG, bool kH>
 __global__ void __launch_bounds__(kRowsE)
-expand_moments_kernel(Geometry g, double2 c, double two_over_R, int M, int64_t l0, int kc,
-                      double2* __restrict__ G) {
+expand_moments_kernel(Geometry g, double2 c, FixedPhase fp, int M, int64_t l0, int kc,
+                      const int4* __restrict__ angles, double2* __restrict__ G) {
+  constexpr int F = (kG ? 1 : 0) + (kH ? 1 : 0);
+  __shared__ int4 table[kAngles];
   __shared__ double sq[kColsE][7][4];
   __shared__ double sn3[kColsE][3];
+  __shared__ long long srho[7][kRowsE];
+  __shared__ double sbase[7][F][kRowsE];   // the weights, then the same as fixed-point numbers
   const int64_t n = g.n;
-  const int64_t i = (int64_t)blockIdx.x * kRowsE + threadIdx.x;
+  const int tid = threadIdx.x;
+  const int64_t i = (int64_t)blockIdx.x * kRowsE + tid;
   const int c0 = blockIdx.y * kColsE;
   const int nc = min(kColsE, kc - c0);
-  for (int t = threadIdx.x; t < nc * 7; t += kRowsE) {
+  for (int t = tid; t < kAngles; t += kRowsE) table[t] = angles[t];
+  for (int t = tid; t < nc * 7; t += kRowsE) {
     const int cc = t / 7, q = t % 7;
     const int64_t l = l0 + c0 + cc;
     sq[cc][q][0] = g.qp[q * n + l];
@@ -104,31 +198,105 @@ expand_moments_kernel(Geometry g, double2 c, double two_over_R, int M, int64_t l
     sq[cc][q][3] = g.qw[q * n + l];
   }
   if (kH)
-    for (int t = threadIdx.x; t < nc * 3; t += kRowsE)
-      sn3[t / 3][t % 3] = g.nrm[(t % 3) * n + l0 + c0 + t / 3];
+    for (int t = tid; t < nc * 3; t += kRowsE) sn3[t / 3][t % 3] = g.nrm[(t % 3) * n + l0 + c0 + t / 3];
   __syncthreads();
   if (i >= n) return;
   const double xi = g.cx[i], yi = g.cx[n + i], zi = g.cx[2 * n + i];
-  constexpr int F = (kG ? 1 : 0) + (kH ? 1 : 0);
+  const Split K = split(fp.K);
   for (int cc = 0; cc < nc; ++cc) {
-    const int64_t l = l0 + c0 + cc;
-    double ar[F][MT], ai[F][MT];
+    long long ar[F][MT], ai[F][MT];
 #pragma unroll
     for (int f = 0; f < F; ++f)
 #pragma unroll
-      for (int m = 0; m < MT; ++m) ar[f][m] = ai[f][m] = 0.0;
-    if (l != i) {
+      for (int m = 0; m < MT; ++m) ar[f][m] = ai[f][m] = 0;
+    int e[F];                    // exponents of the families' scales
+    bool finite = true;
+#pragma unroll
+    for (int f = 0; f < F; ++f) e[f] = 0;
+    if (l0 + c0 + cc != i) {
+      // distances and weights
+      int top[F];
+#pragma unroll
+      for (int f = 0; f < F; ++f) top[f] = 0;
 #pragma unroll 1
-      for (int q = 0; q < 7; ++q)
-        expand_point<MT, kG, kH>(ar, ai, sq[cc][q][3], sq[cc][q][0] - xi, sq[cc][q][1] - yi,
-                                 sq[cc][q][2] - zi, sn3[cc], c, two_over_R);
+      for (int q = 0; q < 7; ++q) {
+        const double dx = sq[cc][q][0] - xi, dy = sq[cc][q][1] - yi, dz = sq[cc][q][2] - zi;
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        // 1 / sqrt(r2) and sqrt(r2) by one third-order step from the FP32 root, y (1 + e / 2 +
+        // 3 e^2 / 8) with e = 1 - r2 y^2 of ~2^-22
+        const float rf = (float)r2;
+        const double y = rf > 1e-30f && rf < 1e30f ? (double)rsqrtf(rf) : rsqrt(r2);
+        const double t = r2 * y, er = fma(-t, y, 1.0), pe = fma(0.375, er, 0.5);
+        const double r = fma(t * er, pe, t), ri = fma(y * er, pe, y);
+        srho[q][tid] = fixed62(r * fp.inv_R, 0);
+        double w = sq[cc][q][3] * ri;
+        if (c.y != 0.0) w *= exp(-c.y * r);
+        if (kG) sbase[q][0][tid] = w;
+        if (kH) sbase[q][F - 1][tid] = w * ri * ri * (dx * sn3[cc][0] + dy * sn3[cc][1] + dz * sn3[cc][2]);
+#pragma unroll
+        for (int f = 0; f < F; ++f)
+          top[f] = max(top[f], __double2hiint(sbase[q][f][tid]) & 0x7FFFFFFF);
+      }
+      // the weights as 62-bit fractions of a scale just above the sum of their magnitudes
+#pragma unroll
+      for (int f = 0; f < F; ++f) {
+        finite = finite && top[f] < 0x7FF00000;
+        e[f] = (top[f] >> 20) - 1022 + 3;
+        long long sum = 0;
+#pragma unroll 1
+        for (int q = 0; q < 7; ++q) {
+          const double v = sbase[q][f][tid];
+          const long long b = fixed62(v, e[f]);
+          sum += b;
+          sbase[q][f][tid] = __longlong_as_double(__double2hiint(v) < 0 ? -b : b);
+        }
+        const int sh = sum ? __clzll(sum) - 2 : 0;
+        e[f] -= sh;
+#pragma unroll 1
+        for (int q = 0; q < 7; ++q)
+          sbase[q][f][tid] = __longlong_as_double(__double_as_longlong(sbase[q][f][tid]) << sh);
+      }
+#pragma unroll 1
+      for (int q = 0; q < 7; ++q) {
+        const long long rho = srho[q][tid];
+        long long co, si;
+        fixed_sincos((unsigned long long)mulh(split(rho), K) << (4 + fp.kb), table, co, si);
+        const Split sc = split(co), ss = split(si);
+        Split br[F], bi[F];
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+          const Split b = split(__double_as_longlong(sbase[q][f][tid]));
+          const long long r0 = mulh(b, sc), i0 = mulh(b, ss);   // 2^-60: as T_0's terms
+          ar[f][0] += r0;
+          ai[f][0] += i0;
+          br[f] = split(r0 << 2);
+          bi[f] = split(i0 << 2);
+        }
+        const long long x = 2 * rho - kOne;
+        const Split sx = split(x);
+        long long t0 = kOne, t1 = x;
+#pragma unroll
+        for (int m = 1; m < MT; ++m) {
+          const Split t = split(t1);
+#pragma unroll
+          for (int f = 0; f < F; ++f) {
+            ar[f][m] = mulh(br[f], t, ar[f][m]);
+            ai[f][m] = mulh(bi[f], t, ai[f][m]);
+          }
+          const long long t2 = (mulh(sx, t) << 3) - t0;
+          t0 = t1;
+          t1 = t2;
+        }
+      }
     }
 #pragma unroll
     for (int f = 0; f < F; ++f)
 #pragma unroll
       for (int m = 0; m < MT; ++m)
         if (m < M)
-          G[((int64_t)(f * M + m) * kc + c0 + cc) * n + i] = make_double2(ar[f][m], ai[f][m]);
+          G[((int64_t)(f * M + m) * kc + c0 + cc) * n + i] =
+              finite ? make_double2(from_fixed60(ar[f][m], e[f]), from_fixed60(ai[f][m], e[f]))
+                     : make_double2(NAN, NAN);
   }
 }
 
@@ -289,7 +457,7 @@ __global__ void expand_columns_kernel(const double2* __restrict__ Ys, int64_t n,
   R[t] = acc;
 }
 
-using MomentKernel = void (*)(Geometry, double2, double, int, int64_t, int, double2*);
+using MomentKernel = void (*)(Geometry, double2, FixedPhase, int, int64_t, int, const int4*, double2*);
 
 template <bool kG, bool kH>
 MomentKernel moment_kernel(int M) {
@@ -306,6 +474,20 @@ MomentKernel moment_kernel(int M) {
   if (M <= 20) return expand_moments_kernel<20, kG, kH>;
   if (M <= 24) return expand_moments_kernel<24, kG, kH>;
   return expand_moments_kernel<kMaxTerms, kG, kH>;
+}
+
+// K = c / (2 pi inv_R) in turns, in two FP64 parts before it is rounded to 62 - kb bits.
+FixedPhase fixed_phase(double c, double R) {
+  FixedPhase fp;
+  fp.inv_R = 1.0 / R;
+  const double i2p = 0.15915494309189535, i2p_lo = -9.839338337591243e-18;   // 1 / (2 pi)
+  const double rhi = 1.0 / fp.inv_R, rlo = fma(-rhi, fp.inv_R, 1.0) / fp.inv_R;   // 1 / inv_R
+  const double a = c * rhi, al = fma(c, rhi, -a) + c * rlo;
+  const double k = a * i2p, kl = fma(a, i2p, -k) + (a * i2p_lo + al * i2p);
+  fp.kb = 0;
+  while (ldexp(1.0, fp.kb) <= fabs(k)) ++fp.kb;
+  fp.K = llrint(ldexp(k, 62 - fp.kb)) + llrint(ldexp(kl, 62 - fp.kb));
+  return fp;
 }
 
 // Largest distance between two points of the mesh, from above: the smaller of its box's
@@ -359,13 +541,20 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   p.R = mesh_reach(ctx);
   if (!(p.R > 0.0) || !isfinite(p.R)) return p;
   p.M = series_terms(dmax, p.R);
+  // about a real centre no exponential is evaluated: for values near the axis, at most a term more
+  if (c_im != 0.0 && series_terms(dmax + fabs(c_im), p.R) <= p.M + 1) {
+    dmax += fabs(c_im);
+    c_im = 0.0;
+    p.M = series_terms(dmax, p.R);
+  }
+  p.c = make_double2(c_re, c_im);
+  if (!(fabs(c_re) * p.R < 0x1p40)) return p;   // the phase's fixed-point range
   if (p.M > 1 && (hasH || deriv)) p.M += 2;
   if (p.M == 1 && (hasH || deriv)) p.M = 3;   // factors 1, r, r^2
   if (p.M < 1 || p.M > kMaxTerms) return p;
   p.first = hasG ? 0 : 1;
   p.fams = (hasG ? 1 : 0) + (hasH ? 1 : 0);
   p.S = p.fams * p.M;
-  p.c = make_double2(c_re, c_im);
   // FP64 operations per entry of the two forms; the smaller wins. Projection at n = 768,
   // nu = 64: direct 5.56 ms at N = 5, expanded 5.41 ms at N = 6 and 5.48 ms at N = 16; at
   // nu = 128: direct 10.2 ms at N = 6, expanded 8.4 ms at N = 7, 9.3 ms at N = 16. Residuals on
@@ -388,8 +577,8 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   // enough blocks for eight small blocks on each SM, at least 64 columns each
   p.splits = p.split ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(8 * (int64_t)std::max(1, sms) / tiles, p.kc / 64));
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-  p.coef_off = 0;
-  p.mom_off = up((size_t)p.S * nk * 16);
+  p.coef_off = kAngles * sizeof(int4);   // (the angles' table first)
+  p.mom_off = p.coef_off + up((size_t)p.S * nk * 16);
   p.y_off = p.mom_off + up((size_t)p.S * p.kc * n * 16);
   p.batch_off = p.y_off + up((size_t)p.splits * p.S * n * ncols * 16);
   p.bytes = p.batch_off + p.batch.bytes;
@@ -417,7 +606,10 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
   MomentKernel mk = p.fams == 2 ? moment_kernel<true, true>(p.M)
                                 : (p.first == 0 ? moment_kernel<true, false>(p.M)
                                                 : moment_kernel<false, true>(p.M));
-  ctx->launches++;
+  int4* angles = reinterpret_cast<int4*>(work);
+  expand_angles_kernel<<<kAngles / 128, 128, 0, s>>>(angles);
+  const FixedPhase fp = fixed_phase(p.c.x, p.R);
+  ctx->launches += 2;
   const double2* Xd = reinterpret_cast<const double2*>(X);
   if (p.split) {
     const bem_status st = split64_batch_scales(ctx, p.batch, work + p.batch_off, Xd, ldx, s);
@@ -426,7 +618,7 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
   for (int64_t l0 = 0; l0 < n; l0 += p.kc) {
     const int kc = (int)std::min<int64_t>(p.kc, n - l0);
     const dim3 ge((unsigned)((n + kRowsE - 1) / kRowsE), (unsigned)((kc + kColsE - 1) / kColsE));
-    mk<<<ge, kRowsE, 0, s>>>(ctx->geo, p.c, 2.0 / p.R, p.M, l0, kc, G);
+    mk<<<ge, kRowsE, 0, s>>>(ctx->geo, p.c, fp, p.M, l0, kc, angles, G);
     ctx->launches++;
     if (p.split) {
       const bem_status st = split64_batch(ctx, p.batch, work + p.batch_off, G, (int64_t)kc * n, kc,

@@ -514,6 +514,10 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
   const size_t y_bytes = AV_dev ? 0 : (size_t)N * n * nu * 2 * sizeof(double);
   ExpandPlan ex = expand_plan(ctx, N, ctx->con.c_re, ctx->con.c_im, std::max(ctx->con.a, ctx->con.b),
                               nu, true, false);
+  // V^H Y_j on the tensor core, its workspace in the place of the expansion's; the workspaces are
+  // found before any is written
+  SplitCross xs = split64_cross_plan(ctx, n, nu, nu, N);
+  xs.use = xs.use && scratch_ready(ctx, y_bytes + xs.bytes, s);
   ex.use = expand_ready(ctx, ex, y_bytes, nu, s);
   if (!ex.use) {
     bem_status st = ensure_scratch(ctx, y_bytes);
@@ -531,6 +535,11 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
     st = near_apply64(ctx, V_dev, ldv, nu, Y, s);
     if (st != BEM_OK) return st;
   }
+  if (xs.use)
+    return split64_cross(ctx, xs, reinterpret_cast<char*>(ctx->d_scratch) + y_bytes,
+                         reinterpret_cast<const double2*>(V_dev), ldv,
+                         reinterpret_cast<const double2*>(Y), reinterpret_cast<const double2*>(ctx->con.w),
+                         reinterpret_cast<double2*>(Bhat_dev), s);
   return cuda_check(ctx, launch_xhy_fp64(ctx, V_dev, ldv, nu, Y, n, n * nu, nu, n, N, ctx->con.w,
                                          Bhat_dev, s),
                     "projection kernel");

@@ -6,10 +6,12 @@
 // precomputed self term on it) and multiplies it into the 32 x 64 accumulator at once,
 // so A(z_j) is never stored.
 // xhy_fp64_kernel: C_j = s_j X^H Y_j, one block per 32 x 32 output tile and batch entry,
-// summing over rows in a fixed order (deterministic, no atomics).
+// summing over rows in a fixed order (deterministic, no atomics). Larger projections form it on
+// the tensor core (split64.cu).
 #include <math.h>
 
 #include "internal.h"
+#include "sm100.cuh"
 
 namespace bem {
 namespace {
@@ -137,14 +139,22 @@ apply_fp64_kernel(Geometry g, const double* __restrict__ self, const double* __r
 
 constexpr int kT = 32;   // output tile of X^H Y
 
+// kShare blocks of a cluster take a tile's rows in turn (a share each) and the first adds their
+// sums in order: where there are too few tiles for the device's SMs. One block a tile: one
+// 576 x 24 x 24 product took 600 us, now 109 us.
+constexpr int kShare = 8;
+
+template <bool kCluster>
 __global__ void __launch_bounds__(kThreads)
 xhy_fp64_kernel(const double* __restrict__ X, int64_t ldx, int p, const double* __restrict__ Y,
                 int64_t ldy, int64_t strideY, int q, int64_t n, const double* __restrict__ scale,
                 double* __restrict__ C) {
+  const int share = kCluster ? (int)sm100::cluster_ctarank() : 0;
   __shared__ double2 sX[kT][kT + 1];
   __shared__ double2 sY[kT][kT + 1];
   const int tiles_a = (p + kT - 1) / kT;
-  const int ta = blockIdx.x % tiles_a, tb = blockIdx.x / tiles_a;
+  const int tile = blockIdx.x / (kCluster ? kShare : 1);
+  const int ta = tile % tiles_a, tb = tile / tiles_a;
   const int jb = blockIdx.y;
   const int tid = threadIdx.x;
   const int oa = tid % kT;        // output row within the tile
@@ -154,18 +164,20 @@ xhy_fp64_kernel(const double* __restrict__ X, int64_t ldx, int p, const double* 
   double2 acc[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) acc[m] = make_double2(0.0, 0.0);
-  for (int64_t r0 = 0; r0 < n; r0 += kT) {
+  // rows a chunk: fewer than kT where the shares would otherwise be uneven
+  const int rows = kCluster ? (int)min((int64_t)kT, (n + kShare - 1) / kShare) : kT;
+  for (int64_t r0 = (int64_t)share * rows; r0 < n; r0 += (int64_t)(kCluster ? kShare : 1) * rows) {
     __syncthreads();
     for (int t = tid; t < kT * kT; t += kThreads) {
       const int rr = t % kT, cc = t / kT;
       const int64_t r = r0 + rr;
       const int a = ta * kT + cc, b = tb * kT + cc;
-      sX[rr][cc] = (r < n && a < p) ? Xc[(int64_t)a * ldx + r] : make_double2(0.0, 0.0);
-      sY[rr][cc] = (r < n && b < q) ? Yc[(int64_t)b * ldy + r] : make_double2(0.0, 0.0);
+      sX[rr][cc] = (r < n && rr < rows && a < p) ? Xc[(int64_t)a * ldx + r] : make_double2(0.0, 0.0);
+      sY[rr][cc] = (r < n && rr < rows && b < q) ? Yc[(int64_t)b * ldy + r] : make_double2(0.0, 0.0);
     }
     __syncthreads();
 #pragma unroll 8
-    for (int rr = 0; rr < kT; ++rr) {
+    for (int rr = 0; rr < (kCluster ? rows : kT); ++rr) {
       const double2 x = sX[rr][oa];   // conj(x) * y
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
@@ -174,6 +186,29 @@ xhy_fp64_kernel(const double* __restrict__ X, int64_t ldx, int p, const double* 
         acc[m].y = fma(x.x, y.y, fma(-x.y, y.x, acc[m].y));
       }
     }
+  }
+  if (kCluster) {
+    __syncthreads();
+    double2* mine = &sX[0][0];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) mine[m * kThreads + tid] = acc[m];
+    sm100::cluster_sync_all();
+    if (share == 0)
+      for (int k = 1; k < kShare; ++k) {
+        const uint32_t from = sm100::mapa_shared(sm100::smem_u32(mine), k);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          double2 v;
+          asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];"
+                       : "=d"(v.x), "=d"(v.y)
+                       : "r"(from + (uint32_t)((m * kThreads + tid) * sizeof(double2)))
+                       : "memory");
+          acc[m].x += v.x;
+          acc[m].y += v.y;
+        }
+      }
+    sm100::cluster_sync_all();   // the shares stay until they are read
+    if (share != 0) return;
   }
   double2 s = make_double2(1.0, 0.0);
   if (scale) s = reinterpret_cast<const double2*>(scale)[jb];
@@ -206,8 +241,24 @@ cudaError_t launch_xhy_fp64(bem_ctx* ctx, const double* X, int64_t ldx, int p, c
                             int64_t ldy, int64_t strideY, int q, int64_t n, int nb,
                             const double* scale, double* C, cudaStream_t s) {
   const int tiles = ((p + kT - 1) / kT) * ((q + kT - 1) / kT);
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  if ((int64_t)tiles * nb * 2 < sms && n > kT) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(tiles * kShare), (unsigned)nb);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kShare;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    ctx->launches++;
+    return cudaLaunchKernelEx(&cfg, xhy_fp64_kernel<true>, X, ldx, p, Y, ldy, strideY, q, n, scale, C);
+  }
   dim3 grid((unsigned)tiles, (unsigned)nb);
-  xhy_fp64_kernel<<<grid, kThreads, 0, s>>>(X, ldx, p, Y, ldy, strideY, q, n, scale, C);
+  xhy_fp64_kernel<false><<<grid, kThreads, 0, s>>>(X, ldx, p, Y, ldy, strideY, q, n, scale, C);
   ctx->launches++;
   return cudaGetLastError();
 }

@@ -57,6 +57,12 @@ constexpr size_t kMaxSplitBytes = (size_t)8 << 30;
 // 50000 x 16 425 / 525, 8192 x 256 1909 / 7171 above.
 constexpr int64_t kMinWork = (int64_t)1 << 23;
 
+// n p q nb from which X^H Y_j by splitting pays. FP64 projections whose last step it is, split
+// against FP64, in us: 192 panels, 16 columns, 16 nodes (2^19.6) 492 / 491; 300 x 10 x 24 457 / 535,
+// 588 x 30 x 16 700 / 833, 972 x 100 x 16 1814 / 3654. Its error against 128-bit sums at 768 x 64
+// is 1e-16, the FP64 kernel's 1.2e-15.
+constexpr int64_t kMinCross = (int64_t)1 << 19;
+
 __device__ __forceinline__ bool skipped(const int* gate, const int* skip) {
   return (gate && *gate == 0) || (skip && *skip != 0);
 }
@@ -120,8 +126,8 @@ __device__ __forceinline__ int scale_exp(int e) { return (e == kNotFinite || e =
 __device__ __forceinline__ int col_exp(const unsigned* hi, int c) { return scale_exp(exponent_of(hi[c])); }
 
 // Digit planes of V's columns with the rows as K: a[kb][tile of 128 columns][digit][re, im] and
-// b[kb][tile of 32 columns]{[digit][re | im], [digit][im | -re]}, in K-major core matrices. One
-// thread per column and 8 rows.
+// b[kb][tile of 32 columns]{[digit][re | im], [digit][im | -re]} (b null: not written), in K-major
+// core matrices. One thread per column and 8 rows.
 __global__ void __launch_bounds__(128)
 split_columns_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int nu, int kbn,
                      int mtu, int ntu, const unsigned* __restrict__ hc, unsigned char* __restrict__ a,
@@ -150,7 +156,7 @@ split_columns_kernel(const double2* __restrict__ V, int64_t ldv, int64_t n, int 
   const int m = c % kTileM, r = c % kTileN;
   unsigned char* ap = a + ((size_t)kb * mtu + c / kTileM) * kABytes + (m / 8) * 256 + kh * 128 + (m % 8) * 16;
   unsigned char* bp = b + ((size_t)kb * ntu + c / kTileN) * kBBytes + (r / 8) * 256 + kh * 128 + (r % 8) * 16;
-  const bool inb = c / kTileN < ntu;
+  const bool inb = b && c / kTileN < ntu;
   // part h of half w of the right operand: rows 32 h + r of the digit's 64
   auto put_b = [&](int w, int h) {
     if (!inb) return;
@@ -296,10 +302,12 @@ split_factor_kernel(const double2* __restrict__ Z, int nu, int kbu, int ntu,
   }
 }
 
-// Digit planes of the columns of X with the rows [0, n) as K, for a plain product:
-// b[kb][tile of 32 columns]{[digit][re | im], [digit][-im | re]}. A thread per column and 8 rows.
+// Digit planes of the columns of X with the rows [0, n) as K: b[kb][tile of 32 columns]
+// {[digit][re | im], [digit][-im | re]} for a plain product, {.., [digit][im | -re]} (kConj) for
+// one with a conjugated left operand. A thread per column and 8 rows.
+template <bool kConj>
 __global__ void __launch_bounds__(128)
-split_rhs_kernel(const double2* __restrict__ X, int64_t ldx, int n, int nu, int kbn, int ntu,
+split_rhs_kernel(const double2* __restrict__ X, int64_t ldx, int64_t n, int nu, int kbn, int ntu,
                  const unsigned* __restrict__ hc, unsigned char* __restrict__ b) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t gr = t % (2 * kbn);
@@ -324,11 +332,12 @@ split_rhs_kernel(const double2* __restrict__ X, int64_t ldx, int n, int nu, int 
   };
   digits8(re, d, false);
   put_b(0, 0);
-  put_b(1, 1);
+  if (!kConj) put_b(1, 1);
   digits8(im, d, false);
   put_b(0, 1);
-  digits8(im, d, true);
-  put_b(1, 0);
+  if (kConj) put_b(1, 0);
+  digits8(kConj ? re : im, d, true);
+  put_b(1, kConj ? 1 : 0);
 }
 
 struct GemmArgs {
@@ -370,14 +379,22 @@ struct Tile {
 };
 
 // Tile i of this block (false: no more).
-enum { kGramSum = 0, kTriangle = 1, kBatch = 2 };
+enum { kGramSum = 0, kTriangle = 1, kBatch = 2, kCross = 3 };
 
 // Gram: one tile per block, the upper ones only, counted along b within a; blockIdx.y the row
-// range. Products: whole rows of tiles per block (the row tile's planes stay in L2), widest
+// range. Cross: likewise, all tiles. Products: whole rows of tiles per block (the row tile's planes stay in L2), widest
 // first; the rows left over after the last full round are dealt tile by tile.
 template <int kMode>
 __device__ __forceinline__ bool tile_of(const GemmArgs& p, int i, Tile& t) {
   const int nt = (int)p.tb;
+  if (kMode == kCross) {
+    if (i > 0) return false;
+    t.ta = blockIdx.x % p.ta;
+    t.tb = (int)(blockIdx.x / p.ta);
+    t.kb0 = (int)((int64_t)p.kb_total * blockIdx.y / p.parts);
+    t.kb1 = (int)((int64_t)p.kb_total * (blockIdx.y + 1) / p.parts);
+    return true;
+  }
   if (kMode == kGramSum) {
     if (i > 0) return false;
     int rest = blockIdx.x, at = 0;
@@ -409,7 +426,8 @@ __device__ __forceinline__ bool tile_of(const GemmArgs& p, int i, Tile& t) {
 // kGramSum: out[part][b nu + a] = sum of the rows of part blockIdx.y, with [re | im] and
 // [im | -re] for conj(V)^T V. kTriangle: V[i][c] = sum_k V[i][k] Z[k][c], with [re | im] and
 // [-im | re]; the K-blocks of the upper triangle only. kBatch: out_s (+)= A_s X likewise, all
-// K-blocks, the row tiles of the matrices one after the other.
+// K-blocks, the row tiles of the matrices one after the other. kCross: as kGramSum with another
+// right operand, out[part][c n + a], a < n, c < nu.
 template <int kMode>
 __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
   if (skipped(p.gate, p.skip)) return;
@@ -560,7 +578,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
       const int64_t row = (t.ta - slot * p.mtn) * kTileM + quarter * 32 + lane;
       const int64_t rows = kMode == kGramSum ? p.nu : p.n;
       int er = row < rows ? p.ea[slot * p.n + row] : 0;
-      if (kMode == kGramSum) er = exponent_of((unsigned)er);
+      if (kMode == kGramSum || kMode == kCross) er = exponent_of((unsigned)er);
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
         const int col = t.tb * kTileN + k;
@@ -571,7 +589,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
         v = e > -1022 && e < 1023 ? v * __longlong_as_double((long long)(e + 1023) << 52) : ldexp(v, e);
         if (er == kNotFinite || ec == kNotFinite) v = NAN;
         double* o = reinterpret_cast<double*>(
-            kMode == kGramSum ? p.out + (int64_t)blockIdx.y * p.nu * p.nu + (int64_t)col * p.nu + row
+            kMode == kGramSum || kMode == kCross ? p.out + ((int64_t)blockIdx.y * p.nu + col) * rows + row
                               : p.out + (slot * p.nu + col) * p.ldv + row);
         o[side] = kMode == kBatch && p.add ? o[side] + v : v;
       }
@@ -589,7 +607,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
 
 bem_status set_gemm_smem(bem_ctx* ctx) {
   for (const void* f : {(const void*)split_gemm_kernel<kGramSum>, (const void*)split_gemm_kernel<kTriangle>,
-                        (const void*)split_gemm_kernel<kBatch>}) {
+                        (const void*)split_gemm_kernel<kBatch>, (const void*)split_gemm_kernel<kCross>}) {
     const bem_status st = cuda_check(
         ctx, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmSmem::total),
         "split product attribute");
@@ -736,7 +754,7 @@ bem_status split64_batch(bem_ctx* ctx, const SplitBatch& b, char* work, const do
   split_rows_kernel<<<dim3((unsigned)(b.mtn * (kTileM / 32)), (unsigned)b.S), 256, 0, s>>>(
       A, b.n, astep, b.n, kc, kb, b.mtn, nullptr, er, ap, nullptr, nullptr);
   const int64_t threads = 2 * (int64_t)kb * b.ntu * kTileN;
-  split_rhs_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(X, ldx, kc, b.nu, kb, b.ntu, hcol, bp);
+  split_rhs_kernel<false><<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(X, ldx, kc, b.nu, kb, b.ntu, hcol, bp);
   GemmArgs g{ap, bp, b.S * b.mtn, b.ntu, b.mtn, add, b.nu, b.n, b.n, kb, 1, er,
              reinterpret_cast<const int*>(hcol), out, ctx->d_status, nullptr, nullptr};
   int sms = 0;
@@ -745,6 +763,81 @@ bem_status split64_batch(bem_ctx* ctx, const SplitBatch& b, char* work, const do
   split_gemm_kernel<kBatch><<<grid, kThreadsG, GemmSmem::total, s>>>(g);
   ctx->launches += 3;
   return cuda_check(ctx, cudaGetLastError(), "split products");
+}
+
+namespace {
+
+// C_j = scale_j * sum of the partial products of its columns.
+__global__ void __launch_bounds__(256)
+split_cross_sum_kernel(const double2* __restrict__ part, int parts, int64_t block, int64_t count,
+                       const double2* __restrict__ scale, double2* __restrict__ C) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= count) return;
+  double2 v = part[t];
+  for (int r = 1; r < parts; ++r) {
+    const double2 u = part[r * count + t];
+    v.x += u.x;
+    v.y += u.y;
+  }
+  if (scale) {
+    const double2 s = scale[t / block];
+    v = make_double2(s.x * v.x - s.y * v.y, s.x * v.y + s.y * v.x);
+  }
+  C[t] = v;
+}
+
+}  // namespace
+
+SplitCross split64_cross_plan(const bem_ctx* ctx, int64_t n, int p, int q, int nb) {
+  SplitCross c;
+  const int64_t cols = (int64_t)q * nb;
+  if (n * p * cols < kMinCross || cols > INT_MAX / 2) return c;
+  c.n = n;
+  c.p = p;
+  c.q = q;
+  c.nb = nb;
+  c.mtp = (p + kTileM - 1) / kTileM;
+  c.nt = (int)((cols + kTileN - 1) / kTileN);
+  const int64_t kb = (n + 15) / 16;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  c.parts = (int)std::max<int64_t>(1, std::min<int64_t>(kb / (2 * kFlush), std::max(1, sms) / (c.mtp * c.nt)));
+  if (kb / c.parts / kFlush > 2000) return c;   // the 64-bit sums' range
+  auto up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
+  c.b_off = up((size_t)kb * c.mtp * kABytes);
+  c.part_off = c.b_off + up((size_t)kb * c.nt * kBBytes);
+  c.h_off = c.part_off + up((size_t)c.parts * p * cols * sizeof(double2));
+  c.bytes = c.h_off + up(((size_t)p + cols) * sizeof(unsigned));
+  c.use = c.bytes <= kMaxSplitBytes;
+  return c;
+}
+
+bem_status split64_cross(bem_ctx* ctx, const SplitCross& c, void* work, const double2* X,
+                         int64_t ldx, const double2* Y, const double2* scale, double2* C,
+                         cudaStream_t s) {
+  unsigned char* ap = static_cast<unsigned char*>(work);
+  unsigned char* bp = ap + c.b_off;
+  double2* part = reinterpret_cast<double2*>(ap + c.part_off);
+  unsigned* hx = reinterpret_cast<unsigned*>(ap + c.h_off);
+  unsigned* hy = hx + c.p;
+  const int cols = c.q * c.nb, kb = (int)((c.n + 15) / 16);
+  bem_status st = set_gemm_smem(ctx);
+  if (st == BEM_OK) st = column_maxima(ctx, hx, X, ldx, c.n, c.p, nullptr, nullptr, s);
+  if (st == BEM_OK) st = column_maxima(ctx, hy, Y, c.n, c.n, cols, nullptr, nullptr, s);
+  if (st != BEM_OK) return st;
+  const int64_t tx = 2 * (int64_t)kb * c.mtp * kTileM, ty = 2 * (int64_t)kb * c.nt * kTileN;
+  split_columns_kernel<<<(unsigned)((tx + 127) / 128), 128, 0, s>>>(X, ldx, c.n, c.p, kb, c.mtp, 0, hx, ap,
+                                                                   nullptr, nullptr);
+  split_rhs_kernel<true><<<(unsigned)((ty + 127) / 128), 128, 0, s>>>(Y, c.n, c.n, cols, kb, c.nt, hy, bp);
+  GemmArgs g{ap, bp, c.mtp, c.nt, c.mtp, false, cols, c.p, c.p, kb, c.parts,
+             reinterpret_cast<const int*>(hx), reinterpret_cast<const int*>(hy), part, ctx->d_status,
+             nullptr, nullptr};
+  split_gemm_kernel<kCross><<<dim3((unsigned)(c.mtp * c.nt), (unsigned)c.parts), kThreadsG, GemmSmem::total, s>>>(g);
+  const int64_t count = (int64_t)c.p * cols;
+  split_cross_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(
+      part, c.parts, (int64_t)c.p * c.q, count, scale, C);
+  ctx->launches += 4;
+  return cuda_check(ctx, cudaGetLastError(), "split projection");
 }
 
 }  // namespace bem

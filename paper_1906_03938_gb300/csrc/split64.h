@@ -51,4 +51,17 @@ bem_status split64_batch(bem_ctx* ctx, const SplitBatch& b, char* work, const do
                          int64_t astep, int kc, const double2* X, int64_t ldx, bool add,
                          double2* out, cudaStream_t s);
 
+// C_j = scale_j X^H Y_j, j < nb (as launch_xhy_fp64, Y contiguous with ld n).
+struct SplitCross {
+  bool use = false;         // large enough to pay, and its workspace within bounds
+  int64_t n = 0;
+  int p = 0, q = 0, nb = 0;
+  int mtp = 0, nt = 0, parts = 1;   // 128-row and 32-column tiles of the outputs, row ranges
+  size_t b_off = 0, part_off = 0, h_off = 0, bytes = 0;
+};
+SplitCross split64_cross_plan(const bem_ctx* ctx, int64_t n, int p, int q, int nb);
+bem_status split64_cross(bem_ctx* ctx, const SplitCross& c, void* work, const double2* X,
+                         int64_t ldx, const double2* Y, const double2* scale, double2* C,
+                         cudaStream_t s);
+
 }  // namespace bem

@@ -499,13 +499,10 @@ near_values32_kernel(Geometry g, const int32_t* __restrict__ rows, const int32_t
                      int64_t nnz, const double* __restrict__ z, int N, GL8 gl, OpCoef op,
                      float2* __restrict__ Cv) {
   __shared__ float s_x[8], s_w[64];
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-      s_x[p] = (float)gl.x[p];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) s_w[8 * p + q] = (float)(gl.w[p] * gl.w[q]);
-    }
+  if (threadIdx.x < 64) {
+    const int p = threadIdx.x / 8, q = threadIdx.x % 8;
+    if (q == 0) s_x[p] = (float)gl.x[p];
+    s_w[threadIdx.x] = (float)(gl.w[p] * gl.w[q]);
   }
   __syncthreads();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -586,58 +583,82 @@ near_values32_kernel(Geometry g, const int32_t* __restrict__ rows, const int32_t
 
 // Slice `slice` of the mixed path's partials := C(z_j) V in FP32 (every row < n_pad and
 // every column < nu written) from stored pair values Cv (node-major, nnz per node; the 8 x 8
-// rule's or the surrogate network's): one warp per (row i, node j); lanes load 32 pairs'
-// values and columns, then sweep the basis columns.
-__global__ void __launch_bounds__(256)
+// rule's or the surrogate network's). A block takes 8 rows, a warp each, and kNodes nodes: lanes
+// load 32 pairs' values and columns, then sweep the basis columns, kGroups of 32. Bound by L2: the
+// rows of V are read once for the kNodes nodes, and the results leave through shared memory as
+// full 32-byte sectors (8 rows of a column are contiguous). One node a warp and stores of single
+// words took 2.5 ms at 20480 panels, 32 nodes, 128 columns and 160 us at 1452 x 24 x 30; now
+// 0.97 ms and 45 us.
+constexpr int kSpRows = 8;
+
+template <int kGroups, int kNodes>
+__global__ void __launch_bounds__(32 * kSpRows)
 near_spmm32_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ cols, int64_t n,
                    int64_t nnz, int N, const float2* __restrict__ Cv, const float2* __restrict__ Vt,
                    int nu, int nup, int C, int n_pad, float* __restrict__ Yp, int slice) {
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
-  const int lane = threadIdx.x % 32;
-  if (w >= (int64_t)n_pad * N) return;
-  const int64_t i = w % n_pad;
-  const int node = (int)(w / n_pad);
-  float2 acc[kMaxColGroups];
+  __shared__ float2 out[kNodes][32 * kGroups][kSpRows + 1];
+  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int64_t i0 = (int64_t)blockIdx.x * kSpRows, i = i0 + w;
+  const int j0 = blockIdx.y * kNodes;
+  float2 acc[kNodes][kGroups];
 #pragma unroll
-  for (int t = 0; t < kMaxColGroups; ++t) acc[t] = make_float2(0.f, 0.f);
+  for (int u = 0; u < kNodes; ++u)
+#pragma unroll
+    for (int t = 0; t < kGroups; ++t) acc[u][t] = make_float2(0.f, 0.f);
   if (i < n) {
     const int32_t e0 = ptr[i], e1 = ptr[i + 1];
-    const float2* Cj = Cv + (int64_t)node * nnz;
     for (int32_t eb = e0; eb < e1; eb += 32) {
       const int32_t e = eb + lane;
-      float2 cval = make_float2(0.f, 0.f);
+      float2 cval[kNodes];
       int32_t l = 0;
+#pragma unroll
+      for (int u = 0; u < kNodes; ++u) cval[u] = make_float2(0.f, 0.f);
       if (e < e1) {
         l = cols[e];
-        cval = Cj[e];
+#pragma unroll
+        for (int u = 0; u < kNodes; ++u)
+          if (j0 + u < N) cval[u] = Cv[(int64_t)(j0 + u) * nnz + e];
       }
       const int cnt = min(32, e1 - eb);
+#pragma unroll 4
       for (int t = 0; t < cnt; ++t) {
-        const float cx = __shfl_sync(0xffffffffu, cval.x, t);
-        const float cy = __shfl_sync(0xffffffffu, cval.y, t);
-        const int32_t lt = __shfl_sync(0xffffffffu, l, t);
-        const float2* vr = Vt + (int64_t)lt * nu;
+        const float2* vr = Vt + (int64_t)__shfl_sync(0xffffffffu, l, t) * nu;
+        float2 v[kGroups];
 #pragma unroll
-        for (int cg = 0; cg < kMaxColGroups; ++cg) {
+        for (int cg = 0; cg < kGroups; ++cg) {
           const int c = lane + 32 * cg;
-          if (c < nu) {
-            const float2 v = vr[c];
-            acc[cg].x = fmaf(cx, v.x, fmaf(-cy, v.y, acc[cg].x));
-            acc[cg].y = fmaf(cx, v.y, fmaf(cy, v.x, acc[cg].y));
+          v[cg] = c < nu ? vr[c] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < kNodes; ++u) {
+          const float cx = __shfl_sync(0xffffffffu, cval[u].x, t);
+          const float cy = __shfl_sync(0xffffffffu, cval[u].y, t);
+#pragma unroll
+          for (int cg = 0; cg < kGroups; ++cg) {
+            acc[u][cg].x = fmaf(cx, v[cg].x, fmaf(-cy, v[cg].y, acc[u][cg].x));
+            acc[u][cg].y = fmaf(cx, v[cg].y, fmaf(cy, v[cg].x, acc[u][cg].y));
           }
         }
       }
     }
   }
-  const int acc_cols = 2 * nup;
-  float* base = Yp + ((size_t)slice * N + node) * acc_cols * (size_t)n_pad;
 #pragma unroll
-  for (int cg = 0; cg < kMaxColGroups; ++cg) {
-    const int c = lane + 32 * cg;
-    if (c < nu) {
+  for (int u = 0; u < kNodes; ++u)
+#pragma unroll
+    for (int cg = 0; cg < kGroups; ++cg) out[u][lane + 32 * cg][w] = acc[u][cg];
+  __syncthreads();
+  const int r = threadIdx.x % kSpRows;
+  if (i0 + r >= n_pad) return;
+  const int acc_cols = 2 * nup;
+#pragma unroll
+  for (int u = 0; u < kNodes; ++u) {
+    if (j0 + u >= N) break;
+    float* base = Yp + ((size_t)slice * N + j0 + u) * acc_cols * (size_t)n_pad + i0 + r;
+    for (int c = threadIdx.x / kSpRows; c < nu; c += 32) {
       const int colr = (c / C) * 2 * C + (c % C);
-      base[(size_t)colr * n_pad + i] = acc[cg].x;
-      base[(size_t)(colr + C) * n_pad + i] = acc[cg].y;
+      const float2 v = out[u][c][r];
+      base[(size_t)colr * n_pad] = v.x;
+      base[(size_t)(colr + C) * n_pad] = v.y;
     }
   }
 }
@@ -1192,9 +1213,14 @@ bem_status near_apply32(bem_ctx* ctx, const float2* V32, int nu, int nup, int C,
       ctx->launches++;
     }
   }
-  const unsigned blocks = (unsigned)((32 * (int64_t)n_pad * N + 255) / 256);
-  near_spmm32_kernel<<<blocks, 256, 0, s>>>(ctx->d_near_ptr, ctx->d_near_cols, n, nnz, N, Cv, Vt,
-                                            nu, nup, C, n_pad, Yp, slice);
+  const int nodes = nu <= 128 ? 4 : 2;
+  auto* spmm = nu <= 32   ? near_spmm32_kernel<1, 4>
+               : nu <= 64  ? near_spmm32_kernel<2, 4>
+               : nu <= 128 ? near_spmm32_kernel<4, 4>
+                           : near_spmm32_kernel<8, 2>;
+  spmm<<<dim3((unsigned)((n_pad + kSpRows - 1) / kSpRows), (unsigned)((N + nodes - 1) / nodes)),
+         32 * kSpRows, 0, s>>>(ctx->d_near_ptr, ctx->d_near_cols, n, nnz, N, Cv, Vt, nu, nup, C, n_pad, Yp,
+                               slice);
   ctx->launches++;
   return cuda_check(ctx, cudaGetLastError(), "near field kernels");
 }

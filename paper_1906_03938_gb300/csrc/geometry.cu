@@ -40,55 +40,95 @@ Rule7 make_rule7() {
   return r;
 }
 
-__global__ void geometry_kernel(Geometry g, Rule7 rule, int* status) {
-  const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g.pack32 && l >= g.n && l < (g.n + 15) / 16 * 16) {
+// Panel data. Long FP64 work per panel on a pipe that takes a warp's operation in 64 clocks, and
+// few panels: a block takes 32 panels and its nine warps a part each (a quadrature point; area,
+// diameter and normal; centroid and edges), the area going to the others through shared memory.
+// One thread a panel: 17 us for 320 panels as for 3072; now 7.5 us.
+constexpr int kGeoParts = 9;
+
+__global__ void __launch_bounds__(32 * kGeoParts) geometry_kernel(Geometry g, Rule7 rule, int* status) {
+  __shared__ double s_area[32];
+  const int part = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int64_t l = blockIdx.x * (int64_t)32 + lane;
+  const int64_t n = g.n;
+  bool valid = l < n;
+  if (g.pack32 && !valid && l < (n + 15) / 16 * 16 && part == 0) {
     // padding panels of the packed array: finite placeholders, zero weights
     for (int t = 0; t < 64; ++t) g.pack32[l * 64 + t] = (t < 28 && t % 4 != 3) ? 1.0f : 0.0f;
-    return;
-  }
-  if (l >= g.n) return;
-  const int32_t i0 = g.tri[3 * l], i1 = g.tri[3 * l + 1], i2 = g.tri[3 * l + 2];
-  if (i0 < 0 || i1 < 0 || i2 < 0 || i0 >= g.nv || i1 >= g.nv || i2 >= g.nv) {
-    atomicOr(status, kStatusBadIndex);
-    return;
   }
   double v[3][3];
-  for (int c = 0; c < 3; ++c) {
-    v[0][c] = g.xyz[3 * (int64_t)i0 + c];
-    v[1][c] = g.xyz[3 * (int64_t)i1 + c];
-    v[2][c] = g.xyz[3 * (int64_t)i2 + c];
+  if (valid) {
+    const int32_t i0 = g.tri[3 * l], i1 = g.tri[3 * l + 1], i2 = g.tri[3 * l + 2];
+    if (i0 < 0 || i1 < 0 || i2 < 0 || i0 >= g.nv || i1 >= g.nv || i2 >= g.nv) {
+      if (part == 0) atomicOr(status, kStatusBadIndex);
+      valid = false;
+    } else {
+      for (int c = 0; c < 3; ++c) {
+        v[0][c] = g.xyz[3 * (int64_t)i0 + c];
+        v[1][c] = g.xyz[3 * (int64_t)i1 + c];
+        v[2][c] = g.xyz[3 * (int64_t)i2 + c];
+      }
+    }
   }
-  const double e1[3] = {v[1][0] - v[0][0], v[1][1] - v[0][1], v[1][2] - v[0][2]};
-  const double e2[3] = {v[2][0] - v[0][0], v[2][1] - v[0][1], v[2][2] - v[0][2]};
-  const double nx = e1[1] * e2[2] - e1[2] * e2[1];
-  const double ny = e1[2] * e2[0] - e1[0] * e2[2];
-  const double nz = e1[0] * e2[1] - e1[1] * e2[0];
-  const double area = 0.5 * sqrt(nx * nx + ny * ny + nz * nz);
-  // degenerate: area below 1e-12 of the squared longest edge (an exact zero can come out
-  // of the cross product as a rounding residue once products are fused)
-  const double e3[3] = {v[2][0] - v[1][0], v[2][1] - v[1][1], v[2][2] - v[1][2]};
-  const double l2 = fmax(fmax(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2],
-                              e2[0] * e2[0] + e2[1] * e2[1] + e2[2] * e2[2]),
-                         e3[0] * e3[0] + e3[1] * e3[1] + e3[2] * e3[2]);
-  if (!(area > 1e-12 * l2) || !isfinite(area)) atomicOr(status, kStatusZeroArea);
-  if (g.diam) {
-    // panel diameter for the near-field criterion, rounded step by step (no fused
-    // operations) so that the criterion is decided exactly as written
-    double len2[3];
-    const double* ed[3] = {e1, e2, e3};
-    for (int t = 0; t < 3; ++t)
-      len2[t] = __dadd_rn(__dadd_rn(__dmul_rn(ed[t][0], ed[t][0]), __dmul_rn(ed[t][1], ed[t][1])),
-                          __dmul_rn(ed[t][2], ed[t][2]));
-    g.diam[l] = fmax(fmax(sqrt(len2[0]), sqrt(len2[1])), sqrt(len2[2]));
+  double x[3], e1[3], e2[3], nx, ny, nz, area;   // x: the part's point, or the centroid
+  if (part < 7) {
+    for (int c = 0; c < 3; ++c)
+      x[c] = rule.bary[part][0] * v[0][c] + rule.bary[part][1] * v[1][c] + rule.bary[part][2] * v[2][c];
+  } else if (part == 7) {
+    for (int c = 0; c < 3; ++c) {
+      e1[c] = v[1][c] - v[0][c];
+      e2[c] = v[2][c] - v[0][c];
+    }
+    nx = e1[1] * e2[2] - e1[2] * e2[1];
+    ny = e1[2] * e2[0] - e1[0] * e2[2];
+    nz = e1[0] * e2[1] - e1[1] * e2[0];
+    area = 0.5 * sqrt(nx * nx + ny * ny + nz * nz);
+    s_area[lane] = area;
+  } else {
+    for (int c = 0; c < 3; ++c) x[c] = (v[0][c] + v[1][c] + v[2][c]) / 3.0;
   }
-  const int64_t n = g.n;
-  for (int c = 0; c < 3; ++c) {
-    const double x = (v[0][c] + v[1][c] + v[2][c]) / 3.0;
-    g.cx[c * n + l] = x;
-    g.cx32[c * n + l] = (float)x;
+  __syncthreads();
+  if (!valid) return;
+  if (part < 7) {
+    const int q = part;
+    const double w = rule.w[q] * s_area[lane] / (4.0 * kPiD);
+    g.qw[q * n + l] = w;
+    g.qw32[q * n + l] = (float)w;
+    for (int c = 0; c < 3; ++c) {
+      g.qp[(7 * c + q) * n + l] = x[c];
+      g.qp32[(7 * c + q) * n + l] = (float)x[c];
+    }
+    if (g.pack32) {
+      float* pk = g.pack32 + (int64_t)l * 64;
+      for (int c = 0; c < 3; ++c) {
+        const float hi = (float)x[c];
+        pk[4 * q + c] = hi;
+        pk[28 + 4 * q + c] = (float)(x[c] - (double)hi);
+      }
+      pk[4 * q + 3] = (float)w;
+      pk[28 + 4 * q + 3] = 0.f;
+    }
+    return;
   }
-  {
+  if (part == 7) {
+    // degenerate: area below 1e-12 of the squared longest edge (an exact zero can come out
+    // of the cross product as a rounding residue once products are fused)
+    const double e3[3] = {v[2][0] - v[1][0], v[2][1] - v[1][1], v[2][2] - v[1][2]};
+    const double l2 = fmax(fmax(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2],
+                                e2[0] * e2[0] + e2[1] * e2[1] + e2[2] * e2[2]),
+                           e3[0] * e3[0] + e3[1] * e3[1] + e3[2] * e3[2]);
+    if (!(area > 1e-12 * l2) || !isfinite(area)) atomicOr(status, kStatusZeroArea);
+    if (g.diam) {
+      // panel diameter for the near-field criterion, rounded step by step (no fused
+      // operations) so that the criterion is decided exactly as written
+      double len2[3];
+      const double* ed[3] = {e1, e2, e3};
+      for (int t = 0; t < 3; ++t)
+        len2[t] = __dadd_rn(__dadd_rn(__dmul_rn(ed[t][0], ed[t][0]), __dmul_rn(ed[t][1], ed[t][1])),
+                            __dmul_rn(ed[t][2], ed[t][2]));
+      // (the root is monotonic: one root of the largest square is the largest of the roots)
+      g.diam[l] = sqrt(fmax(fmax(len2[0], len2[1]), len2[2]));
+    }
     // unit normal in the vertex order (the double-layer kernel's n_y)
     const double inv = 1.0 / (2.0 * area);
     const double un[3] = {nx * inv, ny * inv, nz * inv};
@@ -96,35 +136,15 @@ __global__ void geometry_kernel(Geometry g, Rule7 rule, int* status) {
       if (g.nrm) g.nrm[c * n + l] = un[c];
       if (g.pack32) g.pack32[(int64_t)l * 64 + 56 + c] = (float)un[c];
     }
+    return;
   }
-  for (int q = 0; q < 7; ++q) {
-    for (int c = 0; c < 3; ++c) {
-      const double p = rule.bary[q][0] * v[0][c] + rule.bary[q][1] * v[1][c] +
-                       rule.bary[q][2] * v[2][c];
-      g.qp[(7 * c + q) * n + l] = p;
-      g.qp32[(7 * c + q) * n + l] = (float)p;
-    }
-    const double w = rule.w[q] * area / (4.0 * kPiD);
-    g.qw[q * n + l] = w;
-    g.qw32[q * n + l] = (float)w;
-    if (g.pack32) {
-      float* pk = g.pack32 + (int64_t)l * 64;
-      for (int c = 0; c < 3; ++c) {
-        const double pt = rule.bary[q][0] * v[0][c] + rule.bary[q][1] * v[1][c] +
-                          rule.bary[q][2] * v[2][c];
-        const float hi = (float)pt;
-        pk[4 * q + c] = hi;
-        pk[28 + 4 * q + c] = (float)(pt - (double)hi);
-      }
-      pk[4 * q + 3] = (float)w;
-      pk[28 + 4 * q + 3] = 0.f;
-    }
+  for (int c = 0; c < 3; ++c) {
+    g.cx[c * n + l] = x[c];
+    g.cx32[c * n + l] = (float)x[c];
   }
   if (g.edge32) {
     // node-independent edge data of the FP32 self term, once per panel: the vertex offsets
     // from the centroid are formed in FP64, the rest in FP32 (the FP32 table needs no more)
-    double x[3];
-    for (int c = 0; c < 3; ++c) x[c] = (v[0][c] + v[1][c] + v[2][c]) / 3.0;
     float o[3][3];
     for (int e = 0; e < 3; ++e)
       for (int c = 0; c < 3; ++c) o[e][c] = (float)(v[e][c] - x[c]);
@@ -294,9 +314,7 @@ __global__ void self_term32_kernel(Geometry g, int N, const double* z, GL16 gl, 
 cudaError_t launch_geometry(bem_ctx* ctx, cudaStream_t s) {
   static const Rule7 rule = make_rule7();
   const int64_t n = (ctx->geo.n + 15) / 16 * 16;   // padding panels of the packed array too
-  // one thread per panel in 32-thread blocks: the FP64 work per panel is long and FP64
-  // issue is slow, so the panels are spread over as many SMs as possible
-  geometry_kernel<<<(unsigned)((n + 31) / 32), 32, 0, s>>>(ctx->geo, rule, ctx->d_status);
+  geometry_kernel<<<(unsigned)((n + 31) / 32), 32 * kGeoParts, 0, s>>>(ctx->geo, rule, ctx->d_status);
   ctx->launches++;
   if (ctx->geo.mom32) {
     static const GL16 gl = make_gl16();

@@ -88,21 +88,30 @@ __device__ __forceinline__ long long fixed55(double x, int e) {
 }
 
 // The digits of q = fixed55(x) for eight values, as rows of BF16: out[s] holds digit s of the
-// eight. neg: of -x.
+// eight. neg: of -x. With 128 added to every digit but the first they are the bytes of q, which
+// become numbers as the low mantissa byte of 2^23 (no conversions, which run at an eighth of the
+// rate).
 __device__ __forceinline__ void digits8(const long long (&q)[8], uint4 (&out)[kDigits], bool neg) {
-  long long r[8];
+  uint32_t lo[8], hi[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) r[j] = neg ? -q[j] : q[j];
+  for (int j = 0; j < 8; ++j) {
+    const long long r = (neg ? -q[j] : q[j]) + 0x0000808080808080ll;
+    lo[j] = (uint32_t)r;
+    hi[j] = (uint32_t)(r >> 32);
+  }
 #pragma unroll
-  for (int s = kDigits - 1; s >= 0; --s) {
+  for (int s = 0; s < kDigits; ++s) {
     uint32_t h[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const int d = s > 0 ? ((int)(r[j] + 128) & 255) - 128 : (int)r[j];
-      r[j] = (r[j] - d) >> 8;
-      h[j] = __float_as_uint((float)d) >> 16;   // |d| <= 128: exact
+      uint32_t m;   // 2^23 + 128 + digit
+      if (s == 0) m = 0x4B000000u + (uint32_t)(((int)hi[j] >> 16) + 128);
+      else if (s < 3) m = __byte_perm(hi[j], 0x4B000000u, 0x7440u | (2 - s));
+      else m = __byte_perm(lo[j], 0x4B000000u, 0x7440u | (6 - s));
+      h[j] = __float_as_uint(__uint_as_float(m) - 8388736.f);
     }
-    out[s] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+    out[s] = make_uint4(__byte_perm(h[0], h[1], 0x7632), __byte_perm(h[2], h[3], 0x7632),
+                        __byte_perm(h[4], h[5], 0x7632), __byte_perm(h[6], h[7], 0x7632));
   }
 }
 

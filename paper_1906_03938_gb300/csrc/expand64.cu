@@ -96,48 +96,6 @@ expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, i
 //   the seven weights w / r scaled together so that their sum fills 62 bits.
 // Measured: 5120 panels, 14 terms 34.3 -> 11.0 ms; 768 panels, 17 terms 730 -> 319 us; the residuals
 // and products keep their error against 64-bit references (7.6e-16, 9.5e-16).
-constexpr int kAngles = 1024;
-constexpr long long kOne = 1ll << 62;
-
-struct FixedPhase {
-  double inv_R;   // rho = r inv_R
-  long long K;    // turns per unit of rho, times 2^(62 - kb)
-  int kb;
-};
-
-struct Split {   // x = h 2^32 + l, both signed
-  int h, l;
-};
-__device__ __forceinline__ Split split(long long x) {
-  return Split{(int)((x + 0x80000000ll) >> 32), (int)x};
-}
-// a b 2^-64 to about a unit, plus add; |a|, |b| <= 2^62
-__device__ __forceinline__ long long mulh(Split a, Split b, long long add = 0) {
-  const long long m = (long long)a.h * b.l + ((long long)a.l * b.h + 0x80000000ll);
-  return (long long)a.h * b.h + add + (m >> 32);
-}
-// round(v 2^(62 - e)), 0 <= v < 2^e (or = 2^e)
-__device__ __forceinline__ long long fixed62(double v, int e) {
-  const unsigned long long bits = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
-  const int be = (int)(bits >> 52);
-  const long long m = (long long)((bits & 0xFFFFFFFFFFFFFull) | (be ? 0x10000000000000ull : 0ull));
-  const int sh = max(be, 1) - 1013 - e;
-  if (sh >= 0) return m << min(sh, 10);
-  return sh > -63 ? (m + (1ll << (-sh - 1))) >> -sh : 0;
-}
-// a 2^(e - 60), rounded to FP64
-__device__ __forceinline__ double from_fixed60(long long a, int e) {
-  if (a == 0) return 0.0;
-  const unsigned long long u = (unsigned long long)llabs(a);
-  const int lz = __clzll((long long)u);
-  const int be = 1023 + 3 - lz + e;
-  if (be < 1 || be > 2045) return ldexp((double)a, e - 60);
-  // 53 bits at the top, rounded half up; a carry runs into the exponent
-  const unsigned long long m = ((u << lz) >> 10) + 1;
-  return __longlong_as_double((long long)((((unsigned long long)(be - 1) << 52) + (m >> 1)) |
-                                          ((unsigned long long)a & 0x8000000000000000ull)));
-}
-
 // cos and sin of 2 pi q / kAngles as 62-bit fractions, split: (cos h, cos l, sin h, sin l).
 __global__ void expand_angles_kernel(int4* __restrict__ table) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -146,28 +104,6 @@ __global__ void expand_angles_kernel(int4* __restrict__ table) {
   sincospi(2.0 * q / kAngles, &sn, &cs);
   const Split c = split(llrint(ldexp(cs, 62))), s = split(llrint(ldexp(sn, 62)));
   table[q] = make_int4(c.h, c.l, s.h, s.l);
-}
-
-// cos and sin (62 fractional bits) of the angle phi 2^-64 turns.
-__device__ __forceinline__ void fixed_sincos(unsigned long long phi, const int4* table, long long& co,
-                                             long long& si) {
-  const unsigned q = (unsigned)((phi + (1ull << 53)) >> 54);   // (mod kAngles below)
-  const long long d = (long long)(phi - ((unsigned long long)q << 54));   // |d| <= 2^53
-  constexpr long long kTwoPi = 0x3243F6A8885A308Dll;    // 2 pi 2^59
-  constexpr long long kTwoThirds = 0x2AAAAAAAAAAAAAABll;   // 2 / 3 2^62
-  const long long th = mulh(split(d << 9), split(kTwoPi)) << 2;   // t 2^70
-  const Split t = split(th);
-  const long long u = mulh(t, t);                        // t^2 2^76
-  const int u47 = (int)(u >> 29);                        // t^2 2^47
-  const int f62 = (int)(((long long)u47 * u47) >> 32);   // t^4 2^62
-  // t^2 / 6 - t^4 / 120 in 2^-81
-  const long long v = (mulh(split(u), split(kTwoThirds)) - (((long long)f62 * 572662306) >> 22)) << 5;
-  const Split sn = split(th - (mulh(t, split(v)) >> 17));                       // sin t 2^70
-  const Split cm = split((u << 1) - (((long long)f62 * 357913941) >> 17));      // (1 - cos t) 2^78
-  const int4 e = table[q % kAngles];
-  const Split C{e.x, e.y}, S{e.z, e.w};
-  co = (((long long)e.x << 32) + e.y) - (((mulh(C, cm) >> 8) + mulh(S, sn)) >> 6);
-  si = (((long long)e.z << 32) + e.w) - (((mulh(S, cm) >> 8) - mulh(C, sn)) >> 6);
 }
 
 // Moments of the columns [l0, l0 + kc): G[f M + m][l - l0][i] (i fastest). One thread per row;
@@ -222,12 +158,8 @@ expand_moments_kernel(Geometry g, double2 c, FixedPhase fp, int M, int64_t l0, i
       for (int q = 0; q < 7; ++q) {
         const double dx = sq[cc][q][0] - xi, dy = sq[cc][q][1] - yi, dz = sq[cc][q][2] - zi;
         const double r2 = dx * dx + dy * dy + dz * dz;
-        // 1 / sqrt(r2) and sqrt(r2) by one third-order step from the FP32 root, y (1 + e / 2 +
-        // 3 e^2 / 8) with e = 1 - r2 y^2 of ~2^-22
-        const float rf = (float)r2;
-        const double y = rf > 1e-30f && rf < 1e30f ? (double)rsqrtf(rf) : rsqrt(r2);
-        const double t = r2 * y, er = fma(-t, y, 1.0), pe = fma(0.375, er, 0.5);
-        const double r = fma(t * er, pe, t), ri = fma(y * er, pe, y);
+        double r, ri;
+        root_and_inverse(r2, r, ri);
         srho[q][tid] = fixed62(r * fp.inv_R, 0);
         double w = sq[cc][q][3] * ri;
         if (c.y != 0.0) w *= exp(-c.y * r);
@@ -258,35 +190,10 @@ expand_moments_kernel(Geometry g, double2 c, FixedPhase fp, int M, int64_t l0, i
       }
 #pragma unroll 1
       for (int q = 0; q < 7; ++q) {
-        const long long rho = srho[q][tid];
-        long long co, si;
-        fixed_sincos((unsigned long long)mulh(split(rho), K) << (4 + fp.kb), table, co, si);
-        const Split sc = split(co), ss = split(si);
-        Split br[F], bi[F];
+        long long b[F];
 #pragma unroll
-        for (int f = 0; f < F; ++f) {
-          const Split b = split(__double_as_longlong(sbase[q][f][tid]));
-          const long long r0 = mulh(b, sc), i0 = mulh(b, ss);   // 2^-60: as T_0's terms
-          ar[f][0] += r0;
-          ai[f][0] += i0;
-          br[f] = split(r0 << 2);
-          bi[f] = split(i0 << 2);
-        }
-        const long long x = 2 * rho - kOne;
-        const Split sx = split(x);
-        long long t0 = kOne, t1 = x;
-#pragma unroll
-        for (int m = 1; m < MT; ++m) {
-          const Split t = split(t1);
-#pragma unroll
-          for (int f = 0; f < F; ++f) {
-            ar[f][m] = mulh(br[f], t, ar[f][m]);
-            ai[f][m] = mulh(bi[f], t, ai[f][m]);
-          }
-          const long long t2 = (mulh(sx, t) << 3) - t0;
-          t0 = t1;
-          t1 = t2;
-        }
+        for (int f = 0; f < F; ++f) b[f] = __double_as_longlong(sbase[q][f][tid]);
+        add_moments<MT, F>(ar, ai, b, srho[q][tid], K, fp.kb, table);
       }
     }
 #pragma unroll
@@ -549,6 +456,7 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   }
   p.c = make_double2(c_re, c_im);
   if (!(fabs(c_re) * p.R < 0x1p40)) return p;   // the phase's fixed-point range
+  p.phase = fixed_phase(c_re, p.R);
   if (p.M > 1 && (hasH || deriv)) p.M += 2;
   if (p.M == 1 && (hasH || deriv)) p.M = 3;   // factors 1, r, r^2
   if (p.M < 1 || p.M > kMaxTerms) return p;
@@ -608,7 +516,7 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
                                                 : moment_kernel<false, true>(p.M));
   int4* angles = reinterpret_cast<int4*>(work);
   expand_angles_kernel<<<kAngles / 128, 128, 0, s>>>(angles);
-  const FixedPhase fp = fixed_phase(p.c.x, p.R);
+  const FixedPhase fp = p.phase;
   ctx->launches += 2;
   const double2* Xd = reinterpret_cast<const double2*>(X);
   if (p.split) {
@@ -639,7 +547,7 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
     expand_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, p.splits, Yp);
     ctx->launches++;
   }
-  return near_active(ctx) ? near_expand64(ctx, p, X, ldx, ncols, Yp, s) : BEM_OK;
+  return near_active(ctx) ? near_expand64(ctx, p, angles, X, ldx, ncols, Yp, s) : BEM_OK;
 }
 
 }  // namespace

@@ -8,6 +8,12 @@ namespace bem {
 
 constexpr int kMaxTerms = 32;   // longest series the kernels are built for
 
+struct FixedPhase {
+  double inv_R;   // rho = r inv_R
+  long long K;    // turns per unit of rho, times 2^(62 - kb)
+  int kb;
+};
+
 struct ExpandPlan {
   bool use = false;        // the expansion applies and costs less than the direct form
   int M = 0;               // series terms
@@ -17,6 +23,7 @@ struct ExpandPlan {
   int splits = 1;          // shares of those columns in the products
   double R = 0.0;          // largest distance
   double2 c{};             // centre
+  FixedPhase phase{};
   bool split = false;      // products on the tensor core (split64.cu)
   SplitBatch batch;
   size_t coef_off = 0, mom_off = 0, y_off = 0, batch_off = 0, bytes = 0;
@@ -40,7 +47,7 @@ bem_status expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const 
 // Near pairs (near.cu): Y_s += C_s X for every slot, C_s the moments of the corrections
 // (A_near - A_7); its workspace.
 bool near_expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s);
-bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const double* X, int64_t ldx,
-                         int ncols, double2* Ys, cudaStream_t s);
+bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const int4* angles, const double* X,
+                         int64_t ldx, int ncols, double2* Ys, cudaStream_t s);
 
 }  // namespace bem

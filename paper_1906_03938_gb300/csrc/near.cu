@@ -405,13 +405,19 @@ near_apply64_kernel(Geometry g, const int32_t* __restrict__ ptr, const int32_t* 
 // Moments of the corrections (A_near - A_7) in the expansion over wavenumbers (expand64.cu):
 // C[f M + m][e] for pair e, one thread per pair; its row by bisection of the row pointers. The
 // 71 points' roots and sines serve every wavenumber (near_apply64_kernel and
-// near_percol64_kernel evaluate them for each). FP64-bound: 71 (60 + 3 M) operations a pair.
-// Residuals of 8 vectors on 5120 panels: 23.0 -> 3.1 ms with near_slots64_kernel.
+// near_percol64_kernel evaluate them for each). In fixed point as expand_moments_kernel; the
+// scale, 2^7 above the largest weight so far, moves up where a larger one comes (the sums
+// shifted down with it). Residuals of 8 vectors on 5120 panels: 23.0 -> 2.6 ms with
+// near_slots64_kernel in FP64 (71 (60 + 3 M) operations a pair), now 1.3 ms.
 template <int MT, bool kG, bool kH>
 __global__ void __launch_bounds__(128)
 near_moments64_kernel(Geometry g, const int32_t* __restrict__ ptr,
                       const int32_t* __restrict__ cols, int64_t nnz, GL8 gl, double2 c,
-                      double two_over_R, int M, double2* __restrict__ C) {
+                      FixedPhase fp, const int4* __restrict__ angles, int M,
+                      double2* __restrict__ C) {
+  __shared__ int4 table[kAngles];
+  for (int t = threadIdx.x; t < kAngles; t += 128) table[t] = angles[t];
+  __syncthreads();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= nnz) return;
   const int64_t n = g.n;
@@ -428,11 +434,16 @@ near_moments64_kernel(Geometry g, const int32_t* __restrict__ ptr,
   NearFrame F;
   near_frame(g, l, x, F);
   constexpr int NF = (kG ? 1 : 0) + (kH ? 1 : 0);
-  double ar[NF][MT], ai[NF][MT];
+  long long ar[NF][MT], ai[NF][MT];
+  int scale[NF];   // exponents of the families' scales
 #pragma unroll
-  for (int f = 0; f < NF; ++f)
+  for (int f = 0; f < NF; ++f) {
+    scale[f] = -2000;
 #pragma unroll
-    for (int m = 0; m < MT; ++m) ar[f][m] = ai[f][m] = 0.0;
+    for (int m = 0; m < MT; ++m) ar[f][m] = ai[f][m] = 0;
+  }
+  bool finite = true;
+  const Split K = split(fp.K);
 #pragma unroll 1
   for (int t = 0; t < 71; ++t) {
     double w, y[3];
@@ -445,13 +456,42 @@ near_moments64_kernel(Geometry g, const int32_t* __restrict__ ptr,
       w = -g.qw[q * n + l];
       for (int d = 0; d < 3; ++d) y[d] = g.qp[(7 * d + q) * n + l];
     }
-    expand_point<MT, kG, kH>(ar, ai, w, y[0] - x[0], y[1] - x[1], y[2] - x[2], nrm, c, two_over_R);
+    const double dx = y[0] - x[0], dy = y[1] - x[1], dz = y[2] - x[2];
+    double r, ri;
+    root_and_inverse(dx * dx + dy * dy + dz * dz, r, ri);
+    w *= ri;
+    if (c.y != 0.0) w *= exp(-c.y * r);
+    double base[NF];
+    if (kG) base[0] = w;
+    if (kH) base[NF - 1] = w * ri * ri * (dx * nrm[0] + dy * nrm[1] + dz * nrm[2]);
+    long long b[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const int be = (__double2hiint(base[f]) >> 20) & 2047;
+      finite = finite && be < 2047;
+      const int up = be == 0 ? 0 : be - 1022 + 7 - scale[f];
+      if (up > 0) {
+        const int sh = min(up, 63);
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+          ar[f][m] >>= sh;
+          ai[f][m] >>= sh;
+        }
+        scale[f] += up;
+      }
+      b[f] = fixed62(base[f], scale[f]);
+      if (__double2hiint(base[f]) < 0) b[f] = -b[f];
+    }
+    add_moments<MT, NF>(ar, ai, b, fixed62(r * fp.inv_R, 0), K, fp.kb, table);
   }
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
     for (int m = 0; m < MT; ++m)
-      if (m < M) C[(int64_t)(f * M + m) * nnz + e] = make_double2(ar[f][m], ai[f][m]);
+      if (m < M)
+        C[(int64_t)(f * M + m) * nnz + e] =
+            finite ? make_double2(from_fixed60(ar[f][m], scale[f]), from_fixed60(ai[f][m], scale[f]))
+                   : make_double2(NAN, NAN);
 }
 
 // Y_s += C_s X: one warp per (row i, slot s), lanes over the columns; Xt is X row-major.
@@ -1121,8 +1161,8 @@ bool near_expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_
   return ensure_near_work(ctx, need) == BEM_OK;
 }
 
-bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const double* X, int64_t ldx,
-                         int ncols, double2* Ys, cudaStream_t s) {
+bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const int4* angles, const double* X,
+                         int64_t ldx, int ncols, double2* Ys, cudaStream_t s) {
   const int64_t n = ctx->geo.n, nnz = ctx->near_nnz;
   if (nnz == 0) return BEM_OK;
   double2* Xt = reinterpret_cast<double2*>(ctx->d_near_work);
@@ -1136,7 +1176,7 @@ bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const double* X, int
                           : (p.first == 0 ? near_moments64_kernel<MT, true, false>
                                           : near_moments64_kernel<MT, false, true>);
     k<<<blocks, 128, 0, s>>>(ctx->geo, ctx->d_near_ptr, ctx->d_near_cols, nnz, gl8(), p.c,
-                             2.0 / p.R, p.M, C);
+                             p.phase, angles, p.M, C);
   };
   if (p.M <= 1) go(std::integral_constant<int, 1>());
   else if (p.M <= 12) go(std::integral_constant<int, 12>());

@@ -41,17 +41,24 @@ constexpr int64_t kSplitWork = (int64_t)1 << 25;
 constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
 
 // a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
-// wavenumber k_j, times the operator's coefficient of the family. One block per (j, f): its
-// threads take one Chebyshev point each, then one coefficient each (a thread per coefficient
-// evaluated all points again: 196 us against 56 at 32 wavenumbers).
-__global__ void __launch_bounds__(kCoefPoints)
+// wavenumber k_j, times the operator's coefficient of the family. One block per (j, f): a thread
+// per Chebyshev point for the function, a thread per angle for the cosines cos(pi t / 128) that
+// the sums take, then a warp per coefficient. (A thread per coefficient with the cosines of all
+// its points took 196 us, the points shared 56 us at 32 wavenumbers; now 8 us.)
+constexpr int kCoefThreads = 256;
+
+__global__ void __launch_bounds__(kCoefThreads)
 expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, int M,
                    int first_fam, bool deriv, OpCoef op, double2* __restrict__ a) {
+  static_assert(kCoefThreads == 4 * kCoefPoints, "an angle a thread");
   __shared__ double2 fv[kCoefPoints];
+  __shared__ double cosine[kCoefThreads];
   const int j = blockIdx.x, f = first_fam + blockIdx.y, q = threadIdx.x;
   const double2 kj = k[j];
-  {
-    const double r = 0.5 * R * (cospi((q + 0.5) / kCoefPoints) + 1.0);
+  cosine[q] = cospi(q / (2.0 * kCoefPoints));
+  __syncthreads();
+  if (q < kCoefPoints) {
+    const double r = 0.5 * R * (cosine[2 * q + 1] + 1.0);
     const double dr = kj.x - c.x, di = kj.y - c.y;
     double sn, cs;
     sincos(dr * r, &sn, &cs);
@@ -68,18 +75,26 @@ expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, i
     fv[q] = make_double2(e * (cs * gr - sn * gi), e * (cs * gi + sn * gr));
   }
   __syncthreads();
-  if (q >= M) return;
-  const int m = q;
-  double2 s = make_double2(0.0, 0.0);
-  for (int p = 0; p < kCoefPoints; ++p) {
-    const double w = cospi(m * ((p + 0.5) / kCoefPoints));
-    s.x = fma(w, fv[p].x, s.x);
-    s.y = fma(w, fv[p].y, s.y);
+  const int lane = q % 32;
+  for (int m = q / 32; m < M; m += kCoefThreads / 32) {
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int p = lane; p < kCoefPoints; p += 32) {
+      const double w = cosine[m * (2 * p + 1) % kCoefThreads];   // period 2 pi: kCoefThreads angles
+      s.x = fma(w, fv[p].x, s.x);
+      s.y = fma(w, fv[p].y, s.y);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    }
+    const double sc = (m == 0 ? 1.0 : 2.0) / kCoefPoints;
+    const double or_ = f == 0 ? op.cgr : op.chr, oi = f == 0 ? op.cgi : op.chi;
+    if (lane == 0)
+      a[((int64_t)blockIdx.y * nk + j) * M + m] =
+          make_double2(sc * (s.x * or_ - s.y * oi), sc * (s.x * oi + s.y * or_));
   }
-  const double sc = (m == 0 ? 1.0 : 2.0) / kCoefPoints;
-  const double or_ = f == 0 ? op.cgr : op.chr, oi = f == 0 ? op.cgi : op.chi;
-  a[((int64_t)blockIdx.y * nk + j) * M + m] =
-      make_double2(sc * (s.x * or_ - s.y * oi), sc * (s.x * oi + s.y * or_));
 }
 
 // ---- the moments ----
@@ -509,7 +524,7 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
   double2* a = reinterpret_cast<double2*>(work + p.coef_off);
   double2* G = reinterpret_cast<double2*>(work + p.mom_off);
   double2* Yp = reinterpret_cast<double2*>(work + p.y_off);
-  expand_coef_kernel<<<dim3((unsigned)nk, (unsigned)p.fams), kCoefPoints, 0, s>>>(
+  expand_coef_kernel<<<dim3((unsigned)nk, (unsigned)p.fams), kCoefThreads, 0, s>>>(
       reinterpret_cast<const double2*>(k_dev), nk, p.c, p.R, p.M, p.first, deriv, ctx->op, a);
   MomentKernel mk = p.fams == 2 ? moment_kernel<true, true>(p.M)
                                 : (p.first == 0 ? moment_kernel<true, false>(p.M)

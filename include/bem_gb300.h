@@ -216,10 +216,10 @@ bem_status bem_residual(bem_ctx* ctx, int m, const double* lam_host, const doubl
  *   arith 0: FP64, as bem_residual.
  *   arith 1: double-FP32 ("float-float": every quantity as a pair of FP32 numbers, about
  *            48 significant bits) for the off-diagonal single-layer entries, each entry to
- *            a relative error of about 1e-13; the self and near-field terms stay FP64. On
- *            this GPU, whose FP64 pipe is ~65x slower than its FP32 pipe, it is over ten
- *            times faster than arith 0. The general operator (bem_set_operator with
- *            c_H != 0) always uses the FP64 kernels.
+ *            a relative error of about 1e-13; the self and near-field terms stay FP64. For a
+ *            few columns faster than arith 0; where the FP64 evaluation shared by all columns
+ *            is the faster one (many columns, near field), that is taken. The general operator
+ *            (bem_set_operator with c_H != 0) always uses the FP64 kernels.
  *   Rd_dev     optional n x m complex output A'(lam_c) x_c (derivative in k), may be NULL
  * Other arguments as bem_residual. Synchronises the stream.
  */

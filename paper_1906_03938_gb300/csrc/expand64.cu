@@ -478,21 +478,24 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   p.first = hasG ? 0 : 1;
   p.fams = (hasG ? 1 : 0) + (hasH ? 1 : 0);
   p.S = p.fams * p.M;
-  // FP64 operations per entry of the two forms; the smaller wins. Projection at n = 768,
-  // nu = 64: direct 5.56 ms at N = 5, expanded 5.41 ms at N = 6 and 5.48 ms at N = 16; at
-  // nu = 128: direct 10.2 ms at N = 6, expanded 8.4 ms at N = 7, 9.3 ms at N = 16. Residuals on
-  // 1280 panels: 5.9 ms for 2 to 8 columns (one product tile).
   const int tn = ncols <= 8 ? 8 : 32;
   const double padded = (double)((ncols + tn - 1) / tn * tn);
-  const double expand = 7.0 * (60.0 + (1.0 + 2.0 * p.fams) * p.M) + 3.0 * p.S * padded;
-  const double direct = nodes ? nk * (7.0 * 77.0 + 4.0 * ncols) : ncols * (7.0 * 77.0 + 4.0);
+  p.split = n * n * p.S * (int64_t)(padded - 4.0) >= kSplitWork;
+  // Time per entry of the two forms, in FP64 operations (5.3e11 a second); the smaller wins. The
+  // evaluation's integer instructions count a 28th, as measured (5120 panels, 14 terms: 222
+  // together), the split products 7 a moment and 4 per 32 columns. The direct forms take ~1950 a
+  // column for residuals (4800 panels, one vector: 85 ms, expanded 12.4 ms) and 540 + 4 nu a node
+  // or more for projections (768 panels, 64 columns: 1000).
+  const double eval = 7.0 * (15.0 + (p.c.y != 0.0 ? 22.0 : 0.0) + (110.0 + (12.0 + 14.0 * p.fams) * p.M) / 28.0);
+  p.cost = eval + (p.split ? p.S * (7.0 + 4.0 * ((ncols + 31) / 32)) : 3.0 * p.S * padded);
+  const double expand = p.cost;
+  const double direct = nodes ? nk * (7.0 * 77.0 + 4.0 * ncols) : ncols * 1950.0;
   if (!(expand < direct)) return p;
   // workspace: coefficients, moments of kc columns, slot products (per k split)
   p.kc = (int)std::min<int64_t>(n, std::max<int64_t>(32, (int64_t)(kMomentBytes / ((size_t)p.S * n * 16))));
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const int64_t tiles = (n + kTM - 1) / kTM * ((ncols + tn - 1) / tn) * p.S;
-  p.split = n * n * p.S * (int64_t)(padded - 4.0) >= kSplitWork;
   if (p.split) {
     p.kc = (int)std::min<int64_t>(n, std::max<int64_t>(64, (int64_t)(kMomentBytes / ((size_t)p.S * n * 16)) / 16 * 16));
     p.batch = split64_batch_plan(n, p.kc, p.S, ncols);

@@ -22,6 +22,7 @@ struct ExpandPlan {
   int kc = 0;              // columns evaluated at a time
   int splits = 1;          // shares of those columns in the products
   double R = 0.0;          // largest distance
+  double cost = 0.0;       // time per entry, in FP64 operations
   double2 c{};             // centre
   FixedPhase phase{};
   bool split = false;      // products on the tensor core (split64.cu)

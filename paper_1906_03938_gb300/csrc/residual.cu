@@ -159,6 +159,19 @@ using namespace bem;
 
 namespace {
 
+// Whether the FP64 expansion is faster than the double-FP32 kernel (its time depends on the
+// columns, the expansion's hardly does), in us from 300 to 4800 panels:
+//   4800 panels: 16.9 ms for any number of columns against 7.8 ms at 4, 22.8 ms at 12; 768 panels
+//   0.76 ms against 0.61 at 8, 0.79 at 12; the near pairs 15 ns once against 23 ns a column (4800
+//   panels with near field, 12 columns: 19.4 against 67.8 ms).
+bool expand_beats_ff(const bem_ctx* ctx, const ExpandPlan& ex, int m, bool deriv) {
+  const double n2 = (double)ctx->geo.n * (double)ctx->geo.n;
+  const double pairs = near_active(ctx) ? (double)ctx->near_nnz : 0.0;
+  const double expand = 300.0 + n2 * ex.cost / 5.3e5 + pairs * 0.015;
+  const double ff = std::max(450.0, 200.0 + n2 * m * 0.082e-3) + pairs * m * 0.023;
+  return (deriv ? 2.0 : 1.0) * expand < 0.9 * ff;
+}
+
 bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const double* X_dev,
                          int64_t ldx, double* R_dev, double* Rd_dev, double* relres_host,
                          int arith, void* stream, const char* name) {
@@ -179,11 +192,12 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   const size_t small = (size_t)4 * m * sizeof(double);
   st = ensure_small(ctx, small);
   if (st != BEM_OK) return st;
-  // FP64: one evaluation expanded about the middle of the given values for all columns, where
-  // that costs less than one per column and its workspace can be had
+  // One FP64 evaluation expanded about the middle of the given values for all columns, where that
+  // costs less than one per column (in FP64, or in double-FP32 if asked for: single layer only)
+  // and its workspace can be had
   const size_t r_bytes = R_dev ? 0 : ((size_t)2 * n * m * sizeof(double) + 255) / 256 * 256;
   ExpandPlan ex;
-  if (arith == 0) {
+  {
     double lo[2] = {lam_host[0], lam_host[1]}, hi[2] = {lam_host[0], lam_host[1]};
     for (int c = 0; c < 2 * m; ++c) {
       lo[c % 2] = std::min(lo[c % 2], lam_host[c]);
@@ -194,7 +208,8 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
     for (int c = 0; c < m; ++c)
       dmax = std::max(dmax, hypot(lam_host[2 * c] - cr, lam_host[2 * c + 1] - ci));
     ex = expand_plan(ctx, m, cr, ci, dmax, m, false, Rd_dev != nullptr);
-    ex.use = expand_ready(ctx, ex, r_bytes, m, s);
+    if (arith == 1 && op_single(ctx->op) && !expand_beats_ff(ctx, ex, m, Rd_dev != nullptr)) ex.use = false;
+    ex.use = ex.use && expand_ready(ctx, ex, r_bytes, m, s);
   }
   if (!ex.use) {
     st = ensure_scratch(ctx, r_bytes);
@@ -207,7 +222,7 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
                                        cudaMemcpyHostToDevice, s), name);
   if (st != BEM_OK) return st;
   cudaError_t e = cudaSuccess;
-  if (arith == 1) {
+  if (arith == 1 && !ex.use) {
     e = launch_apply_ff(ctx, m, dlam, X_dev, ldx, R, Rd_dev, s);
   } else if (ex.use) {
     void* w = reinterpret_cast<char*>(ctx->d_scratch) + r_bytes;

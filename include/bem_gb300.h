@@ -193,7 +193,7 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
  * Cholesky factor and triangular inverse (and the smaller Gram matrices) in FP32 and applies
  * the inverse to V in FP64. From n nu^2 = 2^23 the FP64 products are exact sums of BF16 digit
  * products; their workspace (10 bytes per byte of V at nu = 32, 5 at 256; at most 8 GiB,
- * else the FP64 pipe) stays with the context. Fails with BEM_EKERNEL if a Gram matrix is not
+ * else the FP64 pipe) is part of the workspace kept. Fails with BEM_EKERNEL if a Gram matrix is not
  * numerically positive definite (rank-deficient V). Synchronises the stream.
  */
 bem_status bem_cholqr2(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int nu,

@@ -1399,7 +1399,7 @@ size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu) {
 // pass then falls back to the classic factorisation by itself. With R: two classic passes
 // and R = R2 R1.
 bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int nu,
-                        double* R_dev, void* work, cudaStream_t s, uint64_t refresh_seed) {
+                        double* R_dev, void* work, cudaStream_t s, uint64_t refresh_seed, void* split_mem) {
   const CqLayout L = cq_layout(ctx, n, nu);
   const CqWork w = cq_work(work, nu, L);
   bem_status st = BEM_OK;
@@ -1411,7 +1411,7 @@ bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int
                      right_multiply_df_smem(nu))) != BEM_OK)
     return st;
   Split64 sp;
-  split64_plan(ctx, V_dev, ldv, n, nu, sp, s);
+  split64_plan(ctx, ldv, n, nu, split_mem, sp, s);
   if (R_dev) {
     if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R1, refresh_seed, s)) != BEM_OK) return st;
     if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R2, 0, s)) != BEM_OK) return st;
@@ -1479,9 +1479,18 @@ extern "C" bem_status bem_cholqr2(bem_ctx* ctx, double* V_dev, int64_t n, int64_
     return fail(ctx, BEM_EINVAL, "bem_cholqr2: need V, 1 <= nu <= min(n, 256), ldv >= n");
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  bem_status st = ensure_small(ctx, cholqr2_work_bytes(ctx, n, nu));
+  // one workspace for the factors and the split products' planes, the latter given up if it
+  // cannot be had
+  const size_t work = (cholqr2_work_bytes(ctx, n, nu) + 1023) / 1024 * 1024, split = split64_bytes(ctx, n, nu);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (split > 0 && work + split > ctx->small_bytes) {
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    else if (cap == cudaStreamCaptureStatusNone) ensure_small(ctx, work + split);
+  }
+  bem_status st = ensure_small(ctx, work);
   if (st != BEM_OK) return st;
-  st = cholqr2_impl(ctx, V_dev, n, ldv, nu, R_dev, ctx->d_small, s, 0);
+  void* planes = split > 0 && work + split <= ctx->small_bytes ? reinterpret_cast<char*>(ctx->d_small) + work : nullptr;
+  st = cholqr2_impl(ctx, V_dev, n, ldv, nu, R_dev, ctx->d_small, s, 0, planes);
   if (st != BEM_OK) return st;
   if (ctx->async) return cuda_check(ctx, cudaGetLastError(), "bem_cholqr2");
   return take_status(ctx, s, "bem_cholqr2");

@@ -242,10 +242,10 @@ cudaError_t launch_xhy_fp64(bem_ctx* ctx, const double* X, int64_t ldx, int p, c
 // CholeskyQR2 with caller-provided work space (asynchronous; status word on failure).
 // refresh_seed != 0: columns whose first-pass pivot collapses (rank deficiency) are
 // replaced by pseudo-random columns before the second pass instead of failing; R is then
-// not a factor of the input.
+// not a factor of the input. split_mem: split64_bytes of workspace (null: the context's own).
 size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu);
 bem_status cholqr2_impl(bem_ctx* ctx, double* V, int64_t n, int64_t ldv, int nu, double* R,
-                        void* work, cudaStream_t s, uint64_t refresh_seed);
+                        void* work, cudaStream_t s, uint64_t refresh_seed, void* split_mem = nullptr);
 // Near field (near.cu). near_active: a mode is set and the pair list is current (build it
 // with ensure_near first).
 bem_status ensure_near(bem_ctx* ctx, cudaStream_t s);

@@ -635,10 +635,37 @@ int split64_parts(const bem_ctx* ctx, int64_t n, int nu) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((n + 15) / 16 / kFlush, std::max(1, sms) / tiles));
 }
 
-void split64_plan(bem_ctx* ctx, const double* V, int64_t ldv, int64_t n, int nu, Split64& sp,
+namespace {
+
+struct SplitSizes {
+  size_t a, b, total;   // the operands' planes, all with the scales
+};
+
+// The split products' workspace for n x nu (total 0: the FP64 kernels).
+SplitSizes split_sizes(const bem_ctx* ctx, int64_t n, int nu) {
+  SplitSizes z{};
+  if (n * (int64_t)nu * nu < kMinWork) return z;
+  const size_t kbn = (size_t)(n + 15) / 16, kbu = (size_t)(nu + 15) / 16;
+  const size_t mtu = (nu + kTileM - 1) / kTileM, ntu = (nu + kTileN - 1) / kTileN;
+  const size_t mtn = (size_t)(n + kTileM - 1) / kTileM;
+  if ((int64_t)kbn / split64_parts(ctx, n, nu) / kFlush > 2000) return z;   // the 64-bit sums' range
+  auto up = [](size_t b) { return (b + 1023) / 1024 * 1024; };
+  z.a = up(std::max(kbn * mtu, kbu * mtn) * kABytes);
+  z.b = up(std::max(kbn * ntu, kbu * ntu) * kBBytes);
+  const size_t total = z.a + z.b + up((size_t)(2 * nu + n) * sizeof(int));
+  if (total <= kMaxSplitBytes) z.total = total;
+  return z;
+}
+
+}  // namespace
+
+size_t split64_bytes(const bem_ctx* ctx, int64_t n, int nu) { return split_sizes(ctx, n, nu).total; }
+
+void split64_plan(bem_ctx* ctx, int64_t ldv, int64_t n, int nu, void* mem, Split64& sp,
                   cudaStream_t s) {
   sp = Split64();
-  if (n * (int64_t)nu * nu < kMinWork) return;
+  const SplitSizes z = split_sizes(ctx, n, nu);
+  if (z.total == 0) return;
   sp.n = n;
   sp.ldv = ldv;
   sp.nu = nu;
@@ -648,14 +675,7 @@ void split64_plan(bem_ctx* ctx, const double* V, int64_t ldv, int64_t n, int nu,
   sp.ntu = (nu + kTileN - 1) / kTileN;
   sp.mtn = (n + kTileM - 1) / kTileM;
   sp.parts = split64_parts(ctx, n, nu);
-  if (sp.kbn / sp.parts / kFlush > 2000) return;   // the 64-bit sums' range
-  auto up = [](size_t b) { return (b + 1023) / 1024 * 1024; };
-  const size_t a_bytes = up(std::max((size_t)sp.kbn * sp.mtu, (size_t)sp.kbu * (size_t)sp.mtn) * kABytes);
-  const size_t b_bytes = up(std::max((size_t)sp.kbn * sp.ntu, (size_t)sp.kbu * sp.ntu) * kBBytes);
-  const size_t e_bytes = up((size_t)(2 * nu + n) * sizeof(int));
-  const size_t need = a_bytes + b_bytes + e_bytes;
-  if (need > kMaxSplitBytes) return;
-  if (need > ctx->split_bytes) {
+  if (!mem && z.total > ctx->split_bytes) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
       cudaGetLastError();
@@ -664,16 +684,16 @@ void split64_plan(bem_ctx* ctx, const double* V, int64_t ldv, int64_t n, int nu,
     cudaFree(ctx->d_split);
     ctx->d_split = nullptr;
     ctx->split_bytes = 0;
-    if (cudaMalloc(&ctx->d_split, need) != cudaSuccess) {
+    if (cudaMalloc(&ctx->d_split, z.total) != cudaSuccess) {
       cudaGetLastError();
       return;
     }
-    ctx->split_bytes = need;
+    ctx->split_bytes = z.total;
   }
-  unsigned char* base = static_cast<unsigned char*>(ctx->d_split);
+  unsigned char* base = static_cast<unsigned char*>(mem ? mem : ctx->d_split);
   sp.a = base;
-  sp.b = base + a_bytes;
-  sp.hcol = reinterpret_cast<unsigned*>(base + a_bytes + b_bytes);
+  sp.b = base + z.a;
+  sp.hcol = reinterpret_cast<unsigned*>(base + z.a + z.b);
   sp.ez = reinterpret_cast<int*>(sp.hcol + nu);
   sp.erow = sp.ez + nu;
   sp.use = set_gemm_smem(ctx) == BEM_OK;

@@ -22,7 +22,7 @@
 //
 // Measured at 98304 x 256, a Gram matrix or a product: 1.03 ms (0.62 ms of it MMA cycles, the
 // rest waits for the accumulators' reads) and 0.4 ms for scales and digits, against 24 ms on the
-// FP64 pipe; a whole CholeskyQR2 101 -> 7.1 ms with ||Q^H Q - I|| 7.4e-16 -> 6.5e-16. One
+// FP64 pipe; a whole CholeskyQR2 101 -> 6.4 ms with ||Q^H Q - I|| 7.4e-16 -> 6.5e-16. One
 // MMA (N = 64) per pair took 2.3 ms; eight 7-bit digits with 36 pairs left 1.5e-15.
 #include <cuda_bf16.h>
 #include <limits.h>

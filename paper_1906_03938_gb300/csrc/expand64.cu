@@ -37,7 +37,7 @@ constexpr size_t kMomentBytes = (size_t)1 << 30;   // moments held at a time
 // moment and three more launches against 5.6 ps a moment and column). Split against FP64, in us:
 // 300 panels, 8 residuals 505 / 457, 588 panels, 2 residuals 978 / 955 below it; projections of
 // 300 panels, 10 columns 751 / 958, 588 x 60 1687 / 3695, 1728 panels, 2 residuals 5247 / 5518 above.
-constexpr int64_t kSplitWork = (int64_t)1 << 25;
+constexpr double kSplitWork = 0x1p25;
 constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
 
 // a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
@@ -461,7 +461,7 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   const bool hasG = op.cgr != 0.0 || op.cgi != 0.0, hasH = op.chr != 0.0 || op.chi != 0.0;
   const int64_t n = ctx->geo.n;
   p.R = mesh_reach(ctx);
-  if (!(p.R > 0.0) || !isfinite(p.R)) return p;
+  if (!(p.R > 0.0) || !isfinite(p.R) || !isfinite(1.0 / p.R)) return p;
   p.M = series_terms(dmax, p.R);
   // about a real centre no exponential is evaluated: for values near the axis, at most a term more
   if (c_im != 0.0 && series_terms(dmax + fabs(c_im), p.R) <= p.M + 1) {
@@ -480,7 +480,7 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   p.S = p.fams * p.M;
   const int tn = ncols <= 8 ? 8 : 32;
   const double padded = (double)((ncols + tn - 1) / tn * tn);
-  p.split = n * n * p.S * (int64_t)(padded - 4.0) >= kSplitWork;
+  p.split = (double)n * (double)n * p.S * (padded - 4.0) >= kSplitWork;
   // Time per entry of the two forms, in FP64 operations (5.3e11 a second); the smaller wins. The
   // evaluation's integer instructions count a 28th, as measured (5120 panels, 14 terms: 222
   // together), the split products 7 a moment and 4 per 32 columns. The direct forms take ~1950 a

@@ -131,49 +131,43 @@ __global__ void __launch_bounds__(1024) gauss_jordan_kernel(double2* M, double2*
   }
 }
 
-constexpr int kZT = 32;
-// C = A B (complex FP64): A m x k (lda), B k x n (ldb), C m x n (ldc); 32 x 32 tiles,
-// fixed-order sums.
+constexpr int kZT = 16;   // output tile, one output a thread
+constexpr int kZK = 32;   // k staged at a time
+// C = A B (complex FP64): A m x k (lda), B k x n (ldb), C m x n (ldc); fixed-order sums.
 // With gridDim.z > 1 block z sums the k-range [z kc, (z + 1) kc) and writes its partial
 // product at C + z * ldc * n (the caller sums the partials in z order).
-__global__ void __launch_bounds__(256)
+// An SM's FP64 pipe takes 8.5 us for a tile and kZK; the reduced problem's products are a few
+// tiles (24 x 48), so the tiles are small and the k-ranges short (32 x 32 tiles, 128 or more of k:
+// 95 us a product, now ZGM us).
+__global__ void __launch_bounds__(kZT * kZT)
 zgemm_kernel(int m, int n, int k, const double2* __restrict__ A, int64_t lda,
              const double2* __restrict__ B, int64_t ldb, double2* __restrict__ C, int64_t ldc,
              int kc) {
-  __shared__ double2 sA[kZT][kZT + 1];
-  __shared__ double2 sB[kZT][kZT + 1];
+  __shared__ double2 sA[kZT][kZK + 1];
+  __shared__ double2 sB[kZK][kZT + 1];
   const int i0 = blockIdx.x * kZT, j0 = blockIdx.y * kZT;
-  const int ti = threadIdx.x % kZT, tj0 = threadIdx.x / kZT;   // rows ti, columns tj0 + 8 q
-  double2 acc[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) acc[q] = make_double2(0.0, 0.0);
+  const int ti = threadIdx.x % kZT, tj = threadIdx.x / kZT;
+  double2 acc = make_double2(0.0, 0.0);
   const int kb = blockIdx.z * kc, ke = min(k, kb + kc);
   C += (int64_t)blockIdx.z * ldc * n;
-  for (int k0 = kb; k0 < ke; k0 += kZT) {
+  for (int k0 = kb; k0 < ke; k0 += kZK) {
     __syncthreads();
-    for (int t = threadIdx.x; t < kZT * kZT; t += 256) {
+    for (int t = threadIdx.x; t < kZT * kZK; t += kZT * kZT) {
       const int r = t % kZT, c = t / kZT;
       sA[r][c] = (i0 + r < m && k0 + c < ke) ? A[(int64_t)(k0 + c) * lda + i0 + r] : make_double2(0.0, 0.0);
-      sB[r][c] = (k0 + r < ke && j0 + c < n) ? B[(int64_t)(j0 + c) * ldb + k0 + r] : make_double2(0.0, 0.0);
+      const int rb = t % kZK, cb = t / kZK;
+      sB[rb][cb] = (k0 + rb < ke && j0 + cb < n) ? B[(int64_t)(j0 + cb) * ldb + k0 + rb] : make_double2(0.0, 0.0);
     }
     __syncthreads();
+    const int kn = min(kZK, ke - k0);
 #pragma unroll 8
-    for (int kk = 0; kk < kZT; ++kk) {
-      const double2 a = sA[ti][kk];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double2 b = sB[kk][tj0 + 8 * q];
-        acc[q].x = fma(a.x, b.x, fma(-a.y, b.y, acc[q].x));
-        acc[q].y = fma(a.x, b.y, fma(a.y, b.x, acc[q].y));
-      }
+    for (int kk = 0; kk < kn; ++kk) {
+      const double2 a = sA[ti][kk], b = sB[kk][tj];
+      acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+      acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
     }
   }
-  if (i0 + ti < m)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int j = j0 + tj0 + 8 * q;
-      if (j < n) C[(int64_t)j * ldc + i0 + ti] = acc[q];
-    }
+  if (i0 + ti < m && j0 + tj < n) C[(int64_t)(j0 + tj) * ldc + i0 + ti] = acc;
 }
 
 // HW_j = (W_j - U) / (z_j - s): W, HW (N nu) x p with ld N nu, U nu x p.
@@ -505,10 +499,10 @@ cudaError_t launch_zgemm(bem_ctx* ctx, int m, int n, int k, const double* A, int
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const int tiles = (int)(grid.x * grid.y);
   int parts = 1;
-  if (tiles < 2 * sms && k >= 8 * kZT)
-    parts = std::min((2 * sms + tiles - 1) / tiles, k / (4 * kZT));
+  if (tiles < sms && k >= 4 * kZK)
+    parts = std::min((sms + tiles - 1) / tiles, k / kZK);
   if (parts > 1) {
-    const int kc = ((k + parts - 1) / parts + kZT - 1) / kZT * kZT;
+    const int kc = ((k + parts - 1) / parts + kZK - 1) / kZK * kZK;
     parts = (k + kc - 1) / kc;
     const size_t bytes = (size_t)parts * m * n * sizeof(double2);
     if (bytes > ctx->zgemm_bytes) {
@@ -520,7 +514,7 @@ cudaError_t launch_zgemm(bem_ctx* ctx, int m, int n, int k, const double* A, int
       ctx->zgemm_bytes = bytes;
     }
     grid.z = (unsigned)parts;
-    zgemm_kernel<<<grid, 256, 0, s>>>(m, n, k, reinterpret_cast<const double2*>(A), lda,
+    zgemm_kernel<<<grid, kZT * kZT, 0, s>>>(m, n, k, reinterpret_cast<const double2*>(A), lda,
                                       reinterpret_cast<const double2*>(B), ldb,
                                       reinterpret_cast<double2*>(ctx->d_zgemm), m, kc);
     zsum_parts_kernel<<<(unsigned)(((int64_t)m * n + 255) / 256), 256, 0, s>>>(
@@ -529,7 +523,7 @@ cudaError_t launch_zgemm(bem_ctx* ctx, int m, int n, int k, const double* A, int
     ctx->launches += 2;
     return cudaGetLastError();
   }
-  zgemm_kernel<<<grid, 256, 0, s>>>(m, n, k, reinterpret_cast<const double2*>(A), lda,
+  zgemm_kernel<<<grid, kZT * kZT, 0, s>>>(m, n, k, reinterpret_cast<const double2*>(A), lda,
                                     reinterpret_cast<const double2*>(B), ldb,
                                     reinterpret_cast<double2*>(C), ldc, k);
   ctx->launches++;

@@ -5,9 +5,9 @@
 // needing the previous one's result in two entries. On one thread every rotation also paid
 // for its ~3 m complex row and column updates (m = 32: 80.6 ms); here A and Z sit in shared
 // memory (m <= 64) and one warp carries the chain: it applies a rotation to the few entries
-// the next one comes from, a lane per column, then a lane per row, and forms the next
-// rotation while the other warps apply this one to everything else, so a rotation costs one
-// barrier and one chain step. m = 32: 80.6 -> 4.7 ms.
+// the next one comes from, a lane per real number, and forms the next rotation while the other
+// warps apply this one to everything else, so a rotation costs one barrier and one chain step.
+// m = 32: 80.6 -> SEIG ms (a lane per entry: 4.7 ms).
 #pragma once
 
 #include "small_eig.h"
@@ -51,6 +51,55 @@ __device__ __forceinline__ void rotate(zc& p, zc& q, double c, zc s) {
   const zc a = p, b = q;
   p = add(scl(a, c), mul(s, b));
   q = sub(scl(b, c), mul(cj(s), a));
+}
+
+// rotate() of the pair p, q by four lanes, each forming a part of it: lane & 2 the q, lane & 1 the
+// imaginary part. Returns the lane's part. The pipe takes 16 clocks a warp's operation however many
+// lanes take part, so a chain of few numbers is shortened by giving every lane one of them: a
+// rotation's 12 operations become 3, and the next one's formation 12 instead of 23.
+__device__ __forceinline__ double rotate_lanes(zc* p, zc* q, bool active, double c, zc s) {
+  const int lane = threadIdx.x % 32;
+  const bool im = lane & 1, second = lane & 2;
+  double v = 0.0;
+  double* mine = &(second ? q : p)->re + (im ? 1 : 0);
+  if (active) {
+    const double* other = &(second ? p : q)->re;
+    const double o1 = other[im ? 1 : 0], o2 = other[im ? 0 : 1];
+    v = fma(im ? s.im : -s.im, o2, fma(second ? -s.re : s.re, o1, c * *mine));
+  }
+  __syncwarp();
+  if (active) *mine = v;
+  __syncwarp();
+  return v;
+}
+
+// givens_fast(x, y) by a warp (x and y in every lane), written by lanes 0 .. 2.
+__device__ __forceinline__ void givens_lanes(zc x, zc y, double& c, zc& s) {
+  const int lane = threadIdx.x % 32;
+  const bool odd = lane & 1;
+  const double re = odd ? y.re : x.re, im = odd ? y.im : x.im, a = fma(re, re, im * im);
+  const int e = (__double2hiint(a) >> 20) - 1023;   // a within 2^-600 .. 2^600
+  if (!__all_sync(0xffffffffu, e > -600 && e < 600)) {
+    double cc;
+    zc ss;
+    givens(x, y, cc, ss);
+    if (lane == 0) {
+      c = cc;
+      s = ss;
+    }
+    return;
+  }
+  // even lanes 1 / |x|, odd ones 1 / sqrt(|x|^2 + |y|^2)
+  const double sum = a + __shfl_xor_sync(0xffffffffu, a, 1);
+  const double r = rsqrt_step(odd ? sum : a);
+  const double w = r * __shfl_xor_sync(0xffffffffu, r, 1);
+  // lane 0: c = |x|^2 w, lanes 1, 2: the parts of s = x conj(y) w
+  const double u1 = odd ? x.re : x.im, u2 = odd ? x.im : -x.re;
+  const double t = fma(u1, y.re, u2 * y.im);
+  const double v = (lane == 0 ? a : t) * w;
+  if (lane == 0) c = v;
+  else if (lane == 1) s.re = v;
+  else if (lane == 2) s.im = v;
 }
 
 #define SE_A(M, i, j) (M)[(int64_t)(j) * ld + (i)]
@@ -196,37 +245,17 @@ __device__ inline int eig_block(int m, zc* gA, zc* gw, zc* gV, zc* gZ) {
       const zc s = sh_s[k & 1];
       const int rmax = (k + 2 < ihi ? k + 2 : ihi);
       if (tid < 32) {
-        // rows k, k+1 of the columns k, k+1 and (the bulge) k-1
-        const int j = tid < 2 ? k + tid : k - 1;
-        if (tid < (k > l ? 3 : 2)) {
-          zc p = SE_A(A, k, j), q = SE_A(A, k + 1, j);
-          rotate(p, q, c, s);
-          SE_A(A, k, j) = p;
-          SE_A(A, k + 1, j) = q;
-        }
-        __syncwarp();
-        // columns k, k+1 of the rows k .. k+2; the next rotation zeroes A(k+2, k) against
-        // A(k+1, k)
-        const int i = k + tid;
-        zc p = mk(0.0, 0.0);
-        if (tid < 3 && i <= rmax) {
-          zc q = SE_A(A, i, k + 1);
-          p = SE_A(A, i, k);
-          rotate(p, q, c, cj(s));
-          SE_A(A, i, k) = p;
-          SE_A(A, i, k + 1) = q;
-        }
-        if (k + 1 < ihi) {
-          const zc x = mk(__shfl_sync(0xffffffffu, p.re, 1), __shfl_sync(0xffffffffu, p.im, 1));
-          const zc y = mk(__shfl_sync(0xffffffffu, p.re, 2), __shfl_sync(0xffffffffu, p.im, 2));
-          double nc;
-          zc ns;
-          givens_fast(x, y, nc, ns);
-          if (tid == 0) {
-            sh_c[(k + 1) & 1] = nc;
-            sh_s[(k + 1) & 1] = ns;
-          }
-        }
+        // rows k, k+1 of the columns k, k+1 and (the bulge) k-1, then columns k, k+1 of the rows
+        // k .. k+2: four lanes an item, a real number each (givens_lanes)
+        const int g = tid / 4, j = g < 2 ? k + g : k - 1;
+        rotate_lanes(&SE_A(A, k, j), &SE_A(A, k + 1, j), g < (k > l ? 3 : 2), c, s);
+        const int i = k + g;
+        const double p = rotate_lanes(&SE_A(A, i, k), &SE_A(A, i, k + 1), g < 3 && i <= rmax, c, cj(s));
+        // the next rotation zeroes A(k+2, k) against A(k+1, k)
+        if (k + 1 < ihi)
+          givens_lanes(mk(__shfl_sync(0xffffffffu, p, 4), __shfl_sync(0xffffffffu, p, 5)),
+                       mk(__shfl_sync(0xffffffffu, p, 8), __shfl_sync(0xffffffffu, p, 9)),
+                       sh_c[(k + 1) & 1], sh_s[(k + 1) & 1]);
       } else {
         // rows k, k+1 of the columns beyond k+1, columns k, k+1 of the rows above k, and of Z
         const int nrow = m - k - 2 > 0 ? m - k - 2 : 0;

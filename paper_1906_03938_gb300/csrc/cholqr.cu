@@ -906,8 +906,9 @@ size_t factor_smem(int mode, int nu) {
 // of cholesky_kernel. entry(r, c): G(r, c), r <= c. Whole block; false on a failed pivot.
 template <int kT, typename Entry>
 __device__ bool eliminate64(const Entry& entry, int nu, double2* __restrict__ Z, int* deficient) {
-  __shared__ double2 col[2][32 * kT];
+  __shared__ double2 col[2][32 * kT], scaled[32 * kT];
   __shared__ double diag[32 * kT];
+  __shared__ long long bound;
   const int tid = threadIdx.x, lane = tid % 32, w = tid / 32;
   const int tr = lane % 8 + 8 * (w % 4), tc = lane / 8 + 4 * (w / 4);
   double2 g[kT][kT];
@@ -927,14 +928,21 @@ __device__ bool eliminate64(const Entry& entry, int nu, double2* __restrict__ Z,
 #pragma unroll
     for (int i = 0; i < kT; ++i) col[0][tr + 32 * i] = g[i][0];
   __syncthreads();
-  double dmax = 0.0;
-  for (int k = 0; k < nu; ++k) dmax = fmax(dmax, diag[k]);
+  // the pivots' bound, compared as integers (positive numbers order alike): operations of every
+  // thread on the FP64 pipe are what this loop cannot afford
+  if (tid < 32) {
+    double dmax = 0.0;
+    for (int k = tid; k < nu; k += 32) dmax = fmax(dmax, diag[k]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, off));
+    if (tid == 0) bound = __double_as_longlong(1e-13 * dmax);
+  }
   __syncthreads();
   bool ok = true;
   for (int k = 0; k < nu; ++k) {
     const double2* s = col[k & 1];
     double d = s[k].x;
-    const bool bad = !(d > 1e-13 * dmax) || !isfinite(d);
+    const bool bad = __double_as_longlong(d) <= bound || (__double2hiint(d) >> 20) == 2047;
     if (bad && !deficient) {
       ok = false;
       break;
@@ -942,7 +950,14 @@ __device__ bool eliminate64(const Entry& entry, int nu, double2* __restrict__ Z,
     if (tid == 0 && deficient) deficient[k] = bad ? 1 : 0;
     if (bad) d = 1.0;   // unit pivot, no update
     if (tid == 0) diag[k] = d;
-    const double rd = 1.0 / d;
+    // column k over the pivot, by as many threads as it has entries (by every thread the division
+    // alone kept the pipe busy for 5000 clocks)
+    if (tid < 32 * kT) {
+      const double rd = 1.0 / d;
+      const double2 l = s[tid];
+      scaled[tid] = tid > k && !bad ? make_double2(l.x * rd, l.y * rd) : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
     double2 a[kT];
 #pragma unroll
     for (int i = 0; i < kT; ++i) a[i] = tr + 32 * i == k ? make_double2(1.0, 0.0) : s[tr + 32 * i];
@@ -950,8 +965,7 @@ __device__ bool eliminate64(const Entry& entry, int nu, double2* __restrict__ Z,
     for (int j = 0; j < kT; ++j) {
       if (32 * j + 31 <= k) continue;
       const int c = tc + 32 * j;
-      double2 l = s[c];
-      l = c > k && !bad ? make_double2(l.x * rd, l.y * rd) : make_double2(0.0, 0.0);
+      const double2 l = scaled[c];
 #pragma unroll
       for (int i = 0; i < kT; ++i) {
         if (i < j && 32 * i > k) continue;

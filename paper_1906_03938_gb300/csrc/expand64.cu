@@ -33,11 +33,12 @@ constexpr int kCoefPoints = 64;    // Chebyshev points of the coefficients' quad
 constexpr int kRowsE = 128;        // rows per block of the evaluation (a thread each)
 constexpr int kColsE = 8;          // columns per block of the evaluation
 constexpr size_t kMomentBytes = (size_t)1 << 30;   // moments held at a time
-// n^2 S (padded columns - 4) from which the split products pay (split64.cu; conversions of 24 ps a
+// n^2 S (padded columns - 4) from which the split products pay (split64.cu; conversions of 20 ps a
 // moment and three more launches against 5.6 ps a moment and column). Split against FP64, in us:
-// 300 panels, 8 residuals 505 / 457, 588 panels, 2 residuals 978 / 955 below it; projections of
-// 300 panels, 10 columns 751 / 958, 588 x 60 1687 / 3695, 1728 panels, 2 residuals 5247 / 5518 above.
-constexpr double kSplitWork = 0x1p25;
+// 192 panels, 4 columns 354 / 335, 300 panels, 8 residuals 380 / 350 below it; projections of 192
+// panels, 16 columns 362 / 450 (2^23.9), 300 x 10 401 / 615, 588 x 60 765 / 2785, residuals of 588
+// panels, 8 vectors 580 / 601, 3072 panels, 2 vectors 5853 / 8346 above.
+constexpr double kSplitWork = 0x1.cp23;
 constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
 
 // a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at

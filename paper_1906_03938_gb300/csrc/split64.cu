@@ -52,9 +52,9 @@ constexpr int kNotFinite = INT_MIN;           // exponent of a scale over non-fi
 constexpr int kZero = -4000;                  // of one over zeros
 constexpr size_t kMaxSplitBytes = (size_t)8 << 30;
 // n nu^2 from which the split products pay (more launches, less work). A CholeskyQR2, split
-// against FP64 products, in us: 4096 x 32 225 / 172, 20000 x 16 300 / 273, 1452 x 64 271 / 238
-// below it; 600 x 128 420 / 502, 12000 x 32 265 / 287, 3072 x 64 284 / 313, 6000 x 48 289 / 428,
-// 50000 x 16 425 / 525, 8192 x 256 1909 / 7171 above.
+// against FP64 products, in us: 4096 x 32 209 / 169, 20000 x 16 285 / 270, 1452 x 64 248 / 233
+// below it; 600 x 128 424 / 498, 12000 x 32 248 / 282, 3072 x 64 260 / 308, 6000 x 48 271 / 418,
+// 50000 x 16 406 / 528, 8192 x 256 1909 / 7171 above.
 constexpr int64_t kMinWork = (int64_t)1 << 23;
 
 // n p q nb from which X^H Y_j by splitting pays. FP64 projections whose last step it is, split

@@ -415,6 +415,18 @@ bem_status bem_set_async(bem_ctx* ctx, int on);
  */
 bem_status bem_set_wait_limit(bem_ctx* ctx, uint32_t polls);
 /*
+ * Largest device workspace buffer the context allocates (operational; the paper has no
+ * counterpart), for programs that share the device's memory with other allocators. The
+ * context keeps its workspaces: FP64 projections and residuals take up to 24 GiB where the
+ * expansion over the wavenumbers is the faster form, CholeskyQR2 up to 8 GiB of digit planes,
+ * the low-rank far field 4 GiB for a group of nodes, and bem_destroy gives them back. Beyond
+ * `bytes` an allocation fails as if the device's memory were short: a call that has a form
+ * needing less takes that one, one that has none returns BEM_ENOMEM. What a call finds large
+ * enough it uses as it is; the mesh's, contour's and batch's own buffers are not workspaces.
+ * 0 (the default): no limit.
+ */
+bem_status bem_set_workspace_limit(bem_ctx* ctx, int64_t bytes);
+/*
  * Split of the fused mixed-precision kernel's transcendental work between two pipes
  * (tuning; the paper has no counterpart). Each entry of A(z_j) sums 7 quadrature points,
  * each needing e^{i Re(z_j) r}: for the first poly_points of them (0..4) its cosine and

@@ -46,6 +46,7 @@ SIGNATURES = {
     "bem_node_order": (_I, [_P, _P, _P]),
     "bem_set_async": (_I, [_P, _I]),
     "bem_set_wait_limit": (_I, [_P, ctypes.c_uint32]),
+    "bem_set_workspace_limit": (_I, [_P, _I64]),
     "bem_set_eval_split": (_I, [_P, _I]),
     "bem_set_refine_residual": (_I, [_P, _I]),
     "bem_set_twin_clusters": (_I, [_P, _I]),
@@ -411,6 +412,11 @@ class Context:
         """Polls of each pipeline-stage wait of the fused kernel before it gives up with
         BEM_ETIMEOUT (0: at once); the default is 1 << 24."""
         self._chk("bem_set_wait_limit", self._lib.bem_set_wait_limit(self._h, int(polls)))
+
+    def set_workspace_limit(self, nbytes=0):
+        """Largest workspace buffer the context allocates (0: no limit): calls take the forms
+        that need less, or fail with BEM_ENOMEM."""
+        self._chk("bem_set_workspace_limit", self._lib.bem_set_workspace_limit(self._h, int(nbytes)))
 
     def set_eval_split(self, poly_points=-1):
         """Quadrature points (0..4 of 7) per entry whose sine and cosine the fused kernel

@@ -22,12 +22,17 @@ bem_status cuda_check(bem_ctx* ctx, cudaError_t e, const char* what) {
   return fail(ctx, BEM_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+cudaError_t workspace_malloc(const bem_ctx* ctx, void** p, size_t bytes) {
+  *p = nullptr;
+  return bytes > ctx->workspace_limit ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+}
+
 bem_status ensure_scratch(bem_ctx* ctx, size_t bytes) {
   if (bytes <= ctx->scratch_bytes) return BEM_OK;
   if (ctx->d_scratch) cudaFree(ctx->d_scratch);
   ctx->d_scratch = nullptr;
   ctx->scratch_bytes = 0;
-  if (cudaMalloc(&ctx->d_scratch, bytes) != cudaSuccess) {
+  if (workspace_malloc(ctx, &ctx->d_scratch, bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(ctx, BEM_ENOMEM, "scratch allocation of " + std::to_string(bytes) + " bytes failed");
   }
@@ -35,14 +40,21 @@ bem_status ensure_scratch(bem_ctx* ctx, size_t bytes) {
   return BEM_OK;
 }
 
-bool scratch_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s) {
-  if (bytes <= ctx->scratch_bytes) return true;
+bool expand_work_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s) {
+  if (bytes <= ctx->expand_bytes) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return false;
   }
-  return ensure_scratch(ctx, bytes) == BEM_OK;
+  cudaFree(ctx->d_expand);
+  ctx->expand_bytes = 0;
+  if (workspace_malloc(ctx, &ctx->d_expand, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  ctx->expand_bytes = bytes;
+  return true;
 }
 
 bem_status ensure_small(bem_ctx* ctx, size_t bytes) {
@@ -50,7 +62,7 @@ bem_status ensure_small(bem_ctx* ctx, size_t bytes) {
   if (ctx->d_small) cudaFree(ctx->d_small);
   ctx->d_small = nullptr;
   ctx->small_bytes = 0;
-  if (cudaMalloc(&ctx->d_small, bytes) != cudaSuccess) {
+  if (workspace_malloc(ctx, &ctx->d_small, bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(ctx, BEM_ENOMEM, "workspace allocation failed");
   }
@@ -229,6 +241,7 @@ void bem_destroy(bem_ctx* ctx) {
   cudaFree(ctx->d_lu_work);
   cudaFree(ctx->d_ff);
   cudaFree(ctx->d_split);
+  cudaFree(ctx->d_expand);
   cudaFree(ctx->d_zgemm);
   release_cublas(ctx);
   cudaFree(ctx->d_solve);
@@ -283,6 +296,12 @@ bem_status bem_set_async(bem_ctx* ctx, int on) {
 bem_status bem_set_wait_limit(bem_ctx* ctx, uint32_t polls) {
   if (!ctx) return BEM_EINVAL;
   ctx->stage_wait_limit = polls;
+  return BEM_OK;
+}
+
+bem_status bem_set_workspace_limit(bem_ctx* ctx, int64_t bytes) {
+  if (!ctx || bytes < 0) return fail(ctx, BEM_EINVAL, "bem_set_workspace_limit: need bytes >= 0");
+  ctx->workspace_limit = bytes == 0 ? SIZE_MAX : (size_t)bytes;
   return BEM_OK;
 }
 
@@ -509,25 +528,24 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
     return project_hmatrix(ctx, V_dev, ldv, nu, Bhat_dev, AV_dev, s);
   st0 = ensure_self64(ctx, s);
   if (st0 != BEM_OK) return st0;
-  // one evaluation expanded over the nodes where that costs less than one per node, and its
-  // workspace can be had (a stream capture allocates nothing)
   const size_t y_bytes = AV_dev ? 0 : (size_t)N * n * nu * 2 * sizeof(double);
+  st0 = ensure_scratch(ctx, y_bytes);
+  if (st0 != BEM_OK) return st0;
+  // One evaluation expanded over the nodes where that costs less than one per node, and V^H Y_j on
+  // the tensor core, where their workspace (the one after the other in the same buffer) can be had.
+  // A growth that fails gives up what there was, so the forms are settled by the buffer's size
+  // after the last one.
   ExpandPlan ex = expand_plan(ctx, N, ctx->con.c_re, ctx->con.c_im, std::max(ctx->con.a, ctx->con.b),
                               nu, true, false);
-  // V^H Y_j on the tensor core, its workspace in the place of the expansion's; the workspaces are
-  // found before any is written
   SplitCross xs = split64_cross_plan(ctx, n, nu, nu, N);
-  xs.use = xs.use && scratch_ready(ctx, y_bytes + xs.bytes, s);
-  ex.use = expand_ready(ctx, ex, y_bytes, nu, s);
-  if (!ex.use) {
-    bem_status st = ensure_scratch(ctx, y_bytes);
-    if (st != BEM_OK) return st;
-  }
+  ex.use = expand_ready(ctx, ex, nu, s);
+  xs.use = xs.use && expand_work_ready(ctx, xs.bytes, s);
+  ex.use = ex.use && expand_work_ready(ctx, ex.bytes, s);
+  xs.use = xs.use && ctx->expand_bytes >= xs.bytes;
   double* Y = AV_dev ? AV_dev : ctx->d_scratch;
   timing_begin(ctx, s);
   bem_status st =
-      ex.use ? expand_apply_nodes(ctx, ex, V_dev, ldv, nu, Y,
-                                  reinterpret_cast<char*>(ctx->d_scratch) + y_bytes, s)
+      ex.use ? expand_apply_nodes(ctx, ex, V_dev, ldv, nu, Y, ctx->d_expand, s)
              : cuda_check(ctx, launch_apply_fp64(ctx, V_dev, ldv, nu, Y, s), "apply kernel");
   timing_end(ctx, s);
   if (st != BEM_OK) return st;
@@ -536,8 +554,7 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
     if (st != BEM_OK) return st;
   }
   if (xs.use)
-    return split64_cross(ctx, xs, reinterpret_cast<char*>(ctx->d_scratch) + y_bytes,
-                         reinterpret_cast<const double2*>(V_dev), ldv,
+    return split64_cross(ctx, xs, ctx->d_expand, reinterpret_cast<const double2*>(V_dev), ldv,
                          reinterpret_cast<const double2*>(Y), reinterpret_cast<const double2*>(ctx->con.w),
                          reinterpret_cast<double2*>(Bhat_dev), s);
   return cuda_check(ctx, launch_xhy_fp64(ctx, V_dev, ldv, nu, Y, n, n * nu, nu, n, N, ctx->con.w,

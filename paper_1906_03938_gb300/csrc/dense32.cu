@@ -790,7 +790,7 @@ bem_status lu32(bem_ctx* ctx, float2* A, int64_t n, int* ipiv, cudaStream_t s) {
     cudaFree(ctx->d_lu_work);
     ctx->d_lu_work = nullptr;
     ctx->lu_work_bytes = 0;
-    if (cudaMalloc(&ctx->d_lu_work, lu_work) != cudaSuccess) {
+    if (workspace_malloc(ctx, &ctx->d_lu_work, lu_work) != cudaSuccess) {
       cudaGetLastError();
       return fail(ctx, BEM_ENOMEM, "lu32: GEMM workspace allocation failed");
     }

@@ -513,9 +513,9 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   return p;
 }
 
-bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, size_t before, int ncols, cudaStream_t s) {
+bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s) {
   return p.use && (!near_active(ctx) || near_expand_ready(ctx, p, ncols, s)) &&
-         scratch_ready(ctx, before + p.bytes, s);
+         expand_work_ready(ctx, p.bytes, s);
 }
 
 namespace {

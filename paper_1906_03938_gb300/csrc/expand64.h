@@ -34,9 +34,9 @@ struct ExpandPlan {
 // every column (nodes), or wavenumber c times column c.
 ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dmax, int ncols,
                        bool nodes, bool deriv);
-// The workspace can be had: plan's bytes behind `before` bytes of the context's scratch, and the
-// near field's. False leaves the caller the direct form.
-bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, size_t before, int ncols, cudaStream_t s);
+// The workspace can be had: plan's bytes in d_expand, and the near field's. False leaves the caller
+// the direct form.
+bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s);
 // Y_j = A(z_j) V for all nodes of the contour (its FP64 self-term table filled), near field
 // included; Y as launch_apply_fp64's. work: plan's bytes.
 bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,

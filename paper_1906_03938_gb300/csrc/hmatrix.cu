@@ -838,7 +838,7 @@ bem_status grow(bem_ctx* ctx, T*& p, size_t& cap, size_t bytes) {
   cudaFree(p);
   p = nullptr;
   cap = 0;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+  if (workspace_malloc(ctx, &p, bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(ctx, BEM_ENOMEM, "low-rank far field: device allocation failed");
   }

@@ -110,6 +110,10 @@ struct bem_ctx {
   size_t lu_work_bytes = 0;
   void* d_split = nullptr;       // digit planes of the split FP64 products (split64.cu)
   size_t split_bytes = 0;
+  // workspace of the FP64 forms that a smaller one replaces (expand64.cu, split64.cu): apart from
+  // d_scratch, which such a call need not touch
+  void* d_expand = nullptr;
+  size_t expand_bytes = 0;
   double* d_ff = nullptr;        // column splits' partial sums of the double-FP32 residuals
   size_t ff_bytes = 0;
   size_t small_bytes = 0;
@@ -149,6 +153,8 @@ struct bem_ctx {
   // polls of each pipeline-stage wait of the fused projection kernel before it gives up
   // (bem_set_wait_limit); the drains before a block releases its memory keep the full bound
   uint32_t stage_wait_limit = bem::kStageWaitDefault;
+  // largest workspace buffer the context allocates (bem_set_workspace_limit)
+  size_t workspace_limit = SIZE_MAX;
   // quadrature points per entry whose sine and cosine the fused kernel takes from the FMA-
   // pipe polynomials (bem_set_eval_split); -1: the measured default of the unit shape
   int poly_points = -1;
@@ -178,11 +184,18 @@ namespace bem {
 bem_status fail(bem_ctx* ctx, bem_status st, const std::string& msg);
 // Map a CUDA error to BEM_ECUDA with a message; BEM_OK if `e` is cudaSuccess.
 bem_status cuda_check(bem_ctx* ctx, cudaError_t e, const char* what);
+// Memory for a workspace of the context; none beyond its limit (bem_set_workspace_limit), as if the
+// device's memory were short.
+cudaError_t workspace_malloc(const bem_ctx* ctx, void** p, size_t bytes);
+template <typename T>
+cudaError_t workspace_malloc(const bem_ctx* ctx, T** p, size_t bytes) {
+  return workspace_malloc(ctx, reinterpret_cast<void**>(p), bytes);
+}
 // Make sure the context's scratch holds at least `bytes`.
 bem_status ensure_scratch(bem_ctx* ctx, size_t bytes);
-// The same where a smaller workspace would do: false if it cannot be had (no memory, or the
-// stream is being captured and the buffer would have to grow).
-bool scratch_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s);
+// Make sure d_expand holds at least `bytes`; false if that cannot be had (no memory: then there is
+// no buffer; or the stream is being captured and the buffer would have to grow: then it stays).
+bool expand_work_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s);
 bem_status ensure_small(bem_ctx* ctx, size_t bytes);
 void release_cublas(bem_ctx* ctx);
 // nodes z and weights w (2 N doubles each, interleaved) of a contour, on the host

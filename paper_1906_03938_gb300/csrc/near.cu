@@ -1066,7 +1066,7 @@ bem_status ensure_near_work(bem_ctx* ctx, size_t bytes) {
   cudaFree(ctx->d_near_work);
   ctx->d_near_work = nullptr;
   ctx->near_work_bytes = 0;
-  if (cudaMalloc(&ctx->d_near_work, bytes) != cudaSuccess) {
+  if (workspace_malloc(ctx, &ctx->d_near_work, bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(ctx, BEM_ENOMEM, "near field: device allocation failed");
   }

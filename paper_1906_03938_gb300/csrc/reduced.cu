@@ -509,7 +509,7 @@ cudaError_t launch_zgemm(bem_ctx* ctx, int m, int n, int k, const double* A, int
       cudaFree(ctx->d_zgemm);
       ctx->d_zgemm = nullptr;
       ctx->zgemm_bytes = 0;
-      cudaError_t e = cudaMalloc(&ctx->d_zgemm, bytes);
+      cudaError_t e = workspace_malloc(ctx, &ctx->d_zgemm, bytes);
       if (e != cudaSuccess) return e;
       ctx->zgemm_bytes = bytes;
     }

@@ -195,7 +195,8 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   // One FP64 evaluation expanded about the middle of the given values for all columns, where that
   // costs less than one per column (in FP64, or in double-FP32 if asked for: single layer only)
   // and its workspace can be had
-  const size_t r_bytes = R_dev ? 0 : ((size_t)2 * n * m * sizeof(double) + 255) / 256 * 256;
+  st = ensure_scratch(ctx, R_dev ? 0 : (size_t)2 * n * m * sizeof(double));
+  if (st != BEM_OK) return st;
   ExpandPlan ex;
   {
     double lo[2] = {lam_host[0], lam_host[1]}, hi[2] = {lam_host[0], lam_host[1]};
@@ -209,11 +210,7 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
       dmax = std::max(dmax, hypot(lam_host[2 * c] - cr, lam_host[2 * c + 1] - ci));
     ex = expand_plan(ctx, m, cr, ci, dmax, m, false, Rd_dev != nullptr);
     if (arith == 1 && op_single(ctx->op) && !expand_beats_ff(ctx, ex, m, Rd_dev != nullptr)) ex.use = false;
-    ex.use = ex.use && expand_ready(ctx, ex, r_bytes, m, s);
-  }
-  if (!ex.use) {
-    st = ensure_scratch(ctx, r_bytes);
-    if (st != BEM_OK) return st;
+    ex.use = ex.use && expand_ready(ctx, ex, m, s);
   }
   double* R = R_dev ? R_dev : ctx->d_scratch;
   double* dlam = ctx->d_small;
@@ -225,10 +222,9 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   if (arith == 1 && !ex.use) {
     e = launch_apply_ff(ctx, m, dlam, X_dev, ldx, R, Rd_dev, s);
   } else if (ex.use) {
-    void* w = reinterpret_cast<char*>(ctx->d_scratch) + r_bytes;
-    st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, false, w, s);
+    st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, false, ctx->d_expand, s);
     if (st == BEM_OK && Rd_dev)
-      st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, Rd_dev, true, w, s);
+      st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, Rd_dev, true, ctx->d_expand, s);
     if (st != BEM_OK) return st;
   } else {
     e = launch_apply_percol64(ctx, m, dlam, X_dev, ldx, R, false, s);

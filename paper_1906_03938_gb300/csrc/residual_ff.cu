@@ -309,7 +309,7 @@ cudaError_t launch_apply_ff(bem_ctx* ctx, int m, const double* lam_dev, const do
       cudaFree(ctx->d_ff);
       ctx->d_ff = nullptr;
       ctx->ff_bytes = 0;
-      if (cudaMalloc(&ctx->d_ff, bytes) == cudaSuccess) ctx->ff_bytes = bytes;
+      if (workspace_malloc(ctx, &ctx->d_ff, bytes) == cudaSuccess) ctx->ff_bytes = bytes;
       else splits = 1;
     }
     cudaGetLastError();

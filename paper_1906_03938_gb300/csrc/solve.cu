@@ -933,7 +933,7 @@ extern "C" bem_status bem_solve(bem_ctx* ctx, const double* V0_dev, int64_t ldv,
     cudaFree(ctx->d_solve);
     ctx->d_solve = nullptr;
     ctx->solve_bytes = 0;
-    if (cudaMalloc(&ctx->d_solve, need) != cudaSuccess) {
+    if (workspace_malloc(ctx, &ctx->d_solve, need) != cudaSuccess) {
       cudaGetLastError();
       return fail(ctx, BEM_ENOMEM, "bem_solve: buffer allocation failed");
     }

@@ -684,7 +684,7 @@ void split64_plan(bem_ctx* ctx, int64_t ldv, int64_t n, int nu, void* mem, Split
     cudaFree(ctx->d_split);
     ctx->d_split = nullptr;
     ctx->split_bytes = 0;
-    if (cudaMalloc(&ctx->d_split, z.total) != cudaSuccess) {
+    if (workspace_malloc(ctx, &ctx->d_split, z.total) != cudaSuccess) {
       cudaGetLastError();
       return;
     }

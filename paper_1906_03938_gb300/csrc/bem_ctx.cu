@@ -538,9 +538,9 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
   ExpandPlan ex = expand_plan(ctx, N, ctx->con.c_re, ctx->con.c_im, std::max(ctx->con.a, ctx->con.b),
                               nu, true, false);
   SplitCross xs = split64_cross_plan(ctx, n, nu, nu, N);
-  ex.use = expand_ready(ctx, ex, nu, s);
+  ex.use = expand_ready(ctx, ex, s);
   xs.use = xs.use && expand_work_ready(ctx, xs.bytes, s);
-  ex.use = ex.use && expand_work_ready(ctx, ex.bytes, s);
+  ex.use = ex.use && expand_ready(ctx, ex, s);
   xs.use = xs.use && ctx->expand_bytes >= xs.bytes;
   double* Y = AV_dev ? AV_dev : ctx->d_scratch;
   timing_begin(ctx, s);

@@ -510,12 +510,13 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   p.batch_off = p.y_off + up((size_t)p.splits * p.S * n * ncols * 16);
   p.bytes = p.batch_off + p.batch.bytes;
   p.use = p.bytes <= kMaxWork;
+  p.near_off = up(p.bytes);
+  if (near_active(ctx)) p.bytes = p.near_off + near_expand_bytes(ctx, p, ncols);
   return p;
 }
 
-bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s) {
-  return p.use && (!near_active(ctx) || near_expand_ready(ctx, p, ncols, s)) &&
-         expand_work_ready(ctx, p.bytes, s);
+bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, cudaStream_t s) {
+  return p.use && expand_work_ready(ctx, p.bytes, s);
 }
 
 namespace {
@@ -566,7 +567,8 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
     expand_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, p.splits, Yp);
     ctx->launches++;
   }
-  return near_active(ctx) ? near_expand64(ctx, p, angles, X, ldx, ncols, Yp, s) : BEM_OK;
+  return near_active(ctx) ? near_expand64(ctx, p, angles, X, ldx, ncols, Yp, work + p.near_off, s)
+                          : BEM_OK;
 }
 
 }  // namespace

@@ -27,16 +27,15 @@ struct ExpandPlan {
   FixedPhase phase{};
   bool split = false;      // products on the tensor core (split64.cu)
   SplitBatch batch;
-  size_t coef_off = 0, mom_off = 0, y_off = 0, batch_off = 0, bytes = 0;
+  size_t coef_off = 0, mom_off = 0, y_off = 0, batch_off = 0, near_off = 0, bytes = 0;
 };
 
 // Plan for nk wavenumbers within dmax of the centre and ncols columns: every wavenumber times
 // every column (nodes), or wavenumber c times column c.
 ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dmax, int ncols,
                        bool nodes, bool deriv);
-// The workspace can be had: plan's bytes in d_expand, and the near field's. False leaves the caller
-// the direct form.
-bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s);
+// The workspace can be had: plan's bytes in d_expand. False leaves the caller the direct form.
+bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, cudaStream_t s);
 // Y_j = A(z_j) V for all nodes of the contour (its FP64 self-term table filled), near field
 // included; Y as launch_apply_fp64's. work: plan's bytes.
 bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
@@ -46,9 +45,9 @@ bem_status expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const 
                                 const double* X, int64_t ldx, double* R, bool deriv, void* work,
                                 cudaStream_t s);
 // Near pairs (near.cu): Y_s += C_s X for every slot, C_s the moments of the corrections
-// (A_near - A_7); its workspace.
-bool near_expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s);
+// (A_near - A_7), in near_expand_bytes of workspace.
+size_t near_expand_bytes(const bem_ctx* ctx, const ExpandPlan& p, int ncols);
 bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const int4* angles, const double* X,
-                         int64_t ldx, int ncols, double2* Ys, cudaStream_t s);
+                         int64_t ldx, int ncols, double2* Ys, void* work, cudaStream_t s);
 
 }  // namespace bem

@@ -1150,22 +1150,15 @@ bem_status near_apply64(bem_ctx* ctx, const double* V, int64_t ldv, int nu, doub
   return cuda_check(ctx, cudaGetLastError(), "near field kernels");
 }
 
-bool near_expand_ready(bem_ctx* ctx, const ExpandPlan& p, int ncols, cudaStream_t s) {
-  const size_t need = ((size_t)ctx->geo.n * ncols + (size_t)p.S * ctx->near_nnz) * sizeof(double2);
-  if (need <= ctx->near_work_bytes) return true;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
-  return ensure_near_work(ctx, need) == BEM_OK;
+size_t near_expand_bytes(const bem_ctx* ctx, const ExpandPlan& p, int ncols) {
+  return ((size_t)ctx->geo.n * ncols + (size_t)p.S * ctx->near_nnz) * sizeof(double2);
 }
 
 bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const int4* angles, const double* X,
-                         int64_t ldx, int ncols, double2* Ys, cudaStream_t s) {
+                         int64_t ldx, int ncols, double2* Ys, void* work, cudaStream_t s) {
   const int64_t n = ctx->geo.n, nnz = ctx->near_nnz;
   if (nnz == 0) return BEM_OK;
-  double2* Xt = reinterpret_cast<double2*>(ctx->d_near_work);
+  double2* Xt = static_cast<double2*>(work);
   double2* C = Xt + (size_t)n * ncols;
   transpose64_kernel<<<(unsigned)((n * ncols + 255) / 256), 256, 0, s>>>(
       reinterpret_cast<const double2*>(X), ldx, n, ncols, Xt);

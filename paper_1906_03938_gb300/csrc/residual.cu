@@ -210,7 +210,7 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
       dmax = std::max(dmax, hypot(lam_host[2 * c] - cr, lam_host[2 * c + 1] - ci));
     ex = expand_plan(ctx, m, cr, ci, dmax, m, false, Rd_dev != nullptr);
     if (arith == 1 && op_single(ctx->op) && !expand_beats_ff(ctx, ex, m, Rd_dev != nullptr)) ex.use = false;
-    ex.use = ex.use && expand_ready(ctx, ex, m, s);
+    ex.use = ex.use && expand_ready(ctx, ex, s);
   }
   double* R = R_dev ? R_dev : ctx->d_scratch;
   double* dlam = ctx->d_small;

@@ -88,3 +88,42 @@ def test_cholqr2_and_residual_take_the_form_that_fits(problem, limit):
     eye = torch.eye(64, dtype=Q.dtype, device=Q.device)
     assert float((Q.mH @ Q - eye).abs().max()) < 64 * 2.0 ** -52
     ctx.close()
+
+
+@pytest.mark.parametrize("near", [0, 1])
+def test_recorded_mixed_projections_survive_fp64_calls(near):
+    """A recorded batch, or a captured projection with near field, holds the addresses of the
+    context's scratch and near-field buffers. Residuals into the caller's buffer and FP64
+    projections with AV given need neither: the recording stays valid and its results the same."""
+    mesh = synth.cube_sphere(7, (1.0, 0.8, 0.55))
+    bem, ctx = _context(mesh)
+    ctx.set_near_field(near)
+    V = bem.fortran(torch.from_numpy(synth.complex_gaussian(mesh.n, 16, 3)).to("cuda:0"))
+    if near:
+        B = torch.empty((N, 16, 16), dtype=torch.complex128, device="cuda:0")
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            ctx.project(V, bem.PREC_MIXED, Bhat=B)
+            s.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=s):
+                ctx.project(V, bem.PREC_MIXED, Bhat=B)
+
+        def run():
+            graph.replay()
+            torch.cuda.synchronize()
+            return [B]
+    else:
+        batch = bem.Batch([ctx], [V])
+        run = batch.run
+    first = [b.clone() for b in run()]
+    X = bem.fortran(torch.from_numpy(synth.complex_gaussian(mesh.n, 64, 4)).to("cuda:0"))
+    ctx.project(X, bem.PREC_FP64, AV=True)
+    ctx.residual_arith(5.0 + 0.01 * np.arange(64), X, arith=0)
+    again = run()
+    torch.cuda.synchronize()
+    ctx.check()
+    for a, b in zip(first, again):
+        assert torch.equal(a, b)
+    ctx.close()

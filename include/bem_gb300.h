@@ -401,8 +401,9 @@ bem_status bem_check(bem_ctx* ctx, void* stream);
  */
 bem_status bem_set_async(bem_ctx* ctx, int on);
 /*
- * Bound of the pipeline-stage waits of the fused mixed-precision projection kernel
- * (operational; the paper has no counterpart): each wait of a block on its shared-memory
+ * Bound of the pipeline-stage waits of the fused mixed-precision projection kernel and of the
+ * FP64 products on the tensor core (FP64 bem_project, bem_cholqr2 and bem_residual at the sizes
+ * that take them; operational, the paper has no counterpart): each wait of a block on its shared-memory
  * pipeline (copies landed, entries evaluated, tensor-core products done) polls an mbarrier
  * at most `polls` times, with 64 ns sleeps after the first 64 (default 1 << 24, about a
  * second), then records BEM_ETIMEOUT in the device status word, raises the block's abort
@@ -410,8 +411,7 @@ bem_status bem_set_async(bem_ctx* ctx, int on);
  * before a block frees its shared memory and tensor memory keep the default bound whatever
  * this value is, so an aborted block leaves no asynchronous work behind and the context
  * stays usable. polls = 0 makes every stage wait give up at once (a way to exercise the
- * timeout path). Applies to projections planned after the call (bem_project,
- * bem_apply_sum, batches created afterwards).
+ * timeout path). Applies to calls made after this one (batches: created after it).
  */
 bem_status bem_set_wait_limit(bem_ctx* ctx, uint32_t polls);
 /*

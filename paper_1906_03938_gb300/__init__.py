@@ -409,8 +409,8 @@ class Context:
         self._chk("bem_set_async", self._lib.bem_set_async(self._h, 1 if on else 0))
 
     def set_wait_limit(self, polls):
-        """Polls of each pipeline-stage wait of the fused kernel before it gives up with
-        BEM_ETIMEOUT (0: at once); the default is 1 << 24."""
+        """Polls of each pipeline-stage wait of the fused kernel and the FP64 tensor-core
+        products before it gives up with BEM_ETIMEOUT (0: at once); the default is 1 << 24."""
         self._chk("bem_set_wait_limit", self._lib.bem_set_wait_limit(self._h, int(polls)))
 
     def set_workspace_limit(self, nbytes=0):

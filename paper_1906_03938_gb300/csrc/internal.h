@@ -150,8 +150,8 @@ struct bem_ctx {
   cudaEvent_t con_ev = nullptr;
   // asynchronous mode: bem_cholqr2 does not wait for its status word (bem_check reports it)
   bool async = false;
-  // polls of each pipeline-stage wait of the fused projection kernel before it gives up
-  // (bem_set_wait_limit); the drains before a block releases its memory keep the full bound
+  // polls of each pipeline-stage wait of the fused projection kernel and the split products before
+  // it gives up (bem_set_wait_limit); the drains before a block releases its memory keep the full bound
   uint32_t stage_wait_limit = bem::kStageWaitDefault;
   // largest workspace buffer the context allocates (bem_set_workspace_limit)
   size_t workspace_limit = SIZE_MAX;

@@ -47,7 +47,7 @@ constexpr int kStagesG = 2;
 constexpr int kFlush = 4;                     // K-blocks between two flushes of d >= 4 (64 rows)
 constexpr int kFlushWarps = 8;
 constexpr int kThreadsG = 32 * (2 + kFlushWarps);
-constexpr uint32_t kWaitG = kStageWaitDefault;
+constexpr uint32_t kDrainWait = kStageWaitDefault;   // of the waits before a block leaves
 constexpr int kNotFinite = INT_MIN;           // exponent of a scale over non-finite values
 constexpr int kZero = -4000;                  // of one over zeros
 constexpr size_t kMaxSplitBytes = (size_t)8 << 30;
@@ -362,6 +362,7 @@ struct GemmArgs {
   double2* out;        // Gram partial sums, V, or the products of a batch
   int* status;
   const int *gate, *skip;
+  uint32_t wait_limit;   // polls of a pipeline wait
 };
 
 struct GemmSmem {
@@ -370,13 +371,13 @@ struct GemmSmem {
 };
 
 __device__ __forceinline__ bool wait_flag(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          int* status) {
-  for (uint32_t it = 0; it < kWaitG; ++it) {
+                                          const GemmArgs& p) {
+  for (uint32_t it = 0; it < p.wait_limit; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort_flag) return false;
     if (it > 64) __nanosleep(64);
   }
-  atomicOr(status, kStatusTimeout);
+  atomicOr(p.status, kStatusTimeout);
   *abort_flag = 1;
   return false;
 }
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
       for (int i = 0; ok && tile_of<kMode>(p, i, t); ++i)
         for (int kb = t.kb0; kb < t.kb1; ++kb, ++issued) {
           const int s = issued % kStagesG;
-          ok = wait_flag(&empty[s], ((issued / kStagesG) & 1) ^ 1, abort_flag, p.status);
+          ok = wait_flag(&empty[s], ((issued / kStagesG) & 1) ^ 1, abort_flag, p);
           if (!ok) break;
           mbar_arrive_expect_tx(&full[s], kABytes + kBBytes);
           bulk_g2s(smem + GemmSmem::a + s * kABytes, p.a + ((size_t)kb * p.ta + t.ta) * kABytes,
@@ -489,9 +490,9 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
           bulk_g2s(smem + GemmSmem::b + s * kBBytes, p.b + ((size_t)kb * p.tb + t.tb) * kBBytes,
                    kBBytes, &full[s]);
         }
-      if (*abort_flag)   // let copies in flight land (bounded)
-        for (int it = max(0, issued - kStagesG); it < issued; ++it)
-          mbar_wait(&full[it % kStagesG], (it / kStagesG) & 1, kWaitG);
+      // no copy may be in flight when the block leaves, also if the others gave up without it
+      for (int it = max(0, issued - kStagesG); it < issued; ++it)
+        mbar_wait(&full[it % kStagesG], (it / kStagesG) & 1, kDrainWait);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -508,9 +509,9 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
             fresh[g] = at % every == 0;
             last[g] = end || at % every == every - 1;
           }
-          ok = wait_flag(&full[s], (it / kStagesG) & 1, abort_flag, p.status);
+          ok = wait_flag(&full[s], (it / kStagesG) & 1, abort_flag, p);
           for (int g = 0; ok && g < 2; ++g)
-            if (fresh[g] && done[g] > 0) ok = wait_flag(&accfree[g], (done[g] - 1) & 1, abort_flag, p.status);
+            if (fresh[g] && done[g] > 0) ok = wait_flag(&accfree[g], (done[g] - 1) & 1, abort_flag, p);
           if (!ok) break;
           tc_fence_after();
           const uint32_t ab = smem_u32(smem + GemmSmem::a + s * kABytes);
@@ -559,7 +560,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
 #pragma unroll
         for (int g = 1; g >= 0; --g) {
           if (g == 0 && at % (2 * kFlush) != 0 && at < nkb) continue;
-          if (ok) ok = __all_sync(0xffffffffu, wait_flag(&accfull[g], done[g] & 1, abort_flag, p.status));
+          if (ok) ok = __all_sync(0xffffffffu, wait_flag(&accfull[g], done[g] & 1, abort_flag, p));
           if (!ok) continue;
           tc_fence_after();
 #pragma unroll
@@ -607,7 +608,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) split_gemm_kernel(GemmArgs p) {
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
-    if (lane == 0) mbar_wait(drained, 0, kWaitG);   // before the accumulators are released
+    if (lane == 0) mbar_wait(drained, 0, kDrainWait);   // before the accumulators are released
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, 512);
@@ -723,7 +724,7 @@ bem_status split64_gram(bem_ctx* ctx, const Split64& sp, const double2* V, doubl
   int tiles = 0;
   for (int a = 0; a < sp.mtu; ++a) tiles += sp.ntu - a * (kTileM / kTileN);
   GemmArgs g{sp.a, sp.b, sp.mtu, sp.ntu, 0, false, sp.nu, sp.n, sp.ldv, sp.kbn, sp.parts,
-             reinterpret_cast<const int*>(sp.hcol), reinterpret_cast<const int*>(sp.hcol), part, ctx->d_status, gate, nullptr};
+             reinterpret_cast<const int*>(sp.hcol), reinterpret_cast<const int*>(sp.hcol), part, ctx->d_status, gate, nullptr, ctx->stage_wait_limit};
   split_gemm_kernel<kGramSum><<<dim3((unsigned)tiles, (unsigned)sp.parts), kThreadsG, GemmSmem::total, s>>>(g);
   ctx->launches += 2;
   return cuda_check(ctx, cudaGetLastError(), "split Gram matrix");
@@ -740,7 +741,7 @@ bem_status split64_multiply(bem_ctx* ctx, const Split64& sp, bool same, double2*
   split_factor_kernel<<<(unsigned)(sp.ntu * kTileN), 64, 0, s>>>(Z, sp.nu, sp.kbu, sp.ntu, sp.hcol,
                                                                 sp.ez, sp.b, gate, skip);
   GemmArgs g{sp.a, sp.b, sp.mtn, sp.ntu, sp.mtn, false, sp.nu, sp.n, sp.ldv, sp.kbu, 1, sp.erow, sp.ez, V,
-             ctx->d_status, gate, skip};
+             ctx->d_status, gate, skip, ctx->stage_wait_limit};
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const unsigned grid = (unsigned)std::min<int64_t>(std::max(1, sms), sp.mtn * sp.ntu);
@@ -785,7 +786,7 @@ bem_status split64_batch(bem_ctx* ctx, const SplitBatch& b, char* work, const do
   const int64_t threads = 2 * (int64_t)kb * b.ntu * kTileN;
   split_rhs_kernel<false><<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(X, ldx, kc, b.nu, kb, b.ntu, hcol, bp);
   GemmArgs g{ap, bp, b.S * b.mtn, b.ntu, b.mtn, add, b.nu, b.n, b.n, kb, 1, er,
-             reinterpret_cast<const int*>(hcol), out, ctx->d_status, nullptr, nullptr};
+             reinterpret_cast<const int*>(hcol), out, ctx->d_status, nullptr, nullptr, ctx->stage_wait_limit};
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
   const unsigned grid = (unsigned)std::min<int64_t>(std::max(1, sms), g.ta * g.tb);
@@ -860,7 +861,7 @@ bem_status split64_cross(bem_ctx* ctx, const SplitCross& c, void* work, const do
   split_rhs_kernel<true><<<(unsigned)((ty + 127) / 128), 128, 0, s>>>(Y, c.n, c.n, cols, kb, c.nt, hy, bp);
   GemmArgs g{ap, bp, c.mtp, c.nt, c.mtp, false, cols, c.p, c.p, kb, c.parts,
              reinterpret_cast<const int*>(hx), reinterpret_cast<const int*>(hy), part, ctx->d_status,
-             nullptr, nullptr};
+             nullptr, nullptr, ctx->stage_wait_limit};
   split_gemm_kernel<kCross><<<dim3((unsigned)(c.mtp * c.nt), (unsigned)c.parts), kThreadsG, GemmSmem::total, s>>>(g);
   const int64_t count = (int64_t)c.p * cols;
   split_cross_sum_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(

@@ -206,7 +206,8 @@ bem_status bem_cholqr2(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int 
  *   X_dev      n x m complex, column-major, leading dimension ldx
  *   R_dev      optional n x m complex output (leading dimension n), may be NULL
  *   relres_host m doubles receiving ||r_c|| / ||x_c||
- * Synchronises the stream.
+ * Synchronises the stream. BEM_ETIMEOUT if a bounded wait of its products gave up (the results
+ * are then invalid).
  */
 bem_status bem_residual(bem_ctx* ctx, int m, const double* lam_host, const double* X_dev,
                         int64_t ldx, double* R_dev, double* relres_host, void* stream);

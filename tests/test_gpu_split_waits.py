@@ -66,3 +66,23 @@ def test_cholqr2(polls, n, nu, want_R):
     ctx.close()
     eye = torch.eye(nu, dtype=Q.dtype, device=Q.device)
     assert float((Q.mH @ Q - eye).abs().max()) < 64 * 2.0 ** -52   # as tests/test_gpu_split64.py
+
+
+@pytest.mark.parametrize("polls", [0, 1, 8])
+@pytest.mark.parametrize("deriv", [False, True])
+def test_residual(polls, deriv):
+    """1200 panels, 8 vectors: the expansion's products are split ones (n^2 S 28 > 1.5e7)."""
+    import paper_1906_03938_gb300 as bem
+    mesh = synth.cube_sphere(10, (1.0, 0.8, 0.55))
+    X = bem.fortran(torch.from_numpy(synth.complex_gaussian(mesh.n, 8, 6)).to("cuda:0"))
+    lam = 5.0 + 0.1 * np.arange(8) + 0.01j
+    ctx = bem.Context(0)
+    ctx.set_mesh(mesh.xyz, mesh.tri)
+    ref = ctx.residual_arith(lam, X, arith=0, deriv=deriv)[0]
+    ctx.set_wait_limit(polls)
+    for _ in range(3):
+        _timed_out(bem, lambda: ctx.residual_arith(lam, X, arith=0, deriv=deriv), polls == 0)
+    ctx.check()   # the timeout was this call's to report: nothing is left of it
+    ctx.set_wait_limit(1 << 24)
+    assert np.array_equal(ctx.residual_arith(lam, X, arith=0, deriv=deriv)[0], ref)
+    ctx.close()

@@ -145,12 +145,14 @@ near_scan_kernel(Geometry g, int32_t* __restrict__ counts, const int32_t* __rest
         bool in = hit[r] && l < n && i < n && l != i;
         if (in) {
           // the FP32 distance is off by at most 2^-23 sqrt(3) of the coordinates' size and a
-          // few ulps of itself; decided here unless the threshold lies within twice that
+          // few ulps of itself (its square within FP32's range: a mesh of 1e19 or 1e-22 is decided
+          // in FP64); decided here unless the threshold lies within twice that
           const float d = sqrtf(d2[r]), lim = 2.f * fmaxf(fh[r], c.w);
           const float slack = 4.2e-7f * (fm[r] + cm) + 2e-6f * lim;
-          if (d > lim + slack) {
+          const bool ranged = d2[r] > 1e-30f && d2[r] < 1e30f;
+          if (ranged && d > lim + slack) {
             in = false;
-          } else if (!(d < lim - slack)) {
+          } else if (!(ranged && d < lim - slack)) {
             const double xi[3] = {g.cx[i], g.cx[n + i], g.cx[2 * n + i]};
             const double xl[3] = {g.cx[l], g.cx[n + l], g.cx[2 * n + l]};
             in = dist_rn(xi, xl) < 2.0 * fmax(g.diam[i], g.diam[l]);

@@ -1012,33 +1012,24 @@ void free_hmatrix(bem_ctx* ctx) {
   ctx->hm = nullptr;
 }
 
-bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, double* Bhat,
-                           double* AV, cudaStream_t s) {
-  if (!ctx->hm) return fail(ctx, BEM_ESTATE, "bem_project: no low-rank far field set (bem_set_hmatrix)");
+namespace {
+
+// The projection with NB nodes (at most; 0: as group_nodes says) taken together; *taken: how many.
+bem_status project_nodes(bem_ctx* ctx, const double* V, int64_t ldv, int nu, double* Bhat, double* AV,
+                         int NB, int* taken, cudaStream_t s) {
   HMatrix& h = *ctx->hm;
   const int64_t n = ctx->geo.n;
   const int N = ctx->con.N;
-  if (ctx->h_xyz.empty()) return fail(ctx, BEM_ESTATE, "bem_project: no mesh set");
   bem_status st = BEM_OK;
-  if (h.mesh_version != ctx->mesh_version && (st = build_structure(ctx, s)) != BEM_OK) return st;
-  if ((st = ensure_self32(ctx, s)) != BEM_OK) return st;
   const size_t nfar = h.far.size();
   const int nch = nu <= 64 ? 1 : nu <= 128 ? 2 : 4;   // basis columns padded to CW = 64 nch
   const int cw = 64 * nch;
-  int NB = group_nodes(ctx, h, cw);
-  auto group_buffers = [&]() -> bem_status {
-    bem_status r = grow(ctx, h.d_uw, h.uw_bytes, std::max<size_t>(1, NB * h.uw_total) * sizeof(float2));
-    if (r == BEM_OK) r = grow(ctx, h.d_used, h.used_bytes, std::max<size_t>(1, NB * h.used_total));
-    if (r == BEM_OK) r = grow(ctx, h.d_rank, h.rank_cap, std::max<size_t>(1, NB * nfar) * sizeof(int32_t));
-    if (r == BEM_OK) r = grow(ctx, h.d_toff, h.toff_cap, std::max<size_t>(1, NB * nfar) * sizeof(int64_t));
-    return r;
-  };
-  st = group_buffers();
-  if (st != BEM_OK && NB > 1) {   // no room for a group: one node at a time
-    NB = 1;
-    st = group_buffers();
-  }
-  if (st != BEM_OK ||
+  if (NB == 0) NB = group_nodes(ctx, h, cw);
+  *taken = NB;
+  if ((st = grow(ctx, h.d_uw, h.uw_bytes, std::max<size_t>(1, NB * h.uw_total) * sizeof(float2))) != BEM_OK ||
+      (st = grow(ctx, h.d_used, h.used_bytes, std::max<size_t>(1, NB * h.used_total))) != BEM_OK ||
+      (st = grow(ctx, h.d_rank, h.rank_cap, std::max<size_t>(1, NB * nfar) * sizeof(int32_t))) != BEM_OK ||
+      (st = grow(ctx, h.d_toff, h.toff_cap, std::max<size_t>(1, NB * nfar) * sizeof(int64_t))) != BEM_OK ||
       (st = grow(ctx, h.d_vp, h.vp_bytes, (size_t)n * 256 * sizeof(float2))) != BEM_OK)
     return st;
   // the mixed path's FP32 partials (slice 0 of one column split), zeroed: the leaf kernels
@@ -1126,6 +1117,25 @@ bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, d
   h.far_row_terms = row_terms / N;
   h.far_col_terms = col_terms / N;
   return external_end(ctx, fr, nu, Bhat, AV, s);
+}
+
+}  // namespace
+
+bem_status project_hmatrix(bem_ctx* ctx, const double* V, int64_t ldv, int nu, double* Bhat,
+                           double* AV, cudaStream_t s) {
+  if (!ctx->hm) return fail(ctx, BEM_ESTATE, "bem_project: no low-rank far field set (bem_set_hmatrix)");
+  if (ctx->h_xyz.empty()) return fail(ctx, BEM_ESTATE, "bem_project: no mesh set");
+  HMatrix& h = *ctx->hm;
+  bem_status st = BEM_OK;
+  if (h.mesh_version != ctx->mesh_version && (st = build_structure(ctx, s)) != BEM_OK) return st;
+  if ((st = ensure_self32(ctx, s)) != BEM_OK) return st;
+  int taken = 0;
+  st = project_nodes(ctx, V, ldv, nu, Bhat, AV, 0, &taken, s);
+  if (st == BEM_ENOMEM && taken > 1) {   // no room for a group, or beside one: one node at a time
+    free_work(h);
+    st = project_nodes(ctx, V, ldv, nu, Bhat, AV, 1, &taken, s);
+  }
+  return st;
 }
 
 }  // namespace bem

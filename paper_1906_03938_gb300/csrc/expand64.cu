@@ -40,6 +40,11 @@ constexpr size_t kMomentBytes = (size_t)1 << 30;   // moments held at a time
 // panels, 8 vectors 580 / 601, 3072 panels, 2 vectors 5853 / 8346 above.
 constexpr double kSplitWork = 0x1.cp23;
 constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
+// |Re c| R beyond which the direct form runs. The fixed-point phase of every pair is off by up to
+// 2^-59 |Re c| R radians, whatever their distance, the direct form's by 2^-53 k r: for bodies far
+// apart (R of 1e4, 1e6 bodies' sizes at k = 10: 5e-14, 8e-12 in their own entries) that is the
+// larger error. Up to here it is at most 2^-52, an ulp.
+constexpr double kMaxPhase = 128.0;
 
 // a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
 // wavenumber k_j, times the operator's coefficient of the family. One block per (j, f): a thread
@@ -413,22 +418,28 @@ FixedPhase fixed_phase(double c, double R) {
   return fp;
 }
 
-// Largest distance between two points of the mesh, from above: the smaller of its box's
-// diagonal and twice the largest distance of a vertex from the box's centre.
+// Largest distance between two points of the panels (vertices that no panel has do not count), from
+// above: the smaller of their box's diagonal and twice the largest distance of a vertex from the
+// box's centre.
 double mesh_reach(bem_ctx* ctx) {
   if (ctx->reach_version == ctx->mesh_version) return ctx->reach;
   double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   const std::vector<double>& p = ctx->h_xyz;
-  for (size_t t = 0; t < p.size(); ++t) {
-    lo[t % 3] = std::min(lo[t % 3], p[t]);
-    hi[t % 3] = std::max(hi[t % 3], p[t]);
-  }
+  std::vector<char> used(p.size() / 3, 0);
+  for (const int32_t v : ctx->h_tri) used[v] = 1;
+  for (size_t v = 0; v < used.size(); ++v)
+    if (used[v])
+      for (int c = 0; c < 3; ++c) {
+        lo[c] = std::min(lo[c], p[3 * v + c]);
+        hi[c] = std::max(hi[c], p[3 * v + c]);
+      }
   double far2 = 0.0, diag2 = 0.0;
   for (int c = 0; c < 3; ++c) diag2 += (hi[c] - lo[c]) * (hi[c] - lo[c]);
-  for (size_t t = 0; t + 2 < p.size(); t += 3) {
+  for (size_t v = 0; v < used.size(); ++v) {
+    if (!used[v]) continue;
     double d2 = 0.0;
     for (int c = 0; c < 3; ++c) {
-      const double d = p[t + c] - 0.5 * (lo[c] + hi[c]);
+      const double d = p[3 * v + c] - 0.5 * (lo[c] + hi[c]);
       d2 += d * d;
     }
     far2 = std::max(far2, d2);
@@ -471,7 +482,7 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
     p.M = series_terms(dmax, p.R);
   }
   p.c = make_double2(c_re, c_im);
-  if (!(fabs(c_re) * p.R < 0x1p40)) return p;   // the phase's fixed-point range
+  if (!(fabs(c_re) * p.R <= kMaxPhase)) return p;
   p.phase = fixed_phase(c_re, p.R);
   if (p.M > 1 && (hasH || deriv)) p.M += 2;
   if (p.M == 1 && (hasH || deriv)) p.M = 3;   // factors 1, r, r^2

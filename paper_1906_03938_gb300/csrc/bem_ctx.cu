@@ -535,8 +535,7 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
   // the tensor core, where their workspace (the one after the other in the same buffer) can be had.
   // A growth that fails gives up what there was, so the forms are settled by the buffer's size
   // after the last one.
-  ExpandPlan ex = expand_plan(ctx, N, ctx->con.c_re, ctx->con.c_im, std::max(ctx->con.a, ctx->con.b),
-                              nu, true, false);
+  ExpandPlan ex = expand_plan(ctx, N, ctx->con.z_host, ctx->con.c_re, ctx->con.c_im, nu, true, false);
   SplitCross xs = split64_cross_plan(ctx, n, nu, nu, N);
   ex.use = expand_ready(ctx, ex, s);
   xs.use = xs.use && expand_work_ready(ctx, xs.bytes, s);

@@ -45,6 +45,13 @@ constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the
 // apart (R of 1e4, 1e6 bodies' sizes at k = 10: 5e-14, 8e-12 in their own entries) that is the
 // larger error. Up to here it is at most 2^-52, an ulp.
 constexpr double kMaxPhase = 128.0;
+// max |Im (k - c)| R beyond which the direct form runs. The series of e^{i (k - c) r} has coefficients
+// of up to e^{|Im (k - c)| R} whatever r, so the moments' rounding enters near entries that much
+// larger. Against 128-bit products on the unit sphere (R = 2), 16 nodes: dense bases, error of a
+// column's largest entry, expanded / direct: 1.2e-15 / 1.4e-15 at 1.6, 1.7e-15 / 1.6e-15 at 3.2,
+// 1.7e-15 / 2.1e-15 at 4.0, but 1.8e-15 / 1.2e-15 at 4.8; of (|A| |x|)_i for vectors of four panels
+// 1.0e-15 / 6e-16, 2.4e-15 / 7e-16, 4.0e-15 / 8e-16 and 7.6e-15 / 8e-16 (5.6: 1.7e-14).
+constexpr double kMaxGrowth = 4.0;
 
 // a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
 // wavenumber k_j, times the operator's coefficient of the family. One block per (j, f): a thread
@@ -466,7 +473,7 @@ int series_terms(double dmax, double R) {
 
 }  // namespace
 
-ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dmax, int ncols,
+ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, double c_im, int ncols,
                        bool nodes, bool deriv) {
   ExpandPlan p;
   const OpCoef& op = ctx->op;
@@ -474,13 +481,21 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dm
   const int64_t n = ctx->geo.n;
   p.R = mesh_reach(ctx);
   if (!(p.R > 0.0) || !isfinite(p.R) || !isfinite(1.0 / p.R)) return p;
+  double dmax = 0.0, growth = 0.0;
+  for (int j = 0; j < nk; ++j) {
+    dmax = std::max(dmax, hypot(k[2 * j] - c_re, k[2 * j + 1] - c_im));
+    growth = std::max(growth, fabs(k[2 * j + 1] - c_im));
+  }
   p.M = series_terms(dmax, p.R);
   // about a real centre no exponential is evaluated: for values near the axis, at most a term more
-  if (c_im != 0.0 && series_terms(dmax + fabs(c_im), p.R) <= p.M + 1) {
+  if (c_im != 0.0 && series_terms(dmax + fabs(c_im), p.R) <= p.M + 1 &&
+      (growth + fabs(c_im)) * p.R <= kMaxGrowth) {
     dmax += fabs(c_im);
+    growth += fabs(c_im);
     c_im = 0.0;
     p.M = series_terms(dmax, p.R);
   }
+  if (!(growth * p.R <= kMaxGrowth)) return p;
   p.c = make_double2(c_re, c_im);
   if (!(fabs(c_re) * p.R <= kMaxPhase)) return p;
   p.phase = fixed_phase(c_re, p.R);

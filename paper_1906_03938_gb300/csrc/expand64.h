@@ -30,9 +30,9 @@ struct ExpandPlan {
   size_t coef_off = 0, mom_off = 0, y_off = 0, batch_off = 0, near_off = 0, bytes = 0;
 };
 
-// Plan for nk wavenumbers within dmax of the centre and ncols columns: every wavenumber times
-// every column (nodes), or wavenumber c times column c.
-ExpandPlan expand_plan(bem_ctx* ctx, int nk, double c_re, double c_im, double dmax, int ncols,
+// Plan for the nk wavenumbers k (re, im on the host), expanded about (c_re, c_im), and ncols columns:
+// every wavenumber times every column (nodes), or wavenumber c times column c.
+ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, double c_im, int ncols,
                        bool nodes, bool deriv);
 // The workspace can be had: plan's bytes in d_expand. False leaves the caller the direct form.
 bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, cudaStream_t s);

@@ -204,11 +204,8 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
       lo[c % 2] = std::min(lo[c % 2], lam_host[c]);
       hi[c % 2] = std::max(hi[c % 2], lam_host[c]);
     }
-    const double cr = 0.5 * (lo[0] + hi[0]), ci = 0.5 * (lo[1] + hi[1]);
-    double dmax = 0.0;
-    for (int c = 0; c < m; ++c)
-      dmax = std::max(dmax, hypot(lam_host[2 * c] - cr, lam_host[2 * c + 1] - ci));
-    ex = expand_plan(ctx, m, cr, ci, dmax, m, false, Rd_dev != nullptr);
+    ex = expand_plan(ctx, m, lam_host, 0.5 * (lo[0] + hi[0]), 0.5 * (lo[1] + hi[1]), m, false,
+                     Rd_dev != nullptr);
     if (arith == 1 && op_single(ctx->op) && !expand_beats_ff(ctx, ex, m, Rd_dev != nullptr)) ex.use = false;
     ex.use = ex.use && expand_ready(ctx, ex, s);
   }

@@ -25,15 +25,6 @@ __host__ inline size_t eig_smem(int m) {
 // a warp for the chain, the others for the 2 m rows and columns of a rotation
 __host__ inline int eig_threads(int m) { return 32 + 2 * (m < 32 ? 32 : (m + 31) / 32 * 32); }
 
-// 1 / sqrt(a) for a in the range givens_fast admits: the hardware's estimate (20 bits or more)
-// and one third-order step, e = 1 - a y^2, y (1 + e / 2 + 3 e^2 / 8): error below e^3.
-__device__ __forceinline__ double rsqrt_step(double a) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const double e = fma(-a * y, y, 1.0);
-  return fma(y * e, fma(e, 0.375, 0.5), y);
-}
-
 // Givens rotation as small::givens, by reciprocal square roots where the squares are safe.
 __device__ inline void givens_fast(zc x, zc y, double& c, zc& s) {
   const double ax2 = abs2(x), ay2 = abs2(y);
@@ -41,7 +32,7 @@ __device__ inline void givens_fast(zc x, zc y, double& c, zc& s) {
     givens(x, y, c, s);
     return;
   }
-  const double w = rsqrt_step(ax2) * rsqrt_step(ax2 + ay2);
+  const double w = rsqrt(ax2) * rsqrt(ax2 + ay2);
   c = ax2 * w;
   s = scl(mul(x, cj(y)), w);
 }
@@ -91,7 +82,7 @@ __device__ __forceinline__ void givens_lanes(zc x, zc y, double& c, zc& s) {
   }
   // even lanes 1 / |x|, odd ones 1 / sqrt(|x|^2 + |y|^2)
   const double sum = a + __shfl_xor_sync(0xffffffffu, a, 1);
-  const double r = rsqrt_step(odd ? sum : a);
+  const double r = rsqrt(odd ? sum : a);
   const double w = r * __shfl_xor_sync(0xffffffffu, r, 1);
   // lane 0: c = |x|^2 w, lanes 1, 2: the parts of s = x conj(y) w
   const double u1 = odd ? x.re : x.im, u2 = odd ? x.im : -x.re;

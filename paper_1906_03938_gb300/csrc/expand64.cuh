@@ -65,8 +65,9 @@ __device__ __forceinline__ void fixed_sincos(unsigned long long phi, const int4*
   si = (((long long)e.z << 32) + e.w) - (((mulh(S, cm) >> 8) - mulh(C, sn)) >> 6);
 }
 
-// 1 / sqrt(r2) and sqrt(r2) by one third-order step from the FP32 root, y (1 + e / 2 +
-// 3 e^2 / 8) with e = 1 - r2 y^2 of ~2^-22.
+// 1 / sqrt(r2) and sqrt(r2) from the FP32 root y by one step of Householder's third-order iteration,
+// (1 - e)^(-1/2) = 1 + e / 2 + 3 e^2 / 8 + .. with e = 1 - r2 y^2 below 2^-20.8; both to 1.6 units of
+// 2^-53.
 __device__ __forceinline__ void root_and_inverse(double r2, double& r, double& ri) {
   const float rf = (float)r2;
   const double y = rf > 1e-30f && rf < 1e30f ? (double)rsqrtf(rf) : rsqrt(r2);

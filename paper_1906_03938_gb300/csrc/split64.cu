@@ -9,7 +9,11 @@
 // 2^-61 of the scales' product a term. The accumulators are added to 64-bit integers in
 // registers (d >= 4 every 64 rows, d < 4, which collect fewer pairs, every 128), so a whole sum
 // is exact until its single conversion to FP64: the errors are the digits' cut and that
-// rounding, no larger than those of FP64 sums.
+// rounding. The cut is one of the whole column (or row): a sum of K terms is off by up to
+// 2.1 K 2^-53 max|a| max|b|, the bound of an FP64 sum of entries that are all as large. Entries far
+// below their column's largest keep fewer bits (2^-20 of it: 36), so this bound holds normwise where
+// an FP64 sum's holds term by term; for Gaussian columns the sums are more exact than FP64's
+// (X^H Y_j at 768 x 64 1e-16 against 1.2e-15).
 //
 // split_gemm_kernel: a block owns 128 x 32 complex outputs, [Re | Im] of the 32 columns as the
 // 64 columns of each accumulator (8 x 64 = all 512 TMEM columns). Per 16-deep K-block two bulk

@@ -380,7 +380,9 @@ __device__ void chol_inv32_block(const double2* Gg, int ldg, int nu, const doubl
 template <int kT>
 __global__ void __launch_bounds__(1024)
 chol_inv32_kernel(const double2* __restrict__ Gg, int ldg, int nu, const double2* __restrict__ Gd,
-                  int nd, double2* __restrict__ Z, int ldz, int* fallback) {
+                  int nd, double2* __restrict__ Z, int ldz, int* fallback, const int* gate) {
+  if ((gate && *gate == 0) || *fallback != 0) return;
+  __syncthreads();   // (read by every thread before one may set it)
   chol_inv32_block<32, kT>(Gg, ldg, nu, Gd, nd, Z, ldz, fallback);
 }
 
@@ -394,7 +396,9 @@ constexpr int kChol32 = 128;
 template <int kMode>
 __global__ void __launch_bounds__(256)
 chol_block32_kernel(const double2* __restrict__ G, double2* __restrict__ Z, int nu,
-                    double2* __restrict__ W, double2* __restrict__ S, double2* __restrict__ T) {
+                    double2* __restrict__ W, double2* __restrict__ S, double2* __restrict__ T,
+                    const int* fallback, const int* gate) {
+  if ((gate && *gate == 0) || *fallback != 0) return;
   constexpr int h = kChol32;
   const int r = nu - h;
   const int i = blockIdx.x * 16 + threadIdx.x % 16, j = blockIdx.y * 16 + threadIdx.x / 16;
@@ -540,8 +544,9 @@ near_tile_kernel(const double2* __restrict__ G, const double2* __restrict__ Y,
 // The first step, Y1 = -U(E + Y0^H E + E Y0 + Y0^H Y0), Y0 = -U(E). E = -(Y0 + Y0^H), so the
 // second-order terms are -(Y0^H Y0 + Y0^2 + (Y0^2)^H), triangular products with a third of the
 // terms. Every block first sums the block sums of |E|^2 in order:
-//  ||E||_F > eps_max: the near-identity route is abandoned (*classic = 1) and the classic
-//    Cholesky factorisation runs instead;
+//  ||E||_F > eps_max: the near-identity route is abandoned (*classic = 1) and a Cholesky
+//    factorisation runs instead, in FP64 (classic[1] = 1) unless refused is given and *refused == 0
+//    (see near_pass);
 //  ||E||_F <= eps_small: Y1 is exact to rounding (its error is O(||E||^3)), Z = I + Y1 is
 //    written here and the second step is skipped (*done = 1). The second-order terms are then
 //    below 1e-10 and their rounding in FP32 (6e-18) far below Z's own in FP64, so they are
@@ -586,7 +591,7 @@ __device__ __forceinline__ T2 near_second_order(const double2* __restrict__ G, i
 __global__ void __launch_bounds__(64)
 near_y1_kernel(const double2* __restrict__ G, const float* __restrict__ epsp, int nparts, int nu,
                float eps_max, float eps_small, double2* __restrict__ Y, double2* __restrict__ Z,
-               int* classic, int* done, const int* gate) {
+               int* classic, int* done, const int* refused, const int* gate) {
   if (gate && *gate == 0) return;
   __shared__ float red[64];
   const int tid = threadIdx.x;
@@ -604,6 +609,7 @@ near_y1_kernel(const double2* __restrict__ G, const float* __restrict__ epsp, in
     if (first) {
       *classic = 1;
       *done = 1;
+      if (!refused || *refused != 0) classic[1] = 1;
     }
     return;
   }
@@ -1313,13 +1319,35 @@ bem_status small_factor(bem_ctx* ctx, const CqWork& w, int parts, int nu, int* f
   return BEM_OK;
 }
 
+// Z = R^{-1} of w.G in FP32 for nu > kSmallNu, in one or two diagonal blocks; *fallback is set
+// where a pivot is too small. Skipped when gate is given and *gate == 0, or *fallback != 0 (the
+// rest is, once it is set).
+void factor32(bem_ctx* ctx, const CqWork& w, int nu, int* fallback, const int* gate, cudaStream_t s) {
+  const int h = std::min(nu, kChol32), r = nu - h;   // diagonal blocks
+  auto inverse32 = [&](const double2* G, int ldg, int m, double2* Z) {
+    auto* kernel = m <= 32 ? chol_inv32_kernel<1> : m <= 64 ? chol_inv32_kernel<2> : chol_inv32_kernel<4>;
+    kernel<<<1, 1024, 0, s>>>(G, ldg, m, w.G, nu, Z, nu, fallback, gate);
+    ctx->launches++;
+  };
+  inverse32(w.G, nu, h, w.Z);
+  if (r == 0) return;
+  const dim3 gh((unsigned)((h + 15) / 16), (unsigned)((r + 15) / 16)), gr(gh.y, gh.y);
+  chol_block32_kernel<0><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y, fallback, gate);
+  chol_block32_kernel<1><<<gr, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y, fallback, gate);
+  inverse32(w.Q, r, r, w.Z + (size_t)h * nu + h);
+  chol_block32_kernel<2><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y, fallback, gate);
+  chol_block32_kernel<3><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y, fallback, gate);
+  ctx->launches += 4;
+}
+
 // One FP64 pass V <- V R^{-1} whose Gram matrix is expected near the identity: the
 // near-identity factor, or the classic Cholesky factorisation and triangular inverse when
-// ||G - I||_F > kNearEps (flag *classic, set on the device). Everything is skipped unless
-// *gate != 0 (gate null: always runs).
+// ||G - I||_F > kNearEps (flag *classic, set on the device; three ints). Everything is skipped
+// unless *gate != 0 (gate null: always runs). refused, if given: where *refused == 0 and another
+// near pass follows this one, the factor is an FP32 one again (nu > kSmallNu; FP64 if it fails).
 bem_status near_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu,
                      const CqLayout& L, const CqWork& w, const Split64& sp, const int* gate,
-                     int* classic, cudaStream_t s) {
+                     int* classic, const int* refused, cudaStream_t s) {
   double2* V = reinterpret_cast<double2*>(V_dev);
   const unsigned rb = (unsigned)((n + kRMRows - 1) / kRMRows);
   int parts;
@@ -1342,9 +1370,10 @@ bem_status near_pass(bem_ctx* ctx, double* V_dev, int64_t ldv, int64_t n, int nu
   const unsigned nt = (unsigned)((nu + kNT - 1) / kNT);
   const dim3 tgrid(nt, nt);
   near_y1_kernel<<<tgrid, 64, 0, s>>>(w.G, w.epsp, (int)L.sum_blocks, nu, kNearEps, kNearEpsSmall,
-                                      w.Y, w.Z, classic, done, gate);
-  cholesky_kernel<<<1, 1024, 0, s>>>(w.G, nu, ctx->d_status, nullptr, classic);
-  triangular_inverse_kernel<<<nu, 128, 0, s>>>(w.G, nu, w.Z, classic);
+                                      w.Y, w.Z, classic, done, refused, gate);
+  if (refused) factor32(ctx, w, nu, classic + 1, classic, s);
+  cholesky_kernel<<<1, 1024, 0, s>>>(w.G, nu, ctx->d_status, nullptr, classic + 1);
+  triangular_inverse_kernel<<<nu, 128, 0, s>>>(w.G, nu, w.Z, classic + 1);
   near_tile_kernel<1><<<tgrid, 64, 0, s>>>(w.G, w.Y, nullptr, nullptr, nu, w.P1, w.Q1, nullptr,
                                            gate, done);
   near_tile_kernel<2><<<tgrid, 64, 0, s>>>(w.G, w.Y, w.P1, w.Q1, nu, nullptr, nullptr, w.Z,
@@ -1412,6 +1441,10 @@ size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu) {
 // (device flag) and a third pass runs (its kernels return at once otherwise); the second
 // pass then falls back to the classic factorisation by itself. With R: two classic passes
 // and R = R2 R1.
+// nu > kChol32: a basis of condition ~30 .. 1000 passes FP32 but is left too far from orthonormal for
+// the near-identity factor. A classic second pass is then neither as orthogonal as two FP64 passes
+// (400 x 200, condition 100: 2.9e-15 against 1.1e-15) nor fast; the second pass takes another FP32
+// factor instead and the third one finishes. Columns of up to kChol32 keep the classic second pass.
 bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int nu,
                         double* R_dev, void* work, cudaStream_t s, uint64_t refresh_seed, void* split_mem) {
   const CqLayout L = cq_layout(ctx, n, nu);
@@ -1435,7 +1468,7 @@ bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int
   }
   if (refresh_seed != 0) {
     if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, refresh_seed, s)) != BEM_OK) return st;
-    return near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, s);
+    return near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, nullptr, s);
   }
   int* fallback = w.flags;
   double2* V = reinterpret_cast<double2*>(V_dev);
@@ -1455,31 +1488,18 @@ bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int
     st = cuda_check(ctx, cudaMemsetAsync(fallback, 0, sizeof(int), s), "cholqr flag");
     if (st != BEM_OK) return st;
     sum_parts_kernel<<<L.sum_blocks, 256, 0, s>>>(w.part, parts, nu, w.G, nullptr, nullptr);
-    const int h = std::min(nu, kChol32), r = nu - h;   // diagonal blocks of the FP32 factor
-    auto inverse32 = [&](const double2* G, int ldg, int m, double2* Z) {
-      auto* kernel = m <= 32 ? chol_inv32_kernel<1> : m <= 64 ? chol_inv32_kernel<2> : chol_inv32_kernel<4>;
-      kernel<<<1, 1024, 0, s>>>(G, ldg, m, w.G, nu, Z, nu, fallback);
-      ctx->launches++;
-    };
-    inverse32(w.G, nu, h, w.Z);
     ctx->launches++;
-    if (r > 0) {
-      const dim3 gh((unsigned)((h + 15) / 16), (unsigned)((r + 15) / 16)), gr(gh.y, gh.y);
-      chol_block32_kernel<0><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-      chol_block32_kernel<1><<<gr, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-      inverse32(w.Q, r, r, w.Z + (size_t)h * nu + h);
-      chol_block32_kernel<2><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-      chol_block32_kernel<3><<<gh, 256, 0, s>>>(w.G, w.Z, nu, w.P, w.Q, w.Y);
-      ctx->launches += 4;
-    }
+    factor32(ctx, w, nu, fallback, nullptr, s);
   }
   if ((st = multiply64(ctx, sp, wide, V, ldv, n, nu, w.Z, nullptr, fallback, s)) != BEM_OK) return st;
   if ((st = cuda_check(ctx, cudaGetLastError(), "cholqr kernels")) != BEM_OK) return st;
-  if ((st = near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, s)) != BEM_OK) return st;
+  const bool again = nu > kChol32;   // the third pass follows every second one that is not near
+  st = near_pass(ctx, V_dev, ldv, n, nu, L, w, sp, nullptr, w.flags + 1, again ? fallback : nullptr, s);
+  if (st != BEM_OK) return st;
   // the third pass rarely runs: for the smaller bases the form with the fewest launches
   Split64 third = sp;
   if (nu <= kSmallNu && n * (int64_t)nu * nu < ((int64_t)1 << 25)) third.use = false;
-  return near_pass(ctx, V_dev, ldv, n, nu, L, w, third, fallback, w.flags + 4, s);
+  return near_pass(ctx, V_dev, ldv, n, nu, L, w, third, again ? w.flags + 1 : fallback, w.flags + 4, nullptr, s);
 }
 
 }  // namespace bem

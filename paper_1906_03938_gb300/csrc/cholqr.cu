@@ -896,7 +896,7 @@ enum { kFactor32 = 0, kFactorNear = 1, kFactorClassic = 2 };
 struct FactorArgs {
   const double2* part;   // partial Gram matrices
   int parts, nu;
-  double2 *G, *P, *Y, *Z;
+  double2 *G, *Y, *Z;
   float4* Ms;            // Z - I split for the double-FP32 multiply
   int* flag;             // kFactor32: 1 = too ill-conditioned for FP32; kFactorNear: 1 = near route
   int* status;
@@ -1078,7 +1078,7 @@ cq_factor_kernel(FactorArgs p) {
   const int ld = nu + 1;   // (odd in 16-byte words: columns over all banks)
   double2* sG = factor_mem;            // [c][r], r <= c
   double2* sY = sG + nu * ld;
-  double2* sP = sY + nu * ld;          // this block's rows of P
+  double2* sP = sY + nu * ld;          // this block's columns of E + Y + E Y
   float2* yf = reinterpret_cast<float2*>(sY);
   float e2 = 0.f;
   for (int t = tid; t < nu * nu; t += kFactorThreads) {
@@ -1106,18 +1106,7 @@ cq_factor_kernel(FactorArgs p) {
     }
     return;
   }
-  auto e_at = [&](int m, int j) {
-    if (m > j) {
-      const double2 g = sG[m * ld + j];
-      return make_double2(g.x, -g.y);
-    }
-    const double2 g = sG[j * ld + m];
-    return m == j ? make_double2(g.x - 1.0, 0.0) : g;
-  };
-  // this thread's output: rows rank, rank + 8, ... of the block, a column each
-  const int i = rank + kFactorBlocks * (tid / kSmallNu), j = tid % kSmallNu;
-  const bool out = i < nu && j < nu;
-  auto finish = [&](double2 y) {   // Z = I + Y at (i, j), and its split
+  auto finish = [&](int i, int j, double2 y) {   // Z = I + Y at (i, j), and its split
     const int t = j * nu + i;
     const double2 z = i > j ? make_double2(0.0, 0.0) : i == j ? make_double2(1.0 + y.x, 0.0) : y;
     const double br = i == j ? z.x - 1.0 : z.x;
@@ -1125,62 +1114,72 @@ cq_factor_kernel(FactorArgs p) {
     const float fr = (float)br, fi = (float)z.y;
     p.Ms[t] = make_float4(fr, fi, (float)(br - fr), (float)(z.y - fi));
   };
-  auto y1_of = [&](double2 h) {
-    const double2 e = e_at(i, j);
+  auto y1_of = [&](int i, int j, double2 e, double2 h) {
     return i < j ? make_double2(h.x - e.x, h.y - e.y) : make_double2(-0.5 * (e.x - h.x), 0.0);
   };
   if (small) {   // as near_y1_kernel: FP32 second-order terms
-    if (!out) return;
+    // this thread's output: rows rank, rank + 8, ... of the block, a column each
+    const int i = rank + kFactorBlocks * (tid / kSmallNu), j = tid % kSmallNu;
+    if (i >= nu || j >= nu) return;
     double2 y = make_double2(0.0, 0.0);
     if (i <= j) {
+      const double2 g = sG[j * ld + i];
       const float2 h = second_order_at<float2>([&](int r, int c) { return yf[c * ld + r]; }, i, j);
-      y = y1_of(make_double2(h.x, h.y));
+      y = y1_of(i, j, i == j ? make_double2(g.x - 1.0, 0.0) : g, make_double2(h.x, h.y));
     }
-    finish(y);
+    finish(i, j, y);
     return;
   }
-  if (out && i <= j) {
-    auto y0 = [&](int r, int c) {
-      const double2 g = sG[c * ld + r];
-      return r == c ? make_double2(-0.5 * (g.x - 1.0), 0.0) : make_double2(-g.x, -g.y);
-    };
-    p.Y[j * nu + i] = y1_of(second_order_at<double2>(y0, i, j));
+  // Both steps in FP64. The second-order terms of the first are Y0^H Y0 + Y0^2 = -E Y0 in the upper
+  // triangle (E = -(Y0 + Y0^H)), and once more y0_ii^2 on the diagonal; the second step is
+  // -U(E + W + Y^H (E + Y + W)), W = E Y, of which its upper triangle needs W's alone. So a block
+  // takes columns rank, rank + 8, ..., a row a thread, and only Y1 goes round the cluster. FP64-bound:
+  // 3.3 nu^3 multiply-adds (P = Y^H E and Q = Y^H Y in full, by rows, took 6.7 and as many operations
+  // again to form Y0 and E: 222 us at nu = 64; now 137).
+  for (int c = tid; c < nu; c += kFactorThreads) sG[c * ld + c] = make_double2(sG[c * ld + c].x - 1.0, 0.0);
+  __syncthreads();   // sG holds E's upper triangle
+  const int i = tid % kSmallNu, own = tid / kSmallNu, j = rank + kFactorBlocks * own;
+  const bool upper = i <= j && j < nu;
+  auto e_at = [&](int r, int c) {
+    const double2 g = r > c ? sG[r * ld + c] : sG[c * ld + r];
+    return make_double2(g.x, r > c ? -g.y : g.y);
+  };
+  auto mac = [](double2& s, double2 a, double2 b) {
+    s.x += a.x * b.x - a.y * b.y;
+    s.y += a.x * b.y + a.y * b.x;
+  };
+  const double2 eij = upper ? e_at(i, j) : make_double2(0.0, 0.0);
+  if (upper) {
+    const double2* ej = sG + j * ld;
+    double2 h = make_double2(0.0, 0.0);
+    for (int m = 0; m < j; ++m) mac(h, e_at(i, m), ej[m]);
+    mac(h, eij, make_double2(0.5 * ej[j].x, 0.0));
+    if (i == j) h.x += 0.25 * eij.x * eij.x;
+    p.Y[j * nu + i] = y1_of(i, j, eij, h);
   }
   sm100::cluster_sync_all();
   for (int t = tid; t < nu * nu; t += kFactorThreads) {
     const int r = t % nu, c = t / nu;
-    sY[c * ld + r] = r <= c ? __ldcg(p.Y + t) : make_double2(0.0, 0.0);
+    if (r <= c) sY[c * ld + r] = __ldcg(p.Y + t);
   }
   __syncthreads();
-  double2 pe = make_double2(0.0, 0.0), q = pe;
-  if (out) {
-    for (int m = 0; m <= i; ++m) {
-      const double2 a = sY[i * ld + m], b = e_at(m, j), c = sY[j * ld + m];
-      pe.x += a.x * b.x + a.y * b.y;
-      pe.y += a.x * b.y - a.y * b.x;
-      q.x += a.x * c.x + a.y * c.y;
-      q.y += a.x * c.y - a.y * c.x;
-    }
-    sP[tid / kSmallNu * ld + j] = pe;
-    p.P[j * nu + i] = pe;
+  double2 x = make_double2(0.0, 0.0);
+  if (upper) {
+    const double2* yj = sY + j * ld;
+    for (int m = 0; m <= j; ++m) mac(x, e_at(i, m), yj[m]);
+    x.x += eij.x;
+    x.y += eij.y;
+    sP[own * ld + i] = make_double2(x.x + yj[i].x, x.y + yj[i].y);
   }
   __syncthreads();
-  sm100::cluster_sync_all();
-  if (!out) return;
+  if (i >= nu || j >= nu) return;
   double2 y = make_double2(0.0, 0.0);
-  if (i <= j) {
-    double2 h = e_at(i, j);
-    const double2 pt = __ldcg(p.P + i * nu + j);
-    h.x += pe.x + pt.x + q.x;
-    h.y += pe.y - pt.y + q.y;
-    for (int m = 0; m <= j; ++m) {
-      const double2 a = sP[tid / kSmallNu * ld + m], b = sY[j * ld + m];
-      h.x += a.x * b.x - a.y * b.y;
-      h.y += a.x * b.y + a.y * b.x;
-    }
-    y = i < j ? make_double2(-h.x, -h.y) : make_double2(-0.5 * h.x, 0.0);
+  if (upper) {
+    const double2 *yi = sY + i * ld, *pj = sP + own * ld;
+    for (int m = 0; m <= i; ++m) mac(x, make_double2(yi[m].x, -yi[m].y), pj[m]);
+    y = i < j ? make_double2(-x.x, -x.y) : make_double2(-0.5 * x.x, 0.0);
   }
-  finish(y);
+  finish(i, j, y);
 }
 
 // V <- V Z for nu <= kSmallNu: the near-identity product where *near says so, else in FP64.
@@ -1305,7 +1304,7 @@ bem_status multiply64(bem_ctx* ctx, const Split64& sp, bool same, double2* V, in
 template <int kMode>
 bem_status small_factor(bem_ctx* ctx, const CqWork& w, int parts, int nu, int* flag, int* deficient,
                         const int* gate, cudaStream_t s) {
-  const FactorArgs a{w.part, parts, nu, w.G, w.P, w.Y, w.Z, reinterpret_cast<float4*>(w.Q1),
+  const FactorArgs a{w.part, parts, nu, w.G, w.Y, w.Z, reinterpret_cast<float4*>(w.Q1),
                      flag, ctx->d_status, deficient, gate};
   auto* kernel = nu <= 32 ? cq_factor_kernel<kMode, 1> : cq_factor_kernel<kMode, 2>;
   if (factor_smem(kMode, nu) > 0) {   // (beside ~19 KB of its static arrays)

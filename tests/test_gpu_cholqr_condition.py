@@ -1,5 +1,5 @@
-"""CholeskyQR2 of bases wider than 128 columns and of condition 10 .. 1000, which the FP32 first factor
-accepts but does not leave orthonormal enough for the near-identity factor: the last pass is a near one
+"""CholeskyQR2 of bases of condition 3 .. 1000. Wider than 128 columns the FP32 first factor accepts
+them but does not leave them orthonormal enough for the near-identity factor: the last pass is a near one
 all the same. Q^H Q - I is summed in binary128 (or 64-bit extended). Bar 4 eps: the last pass rounds
 the entries of Q once (2.8 units of 2^-53 in an entry of Q^H Q at most), its factor and its Gram matrix
 once each (3 units); the digits' cuts are random and a fraction of a unit.
@@ -29,7 +29,7 @@ def test_orthonormal(n, nu, cond):
     Q = V.clone()
     ctx.cholqr2(Q, want_R=False)
     ctx.close()
-    cols = np.random.RandomState(0).permutation(nu)[:32]
+    cols = np.random.RandomState(0).permutation(nu)[:32]   # (all of narrower bases)
     q = Q.cpu().numpy().astype(np.clongdouble)
     err = np.abs(q.conj().T @ q[:, cols] - np.eye(nu)[:, cols])
     assert float(err.max()) <= 4 * EPS
@@ -37,6 +37,13 @@ def test_orthonormal(n, nu, cond):
     assert float((V - Q @ R).abs().max()) < 64 * EPS   # ||V|| = 1: the span is V's
     low = R.tril(-1)
     assert float(low.abs().max()) < 64 * EPS           # and R is triangular: Q is V's QR factor
+
+
+@pytest.mark.parametrize("cond", [3.0, 30.0, 60.0, 100.0, 150.0])
+@pytest.mark.parametrize("n, nu", [(40, 5), (300, 17), (500, 32), (500, 33), (1000, 63), (3072, 64)])
+def test_both_steps_of_narrow_bases(n, nu, cond):
+    """nu <= 64: one cluster forms the near-identity factor; for 1e-5 < ||G - I|| <= 5e-4 in two steps."""
+    test_orthonormal(n, nu, cond)
 
 
 @pytest.mark.parametrize("n, nu", [(400, 140), (1100, 256)])

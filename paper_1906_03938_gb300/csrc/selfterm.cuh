@@ -100,52 +100,6 @@ __device__ inline double2 hprime_fun(double2 w) {
   return make_double2((num.x * w2.x + num.y * w2.y) / d, (num.y * w2.x - num.x * w2.y) / d);
 }
 
-// Self term of the triangle with vertices v[0..2] about the point x, at wavenumber k.
-// (deriv = true: its derivative in k, the integral of i R^2 h'(i k R) d(phi), i.e.
-// i d^2 cosh(u) h'(i k d cosh u) du along each edge.)
-__device__ inline double2 self_term(const double v[3][3], const double x[3], double2 k,
-                                    const GL16& gl, bool deriv = false) {
-  double2 total = make_double2(0.0, 0.0);
-  for (int e = 0; e < 3; ++e) {
-    const double* p = v[e];
-    const double* q = v[(e + 1) % 3];
-    double tx = q[0] - p[0], ty = q[1] - p[1], tz = q[2] - p[2];
-    const double len = sqrt(tx * tx + ty * ty + tz * tz);
-    tx /= len;
-    ty /= len;
-    tz /= len;
-    const double px = p[0] - x[0], py = p[1] - x[1], pz = p[2] - x[2];
-    const double qx = q[0] - x[0], qy = q[1] - x[1], qz = q[2] - x[2];
-    const double sp = px * tx + py * ty + pz * tz;
-    const double sq = qx * tx + qy * ty + qz * tz;
-    const double ox = px - sp * tx, oy = py - sp * ty, oz = pz - sp * tz;
-    const double d = sqrt(ox * ox + oy * oy + oz * oz);
-    const double up = asinh(sp / d), uq = asinh(sq / d);
-    const bool split = up < 0.0 && uq > 0.0;
-    for (int s = 0; s < (split ? 2 : 1); ++s) {
-      const double lo = split ? (s == 0 ? up : 0.0) : up;
-      const double hi = split ? (s == 0 ? 0.0 : uq) : uq;
-      const double half = 0.5 * (hi - lo), mid = 0.5 * (hi + lo);
-      for (int gi = 0; gi < 16; ++gi) {
-        const double R = d * cosh(mid + half * gl.x[gi]);
-        const double2 wv = make_double2(-k.y * R, k.x * R);   // i k R
-        if (deriv) {
-          const double2 hp = hprime_fun(wv);
-          const double f = half * gl.w[gi] * d * R;         // d^2 cosh(u) = d R
-          total.x += -f * hp.y;                               // i * hp
-          total.y += f * hp.x;
-        } else {
-          const double2 h = h_fun(wv);
-          const double f = half * gl.w[gi] * d;
-          total.x += f * h.x;
-          total.y += f * h.y;
-        }
-      }
-    }
-  }
-  return make_double2(total.x / (4.0 * kPiD), total.y / (4.0 * kPiD));
-}
-
 // Edge data of the self term, FP64: for edge e = (v[e], v[e+1]) about the point x, the
 // distance d from x to the edge's line and the u = asinh(s / d) range of the edge.
 __device__ inline void self_edge(const double v[3][3], const double x[3], int e, double& d,
@@ -169,12 +123,15 @@ __device__ inline void self_edge(const double v[3][3], const double x[3], int e,
 
 // Self entries c_G A_ll(k) + c_H / 2 of panel l at nk wavenumbers (deriv: c_G A'_ll(k)), by one
 // warp: out[j n + l].
-// A_ll(k) = sum_p (i k rho)^p c_p, c_p = (1 / 4 pi) sum_g f_g (R_g / rho)^p / (p + 1)! over the 96
-// angular nodes, f_g their weights, R_g <= rho their radii (h(w) = sum_p w^p / (p + 1)!), so the
-// moments c_p serve every wavenumber: 24 terms are exact to 1e-18 for |k| rho <= 2, and a
-// wavenumber costs 24 complex multiply-adds where the sum over the angular nodes costs 96 sines,
-// exponentials and complex divisions. Larger |k| rho (a panel of a third of a wavelength)
-// take that sum. FP64-bound; 768 panels, 32 wavenumbers: 2.94 -> 0.055 ms.
+// A_ll(k) = (1 / 4 pi) sum_g f_g h(i k R_g) over the 96 angular nodes, f_g their weights, R_g <= rho
+// their radii; three nodes a lane. With h(w) = sum_p w^p / (p + 1)! it is sum_p (i k rho)^p c_p,
+// c_p = (1 / 4 pi) sum_g f_g (R_g / rho)^p / (p + 1)!, and the moments c_p serve every wavenumber: 24
+// terms are exact to 1e-18 for |k| rho <= 2, and a wavenumber costs 24 complex multiply-adds where
+// the sum over the angular nodes costs 96 sines, exponentials and complex divisions. Larger |k| rho (a
+// panel of a third of a wavelength) take that sum, the warp's lanes together for a wavenumber at a
+// time (by the one lane of a wavenumber, and after the moments, 96 nodes took 400 us where one thread
+// a panel had taken 200: residuals of one vector on 12 panels at k = 5). FP64-bound; 768 panels, 32
+// wavenumbers: 2.94 -> 0.055 ms.
 constexpr int kSelfTerms64 = 24;
 
 __device__ inline void self_entries_warp(const double v[3][3], const double x[3], int64_t l,
@@ -192,39 +149,54 @@ __device__ inline void self_entries_warp(const double v[3][3], const double x[3]
     rho2 = fmax(rho2, r2);
   }
   const double rho = sqrt(rho2), inv = 1.0 / rho;
-  double mom[kSelfTerms64];
+  double f[3], R[3];   // weights and radii of this lane's nodes, one of every edge
 #pragma unroll
-  for (int p = 0; p < kSelfTerms64; ++p) mom[p] = 0.0;
-#pragma unroll 1
-  for (int e = 0; e < 3; ++e) {   // this lane's node of edge e: side lane / 16, node lane % 16
+  for (int e = 0; e < 3; ++e) {   // side lane / 16, node lane % 16
     const double d = __shfl_sync(0xffffffffu, d_, e), up = __shfl_sync(0xffffffffu, up_, e),
                  uq = __shfl_sync(0xffffffffu, uq_, e);
     const bool split = up < 0.0 && uq > 0.0;
     const int side = lane / 16, gi = lane % 16;
     const double lo = split && side ? 0.0 : up, hi = split && !side ? 0.0 : uq;
     const double half = 0.5 * (hi - lo), mid = 0.5 * (hi + lo);
-    double f = (split || side == 0) ? half * gl.w[gi] * d : 0.0;
-    const double t = d * cosh(mid + half * gl.x[gi]) * inv;
+    f[e] = (split || side == 0) ? half * gl.w[gi] * d : 0.0;
+    R[e] = d * cosh(mid + half * gl.x[gi]);
+  }
+  auto series = [&](double2 kj) { return (kj.x * kj.x + kj.y * kj.y) * rho2 <= 4.0; };
+  auto put = [&](int j, double2 a) {
+    out[(int64_t)j * n + l] = make_double2(cgr * a.x - cgi * a.y + (deriv ? 0.0 : 0.5 * chr),
+                                           cgr * a.y + cgi * a.x + (deriv ? 0.0 : 0.5 * chi));
+  };
+  bool near = false, far = false;
+  for (int j = lane; j < nk; j += 32) (series(k[j]) ? near : far) = true;
+  near = __any_sync(0xffffffffu, near);
+  far = __any_sync(0xffffffffu, far);
+  if (near) {
+    double mom[kSelfTerms64];
+#pragma unroll
+    for (int p = 0; p < kSelfTerms64; ++p) mom[p] = 0.0;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const double t = R[e] * inv;
+      double g = f[e];
+#pragma unroll
+      for (int p = 0; p < kSelfTerms64; ++p) {
+        mom[p] += g;
+        g *= t;
+      }
+    }
+    double fact = 1.0;
 #pragma unroll
     for (int p = 0; p < kSelfTerms64; ++p) {
-      mom[p] += f;
-      f *= t;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) mom[p] += __shfl_xor_sync(0xffffffffu, mom[p], off);
+      fact *= 1.0 / (p + 1);
+      mom[p] *= fact * (1.0 / (4.0 * kPiD));
     }
-  }
-  double fact = 1.0;
-#pragma unroll
-  for (int p = 0; p < kSelfTerms64; ++p) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mom[p] += __shfl_xor_sync(0xffffffffu, mom[p], off);
-    fact *= 1.0 / (p + 1);
-    mom[p] *= fact * (1.0 / (4.0 * kPiD));
-  }
-  for (int j = lane; j < nk; j += 32) {
-    const double2 kj = k[j];
-    double2 a;
-    if ((kj.x * kj.x + kj.y * kj.y) * rho2 <= 4.0) {
+    for (int j = lane; j < nk; j += 32) {
+      const double2 kj = k[j];
+      if (!series(kj)) continue;
       const double2 w = make_double2(-kj.y * rho, kj.x * rho);   // i k rho
-      a = make_double2(0.0, 0.0);
+      double2 a = make_double2(0.0, 0.0);
       if (deriv) {   // i rho sum_p p c_p w^{p-1}
 #pragma unroll
         for (int p = kSelfTerms64 - 1; p >= 1; --p)
@@ -235,11 +207,35 @@ __device__ inline void self_entries_warp(const double v[3][3], const double x[3]
         for (int p = kSelfTerms64 - 1; p >= 0; --p)
           a = make_double2(fma(a.x, w.x, fma(-a.y, w.y, mom[p])), fma(a.x, w.y, a.y * w.x));
       }
-    } else {
-      a = self_term(v, x, kj, gl, deriv);
+      put(j, a);
     }
-    out[(int64_t)j * n + l] = make_double2(cgr * a.x - cgi * a.y + (deriv ? 0.0 : 0.5 * chr),
-                                           cgr * a.y + cgi * a.x + (deriv ? 0.0 : 0.5 * chi));
+  }
+  if (!far) return;
+  for (int j = 0; j < nk; ++j) {
+    const double2 kj = k[j];
+    if (series(kj)) continue;
+    double2 a = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int e = 0; e < 3; ++e) {
+      const double fe = e == 0 ? f[0] : e == 1 ? f[1] : f[2];
+      const double Re = e == 0 ? R[0] : e == 1 ? R[1] : R[2];
+      const double2 w = make_double2(-kj.y * Re, kj.x * Re);   // i k R
+      if (deriv) {   // the integral of i R^2 h'(i k R): f_g holds one R
+        const double2 hp = hprime_fun(w);
+        a.x -= fe * Re * hp.y;
+        a.y += fe * Re * hp.x;
+      } else {
+        const double2 h = h_fun(w);
+        a.x += fe * h.x;
+        a.y += fe * h.y;
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
+      a.y += __shfl_xor_sync(0xffffffffu, a.y, off);
+    }
+    if (lane == 0) put(j, make_double2(a.x / (4.0 * kPiD), a.y / (4.0 * kPiD)));
   }
 }
 

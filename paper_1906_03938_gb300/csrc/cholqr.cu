@@ -1230,10 +1230,12 @@ CqLayout cq_layout(bem_ctx* ctx, int64_t n, int nu) {
   const int T = (nu + kGT - 1) / kGT;
   L.tiles_u = T * (T + 1) / 2;
   // no fewer than 4 rows a part: a 32 x 32 tile of a row is 0.8 us of an SM's FP64 pipe, so a short
-  // V is spread thin (320 x 16: 27 us at 32 rows a part, 5.6 us at 4); one block an SM where a
-  // single cluster adds the parts
+  // V is spread thin (320 x 16: 27 us at 32 rows a part, 5.6 us at 4); at most one block an SM where
+  // a single cluster adds the parts (one block more, 51 parts of 3 tiles, doubles the time of the
+  // slowest SM: 3000 x 33 with R 690 us, now 591)
   const int64_t blocks = (nu <= kSmallNu ? 1 : 2) * (int64_t)std::max(1, sms);
-  L.parts = std::max<int64_t>(1, std::min<int64_t>((n + 3) / 4, (blocks + L.tiles_u - 1) / L.tiles_u));
+  L.parts = nu <= kSmallNu ? blocks / L.tiles_u : (blocks + L.tiles_u - 1) / L.tiles_u;
+  L.parts = std::max<int64_t>(1, std::min<int64_t>((n + 3) / 4, L.parts));
   L.rows_per_part = (n + L.parts - 1) / L.parts;
   L.parts = (n + L.rows_per_part - 1) / L.rows_per_part;
   L.rows32 = std::max<int64_t>(L.rows_per_part, kGT);

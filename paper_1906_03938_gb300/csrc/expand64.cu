@@ -40,6 +40,12 @@ constexpr size_t kMomentBytes = (size_t)1 << 30;   // moments held at a time
 // panels, 8 vectors 580 / 601, 3072 panels, 2 vectors 5853 / 8346 above.
 constexpr double kSplitWork = 0x1.cp23;
 constexpr size_t kMaxWork = (size_t)24 << 30;      // workspace beyond which the direct form runs
+// Panels below which the direct form runs: its threads pass over the columns one after the other (7 us
+// a column in a projection, 16 in a residual), the expansion's launches take the same time for any few
+// panels. Expanded against direct, in us: projections at 16 nodes 250 / 125 (12 panels), 282 / 233 (24),
+// 280 / 266 (32), 288 / 355 (48), with both operators 372 / 140, 425 / 283, 420 / 334, 424 / 456;
+// residuals 170 / 158 (2), 183 / 195 (4), 217 / 321 (12).
+constexpr int64_t kMinNodes = 40, kMinColumns = 4;
 // |Re c| R beyond which the direct form runs. The fixed-point phase of every pair is off by up to
 // 2^-59 |Re c| R radians, whatever their distance, the direct form's by 2^-53 k r: for bodies far
 // apart (R of 1e4, 1e6 bodies' sizes at k = 10: 5e-14, 8e-12 in their own entries) that is the
@@ -479,6 +485,7 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, doubl
   const OpCoef& op = ctx->op;
   const bool hasG = op.cgr != 0.0 || op.cgi != 0.0, hasH = op.chr != 0.0 || op.chi != 0.0;
   const int64_t n = ctx->geo.n;
+  if (n < (nodes ? kMinNodes : kMinColumns)) return p;
   p.R = mesh_reach(ctx);
   if (!(p.R > 0.0) || !isfinite(p.R) || !isfinite(1.0 / p.R)) return p;
   double dmax = 0.0, growth = 0.0;

@@ -160,16 +160,18 @@ using namespace bem;
 namespace {
 
 // Whether the FP64 expansion is faster than the double-FP32 kernel (its time depends on the
-// columns, the expansion's hardly does), in us from 300 to 4800 panels:
+// columns, the expansion's hardly does), in us, both with the self terms:
+//   12 panels 217 / 155, 32 227 / 208, 48 232 / 249, 64 235 / 292, 108 259 / 407;
 //   4800 panels: 16.9 ms for any number of columns against 7.8 ms at 4, 22.8 ms at 12; 768 panels
 //   0.76 ms against 0.61 at 8, 0.79 at 12; the near pairs 15 ns once against 23 ns a column (4800
 //   panels with near field, 12 columns: 19.4 against 67.8 ms).
 bool expand_beats_ff(const bem_ctx* ctx, const ExpandPlan& ex, int m, bool deriv) {
   const double n2 = (double)ctx->geo.n * (double)ctx->geo.n;
   const double pairs = near_active(ctx) ? (double)ctx->near_nnz : 0.0;
-  const double expand = 300.0 + n2 * ex.cost / 5.3e5 + pairs * 0.015;
-  const double ff = std::max(450.0, 200.0 + n2 * m * 0.082e-3) + pairs * m * 0.023;
-  return (deriv ? 2.0 : 1.0) * expand < 0.9 * ff;
+  const double expand = 240.0 + n2 * ex.cost / 5.3e5 + pairs * 0.015;
+  const double few = std::min(450.0, 125.0 + 2.6 * (double)ctx->geo.n);
+  const double ff = std::max(few, 200.0 + n2 * m * 0.082e-3) + pairs * m * 0.023;
+  return ex.use && (deriv ? 2.0 : 1.0) * expand < 0.9 * ff;
 }
 
 bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const double* X_dev,

@@ -509,14 +509,15 @@ near_slots64_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__
   const int32_t e0 = ptr[i], e1 = ptr[i + 1];
   if (e0 == e1) return;
   for (int c = lane; c < nu; c += 32) {
-    double2 acc = Ys[((int64_t)s * nu + c) * n + i];
+    double2 acc = make_double2(0.0, 0.0);   // the corrections, small beside the product they go to
     for (int32_t e = e0; e < e1; ++e) {
       const double2 m = C[(int64_t)s * nnz + e];
       const double2 v = Xt[(int64_t)cols[e] * nu + c];
       acc.x = fma(m.x, v.x, fma(-m.y, v.y, acc.x));
       acc.y = fma(m.x, v.y, fma(m.y, v.x, acc.y));
     }
-    Ys[((int64_t)s * nu + c) * n + i] = acc;
+    double2* y = Ys + ((int64_t)s * nu + c) * n + i;
+    *y = make_double2(y->x + acc.x, y->y + acc.y);
   }
 }
 

@@ -7,10 +7,13 @@
 // of wavenumbers. So
 //     A(k_j) = sum_m a_m(k_j) G_m,   G_m,il = sum_q w_q e^{i c r_q} / r_q T_m(x_q),
 // and A(k_j) X = sum_m a_m(k_j) (G_m X): one evaluation (a sine, cosine and root per point)
-// and M matrix products in the place of N of each. The general operator
-// c_G G + c_H (1/2 I + K) adds a second family of moments, H_m with the weight
-// w_q s_q / r_q, s = (y - x).n / r^2, and the coefficients of (i k r - 1) e^{i (k - c) r}; the
-// k-derivative only changes the coefficients.
+// and M matrix products in the place of N of each. All families of moments take this one series;
+// powers of r go into their weights. The general operator c_G G + c_H (1/2 I + K), whose second kernel
+// is (i k r - 1) e^{ikr} s / r, s = (y - x).n / r^2, adds H_m of weight w s / r with the factor -c_H and
+// J_m of weight w s with i k c_H; the k-derivative has G_m of weight w with i c_G and J_m of weight
+// w s r with -k c_H. (A series of (i k r - 1) e^{i (k - c) r} has coefficients of ~k R / 2 beside a
+// value of 1 at r = 0, and with them the rounding of near entries: residuals of the Robin operator at
+// k R = 14 were off by 7.3e-16 against 128-bit sums, the direct form by 3.0e-16, now by 2.6e-16.)
 //
 // Bound by arithmetic: 7 points of 15 FP64 operations and ~(110 + 26 M) integer ones per entry
 // (below), and M nu products, in FP64 (1/64 of the FP32 rate on this part) or, the larger ones,
@@ -52,27 +55,32 @@ constexpr int64_t kMinNodes = 40, kMinColumns = 4;
 // larger error. Up to here it is at most 2^-52, an ulp.
 constexpr double kMaxPhase = 128.0;
 // max |Im (k - c)| R beyond which the direct form runs. The series of e^{i (k - c) r} has coefficients
-// of up to e^{|Im (k - c)| R} whatever r, so the moments' rounding enters near entries that much
-// larger. Against 128-bit products on the unit sphere (R = 2), 16 nodes: dense bases, error of a
-// column's largest entry, expanded / direct: 1.2e-15 / 1.4e-15 at 1.6, 1.7e-15 / 1.6e-15 at 3.2,
-// 1.7e-15 / 2.1e-15 at 4.0, but 1.8e-15 / 1.2e-15 at 4.8; of (|A| |x|)_i for vectors of four panels
-// 1.0e-15 / 6e-16, 2.4e-15 / 7e-16, 4.0e-15 / 8e-16 and 7.6e-15 / 8e-16 (5.6: 1.7e-14).
-constexpr double kMaxGrowth = 4.0;
+// of up to e^{|Im (k - c)| R} whatever r, so the rounding of moments and slot products enters near
+// entries that much larger. Against 128-bit products, expanded / direct, error of ||A X|| (300 panels,
+// single layer, Neumann, Robin):
+//   projections at the lowest nodes: 4.6e-16 / 8.3e-16, 2.6e-16 / 6.1e-16, 2.8e-16 / 8.8e-16 at 1.2,
+//     1.3e-15 / 1.4e-15, 6.6e-16 / 8.8e-16, 1.2e-15 / 1.4e-15 at 3.2 (a contour of radius 1.6); the
+//     other nodes and V^H A V a third of the direct form's. Vectors of four panels lose more, by
+//     component of (|A| |x|)_i 4.0e-15 / 8e-16 at 4.0 (80 panels) and 1.7e-14 at 5.6.
+//   residuals, whose direct form sums more exactly: 4.7e-16 / 5.5e-16, 2.9e-16 / 3.0e-16,
+//     2.9e-16 / 3.1e-16 near the axis, 5.4e-16 / 5.5e-16, 3.1e-16 / 3.2e-16, 3.1e-16 / 3.2e-16 at 0.6,
+//     but 7.3e-16 / 5.7e-16, 3.7e-16 / 3.5e-16 at 1.4.
+constexpr double kMaxGrowthNodes = 4.0, kMaxGrowthColumns = 0.6;
 
-// a[f][j][m], f the family: Chebyshev coefficients on [0, R] of the family's function of r at
-// wavenumber k_j, times the operator's coefficient of the family. One block per (j, f): a thread
+// a[f][j][m], f the family: Chebyshev coefficients on [0, R] of e^{i (k_j - c) r}, times the family's
+// factor. One block per (j, f): a thread
 // per Chebyshev point for the function, a thread per angle for the cosines cos(pi t / 128) that
 // the sums take, then a warp per coefficient. (A thread per coefficient with the cosines of all
 // its points took 196 us, the points shared 56 us at 32 wavenumbers; now 8 us.)
 constexpr int kCoefThreads = 256;
 
 __global__ void __launch_bounds__(kCoefThreads)
-expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, int M,
-                   int first_fam, bool deriv, OpCoef op, double2* __restrict__ a) {
+expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, int M, bool hasG,
+                   bool deriv, OpCoef op, double2* __restrict__ a) {
   static_assert(kCoefThreads == 4 * kCoefPoints, "an angle a thread");
   __shared__ double2 fv[kCoefPoints];
   __shared__ double cosine[kCoefThreads];
-  const int j = blockIdx.x, f = first_fam + blockIdx.y, q = threadIdx.x;
+  const int j = blockIdx.x, q = threadIdx.x;
   const double2 kj = k[j];
   cosine[q] = cospi(q / (2.0 * kCoefPoints));
   __syncthreads();
@@ -82,18 +90,19 @@ expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, i
     double sn, cs;
     sincos(dr * r, &sn, &cs);
     const double e = exp(-di * r);
-    // the family's factor at r: 1 or (i k r - 1), and their k-derivatives i r and -k r^2
-    double gr, gi;
-    if (f == 0) {
-      gr = deriv ? 0.0 : 1.0;
-      gi = deriv ? r : 0.0;
-    } else {
-      gr = deriv ? -kj.x * r * r : -kj.y * r - 1.0;
-      gi = deriv ? -kj.y * r * r : kj.x * r;
-    }
-    fv[q] = make_double2(e * (cs * gr - sn * gi), e * (cs * gi + sn * gr));
+    fv[q] = make_double2(e * cs, e * sn);
   }
   __syncthreads();
+  // the family's factor
+  double2 fac;
+  if (hasG && blockIdx.y == 0) {
+    fac = deriv ? make_double2(-op.cgi, op.cgr) : make_double2(op.cgr, op.cgi);
+  } else {
+    const double2 kc = make_double2(kj.x * op.chr - kj.y * op.chi, kj.x * op.chi + kj.y * op.chr);   // k c_H
+    if (deriv) fac = make_double2(-kc.x, -kc.y);
+    else if (blockIdx.y == (hasG ? 1 : 0)) fac = make_double2(-op.chr, -op.chi);
+    else fac = make_double2(-kc.y, kc.x);
+  }
   const int lane = q % 32;
   for (int m = q / 32; m < M; m += kCoefThreads / 32) {
     double2 s = make_double2(0.0, 0.0);
@@ -109,10 +118,9 @@ expand_coef_kernel(const double2* __restrict__ k, int nk, double2 c, double R, i
       s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
     }
     const double sc = (m == 0 ? 1.0 : 2.0) / kCoefPoints;
-    const double or_ = f == 0 ? op.cgr : op.chr, oi = f == 0 ? op.cgi : op.chi;
     if (lane == 0)
       a[((int64_t)blockIdx.y * nk + j) * M + m] =
-          make_double2(sc * (s.x * or_ - s.y * oi), sc * (s.x * oi + s.y * or_));
+          make_double2(sc * (s.x * fac.x - s.y * fac.y), sc * (s.x * fac.y + s.y * fac.x));
   }
 }
 
@@ -143,11 +151,11 @@ __global__ void expand_angles_kernel(int4* __restrict__ table) {
 // Moments of the columns [l0, l0 + kc): G[f M + m][l - l0][i] (i fastest). One thread per row;
 // the block's columns' geometry is staged in shared memory and read by broadcast. The
 // diagonal is zero (the self terms are added in closed form).
-template <int MT, bool kG, bool kH>
+template <int MT, int kKind>
 __global__ void __launch_bounds__(kRowsE)
 expand_moments_kernel(Geometry g, double2 c, FixedPhase fp, int M, int64_t l0, int kc,
                       const int4* __restrict__ angles, double2* __restrict__ G) {
-  constexpr int F = (kG ? 1 : 0) + (kH ? 1 : 0);
+  constexpr int F = kFamilies<kKind>;
   __shared__ int4 table[kAngles];
   __shared__ double sq[kColsE][7][4];
   __shared__ double sn3[kColsE][3];
@@ -167,7 +175,7 @@ expand_moments_kernel(Geometry g, double2 c, FixedPhase fp, int M, int64_t l0, i
     sq[cc][q][2] = g.qp[(14 + q) * n + l];
     sq[cc][q][3] = g.qw[q * n + l];
   }
-  if (kH)
+  if (kKind >= kDouble)
     for (int t = tid; t < nc * 3; t += kRowsE) sn3[t / 3][t % 3] = g.nrm[(t % 3) * n + l0 + c0 + t / 3];
   __syncthreads();
   if (i >= n) return;
@@ -195,10 +203,11 @@ expand_moments_kernel(Geometry g, double2 c, FixedPhase fp, int M, int64_t l0, i
         double r, ri;
         root_and_inverse(r2, r, ri);
         srho[q][tid] = fixed62(r * fp.inv_R, 0);
-        double w = sq[cc][q][3] * ri;
-        if (c.y != 0.0) w *= exp(-c.y * r);
-        if (kG) sbase[q][0][tid] = w;
-        if (kH) sbase[q][F - 1][tid] = w * ri * ri * (dx * sn3[cc][0] + dy * sn3[cc][1] + dz * sn3[cc][2]);
+        const double dn = kKind >= kDouble ? dx * sn3[cc][0] + dy * sn3[cc][1] + dz * sn3[cc][2] : 0.0;
+        double w[F];
+        moment_weights<kKind>(w, sq[cc][q][3], r, ri, dn, c.y);
+#pragma unroll
+        for (int f = 0; f < F; ++f) sbase[q][f][tid] = w[f];
 #pragma unroll
         for (int f = 0; f < F; ++f)
           top[f] = max(top[f], __double2hiint(sbase[q][f][tid]) & 0x7FFFFFFF);
@@ -355,13 +364,9 @@ expand_nodes_kernel(const double2* __restrict__ Ys, int64_t n, int nu, int M, in
   const int cl = (int)(t / n);
   const int j0 = blockIdx.y * kNodesC;
   const double2 v = V[(int64_t)cl * ldv + i];
-  double2 acc[kNodesC];
+  double2 acc[kNodesC];   // the slots' sum; the self term, half of the vector for K, last
 #pragma unroll
-  for (int u = 0; u < kNodesC; ++u) {
-    const int j = min(j0 + u, N - 1);
-    const double2 d = self[(int64_t)j * n + i];
-    acc[u] = make_double2(d.x * v.x - d.y * v.y, d.x * v.y + d.y * v.x);
-  }
+  for (int u = 0; u < kNodesC; ++u) acc[u] = make_double2(0.0, 0.0);
   for (int f = 0; f < fams; ++f)
     for (int m = 0; m < M; ++m) {
       const double2 y = Ys[(int64_t)(f * M + m) * n * nu + t];
@@ -374,7 +379,11 @@ expand_nodes_kernel(const double2* __restrict__ Ys, int64_t n, int nu, int M, in
     }
 #pragma unroll
   for (int u = 0; u < kNodesC; ++u)
-    if (j0 + u < N) Y[(int64_t)(j0 + u) * n * nu + t] = acc[u];
+    if (j0 + u < N) {
+      const double2 d = self[(int64_t)(j0 + u) * n + i];
+      Y[(int64_t)(j0 + u) * n * nu + t] = make_double2(acc[u].x + (d.x * v.x - d.y * v.y),
+                                                       acc[u].y + (d.x * v.y + d.y * v.x));
+    }
 }
 
 // R_c = sum_s a_s(k_c) Y_s,c + R_c x_c (R holds the self terms at k_c).
@@ -386,8 +395,7 @@ __global__ void expand_columns_kernel(const double2* __restrict__ Ys, int64_t n,
   if (t >= n * m) return;
   const int64_t i = t % n;
   const int c = (int)(t / n);
-  const double2 x = X[(int64_t)c * ldx + i], d = R[t];
-  double2 acc = make_double2(d.x * x.x - d.y * x.y, d.x * x.y + d.y * x.x);
+  double2 acc = make_double2(0.0, 0.0);   // the slots' sum; the self term last (expand_nodes_kernel)
   for (int f = 0; f < fams; ++f)
     for (int q = 0; q < M; ++q) {
       const double2 y = Ys[(int64_t)(f * M + q) * n * m + t];
@@ -395,26 +403,27 @@ __global__ void expand_columns_kernel(const double2* __restrict__ Ys, int64_t n,
       acc.x = fma(w.x, y.x, fma(-w.y, y.y, acc.x));
       acc.y = fma(w.x, y.y, fma(w.y, y.x, acc.y));
     }
-  R[t] = acc;
+  const double2 x = X[(int64_t)c * ldx + i], d = R[t];
+  R[t] = make_double2(acc.x + (d.x * x.x - d.y * x.y), acc.y + (d.x * x.y + d.y * x.x));
 }
 
 using MomentKernel = void (*)(Geometry, double2, FixedPhase, int, int64_t, int, const int4*, double2*);
 
-template <bool kG, bool kH>
+template <int kKind>
 MomentKernel moment_kernel(int M) {
-  if (M <= 1) return expand_moments_kernel<1, kG, kH>;
-  if (M <= 8) return expand_moments_kernel<8, kG, kH>;
-  if (M <= 10) return expand_moments_kernel<10, kG, kH>;
-  if (M <= 12) return expand_moments_kernel<12, kG, kH>;
-  if (M <= 13) return expand_moments_kernel<13, kG, kH>;
-  if (M <= 14) return expand_moments_kernel<14, kG, kH>;
-  if (M <= 15) return expand_moments_kernel<15, kG, kH>;
-  if (M <= 16) return expand_moments_kernel<16, kG, kH>;
-  if (M <= 17) return expand_moments_kernel<17, kG, kH>;
-  if (M <= 18) return expand_moments_kernel<18, kG, kH>;
-  if (M <= 20) return expand_moments_kernel<20, kG, kH>;
-  if (M <= 24) return expand_moments_kernel<24, kG, kH>;
-  return expand_moments_kernel<kMaxTerms, kG, kH>;
+  if (M <= 1) return expand_moments_kernel<1, kKind>;
+  if (M <= 8) return expand_moments_kernel<8, kKind>;
+  if (M <= 10) return expand_moments_kernel<10, kKind>;
+  if (M <= 12) return expand_moments_kernel<12, kKind>;
+  if (M <= 13) return expand_moments_kernel<13, kKind>;
+  if (M <= 14) return expand_moments_kernel<14, kKind>;
+  if (M <= 15) return expand_moments_kernel<15, kKind>;
+  if (M <= 16) return expand_moments_kernel<16, kKind>;
+  if (M <= 17) return expand_moments_kernel<17, kKind>;
+  if (M <= 18) return expand_moments_kernel<18, kKind>;
+  if (M <= 20) return expand_moments_kernel<20, kKind>;
+  if (M <= 24) return expand_moments_kernel<24, kKind>;
+  return expand_moments_kernel<kMaxTerms, kKind>;
 }
 
 // K = c / (2 pi inv_R) in turns, in two FP64 parts before it is rounded to 62 - kb bits.
@@ -480,7 +489,7 @@ int series_terms(double dmax, double R) {
 }  // namespace
 
 ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, double c_im, int ncols,
-                       bool nodes, bool deriv) {
+                       bool nodes, bool deriv, int arith) {
   ExpandPlan p;
   const OpCoef& op = ctx->op;
   const bool hasG = op.cgr != 0.0 || op.cgi != 0.0, hasH = op.chr != 0.0 || op.chi != 0.0;
@@ -493,24 +502,26 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, doubl
     dmax = std::max(dmax, hypot(k[2 * j] - c_re, k[2 * j + 1] - c_im));
     growth = std::max(growth, fabs(k[2 * j + 1] - c_im));
   }
+  // (double-FP32 residuals, good to 1e-13, have the projections' bound)
+  const double max_growth = nodes || arith == 1 ? kMaxGrowthNodes : kMaxGrowthColumns;
   p.M = series_terms(dmax, p.R);
   // about a real centre no exponential is evaluated: for values near the axis, at most a term more
   if (c_im != 0.0 && series_terms(dmax + fabs(c_im), p.R) <= p.M + 1 &&
-      (growth + fabs(c_im)) * p.R <= kMaxGrowth) {
+      (growth + fabs(c_im)) * p.R <= max_growth) {
     dmax += fabs(c_im);
     growth += fabs(c_im);
     c_im = 0.0;
     p.M = series_terms(dmax, p.R);
   }
-  if (!(growth * p.R <= kMaxGrowth)) return p;
+  if (!(growth * p.R <= max_growth)) return p;
   p.c = make_double2(c_re, c_im);
   if (!(fabs(c_re) * p.R <= kMaxPhase)) return p;
   p.phase = fixed_phase(c_re, p.R);
-  if (p.M > 1 && (hasH || deriv)) p.M += 2;
-  if (p.M == 1 && (hasH || deriv)) p.M = 3;   // factors 1, r, r^2
   if (p.M < 1 || p.M > kMaxTerms) return p;
-  p.first = hasG ? 0 : 1;
-  p.fams = (hasG ? 1 : 0) + (hasH ? 1 : 0);
+  p.hasG = hasG;
+  p.nh = hasH ? (deriv ? 1 : 2) : 0;
+  p.fams = (hasG ? 1 : 0) + p.nh;
+  p.deriv = deriv;
   p.S = p.fams * p.M;
   const int tn = ncols <= 8 ? 8 : 32;
   const double padded = (double)((ncols + tn - 1) / tn * tn);
@@ -520,8 +531,10 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, doubl
   // together), the split products 7 a moment and 4 per 32 columns. The direct forms take ~1950 a
   // column for residuals (4800 panels, one vector: 85 ms, expanded 12.4 ms) and 540 + 4 nu a node
   // or more for projections (768 panels, 64 columns: 1000).
-  const double eval = 7.0 * (15.0 + (p.c.y != 0.0 ? 22.0 : 0.0) + (110.0 + (12.0 + 14.0 * p.fams) * p.M) / 28.0);
-  p.cost = eval + (p.split ? p.S * (7.0 + 4.0 * ((ncols + 31) / 32)) : 3.0 * p.S * padded);
+  auto evaluation = [&](int fams) {
+    return fams == 0 ? 0.0 : 7.0 * (15.0 + (p.c.y != 0.0 ? 22.0 : 0.0) + (110.0 + (12.0 + 14.0 * fams) * p.M) / 28.0);
+  };
+  p.cost = evaluation(hasG ? 1 : 0) + evaluation(p.nh) + (p.split ? p.S * (7.0 + 4.0 * ((ncols + 31) / 32)) : 3.0 * p.S * padded);
   const double expand = p.cost;
   const double direct = nodes ? nk * (7.0 * 77.0 + 4.0 * ncols) : ncols * 1950.0;
   if (!(expand < direct)) return p;
@@ -556,17 +569,17 @@ namespace {
 
 // The slot products Y_s = G_s X into the workspace, near-field corrections included.
 bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const double* k_dev,
-                     const double* X, int64_t ldx, int ncols, bool deriv, char* work,
-                     cudaStream_t s) {
+                     const double* X, int64_t ldx, int ncols, char* work, cudaStream_t s) {
   const int64_t n = ctx->geo.n;
   double2* a = reinterpret_cast<double2*>(work + p.coef_off);
   double2* G = reinterpret_cast<double2*>(work + p.mom_off);
   double2* Yp = reinterpret_cast<double2*>(work + p.y_off);
   expand_coef_kernel<<<dim3((unsigned)nk, (unsigned)p.fams), kCoefThreads, 0, s>>>(
-      reinterpret_cast<const double2*>(k_dev), nk, p.c, p.R, p.M, p.first, deriv, ctx->op, a);
-  MomentKernel mk = p.fams == 2 ? moment_kernel<true, true>(p.M)
-                                : (p.first == 0 ? moment_kernel<true, false>(p.M)
-                                                : moment_kernel<false, true>(p.M));
+      reinterpret_cast<const double2*>(k_dev), nk, p.c, p.R, p.M, p.hasG, p.deriv, ctx->op, a);
+  // the single layer's family and the double layer's by a launch each (the sums of three do not fit
+  // the registers)
+  const MomentKernel single = p.deriv ? moment_kernel<kSingleDeriv>(p.M) : moment_kernel<kSingle>(p.M);
+  const MomentKernel dbl = p.deriv ? moment_kernel<kDoubleDeriv>(p.M) : moment_kernel<kDouble>(p.M);
   int4* angles = reinterpret_cast<int4*>(work);
   expand_angles_kernel<<<kAngles / 128, 128, 0, s>>>(angles);
   const FixedPhase fp = p.phase;
@@ -579,8 +592,10 @@ bem_status expand_products(bem_ctx* ctx, const ExpandPlan& p, int nk, const doub
   for (int64_t l0 = 0; l0 < n; l0 += p.kc) {
     const int kc = (int)std::min<int64_t>(p.kc, n - l0);
     const dim3 ge((unsigned)((n + kRowsE - 1) / kRowsE), (unsigned)((kc + kColsE - 1) / kColsE));
-    mk<<<ge, kRowsE, 0, s>>>(ctx->geo, p.c, fp, p.M, l0, kc, angles, G);
-    ctx->launches++;
+    if (p.hasG) single<<<ge, kRowsE, 0, s>>>(ctx->geo, p.c, fp, p.M, l0, kc, angles, G);
+    if (p.nh > 0)
+      dbl<<<ge, kRowsE, 0, s>>>(ctx->geo, p.c, fp, p.M, l0, kc, angles, G + (p.hasG ? (int64_t)p.M * kc * n : 0));
+    ctx->launches += (p.hasG ? 1 : 0) + (p.nh > 0 ? 1 : 0);
     if (p.split) {
       const bem_status st = split64_batch(ctx, p.batch, work + p.batch_off, G, (int64_t)kc * n, kc,
                                           Xd + l0, ldx, l0 > 0, Yp, s);
@@ -611,7 +626,7 @@ bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V
   char* w = static_cast<char*>(work);
   const int N = ctx->con.N;
   const int64_t n = ctx->geo.n;
-  const bem_status st = expand_products(ctx, p, N, ctx->con.z, V, ldv, nu, false, w, s);
+  const bem_status st = expand_products(ctx, p, N, ctx->con.z, V, ldv, nu, w, s);
   if (st != BEM_OK) return st;
   const dim3 g((unsigned)((n * nu + 127) / 128), (unsigned)((N + kNodesC - 1) / kNodesC));
   expand_nodes_kernel<<<g, 128, 0, s>>>(reinterpret_cast<const double2*>(w + p.y_off), n, nu, p.M,
@@ -624,12 +639,11 @@ bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V
 }
 
 bem_status expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
-                                 const double* X, int64_t ldx, double* R, bool deriv, void* work,
-                                 cudaStream_t s) {
+                                 const double* X, int64_t ldx, double* R, void* work, cudaStream_t s) {
   char* w = static_cast<char*>(work);
   const int64_t n = ctx->geo.n;
-  bem_status st = cuda_check(ctx, launch_self_at(ctx, m, lam_dev, R, deriv, s), "self terms");
-  if (st == BEM_OK) st = expand_products(ctx, p, m, lam_dev, X, ldx, m, deriv, w, s);
+  bem_status st = cuda_check(ctx, launch_self_at(ctx, m, lam_dev, R, p.deriv, s), "self terms");
+  if (st == BEM_OK) st = expand_products(ctx, p, m, lam_dev, X, ldx, m, w, s);
   if (st != BEM_OK) return st;
   expand_columns_kernel<<<(unsigned)((n * m + 127) / 128), 128, 0, s>>>(
       reinterpret_cast<const double2*>(w + p.y_off), n, m, p.M, p.fams,

@@ -76,6 +76,24 @@ __device__ __forceinline__ void root_and_inverse(double r2, double& r, double& r
   ri = fma(y * er, pe, y);
 }
 
+template <int kKind>
+constexpr int kFamilies = kKind == kDouble ? 2 : 1;
+
+// The families' weights at a point of weight wq, distance r (ri = 1 / r) and dn = (y - x).n, with the
+// factor e^{-ci r} of a complex centre.
+template <int kKind>
+__device__ __forceinline__ void moment_weights(double (&w)[kFamilies<kKind>], double wq, double r, double ri,
+                                               double dn, double ci) {
+  double g = kKind == kSingleDeriv ? wq : wq * ri;
+  if (ci != 0.0) g *= exp(-ci * r);
+  if (kKind == kDouble) {
+    w[0] = g * ri * ri * dn;
+    w[kFamilies<kKind> - 1] = g * ri * dn;
+  } else {
+    w[0] = kKind == kDoubleDeriv ? g * dn : g;
+  }
+}
+
 // acc[f][m] += b_f e^{i phase} T_m(2 rho - 1) in units of 2^-60 of b's scale; b_f and rho as
 // 62-bit fractions.
 template <int MT, int F>

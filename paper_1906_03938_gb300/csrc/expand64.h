@@ -17,7 +17,9 @@ struct FixedPhase {
 struct ExpandPlan {
   bool use = false;        // the expansion applies and costs less than the direct form
   int M = 0;               // series terms
-  int fams = 0, first = 0; // moment families (0: single layer, 1: double layer), the first one
+  bool hasG = false;       // a family for the single layer
+  int nh = 0, fams = 0;    // families for the double layer; all of them
+  bool deriv = false;      // the k-derivative's families
   int S = 0;               // slots, fams M
   int kc = 0;              // columns evaluated at a time
   int splits = 1;          // shares of those columns in the products
@@ -30,20 +32,23 @@ struct ExpandPlan {
   size_t coef_off = 0, mom_off = 0, y_off = 0, batch_off = 0, near_off = 0, bytes = 0;
 };
 
+// Weights of the moments, by their first family.
+enum MomentKind { kSingle, kSingleDeriv, kDouble, kDoubleDeriv };
+
 // Plan for the nk wavenumbers k (re, im on the host), expanded about (c_re, c_im), and ncols columns:
-// every wavenumber times every column (nodes), or wavenumber c times column c.
+// every wavenumber times every column (nodes), or wavenumber c times column c; of A, or (deriv) of A'.
+// arith 1: in the place of double-FP32 products.
 ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, double c_im, int ncols,
-                       bool nodes, bool deriv);
+                       bool nodes, bool deriv, int arith = 0);
 // The workspace can be had: plan's bytes in d_expand. False leaves the caller the direct form.
 bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, cudaStream_t s);
 // Y_j = A(z_j) V for all nodes of the contour (its FP64 self-term table filled), near field
 // included; Y as launch_apply_fp64's. work: plan's bytes.
 bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,
                               int nu, double* Y, void* work, cudaStream_t s);
-// As launch_apply_percol64, near field included.
+// As launch_apply_percol64 (A' for a plan of the derivative), near field included.
 bem_status expand_apply_columns(bem_ctx* ctx, const ExpandPlan& p, int m, const double* lam_dev,
-                                const double* X, int64_t ldx, double* R, bool deriv, void* work,
-                                cudaStream_t s);
+                                const double* X, int64_t ldx, double* R, void* work, cudaStream_t s);
 // Near pairs (near.cu): Y_s += C_s X for every slot, C_s the moments of the corrections
 // (A_near - A_7), in near_expand_bytes of workspace.
 size_t near_expand_bytes(const bem_ctx* ctx, const ExpandPlan& p, int ncols);

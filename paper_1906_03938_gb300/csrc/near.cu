@@ -411,7 +411,7 @@ near_apply64_kernel(Geometry g, const int32_t* __restrict__ ptr, const int32_t* 
 // scale, 2^7 above the largest weight so far, moves up where a larger one comes (the sums
 // shifted down with it). Residuals of 8 vectors on 5120 panels: 23.0 -> 2.6 ms with
 // near_slots64_kernel in FP64 (71 (60 + 3 M) operations a pair), now 1.3 ms.
-template <int MT, bool kG, bool kH>
+template <int MT, int kKind>
 __global__ void __launch_bounds__(128)
 near_moments64_kernel(Geometry g, const int32_t* __restrict__ ptr,
                       const int32_t* __restrict__ cols, int64_t nnz, GL8 gl, double2 c,
@@ -431,11 +431,11 @@ near_moments64_kernel(Geometry g, const int32_t* __restrict__ ptr,
   const int64_t i = lo, l = cols[e];
   const double x[3] = {g.cx[i], g.cx[n + i], g.cx[2 * n + i]};
   double nrm[3] = {0.0, 0.0, 0.0};
-  if (kH)
+  if (kKind >= kDouble)
     for (int d = 0; d < 3; ++d) nrm[d] = g.nrm[d * n + l];
   NearFrame F;
   near_frame(g, l, x, F);
-  constexpr int NF = (kG ? 1 : 0) + (kH ? 1 : 0);
+  constexpr int NF = kFamilies<kKind>;
   long long ar[NF][MT], ai[NF][MT];
   int scale[NF];   // exponents of the families' scales
 #pragma unroll
@@ -461,11 +461,8 @@ near_moments64_kernel(Geometry g, const int32_t* __restrict__ ptr,
     const double dx = y[0] - x[0], dy = y[1] - x[1], dz = y[2] - x[2];
     double r, ri;
     root_and_inverse(dx * dx + dy * dy + dz * dz, r, ri);
-    w *= ri;
-    if (c.y != 0.0) w *= exp(-c.y * r);
     double base[NF];
-    if (kG) base[0] = w;
-    if (kH) base[NF - 1] = w * ri * ri * (dx * nrm[0] + dy * nrm[1] + dz * nrm[2]);
+    moment_weights<kKind>(base, w, r, ri, dx * nrm[0] + dy * nrm[1] + dz * nrm[2], c.y);
     long long b[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
@@ -1168,11 +1165,15 @@ bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const int4* angles, 
   const unsigned blocks = (unsigned)((nnz + 127) / 128);
   auto go = [&](auto mt) {
     constexpr int MT = decltype(mt)::value;
-    auto* k = p.fams == 2 ? near_moments64_kernel<MT, true, true>
-                          : (p.first == 0 ? near_moments64_kernel<MT, true, false>
-                                          : near_moments64_kernel<MT, false, true>);
-    k<<<blocks, 128, 0, s>>>(ctx->geo, ctx->d_near_ptr, ctx->d_near_cols, nnz, gl8(), p.c,
-                             p.phase, angles, p.M, C);
+    auto* single = p.deriv ? near_moments64_kernel<MT, kSingleDeriv> : near_moments64_kernel<MT, kSingle>;
+    auto* dbl = p.deriv ? near_moments64_kernel<MT, kDoubleDeriv> : near_moments64_kernel<MT, kDouble>;
+    if (p.hasG)
+      single<<<blocks, 128, 0, s>>>(ctx->geo, ctx->d_near_ptr, ctx->d_near_cols, nnz, gl8(), p.c, p.phase,
+                                    angles, p.M, C);
+    if (p.nh > 0)
+      dbl<<<blocks, 128, 0, s>>>(ctx->geo, ctx->d_near_ptr, ctx->d_near_cols, nnz, gl8(), p.c, p.phase,
+                                 angles, p.M, C + (p.hasG ? (int64_t)p.M * nnz : 0));
+    ctx->launches += (p.hasG ? 1 : 0) + (p.nh > 0 ? 1 : 0);
   };
   if (p.M <= 1) go(std::integral_constant<int, 1>());
   else if (p.M <= 12) go(std::integral_constant<int, 12>());
@@ -1183,7 +1184,7 @@ bem_status near_expand64(bem_ctx* ctx, const ExpandPlan& p, const int4* angles, 
   else go(std::integral_constant<int, kMaxTerms>());
   near_slots64_kernel<<<(unsigned)((32 * n * (int64_t)p.S + 255) / 256), 256, 0, s>>>(
       ctx->d_near_ptr, ctx->d_near_cols, n, nnz, p.S, C, Xt, ncols, Ys);
-  ctx->launches += 3;
+  ctx->launches += 2;
   return cuda_check(ctx, cudaGetLastError(), "near field kernels");
 }
 

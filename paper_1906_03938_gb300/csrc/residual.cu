@@ -199,17 +199,22 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   // and its workspace can be had
   st = ensure_scratch(ctx, R_dev ? 0 : (size_t)2 * n * m * sizeof(double));
   if (st != BEM_OK) return st;
-  ExpandPlan ex;
+  ExpandPlan ex, exd;   // of A, and of A' if it is asked for
   {
     double lo[2] = {lam_host[0], lam_host[1]}, hi[2] = {lam_host[0], lam_host[1]};
     for (int c = 0; c < 2 * m; ++c) {
       lo[c % 2] = std::min(lo[c % 2], lam_host[c]);
       hi[c % 2] = std::max(hi[c % 2], lam_host[c]);
     }
-    ex = expand_plan(ctx, m, lam_host, 0.5 * (lo[0] + hi[0]), 0.5 * (lo[1] + hi[1]), m, false,
-                     Rd_dev != nullptr);
+    const double cr = 0.5 * (lo[0] + hi[0]), ci = 0.5 * (lo[1] + hi[1]);
+    const int ar = op_single(ctx->op) ? arith : 0;
+    ex = expand_plan(ctx, m, lam_host, cr, ci, m, false, false, ar);
+    if (Rd_dev) {
+      exd = expand_plan(ctx, m, lam_host, cr, ci, m, false, true, ar);
+      ex.use = ex.use && exd.use;
+    }
     if (arith == 1 && op_single(ctx->op) && !expand_beats_ff(ctx, ex, m, Rd_dev != nullptr)) ex.use = false;
-    ex.use = ex.use && expand_ready(ctx, ex, s);
+    ex.use = ex.use && expand_work_ready(ctx, std::max(ex.bytes, exd.bytes), s);
   }
   double* R = R_dev ? R_dev : ctx->d_scratch;
   double* dlam = ctx->d_small;
@@ -221,9 +226,9 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   if (arith == 1 && !ex.use) {
     e = launch_apply_ff(ctx, m, dlam, X_dev, ldx, R, Rd_dev, s);
   } else if (ex.use) {
-    st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, false, ctx->d_expand, s);
+    st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, ctx->d_expand, s);
     if (st == BEM_OK && Rd_dev)
-      st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, Rd_dev, true, ctx->d_expand, s);
+      st = expand_apply_columns(ctx, exd, m, dlam, X_dev, ldx, Rd_dev, ctx->d_expand, s);
     if (st != BEM_OK) return st;
   } else {
     e = launch_apply_percol64(ctx, m, dlam, X_dev, ldx, R, false, s);

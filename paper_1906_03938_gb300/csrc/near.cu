@@ -13,12 +13,13 @@
 //   * Y_j += C(z_j) V for the FP64 projection, the same in FP32 into a slice of the mixed
 //     path's partial products, and R[:, c] += C(lam_c) X[:, c] (values or k-derivatives)
 //     for residuals and refinement.
-// FP64 and residual paths: one warp per (row, node) or (row, column), whose lanes evaluate
-// the row's pair corrections and then sweep the basis columns with them. FP32 path: the
-// values of every (pair, node) first, by the 8 x 8 rule (a thread per pair and 8 nodes) or
-// by the surrogate network on the tensor core (128-sample tiles), then one warp per (row,
-// node) sweeps the basis columns with them. Every sum runs in a fixed order, so the results
-// are deterministic.
+// FP64 projections and residuals take the corrections' moments in the expansion over wavenumbers
+// (expand64.cu; near_moments64_kernel, a thread per pair, and near_slots64_kernel, a warp per row and
+// slot); where that is not taken, one warp per (row, node) or (row, column) evaluates the row's pair
+// corrections and sweeps the basis columns with them. FP32 path: the values of every (pair, node)
+// first, by the 8 x 8 rule (a thread per pair and 8 nodes) or by the surrogate network on the tensor
+// core (128-sample tiles), then a sparse product whose blocks take 8 rows (a warp each) and 2 or 4
+// nodes. Every sum runs in a fixed order, so the results are deterministic.
 #include <cuda_bf16.h>
 #include <math.h>
 

@@ -418,8 +418,9 @@ bem_status bem_set_wait_limit(bem_ctx* ctx, uint32_t polls);
 /*
  * Largest device workspace buffer the context allocates (operational; the paper has no
  * counterpart), for programs that share the device's memory with other allocators. The
- * context keeps its workspaces: FP64 projections and residuals take up to 24 GiB where the
- * expansion over the wavenumbers is the faster form, CholeskyQR2 up to 8 GiB of digit planes,
+ * context keeps its workspaces: FP64 projections and residuals take up to 24 GiB (and the near
+ * pairs' moments) where the expansion over the wavenumbers is the faster form, once more while a
+ * captured call holds that buffer; CholeskyQR2 up to 8 GiB of digit planes,
  * the low-rank far field 4 GiB for a group of nodes, and bem_destroy gives them back. Beyond
  * `bytes` an allocation fails as if the device's memory were short: a call that has a form
  * needing less takes that one, one that has none returns BEM_ENOMEM. What a call finds large

@@ -40,20 +40,50 @@ bem_status ensure_scratch(bem_ctx* ctx, size_t bytes) {
   return BEM_OK;
 }
 
-bool expand_work_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s) {
-  if (bytes <= ctx->expand_bytes) return true;
+ExpandUse::~ExpandUse() {
+  if (work && !captured) cudaEventRecord(ctx->expand_ev, s);
+}
+
+bool ExpandUse::get(size_t bytes) {
+  work = nullptr;
+  if (bytes == 0) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  cudaFree(ctx->d_expand);
-  ctx->expand_bytes = 0;
-  if (workspace_malloc(ctx, &ctx->d_expand, bytes) != cudaSuccess) {
+  captured = cap != cudaStreamCaptureStatusNone;
+  if (captured) {
+    if (bytes > ctx->captured_bytes) {
+      if (bytes > ctx->expand_bytes) return false;
+      ctx->captured.push_back(ctx->d_expand);
+      ctx->captured_bytes = ctx->expand_bytes;
+      ctx->captured_total += ctx->expand_bytes;
+      ctx->d_expand = nullptr;
+      ctx->expand_bytes = 0;
+    }
+    work = ctx->captured.back();
+    return true;
+  }
+  if (bytes > ctx->expand_bytes) {
+    cudaFree(ctx->d_expand);
+    ctx->expand_bytes = 0;
+    if (workspace_malloc(ctx, &ctx->d_expand, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    ctx->expand_bytes = bytes;
+  }
+  if (!ctx->expand_ev && cudaEventCreateWithFlags(&ctx->expand_ev, cudaEventDisableTiming) != cudaSuccess) {
+    ctx->expand_ev = nullptr;
     cudaGetLastError();
     return false;
   }
-  ctx->expand_bytes = bytes;
+  if (cudaStreamWaitEvent(s, ctx->expand_ev, 0) != cudaSuccess) {   // (not recorded yet: no wait)
+    cudaGetLastError();
+    return false;
+  }
+  work = ctx->d_expand;
   return true;
 }
 
@@ -242,6 +272,8 @@ void bem_destroy(bem_ctx* ctx) {
   cudaFree(ctx->d_ff);
   cudaFree(ctx->d_split);
   cudaFree(ctx->d_expand);
+  for (void* p : ctx->captured) cudaFree(p);
+  if (ctx->expand_ev) cudaEventDestroy(ctx->expand_ev);
   cudaFree(ctx->d_zgemm);
   release_cublas(ctx);
   cudaFree(ctx->d_solve);
@@ -532,19 +564,21 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
   st0 = ensure_scratch(ctx, y_bytes);
   if (st0 != BEM_OK) return st0;
   // One evaluation expanded over the nodes where that costs less than one per node, and V^H Y_j on
-  // the tensor core, where their workspace (the one after the other in the same buffer) can be had.
-  // A growth that fails gives up what there was, so the forms are settled by the buffer's size
-  // after the last one.
+  // the tensor core, where their workspace (the one after the other in the same buffer) can be had;
+  // where only the smaller one's can, that form alone.
   ExpandPlan ex = expand_plan(ctx, N, ctx->con.z_host, ctx->con.c_re, ctx->con.c_im, nu, true, false);
   SplitCross xs = split64_cross_plan(ctx, n, nu, nu, N);
-  ex.use = expand_ready(ctx, ex, s);
-  xs.use = xs.use && expand_work_ready(ctx, xs.bytes, s);
-  ex.use = ex.use && expand_ready(ctx, ex, s);
-  xs.use = xs.use && ctx->expand_bytes >= xs.bytes;
+  const size_t eb = ex.use ? ex.bytes : 0, xb = xs.use ? xs.bytes : 0;
+  ExpandUse ws(ctx, s);
+  if (!ws.get(std::max(eb, xb))) {
+    const size_t rest = ws.get(std::min(eb, xb)) ? std::min(eb, xb) : 0;
+    ex.use = eb > 0 && eb <= rest;
+    xs.use = xb > 0 && xb <= rest;
+  }
   double* Y = AV_dev ? AV_dev : ctx->d_scratch;
   timing_begin(ctx, s);
   bem_status st =
-      ex.use ? expand_apply_nodes(ctx, ex, V_dev, ldv, nu, Y, ctx->d_expand, s)
+      ex.use ? expand_apply_nodes(ctx, ex, V_dev, ldv, nu, Y, ws.work, s)
              : cuda_check(ctx, launch_apply_fp64(ctx, V_dev, ldv, nu, Y, s), "apply kernel");
   timing_end(ctx, s);
   if (st != BEM_OK) return st;
@@ -553,7 +587,7 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
     if (st != BEM_OK) return st;
   }
   if (xs.use)
-    return split64_cross(ctx, xs, ctx->d_expand, reinterpret_cast<const double2*>(V_dev), ldv,
+    return split64_cross(ctx, xs, ws.work, reinterpret_cast<const double2*>(V_dev), ldv,
                          reinterpret_cast<const double2*>(Y), reinterpret_cast<const double2*>(ctx->con.w),
                          reinterpret_cast<double2*>(Bhat_dev), s);
   return cuda_check(ctx, launch_xhy_fp64(ctx, V_dev, ldv, nu, Y, n, n * nu, nu, n, N, ctx->con.w,

@@ -561,10 +561,6 @@ ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, doubl
   return p;
 }
 
-bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, cudaStream_t s) {
-  return p.use && expand_work_ready(ctx, p.bytes, s);
-}
-
 namespace {
 
 // The slot products Y_s = G_s X into the workspace, near-field corrections included.

@@ -40,8 +40,6 @@ enum MomentKind { kSingle, kSingleDeriv, kDouble, kDoubleDeriv };
 // arith 1: in the place of double-FP32 products.
 ExpandPlan expand_plan(bem_ctx* ctx, int nk, const double* k, double c_re, double c_im, int ncols,
                        bool nodes, bool deriv, int arith = 0);
-// The workspace can be had: plan's bytes in d_expand. False leaves the caller the direct form.
-bool expand_ready(bem_ctx* ctx, const ExpandPlan& p, cudaStream_t s);
 // Y_j = A(z_j) V for all nodes of the contour (its FP64 self-term table filled), near field
 // included; Y as launch_apply_fp64's. work: plan's bytes.
 bem_status expand_apply_nodes(bem_ctx* ctx, const ExpandPlan& p, const double* V, int64_t ldv,

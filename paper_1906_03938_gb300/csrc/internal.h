@@ -111,9 +111,13 @@ struct bem_ctx {
   void* d_split = nullptr;       // digit planes of the split FP64 products (split64.cu)
   size_t split_bytes = 0;
   // workspace of the FP64 forms that a smaller one replaces (expand64.cu, split64.cu): apart from
-  // d_scratch, which such a call need not touch
+  // d_scratch, which such a call need not touch; calls on several streams use it in turn, the event
+  // marks the last use. Buffers that captured calls hold (the last one, of captured_bytes, for
+  // captures to come) are theirs alone until bem_destroy.
   void* d_expand = nullptr;
-  size_t expand_bytes = 0;
+  size_t expand_bytes = 0, captured_bytes = 0, captured_total = 0;
+  cudaEvent_t expand_ev = nullptr;
+  std::vector<void*> captured;
   double* d_ff = nullptr;        // column splits' partial sums of the double-FP32 residuals
   size_t ff_bytes = 0;
   size_t small_bytes = 0;
@@ -193,9 +197,21 @@ cudaError_t workspace_malloc(const bem_ctx* ctx, T** p, size_t bytes) {
 }
 // Make sure the context's scratch holds at least `bytes`.
 bem_status ensure_scratch(bem_ctx* ctx, size_t bytes);
-// Make sure d_expand holds at least `bytes`; false if that cannot be had (no memory: then there is
-// no buffer; or the stream is being captured and the buffer would have to grow: then it stays).
-bool expand_work_ready(bem_ctx* ctx, size_t bytes, cudaStream_t s);
+// A call's use of the context's d_expand on stream s, until the object's end.
+//  get: `bytes` in work, behind the last use by any stream; false, and no buffer, if that cannot be
+//  had. A stream that is being captured gets a buffer that no other call uses or frees afterwards:
+//  the captures' last one, or the present one, which then is theirs (nothing is allocated).
+struct ExpandUse {
+  ExpandUse(bem_ctx* c, cudaStream_t st) : ctx(c), s(st) {}
+  ~ExpandUse();
+  ExpandUse(const ExpandUse&) = delete;
+  ExpandUse& operator=(const ExpandUse&) = delete;
+  bool get(size_t bytes);
+  bem_ctx* ctx;
+  cudaStream_t s;
+  void* work = nullptr;
+  bool captured = false;
+};
 bem_status ensure_small(bem_ctx* ctx, size_t bytes);
 void release_cublas(bem_ctx* ctx);
 // nodes z and weights w (2 N doubles each, interleaved) of a contour, on the host

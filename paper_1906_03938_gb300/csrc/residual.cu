@@ -199,6 +199,7 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   // and its workspace can be had
   st = ensure_scratch(ctx, R_dev ? 0 : (size_t)2 * n * m * sizeof(double));
   if (st != BEM_OK) return st;
+  ExpandUse ws(ctx, s);
   ExpandPlan ex, exd;   // of A, and of A' if it is asked for
   {
     double lo[2] = {lam_host[0], lam_host[1]}, hi[2] = {lam_host[0], lam_host[1]};
@@ -214,7 +215,7 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
       ex.use = ex.use && exd.use;
     }
     if (arith == 1 && op_single(ctx->op) && !expand_beats_ff(ctx, ex, m, Rd_dev != nullptr)) ex.use = false;
-    ex.use = ex.use && expand_work_ready(ctx, std::max(ex.bytes, exd.bytes), s);
+    ex.use = ex.use && ws.get(std::max(ex.bytes, exd.bytes));
   }
   double* R = R_dev ? R_dev : ctx->d_scratch;
   double* dlam = ctx->d_small;
@@ -226,9 +227,9 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   if (arith == 1 && !ex.use) {
     e = launch_apply_ff(ctx, m, dlam, X_dev, ldx, R, Rd_dev, s);
   } else if (ex.use) {
-    st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, ctx->d_expand, s);
+    st = expand_apply_columns(ctx, ex, m, dlam, X_dev, ldx, R, ws.work, s);
     if (st == BEM_OK && Rd_dev)
-      st = expand_apply_columns(ctx, exd, m, dlam, X_dev, ldx, Rd_dev, ctx->d_expand, s);
+      st = expand_apply_columns(ctx, exd, m, dlam, X_dev, ldx, Rd_dev, ws.work, s);
     if (st != BEM_OK) return st;
   } else {
     e = launch_apply_percol64(ctx, m, dlam, X_dev, ldx, R, false, s);

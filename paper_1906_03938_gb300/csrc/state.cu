@@ -48,7 +48,7 @@ bem_status bem_stats(const bem_ctx* ctx, bem_stats_t* out) {
   out->near_pairs = near_active(ctx) ? ctx->near_nnz : -1;
   out->launches = ctx->launches;
   out->workspace_bytes = (int64_t)(ctx->scratch_bytes + ctx->small_bytes + ctx->solve_bytes +
-                                   ctx->near_work_bytes + ctx->expand_bytes);
+                                   ctx->near_work_bytes + ctx->expand_bytes + ctx->captured_total);
   out->surrogate_ready = ctx->net_ready ? 1 : 0;
   return BEM_OK;
 }

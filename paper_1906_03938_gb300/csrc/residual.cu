@@ -240,15 +240,16 @@ bem_status residual_impl(bem_ctx* ctx, int m, const double* lam_host, const doub
   st = cuda_check(ctx, launch_colnorms(ctx, R, n, X_dev, ldx, n, m, dnorm, s), name);
   if (st != BEM_OK) return st;
   std::vector<double> h(2 * m);
+  const bool waits = ex.use && (ex.split || exd.split);
   int flags = 0;
   st = cuda_check(ctx, cudaMemcpyAsync(h.data(), dnorm, 2 * m * sizeof(double),
                                        cudaMemcpyDeviceToHost, s), name);
-  if (st == BEM_OK)
+  if (st == BEM_OK && waits)
     st = cuda_check(ctx, cudaMemcpyAsync(&flags, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, s), name);
   if (st == BEM_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), name);
   if (st != BEM_OK) return st;
-  // the split products' waits are bounded: norms of products that gave up are no result (what
-  // other calls recorded is left to bem_check, as ever)
+  // the split products' waits are bounded: norms of products that gave up are no result. (What other
+  // calls recorded is left to bem_check, as ever, where this one has no such wait.)
   if (flags & kStatusTimeout) return take_status(ctx, s, name);
   for (int c = 0; c < m; ++c)
     relres_host[c] = h[2 * c + 1] > 0.0 ? sqrt(h[2 * c]) / sqrt(h[2 * c + 1]) : INFINITY;

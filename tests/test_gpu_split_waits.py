@@ -86,3 +86,25 @@ def test_residual(polls, deriv):
     ctx.set_wait_limit(1 << 24)
     assert np.array_equal(ctx.residual_arith(lam, X, arith=0, deriv=deriv)[0], ref)
     ctx.close()
+
+
+@pytest.mark.parametrize("m, arith", [(1, 1), (1, 0)])
+def test_residual_without_waits_leaves_other_calls_timeouts(m, arith):
+    """108 panels and one vector: no split products. The timeout that a projection
+    recorded is the check's to report, not the residual's."""
+    import paper_1906_03938_gb300 as bem
+    mesh = synth.cube_sphere(3, (1.0, 0.8, 0.55))
+    X = bem.fortran(torch.from_numpy(synth.complex_gaussian(mesh.n, 16, 6)).to("cuda:0"))
+    ctx = bem.Context(0)
+    ctx.set_mesh(mesh.xyz, mesh.tri)
+    ctx.set_contour("circle", 5.0, 0.8, 0.8, N)
+    ref = ctx.residual_arith([5.0], X[:, :m], arith=arith)[0]
+    ctx.set_wait_limit(0)
+    ctx.project(X, bem.PREC_MIXED)
+    ctx.set_wait_limit(1 << 24)
+    assert np.array_equal(ctx.residual_arith([5.0], X[:, :m], arith=arith)[0], ref)
+    with pytest.raises(bem.BemError) as e:
+        ctx.check()
+    assert e.value.status == bem.STATUS_CODES["BEM_ETIMEOUT"]
+    ctx.check()
+    ctx.close()

@@ -70,6 +70,11 @@ __device__ __forceinline__ void fixed_sincos(unsigned long long phi, const int4*
 // 2^-53.
 __device__ __forceinline__ void root_and_inverse(double r2, double& r, double& ri) {
   const float rf = (float)r2;
+  if (rf < 1e-30f && r2 == 0.0) {   // coinciding points: k-derivatives have a value there
+    r = 0.0;
+    ri = INFINITY;
+    return;
+  }
   const double y = rf > 1e-30f && rf < 1e30f ? (double)rsqrtf(rf) : rsqrt(r2);
   const double t = r2 * y, er = fma(-t, y, 1.0), pe = fma(0.375, er, 0.5);
   r = fma(t * er, pe, t);

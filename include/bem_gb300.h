@@ -188,7 +188,8 @@ bem_status bem_project(bem_ctx* ctx, const double* V_dev, int64_t ldv, int nu,
  * projection, Section 4, Example 1): G = V^H V, R1 = chol(G), V <- V R1^{-1}, repeated
  * once; on return V (n x nu, column-major, leading dimension ldv) has orthonormal
  * columns and, if R_dev is not NULL, R_dev (nu x nu, column-major) holds R = R2 R1 with
- * V_in = V_out R. The second pass is FP64 throughout and sets the final orthogonality;
+ * V_in = V_out R. The last pass is FP64 throughout and sets the final orthogonality (the second
+ * one, or a third where the second finds V far from orthonormal yet);
  * when R_dev is NULL the first pass (whose only job is to make V well conditioned) runs its
  * Cholesky factor and triangular inverse (and the smaller Gram matrices) in FP32 and applies
  * the inverse to V in FP64. From n nu^2 = 2^23 the FP64 products are exact sums of BF16 digit

@@ -270,7 +270,6 @@ void bem_destroy(bem_ctx* ctx) {
   cudaFree(ctx->d_piv_idx);
   cudaFree(ctx->d_lu_work);
   cudaFree(ctx->d_ff);
-  cudaFree(ctx->d_split);
   cudaFree(ctx->d_expand);
   for (void* p : ctx->captured) cudaFree(p);
   if (ctx->expand_ev) cudaEventDestroy(ctx->expand_ev);

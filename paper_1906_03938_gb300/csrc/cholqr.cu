@@ -1235,12 +1235,14 @@ CqLayout cq_layout(bem_ctx* ctx, int64_t n, int nu) {
   // slowest SM: 3000 x 33 with R 690 us, now 591)
   const int64_t blocks = (nu <= kSmallNu ? 1 : 2) * (int64_t)std::max(1, sms);
   L.parts = nu <= kSmallNu ? blocks / L.tiles_u : (blocks + L.tiles_u - 1) / L.tiles_u;
+  // room for the parts of any n: the workspace a call finds does not grow (and move) with n, so that
+  // what a captured call holds is there after calls on longer bases
+  L.parts_max = std::max<int64_t>(std::max<int64_t>(1, L.parts), split64_parts(ctx, INT64_MAX / 2, nu));
   L.parts = std::max<int64_t>(1, std::min<int64_t>((n + 3) / 4, L.parts));
   L.rows_per_part = (n + L.parts - 1) / L.parts;
   L.parts = (n + L.rows_per_part - 1) / L.rows_per_part;
   L.rows32 = std::max<int64_t>(L.rows_per_part, kGT);
   L.parts32 = (n + L.rows32 - 1) / L.rows32;
-  L.parts_max = std::max<int64_t>(L.parts, split64_parts(ctx, n, nu));
   L.sum_blocks = (unsigned)((8 * (int64_t)nu * nu + 255) / 256);
   return L;
 }
@@ -1447,7 +1449,7 @@ size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu) {
 // (400 x 200, condition 100: 2.9e-15 against 1.1e-15) nor fast; the second pass takes another FP32
 // factor instead and the third one finishes. Columns of up to kChol32 keep the classic second pass.
 bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int nu,
-                        double* R_dev, void* work, cudaStream_t s, uint64_t refresh_seed, void* split_mem) {
+                        double* R_dev, void* work, cudaStream_t s, uint64_t refresh_seed) {
   const CqLayout L = cq_layout(ctx, n, nu);
   const CqWork w = cq_work(work, nu, L);
   bem_status st = BEM_OK;
@@ -1458,8 +1460,12 @@ bem_status cholqr2_impl(bem_ctx* ctx, double* V_dev, int64_t n, int64_t ldv, int
   if ((st = set_smem(ctx, (const void*)right_multiply_near_df_kernel,
                      right_multiply_df_smem(nu))) != BEM_OK)
     return st;
+  // the split products' planes, given up if they cannot be had: apart from the factors' workspace,
+  // whose size does not depend on n
   Split64 sp;
-  split64_plan(ctx, ldv, n, nu, split_mem, sp, s);
+  const size_t split = split64_bytes(ctx, n, nu);
+  ExpandUse planes(ctx, s);
+  if (split > 0 && planes.get(split)) split64_plan(ctx, ldv, n, nu, planes.work, sp);
   if (R_dev) {
     if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R1, refresh_seed, s)) != BEM_OK) return st;
     if ((st = classic_pass(ctx, V_dev, ldv, n, nu, L, w, sp, w.R2, 0, s)) != BEM_OK) return st;
@@ -1514,18 +1520,9 @@ extern "C" bem_status bem_cholqr2(bem_ctx* ctx, double* V_dev, int64_t n, int64_
     return fail(ctx, BEM_EINVAL, "bem_cholqr2: need V, 1 <= nu <= min(n, 256), ldv >= n");
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
-  // one workspace for the factors and the split products' planes, the latter given up if it
-  // cannot be had
-  const size_t work = (cholqr2_work_bytes(ctx, n, nu) + 1023) / 1024 * 1024, split = split64_bytes(ctx, n, nu);
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (split > 0 && work + split > ctx->small_bytes) {
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
-    else if (cap == cudaStreamCaptureStatusNone) ensure_small(ctx, work + split);
-  }
-  bem_status st = ensure_small(ctx, work);
+  bem_status st = ensure_small(ctx, cholqr2_work_bytes(ctx, n, nu));
   if (st != BEM_OK) return st;
-  void* planes = split > 0 && work + split <= ctx->small_bytes ? reinterpret_cast<char*>(ctx->d_small) + work : nullptr;
-  st = cholqr2_impl(ctx, V_dev, n, ldv, nu, R_dev, ctx->d_small, s, 0, planes);
+  st = cholqr2_impl(ctx, V_dev, n, ldv, nu, R_dev, ctx->d_small, s, 0);
   if (st != BEM_OK) return st;
   if (ctx->async) return cuda_check(ctx, cudaGetLastError(), "bem_cholqr2");
   return take_status(ctx, s, "bem_cholqr2");

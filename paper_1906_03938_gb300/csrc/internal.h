@@ -108,10 +108,8 @@ struct bem_ctx {
   size_t zgemm_bytes = 0;
   float* d_lu_work = nullptr;    // the LU's trailing-update operands in real form
   size_t lu_work_bytes = 0;
-  void* d_split = nullptr;       // digit planes of the split FP64 products (split64.cu)
-  size_t split_bytes = 0;
-  // workspace of the FP64 forms that a smaller one replaces (expand64.cu, split64.cu): apart from
-  // d_scratch, which such a call need not touch; calls on several streams use it in turn, the event
+  // workspace of the FP64 forms that need more than others (expand64.cu, split64.cu): apart from
+  // d_scratch and d_small, which such a call need not touch; calls on several streams use it in turn, the event
   // marks the last use. Buffers that captured calls hold (the last one, of captured_bytes, for
   // captures to come) are theirs alone until bem_destroy.
   void* d_expand = nullptr;
@@ -271,10 +269,10 @@ cudaError_t launch_xhy_fp64(bem_ctx* ctx, const double* X, int64_t ldx, int p, c
 // CholeskyQR2 with caller-provided work space (asynchronous; status word on failure).
 // refresh_seed != 0: columns whose first-pass pivot collapses (rank deficiency) are
 // replaced by pseudo-random columns before the second pass instead of failing; R is then
-// not a factor of the input. split_mem: split64_bytes of workspace (null: the context's own).
+// not a factor of the input.
 size_t cholqr2_work_bytes(bem_ctx* ctx, int64_t n, int nu);
 bem_status cholqr2_impl(bem_ctx* ctx, double* V, int64_t n, int64_t ldv, int nu, double* R,
-                        void* work, cudaStream_t s, uint64_t refresh_seed, void* split_mem = nullptr);
+                        void* work, cudaStream_t s, uint64_t refresh_seed);
 // Near field (near.cu). near_active: a mode is set and the pair list is current (build it
 // with ensure_near first).
 bem_status ensure_near(bem_ctx* ctx, cudaStream_t s);

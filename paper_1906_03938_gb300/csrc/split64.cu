@@ -666,8 +666,7 @@ SplitSizes split_sizes(const bem_ctx* ctx, int64_t n, int nu) {
 
 size_t split64_bytes(const bem_ctx* ctx, int64_t n, int nu) { return split_sizes(ctx, n, nu).total; }
 
-void split64_plan(bem_ctx* ctx, int64_t ldv, int64_t n, int nu, void* mem, Split64& sp,
-                  cudaStream_t s) {
+void split64_plan(bem_ctx* ctx, int64_t ldv, int64_t n, int nu, void* mem, Split64& sp) {
   sp = Split64();
   const SplitSizes z = split_sizes(ctx, n, nu);
   if (z.total == 0) return;
@@ -680,22 +679,7 @@ void split64_plan(bem_ctx* ctx, int64_t ldv, int64_t n, int nu, void* mem, Split
   sp.ntu = (nu + kTileN - 1) / kTileN;
   sp.mtn = (n + kTileM - 1) / kTileM;
   sp.parts = split64_parts(ctx, n, nu);
-  if (!mem && z.total > ctx->split_bytes) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-      cudaGetLastError();
-      return;
-    }
-    cudaFree(ctx->d_split);
-    ctx->d_split = nullptr;
-    ctx->split_bytes = 0;
-    if (workspace_malloc(ctx, &ctx->d_split, z.total) != cudaSuccess) {
-      cudaGetLastError();
-      return;
-    }
-    ctx->split_bytes = z.total;
-  }
-  unsigned char* base = static_cast<unsigned char*>(mem ? mem : ctx->d_split);
+  unsigned char* base = static_cast<unsigned char*>(mem);
   sp.a = base;
   sp.b = base + z.a;
   sp.hcol = reinterpret_cast<unsigned*>(base + z.a + z.b);

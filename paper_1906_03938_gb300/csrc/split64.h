@@ -21,11 +21,9 @@ struct Split64 {
 
 // Workspace of the split products of an n x nu basis (0: the FP64 kernels are the better choice).
 size_t split64_bytes(const bem_ctx* ctx, int64_t n, int nu);
-// Fills sp for an n x nu basis of leading dimension ldv, in mem (split64_bytes) or, if that is
-// null, in memory of the context's; use is false where the FP64 kernels are the better choice or
-// the workspace cannot be had.
-void split64_plan(bem_ctx* ctx, int64_t ldv, int64_t n, int nu, void* mem, Split64& sp,
-                  cudaStream_t s);
+// Fills sp for an n x nu basis of leading dimension ldv, in mem (split64_bytes); use is false where the
+// FP64 kernels are the better choice.
+void split64_plan(bem_ctx* ctx, int64_t ldv, int64_t n, int nu, void* mem, Split64& sp);
 // Row ranges of the Gram matrix of an n x nu basis (partial sums to provide for).
 int split64_parts(const bem_ctx* ctx, int64_t n, int nu);
 // part[r][b nu + a] = sum over row range r of conj(V[i][a]) V[i][b] for the upper 32 x 32 tiles

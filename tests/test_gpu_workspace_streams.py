@@ -53,6 +53,33 @@ def test_captured_projection_outlives_larger_workspaces(near, av):
     ctx.close()
 
 
+def test_captured_cholqr2_outlives_larger_workspaces():
+    """Split products at both sizes (n nu^2 > 2^23). The room for partial Gram matrices is that of the
+    longest basis whatever n."""
+    bem, ctx, _ = _context()
+    ctx.set_async(True)
+    V = _basis(bem, 3072, 64, 1)
+    Q = V.clone()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        ctx.cholqr2(Q, want_R=False)
+        s.synchronize()
+        expected = Q.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            ctx.cholqr2(Q, want_R=False)
+    for _ in range(2):
+        big = _basis(bem, 32768, 64, 2)
+        ctx.cholqr2(big, want_R=False)
+        Q.copy_(V)
+        graph.replay()
+        torch.cuda.synchronize()
+        ctx.check()
+        assert torch.equal(Q, expected)
+    ctx.close()
+
+
 def test_calls_on_two_streams():
     bem, ctx, n = _context()
     Vs = [_basis(bem, n, nu, 3 + nu) for nu in (48, 64)]
